@@ -92,7 +92,7 @@ int ch_hull(const float* pts, int64_t n, int32_t* out_idx, int64_t* out_n, void*
  *   host_offsets  optional HOST copy of offsets (NULL allowed): lets the
  *            library size its launches without reading the device array.
  * Each result equals ch_hull on that set alone.  The batch's points are
- * streamed as one array (extremes, then filter); dense sets of at least 32768
+ * streamed as one array (extremes, then filter); dense sets of at least 16384
  * points are filtered by a star polygon of their own points (Table V's
  * worst case); see ch_batched_counters.
  * Shape of the streamed per-point kernels (threads per block x points per
@@ -117,11 +117,11 @@ int ch_hull_batched(const float* pts, const int64_t* offsets, int32_t k,
  *   out[4 i]      records handed to the hull stage (the filter's survivors,
  *                 the chain end points included),
  *   out[4 i + 1]  vertices of the star polygon that filtered the set (0 when
- *                 none: a sparse set, a set under 32768 points, or a polygon
+ *                 none: a sparse set, a set under 16384 points, or a polygon
  *                 that failed its checks),
  *   out[4 i + 2]  the set's status (CH_OK or a negative ch_status),
- *   out[4 i + 3]  hull stage: 0 one block, 1 the bucketed path, 2 the
- *                 single-hull path.
+ *   out[4 i + 3]  hull stage: 0 one block, 1 chain by chain (a block per
+ *                 queue, or the bucketed path), 2 the single-hull path.
  * k must equal that call's k; out holds 4 k values.  Returns 4 (values per
  * set).  Synchronises the stream.  CH_EINVAL when no batched call of k sets
  * ran on that stream (or out is NULL).

@@ -21,15 +21,18 @@
 //                end points reduced;
 //   bt_hull_small  one block per set: the support-line records, then the
 //                hull of a set with few records in a small footprint;
-//   bt_star_refine  sets with more records than one block holds: a second
+//   bt_star_refine  sets with a queue that one block cannot hold: a second
 //                polygon from the set's records drops those strictly inside;
-//   bt_hull      persistent over the remaining sets: the hull of a set's
+//   bt_hull      persistent over the larger sparse sets: the hull of a set's
 //                records in one block (quickhull rounds and the stitch, as in
-//                the single hull's last block).
-// Sets whose records exceed what one block holds (or are many and near the
-// hull) go through the bucketed large-survivor path together
-// (batched_large.cu); the rare set it cannot finish (a bucket chain longer
-// than kBkChain) is flagged and the host runs the single-hull path on it.
+//                the single hull's last block);
+//   bt_queue_chain  persistent over the queues of the other sets: a queue's
+//                lower chain by one block (qchain.cuh), the set's chains
+//                joined by the block that finishes the fourth.
+// Sets with a queue that no block holds go through the bucketed
+// large-survivor path together (batched_large.cu); the rare set it cannot
+// finish (a bucket chain longer than kBkChain) is flagged and the host runs
+// the single-hull path on it.
 // Each result equals ch_hull on the set alone (local indices).  The device
 // work of one call is captured into a CUDA graph on a private stream; the
 // executable graph of a (device, stream) is updated in place from call to
@@ -41,6 +44,7 @@
 #include "hullcore.cuh"
 #include "launch.h"
 #include "octagon.cuh"
+#include "qchain.cuh"
 #include "records.cuh"
 #include "star.cuh"
 #include "tma.cuh"
@@ -60,10 +64,11 @@ constexpr int kBWarpTileMin = 256;     // points of the smallest warp tile of th
 constexpr int kBOctThreads = 256;      // threads of bt_octagon: a warp per direction
 
 // Star polygon of dense sets (star.cuh): a set of at least kBStarMinPts
-// points has a slot of angular bins and a polygon.  The bins are taken
+// points has a slot of angular bins and a polygon (a smaller set's queues fit
+// bt_queue_chain as they are).  The bins are taken
 // around the centre of the box of the set's extremes, over a sample of
 // kBStarParts evenly spread runs of the set (up to kBStarRun points each).
-constexpr long long kBStarMinPts = 32768;
+constexpr long long kBStarMinPts = 16384;
 constexpr int kBStarParts = 16;
 constexpr int kBStarRun = 16384;
 constexpr int kBDenseSample = 2048;   // points of a set's density test
@@ -89,11 +94,13 @@ struct BArgs {
     StarPoly* star_polys;     // one per slot
     unsigned* star_ctr;       // work lists: [0] dense sets listed, [1] taken by bt_star_build;
                               // [2] / [3] sets for bt_star_refine from the front / back, [4] taken;
-                              // [5] sets for bt_hull, [6] taken; [7] bt_dense's units, [8] taken
+                              // [5] sets for bt_hull, [6] taken; [7] bt_dense's units, [8] taken;
+                              // [9] / [10] sets for bt_queue_chain from the front / back, [11] / [12] queues taken
     int* star_list;           // k entries
     unsigned* unit_base;      // k entries: first bt_dense unit of each listed set
     int* refine_list;         // k entries
     int* hull_list;           // k entries
+    int* q_list;              // k entries: sets for bt_queue_chain, the small ones from the front, the large from the back
     uint32_t* kP;             // the bucketed path's scatter buffer (set regions as keys / vals)
     uint64_t* vP;
 };
@@ -1036,8 +1043,8 @@ __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Second star polygon of a set whose records one block still cannot hold
-// (bt_hull_small's list): its records are the points outside the first
+// Second star polygon of a set with a queue that one block still cannot hold
+// (bt_list_queues' list): its records are the points outside the first
 // polygon (or, for a sparse set, outside the octagon), so binning all of
 // them puts a rim point in nearly every bin.  One block per set, persistent
 // over the list (the sets with more than kBRefineHuge records first):
@@ -1209,14 +1216,36 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_refine(BArgs a) {
 
 // One block per set, in two kernels.  bt_hull_small (every set): the
 // support-line records, then the hull of a set of at most kBSmallRec records
-// in a small shared-memory footprint (several blocks per SM).  bt_hull (the
-// other sets): the hull when one block can hold the records, else the set is
-// flagged for the bucketed path.  A small set whose quickhull rounds exceed
-// their vertex capacity is flagged the same way.
+// in a small shared-memory footprint (several blocks per SM).  bt_hull: the
+// sparse sets with more records than that, while one block can hold them.
+// The other sets, and a small set whose quickhull rounds exceed their vertex
+// capacity, go queue by queue through bt_queue_chain.
 constexpr int kBSmallRec = 2048;        // records of a small set
 constexpr int kBSmallVert = 256;        // quickhull vertices of a small set
 constexpr int kBSmallThreads = 256;
+constexpr int kBDenseRec = 256;         // records of a dense set that the quickhull rounds take at most
 using QhSmall = QhSmemT<kBSmallRec, kBSmallVert>;
+
+// bt_queue_chain's two shapes: a queue of at most kBQSmall records by 256
+// threads in 57 KB of shared memory (four blocks per SM), of at most kBQLarge
+// by 1024 threads in 221 KB.
+constexpr int kBQSmall = 2560, kBQLarge = 10240;
+using QcSmall = QcSmem<kBQSmall, 1024>;
+using QcLarge = QcSmem<kBQLarge, 4096>;
+static_assert(sizeof(QcLarge) <= 225 * 1024, "one block's shared memory");
+
+// One thread: lists set i (total records) for bt_queue_chain, and first for
+// bt_star_refine when a queue has more records than the large shape holds.
+__device__ __forceinline__ void bt_list_queues(const BArgs& a, int i, unsigned total) {
+    unsigned most = 0u;
+    for (int q = 0; q < 4; ++q) most = max(most, *(volatile unsigned*)&a.ctl[i].counts4[q]);
+    if (most <= (unsigned)kBQSmall) a.q_list[atomicAdd(&a.star_ctr[9], 1u)] = i;
+    else a.q_list[a.k - 1 - (int)atomicAdd(&a.star_ctr[10], 1u)] = i;
+    if (most > (unsigned)kBQLarge) {
+        if (total > kBRefineHuge) a.refine_list[atomicAdd(&a.star_ctr[2], 1u)] = i;
+        else a.refine_list[a.k - 1 - (int)atomicAdd(&a.star_ctr[3], 1u)] = i;
+    }
+}
 
 __global__ void __launch_bounds__(kBSmallThreads) bt_hull_small(BArgs a) {
     __shared__ QhSmall q;
@@ -1263,13 +1292,15 @@ __global__ void __launch_bounds__(kBSmallThreads) bt_hull_small(BArgs a) {
         a.vals[rb + s_lpos[tid]] = s_lval[tid];
         atomicAdd(&c->counts4[s_lkey[tid] >> kKeyBits], 1u);
     }
-    if (total > (unsigned)kBSmallRec) {   // bt_hull's, after bt_star_refine's when one block cannot hold them
+    // Records near the hull (a star polygon left them, or more than a quarter
+    // of the points survived the octagon) are mostly vertices, and past a few
+    // hundred they outgrow the quickhull rounds: queue by queue then.
+    const bool dense = c->star_k > 0 || 4ll * total > ni;
+    if (total > (unsigned)kBSmallRec || (dense && total > (unsigned)kBDenseRec)) {
+        __syncthreads();   // the queue counts are complete
         if (tid == 0) {
-            a.hull_list[atomicAdd(&a.star_ctr[5], 1u)] = i;
-            if (total > (unsigned)kMidCap) {
-                if (total > kBRefineHuge) a.refine_list[atomicAdd(&a.star_ctr[2], 1u)] = i;
-                else a.refine_list[a.k - 1 - (int)atomicAdd(&a.star_ctr[3], 1u)] = i;
-            }
+            if (!dense && total <= (unsigned)kMidCap) a.hull_list[atomicAdd(&a.star_ctr[5], 1u)] = i;
+            else bt_list_queues(a, i, total);
         }
         return;
     }
@@ -1287,13 +1318,11 @@ __global__ void __launch_bounds__(kBSmallThreads) bt_hull_small(BArgs a) {
         stitch_cycle(q.ru, q.rv, q.ri, s_mv, q.rs, c, ni, a.out_idx + base, a.out_n + i);
         if (tid == 0) c->done = 1;
     } else if (tid == 0) {
-        a.big[i] = 1;   // too many chain vertices for the small footprint: the bucketed path
-        c->done = 1;
+        bt_list_queues(a, i, total);   // too many chain vertices for the small footprint
     }
 }
 
 constexpr size_t bt_cmax(size_t x, size_t y) { return x > y ? x : y; }
-constexpr int kBQhSkip = 2048;
 constexpr size_t kBHullSmem = bt_cmax(kMidSmemBytes, sizeof(QhSmem));
 
 // Persistent over bt_hull_small's list of the sets with more records than
@@ -1315,16 +1344,6 @@ __global__ void __launch_bounds__(kBHullThreads, 1) bt_hull(BArgs a) {
         const unsigned total = *(volatile unsigned*)&c->count;   // with the line records
         const long long rb = region_base(a, i);
         const long long base = a.offsets[i], ni = a.offsets[i + 1] - base;
-        // More than one block holds, or past kBQhSkip records that are near
-        // the hull (a star polygon left them, or more than a quarter of the
-        // points survived the octagon), whose chains would outgrow the
-        // quickhull rounds' vertex capacity (kQhCap): the bucketed path.
-        const bool dense = c->star_k > 0 || 4ll * total > ni;
-        if (*(volatile int*)&c->done || total > (unsigned)kMidCap || (dense && total > (unsigned)kBQhSkip)) {
-            if (tid == 0 && !*(volatile int*)&c->done) a.big[i] = 1;
-            __syncthreads();
-            continue;
-        }
         QhSmem& q = *reinterpret_cast<QhSmem*>(dyn);
         for (unsigned j = tid; j < total; j += blockDim.x) {
             const uint32_t k = __ldcg(a.keys + rb + j);
@@ -1347,6 +1366,132 @@ __global__ void __launch_bounds__(kBHullThreads, 1) bt_hull(BArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// The queue chains of the listed sets (bt_list_queues), persistent over their
+// queues: a block gathers the queue's records from the set's region, sorts
+// them by u and reduces them to the lower chain in shared memory (qchain.cuh),
+// and leaves the chain in the set's region of the scatter buffer; the block
+// completing a set's fourth chain joins the chains.  A set with a queue over
+// the large shape's capacity (after bt_star_refine) is flagged for the
+// bucketed path.
+// Bound by latency: short scans between barriers, so several small blocks
+// share an SM.  On the 4096-set batch (1247 such sets, 9.4e6 records, 5.6e6
+// hull vertices) both shapes take 0.50 ms together; the bucketed path took
+// 3.4 ms (bucket chains 1.0, merges 2.1) after a second polygon (0.45 ms)
+// that the sets no longer need.
+constexpr int kBQGather = 4;   // records per thread in flight
+
+template <class Q, int T, bool kLarge>
+__global__ void __launch_bounds__(T) bt_queue_chain(BArgs a) {
+    extern __shared__ __align__(16) char dyn[];
+    Q& q = *reinterpret_cast<Q*>(dyn);
+    __shared__ int s_item, s_n, s_last;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const unsigned items = 4u * a.star_ctr[kLarge ? 10 : 9];
+    for (;;) {
+        if (tid == 0) {
+            const unsigned g = atomicAdd(&a.star_ctr[kLarge ? 12 : 11], 1u);
+            const int e = (int)(g >> 2);
+            s_item = g < items ? 4 * (kLarge ? a.q_list[a.k - 1 - e] : a.q_list[e]) + (int)(g & 3u) : -1;
+            s_n = 0;
+        }
+        __syncthreads();
+        const int item = s_item;
+        if (item < 0) return;
+        const int i = item >> 2, qq = item & 3;
+        Ctl* c = a.ctl + i;
+        const long long base = a.offsets[i], ni = a.offsets[i + 1] - base;
+        const long long rb = region_base(a, i);
+        const unsigned m = c->count;
+        unsigned pre[5];   // the queues' records before each queue
+        pre[0] = 0u;
+        bool fits = true;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const unsigned cr = c->counts4[r];
+            pre[r + 1] = pre[r] + cr;
+            fits = fits && cr <= (unsigned)Q::kCap;
+        }
+        if (!fits) {
+            if (tid == 0 && qq == 0) a.big[i] = 1;
+            __syncthreads();
+            continue;
+        }
+        for (unsigned j0 = 0; j0 < m; j0 += T * kBQGather) {
+            uint32_t k[kBQGather];
+            uint64_t w[kBQGather];
+            bool own[kBQGather];
+#pragma unroll
+            for (int e = 0; e < kBQGather; ++e) {
+                const unsigned j = j0 + e * T + tid;
+                k[e] = j < m ? __ldcg(a.keys + rb + j) : 0u;
+                own[e] = j < m && (int)(k[e] >> kKeyBits) == qq;
+            }
+#pragma unroll
+            for (int e = 0; e < kBQGather; ++e) w[e] = own[e] ? __ldcg(a.vals + rb + j0 + e * T + tid) : 0ull;
+#pragma unroll
+            for (int e = 0; e < kBQGather; ++e) {
+                const unsigned bal = __ballot_sync(0xFFFFFFFFu, own[e]);
+                if (!bal) continue;
+                int pos = 0;
+                if (lane == 0) pos = atomicAdd(&s_n, __popc(bal));
+                pos = __shfl_sync(0xFFFFFFFFu, pos, 0) + __popc(bal & lanemask_lt());
+                if (own[e] && pos < Q::kCap) {
+                    q.a[pos] = qc_pack(k[e] & kKeyMask, (unsigned)(w[e] >> 31), (unsigned)pos);
+                    q.si[pos] = (int)(w[e] & 0x7FFFFFFFull);
+                }
+            }
+        }
+        __syncthreads();
+        const int n = min(s_n, Q::kCap);   // counts4[qq], the chain's two end points among them
+        uint32_t ulo, uhi, v;
+        queue_frame(qq, c->oct.vx[2 * qq], c->oct.vy[2 * qq], ulo, v);
+        queue_frame(qq, c->oct.vx[(2 * qq + 2) & 7], c->oct.vy[(2 * qq + 2) & 7], uhi, v);
+        qc_sort<T>(q, n, (int)ulo, (int)uhi);
+        unsigned long long *src = q.b, *dst = q.a;
+        const int len = qc_eliminate<T>(src, dst, n, q.tmp);
+        for (int j = tid; j < len; j += T) {
+            const unsigned long long x = src[j];
+            a.vP[rb + pre[qq] + j] = x >> kQcPosBits;
+            a.kP[rb + pre[qq] + j] = (uint32_t)q.si[qc_pos(x)];
+        }
+        if (tid == 0) c->reg_end[qq] = (unsigned)len;
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            s_last = atomicAdd(&c->blocks_done[3], 1u) == 3u;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!s_last) continue;
+        int off[5];
+        off[0] = 0;
+        for (int r = 0; r < 4; ++r) off[r + 1] = off[r] + max((int)__ldcg(&c->reg_end[r]) - 1, 0);
+        auto get = [&](int r, int j, int& pu, int& pv, int& pi) {
+            const uint64_t x = __ldcg(a.vP + rb + pre[r] + j);
+            pu = (int)(x >> kKeyBits);
+            pv = (int)(x & kKeyMask);
+            pi = (int)__ldcg(a.kP + rb + pre[r] + j);
+        };
+        if (off[4] > kStitchLong) {
+            stitch_long(off, get, ni, c, a.out_idx + base, a.out_n + i);
+        } else {   // few vertices, or a degenerate cycle: one warp, in shared memory
+            int* X = reinterpret_cast<int*>(q.a);
+            int *Y = X + kStitchLong, *V = Y + kStitchLong, *tmp = V + kStitchLong;
+            for (int p = tid; p < off[4]; p += T) {
+                const int r = p >= off[2] ? (p >= off[3] ? 3 : 2) : (p >= off[1] ? 1 : 0);
+                int pu, pv;
+                get(r, p - off[r], pu, pv, V[p]);
+                frame_to_xy(r, pu, pv, X[p], Y[p]);
+            }
+            __syncthreads();
+            stitch_cycle(X, Y, V, off[4], tmp, c, ni, a.out_idx + base, a.out_n + i);
+        }
+        if (tid == 0) a.big[i] = 2;   // finished queue by queue
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Workspace per (device, stream), grow-only.
 struct BWork {
     char* base = nullptr;
@@ -1360,7 +1505,7 @@ static std::map<std::pair<int, cudaStream_t>, BWork> g_bws;
 static size_t bt_align(size_t x) { return (x + 255) / 256 * 256; }
 
 struct BLayout {
-    size_t ctl, keys, vals, rmap, big, redo, star_ctr, star_list, refine_list, hull_list, unit_base, star_slot, star_bins, star_polys;
+    size_t ctl, keys, vals, rmap, big, redo, star_ctr, star_list, refine_list, hull_list, q_list, unit_base, star_slot, star_bins, star_polys;
     size_t seg_nb, seg_bbase, seg_lo, seg_scale, seg_tbase, rt_base, totals;
     size_t bcount, bcur, bstart, blen, bu, bv, bi, kP, vP, cu, cv, ci, clen, ctmap, counters;
     size_t zero_from, zero_to;   // star bins and bucket counters: cleared before each batch
@@ -1394,6 +1539,7 @@ static BLayout bt_layout(long long total, int k, long long big_pts, long long bi
     L.unit_base = take(sizeof(unsigned) * (size_t)k);
     L.refine_list = take(sizeof(int) * (size_t)k);
     L.hull_list = take(sizeof(int) * (size_t)k);
+    L.q_list = take(sizeof(int) * (size_t)k);
     L.star_list = take(sizeof(int) * (size_t)k);
     L.star_slot = take(sizeof(int) * (size_t)k);
     L.star_polys = take(sizeof(StarPoly) * (size_t)slots);
@@ -1534,6 +1680,11 @@ static int bt_configure(int dev, BtDevice* out) {
         cudaFuncSetAttribute(bt_star_refine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBStarSmem) !=
             cudaSuccess ||
         cudaFuncSetAttribute(bt_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBDenseSmem) != cudaSuccess)
+        return CH_ECUDA;
+    if (cudaFuncSetAttribute(bt_queue_chain<QcSmall, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(QcSmall)) != cudaSuccess ||
+        cudaFuncSetAttribute(bt_queue_chain<QcLarge, 1024, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(QcLarge)) != cudaSuccess)
         return CH_ECUDA;
     if (configure_batched_large() != cudaSuccess) return CH_ECUDA;
     bt_occupancy<128, 16>(d.occ[0]);
@@ -1710,6 +1861,11 @@ static int bt_enqueue(const BtCall& c, unsigned char* redo, cudaStream_t s) {
     { ProfScope p("batched_hull_small", s); bt_hull_small<<<c.a.k, kBSmallThreads, 0, s>>>(c.a); }
     { ProfScope p("batched_refine", s); bt_star_refine<<<c.sms, kBStarThreads, kBStarSmem, s>>>(c.a); }
     { ProfScope p("batched_hull", s); bt_hull<<<c.sms, kBHullThreads, kBHullSmem, s>>>(c.a); }
+    {
+        ProfScope p("batched_queues", s);
+        bt_queue_chain<QcSmall, 256, false><<<c.sms * 4, 256, sizeof(QcSmall), s>>>(c.a);
+        bt_queue_chain<QcLarge, 1024, true><<<c.sms, 1024, sizeof(QcLarge), s>>>(c.a);
+    }
     // Sets with more records than one block holds: all together through the
     // bucketed path.
     launch_batched_large(c.b, redo, c.sms, s);
@@ -1936,6 +2092,7 @@ int hull_batched_impl(const float* pts, const int64_t* offsets, int32_t k, int32
     a.star_polys = (StarPoly*)(base + L.star_polys);
     a.refine_list = (int*)(base + L.refine_list);
     a.hull_list = (int*)(base + L.hull_list);
+    a.q_list = (int*)(base + L.q_list);
     a.unit_base = (unsigned*)(base + L.unit_base);
     a.kP = (uint32_t*)(base + L.kP);
     a.vP = (uint64_t*)(base + L.vP);

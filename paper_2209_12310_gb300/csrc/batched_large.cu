@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(1024) btl_prep(BLArgs a) {
     for (int sg = tid; sg < nseg; sg += 1024) {
         const int i = sg >> 2, q = sg & 3;
         unsigned nb = 0u;
-        if (a.big[i]) {
+        if (a.big[i] == 1) {
             const Ctl* c = a.ctl + i;
             nb = bk_buckets_for(c->counts4[q]);
             // Records that a star polygon left are mostly near the hull, a
@@ -94,8 +94,8 @@ __global__ void __launch_bounds__(1024) btl_prep(BLArgs a) {
     }
     for (int i = tid; i < a.k; i += 1024) {
         Ctl* c = a.ctl + i;
-        a.rt_base[i] = a.big[i] ? (c->count + kBLTile - 1) / kBLTile : 0u;
-        if (a.big[i]) {
+        a.rt_base[i] = a.big[i] == 1 ? (c->count + kBLTile - 1) / kBLTile : 0u;
+        if (a.big[i] == 1) {
             c->bk_state = 1;
             c->blocks_done[3] = 0u;
         }
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kChainThreads) btl_chain(BLArgs a) {
 __global__ void btl_flags(BLArgs a, unsigned char* redo) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.k) return;
-    redo[i] = (a.big[i] && (*(volatile int*)&a.ctl[i].bk_state == 2 || a.totals[3] == 0u)) ? 1 : 0;
+    redo[i] = (a.big[i] == 1 && (*(volatile int*)&a.ctl[i].bk_state == 2 || a.totals[3] == 0u)) ? 1 : 0;
 }
 
 static int g_occ_bucket_hull = 1;   // resident btl_bucket_hull blocks per SM (set by configure_batched_large)

@@ -1,0 +1,293 @@
+// qchain.cuh -- a queue's lower chain from its unsorted records by one block:
+// a bucket sort by u in shared memory, then elimination rounds; and the stitch
+// of four long queue chains.
+//
+// Elimination: a point on or above the segment between two other input points
+// of its queue (one on either side in u) is no strict vertex of the lower
+// chain, whatever becomes of those two.  So in one round every thread takes a
+// run of consecutive points, with the point before and the point after the run
+// as fixed context, and reduces it to the lower chain of the run and its
+// context (Andrew's scan, Table I); the runs that are left are packed together
+// and the next round cuts them at other places.  A round that removes nothing
+// has found every triple of neighbours turning strictly left: the chain is
+// convex, hence the lower chain.  Points near the hull (what a star polygon
+// leaves of dense data) need a few rounds.  Where long parts of two chains hide
+// each other the rounds are bounded by doubling the runs, up to one run that
+// holds every point.
+//
+// This replaces, for queues that fit, a warp's quickhull per bucket of 16
+// records and a tree of pairwise merges: those are chains of dependent
+// shared-memory searches with a few lanes at work (1.0 + 2.1 ms of a 7.5 ms
+// batch of 4096 sets), while a round here is a short scan on every thread.
+#pragma once
+
+#include "ch_internal.cuh"
+#include "hullcore.cuh"
+
+namespace ch {
+
+// A point of a chain under construction: u, v (25 bits each) and its slot in
+// the index array (14 bits).  The words order by (u, v).
+constexpr int kQcPosBits = 14;
+constexpr unsigned long long kQcPad = ~0ull;   // sorts last; u never has all bits set
+
+__device__ __forceinline__ unsigned long long qc_pack(unsigned u, unsigned v, unsigned pos) {
+    return ((unsigned long long)u << (kKeyBits + kQcPosBits)) | ((unsigned long long)v << kQcPosBits) | pos;
+}
+__device__ __forceinline__ int qc_u(unsigned long long w) { return (int)(w >> (kKeyBits + kQcPosBits)); }
+__device__ __forceinline__ int qc_v(unsigned long long w) { return (int)(w >> kQcPosBits) & (int)kKeyMask; }
+__device__ __forceinline__ int qc_pos(unsigned long long w) { return (int)(w & ((1ull << kQcPosBits) - 1ull)); }
+
+// CAP points at most (below 2^14), NB buckets at most.
+template <int CAP, int NB>
+struct QcSmem {
+    static_assert(CAP <= (1 << kQcPosBits) - 1 && NB % 32 == 0, "slots and buckets");
+    static constexpr int kCap = CAP, kBuckets = NB;
+    unsigned long long a[CAP], b[CAP];   // contiguous: the bitonic sort uses both
+    int si[CAP];                         // index of the point in slot p
+    unsigned cnt[NB];
+    int tmp[33];
+    int big;
+};
+
+// Order by (u, v), then by the lowest index.
+__device__ __forceinline__ bool qc_less(unsigned long long x, unsigned long long y, const int* si) {
+    const unsigned long long kx = x >> kQcPosBits, ky = y >> kQcPosBits;
+    if (kx != ky) return kx < ky;
+    return x != kQcPad && y != kQcPad && si[qc_pos(x)] < si[qc_pos(y)];
+}
+
+// The n points of q.a (u in [lo, hi]) in order, into q.b.  Whole block of T
+// threads.  Buckets of equal width in u hold about two points each, and a
+// thread sorts a bucket by insertion; when some bucket holds more than
+// kQcBucket (points crowded in u), the whole array goes through a bitonic
+// sort instead.
+constexpr unsigned kQcBucket = 32;
+
+template <int T, class Q>
+__device__ void qc_sort(Q& q, int n, int lo, int hi) {
+    const int tid = threadIdx.x;
+    const int nb = min(Q::kBuckets, n / 2 + 1);
+    const float scale = (float)nb / (float)(hi - lo + 1);
+    auto bucket = [&](unsigned long long w) { return max(0, min(nb - 1, (int)((float)(qc_u(w) - lo) * scale))); };
+    for (int b = tid; b < nb; b += T) q.cnt[b] = 0u;
+    if (tid == 0) q.big = 0;
+    __syncthreads();
+    for (int j = tid; j < n; j += T) atomicAdd(&q.cnt[bucket(q.a[j])], 1u);
+    __syncthreads();
+    const int per = (nb + T - 1) / T, b0 = min(nb, tid * per), b1 = min(nb, b0 + per);
+    unsigned sum = 0u, most = 0u;
+    for (int b = b0; b < b1; ++b) {
+        sum += q.cnt[b];
+        most = max(most, q.cnt[b]);
+    }
+    if (most > kQcBucket) q.big = 1;
+    int tot;
+    unsigned run = (unsigned)block_excl_scan((int)sum, q.tmp, &tot);
+    if (q.big) {   // block-uniform: set before the scan's barriers
+        int P = 1;
+        while (P < n) P <<= 1;   // n <= CAP < 2^14 <= 2 CAP words in a and b
+        unsigned long long* s = q.a;
+        for (int j = n + tid; j < P; j += T) s[j] = kQcPad;
+        __syncthreads();
+        for (int k = 2; k <= P; k <<= 1)
+            for (int d = k >> 1; d > 0; d >>= 1) {
+                for (int i = tid; i < P; i += T) {
+                    const int l = i ^ d;
+                    if (l > i) {
+                        const unsigned long long x = s[i], y = s[l];
+                        const bool up = (i & k) == 0;
+                        if (up ? qc_less(y, x, q.si) : qc_less(x, y, q.si)) {
+                            s[i] = y;
+                            s[l] = x;
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+        for (int j = tid; j < n; j += T) q.b[j] = s[j];   // the points are all in a again: n <= CAP
+        __syncthreads();
+        return;
+    }
+    for (int b = b0; b < b1; ++b) {
+        const unsigned c = q.cnt[b];
+        q.cnt[b] = run;
+        run += c;
+    }
+    __syncthreads();
+    for (int j = tid; j < n; j += T) {
+        const unsigned long long w = q.a[j];
+        q.b[atomicAdd(&q.cnt[bucket(w)], 1u)] = w;
+    }
+    __syncthreads();
+    for (int b = tid; b < nb; b += T) {   // cnt[b] is now the end of bucket b
+        const int s = b ? (int)q.cnt[b - 1] : 0, e = (int)q.cnt[b];
+        for (int i = s + 1; i < e; ++i) {
+            const unsigned long long w = q.b[i];
+            int j = i;
+            for (; j > s; --j) {
+                const unsigned long long x = q.b[j - 1];
+                if (!qc_less(w, x, q.si)) break;
+                q.b[j] = x;
+            }
+            q.b[j] = w;
+        }
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ long long qc_cross(unsigned long long o, unsigned long long a, unsigned long long b) {
+    return cross_uv(qc_u(o), qc_v(o), qc_u(a), qc_v(a), qc_u(b), qc_v(b));
+}
+__device__ __forceinline__ bool qc_same_u(unsigned long long a, unsigned long long b) {
+    return ((a ^ b) >> (kKeyBits + kQcPosBits)) == 0ull;
+}
+
+// The lower chain of the n >= 1 points in src, ordered by (u, v, index):
+// returns its length; src points at it (the two buffers change roles).  Of
+// points of equal u only the first can be a vertex: the others are skipped
+// where they follow it.  Whole block of T threads.  Runs have an odd length,
+// so that the lanes of a warp read different banks.
+constexpr int kQcRun = 5;      // points of a run at least
+constexpr int kQcSteady = 8;   // rounds before the runs grow (twofold every second round)
+
+template <int T>
+__device__ int qc_eliminate(unsigned long long*& src, unsigned long long*& dst, int n, int* s_tmp) {
+    const int tid = threadIdx.x;
+    int least = kQcRun;
+    for (int round = 0;; ++round) {
+        if (round > kQcSteady && (round & 1) && least < n) least = 2 * least + 1;
+        // odd rounds cut half a run later (T - 1 whole runs still hold all points)
+        const int c = max(least, (n + T - 2) / (T - 1)) | 1;
+        const int shift = (round & 1) ? c / 2 : 0;
+        const long long l0 = (long long)tid * c - shift;
+        const int lo = (int)max(0ll, min((long long)n, l0)), hi = (int)max(0ll, min((long long)n, l0 + c));
+        const bool some = lo < hi, ctx = some && lo > 0, after = some && hi < n;
+        const unsigned long long left = ctx ? src[lo - 1] : 0ull;
+        unsigned long long top = left, sec = 0ull;
+        const unsigned long long right = after ? src[hi] : 0ull;
+        __syncthreads();   // every context is read before the runs are rewritten
+        int cnt = 0;                // points kept: src[lo .. lo + cnt)
+        const int below = ctx ? 1 : 0;   // the context is the stack's bottom
+        int depth = below;
+        auto pop_above = [&](unsigned long long w) {
+            while (depth >= 2 && qc_cross(sec, top, w) <= 0) {
+                --depth;
+                --cnt;
+                top = sec;
+                // the element below the new top
+                if (depth >= 2) {
+                    const int e = depth - 2 - below;
+                    sec = e >= 0 ? src[lo + e] : left;
+                }
+            }
+        };
+        for (int j = lo; j < hi; ++j) {
+            const unsigned long long w = src[j];
+            if (depth > 0 && qc_same_u(top, w)) continue;
+            pop_above(w);
+            src[lo + cnt] = w;
+            ++cnt;
+            ++depth;
+            sec = top;
+            top = w;
+        }
+        if (after && !qc_same_u(top, right)) pop_above(right);
+        int tot;
+        const int off = block_excl_scan(cnt, s_tmp, &tot);
+        if (tot == n) return n;   // nothing removed: convex
+        for (int j = 0; j < cnt; ++j) dst[off + j] = src[lo + j];
+        __syncthreads();
+        unsigned long long* t = src;
+        src = dst;
+        dst = t;
+        n = tot;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Joins four queue chains into the output: the cycle of the chains without
+// their last points, off[q] the position of queue q's first point, m = off[4]
+// > kStitchLong in all; get(q, j, u, v, i) reads point j of chain q.  Each
+// chain is strictly convex and the cycle has an area (a degenerate input's
+// chains have two points at most), so only the chains' first points can fail
+// to be strict vertices, and the lexicographically smallest vertex is the
+// first or the second of queue 0 (W, or the lower end of the line x = xmin).
+// So each position's place in the output follows from the at most four
+// positions dropped: one pass, no scan.  Whole block.
+constexpr int kStitchLong = 64;
+
+template <class Get>
+__device__ void stitch_long(const int (&off)[5], Get get, long long n, Ctl* ctl, int32_t* out_idx, int64_t* out_n) {
+    __shared__ int s_drop[4], s_bad, s_start;
+    const int tid = threadIdx.x, m = off[4];
+    auto locate = [&](int p, int& q, int& j) {
+        q = p >= off[2] ? (p >= off[3] ? 3 : 2) : (p >= off[1] ? 1 : 0);
+        j = p - off[q];
+    };
+    auto xy = [&](int p, long long& x, long long& y) {
+        int q, j, u, v, i, X, Y;
+        locate(p, q, j);
+        get(q, j, u, v, i);
+        frame_to_xy(q, u, v, X, Y);
+        x = X;
+        y = Y;
+    };
+    if (tid == 0) s_bad = 0;
+    __syncthreads();
+    if (tid < 4) {
+        s_drop[tid] = INT_MAX;
+        const int p = off[tid];
+        if (off[tid + 1] > p) {   // queue tid has a point in the cycle
+            long long ax, ay, bx, by, cx, cy;
+            xy(p == 0 ? m - 1 : p - 1, ax, ay);
+            xy(p, bx, by);
+            xy(p + 1 == m ? 0 : p + 1, cx, cy);
+            const long long tr = orient64(ax, ay, bx, by, cx, cy);
+            if (tr < 0) s_bad = 1;   // internal consistency check
+            if (tr <= 0) s_drop[tid] = p;
+        }
+    }
+    __syncthreads();
+    const int d0 = s_drop[0], d1 = s_drop[1], d2 = s_drop[2], d3 = s_drop[3];
+    auto dropped_before = [&](int p) { return (d0 < p) + (d1 < p) + (d2 < p) + (d3 < p); };
+    auto dropped = [&](int p) { return p == d0 || p == d1 || p == d2 || p == d3; };
+    const int h = m - dropped_before(INT_MAX);
+    if (tid == 0) {
+        unsigned long long best = ~0ull;
+        int start = 0;
+        for (int e = -2; e < 4; ++e) {
+            const int p = e < 0 ? m + e : e;
+            if (dropped(p)) continue;
+            long long x, y;
+            xy(p, x, y);
+            const unsigned long long k = xy_key(x, y);
+            if (k < best) {
+                best = k;
+                start = p - dropped_before(p);
+            }
+        }
+        s_start = start;
+        if (s_bad || h > n) set_status(ctl, CH_ECUDA);
+    }
+    __syncthreads();
+    if (h > n) {   // cannot happen for a correct hull; never write past out_idx
+        if (tid == 0) *out_n = CH_ECUDA;
+        return;
+    }
+    const int start = s_start;
+    for (int p = tid; p < m; p += blockDim.x) {
+        if (dropped(p)) continue;
+        int q, j, u, v, i;
+        locate(p, q, j);
+        get(q, j, u, v, i);
+        const int r = p - dropped_before(p) - start;
+        out_idx[r < 0 ? r + h : r] = i;
+    }
+    if (tid == 0) {
+        const int st = read_status(ctl);
+        *out_n = st == CH_OK ? (int64_t)h : (int64_t)st;
+    }
+}
+
+}  // namespace ch
