@@ -33,7 +33,7 @@ static int device_info(int dev, DevInfo* out) {
     if (configure_hull_kernels() != cudaSuccess) return CH_ECUDA;
     if (configure_filter_kernels() != cudaSuccess) return CH_ECUDA;
     if (configure_post_kernel() != cudaSuccess) return CH_ECUDA;
-    if (configure_bucket_kernels() != cudaSuccess) return CH_ECUDA;
+    if (configure_queue_kernels() != cudaSuccess) return CH_ECUDA;
     if (configure_star_kernel() != cudaSuccess) return CH_ECUDA;
     if (occupancy_filter(&di.occ_main, &di.occ_lab) != cudaSuccess) return CH_ECUDA;
     if (occupancy_post(&di.occ_post) != cudaSuccess) return CH_ECUDA;
@@ -57,10 +57,7 @@ Layout make_layout(long long n) {
     Layout L{};
     L.cap = n + 16;
     L.sort_tiles = (L.cap + kSortTile - 1) / kSortTile;
-    L.bmax = L.cap / kBkAvg + 4 * kBkMinQ + 8;
-    // chain tiles: sorted records (one per kChainTile) or bucket chains (one
-    // per kBkGroup buckets of each queue), whichever needs more
-    L.ctcap = std::max((L.cap + kChainTile - 1) / kChainTile + 4, L.bmax / kBkGroup + 8);
+    L.ctcap = (L.cap + kChainTile - 1) / kChainTile + 4;   // chain tiles of the sorted records
     size_t o = 0;
     auto take = [&](size_t bytes) {
         const size_t r = o;
@@ -68,12 +65,13 @@ Layout make_layout(long long n) {
         return r;
     };
     // zeroed at allocation: the control block, the sort's look-back status
-    // words and the merge tree's arrival counters (each kernel leaves them
-    // in that state for the next call)
+    // words, the merge tree's arrival counters, the star bins and the tile
+    // counters (each kernel leaves them in that state for the next call)
     L.off_ctl = take(sizeof(Ctl));
     L.off_status = take(8 * (size_t)kDigits * L.sort_tiles);
     L.off_counters = take(4 * (size_t)kMaxLevels * L.ctcap);
     L.off_star_bins = take(star_bins_bytes());   // the star and post passes leave them at zero
+    L.off_tiles = take(tiles_bytes());           // tile_hist_kernel leaves its counters at zero
     L.zero_bytes = o;
     L.off_kA = take(4 * (size_t)L.cap);
     L.off_kB = take(4 * (size_t)L.cap);
@@ -83,14 +81,6 @@ Layout make_layout(long long n) {
     L.off_cv = take(4 * (size_t)L.ctcap * kChainTile);
     L.off_ci = take(4 * (size_t)L.ctcap * kChainTile);
     L.off_clen = take(4 * (size_t)L.ctcap);
-    L.off_bcount = take(4 * (size_t)L.bmax);
-    L.off_bcur = take(4 * (size_t)L.bmax);
-    L.off_bstart = take(4 * (size_t)L.bmax);
-    L.off_bsum = take(4 * ((size_t)L.bmax / 1024 + 2 + 2 * (size_t)kBkCoarseMax + 1));   // block sums, cursors, tiles
-    L.off_blen = take(4 * (size_t)L.bmax);
-    L.off_bu = take(4 * (size_t)L.bmax * kBkChain);
-    L.off_bv = take(4 * (size_t)L.bmax * kBkChain);
-    L.off_bi = take(4 * (size_t)L.bmax * kBkChain);
     L.total = o;
     return L;
 }
@@ -279,9 +269,9 @@ static void prof_drain() {
 // ---------------------------------------------------------------------------
 // The launch sequence of one hull (n >= 1) on an allocated workspace, in two
 // parts: the filter (init .. post), after which small survivor sets are done,
-// and the large-survivor path (buckets, the sort fallback, the chain merge).
-// `cond`, when non-zero, is a graph condition the post pass raises when the
-// second part has work (see the CUDA-graph cache below).
+// and the large-survivor path (queues, tiles, the sort).  `cond`, when
+// non-zero, is a graph condition the post pass sets when the second part has
+// work (see the CUDA-graph cache below).
 struct HullLaunch {
     DevInfo di;
     Ctl* ctl;
@@ -355,13 +345,19 @@ static void enqueue_filter_part(const float* pts, long long n, int32_t* out_idx,
     }
 }
 
+// The large-survivor part of a call: the queues that fit a block each (bodies
+// & 1), the tiled queues and the sort (bodies & 2).  Each kernel returns at once
+// when the call took another path; a captured graph holds the two bodies apart
+// and runs the one that the post pass chose.
 static void enqueue_large_part(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s,
-                               char* base, const Layout& L, const HullLaunch& h) {
+                               char* base, const Layout& L, const HullLaunch& h, int bodies) {
     Ctl* ctl = h.ctl;
     unsigned long long* status = (unsigned long long*)(base + L.off_status);
-    launch_bucket_pass(ctl, h.kA, h.vA, h.kB, h.vB, (unsigned*)(base + L.off_bcount), (unsigned*)(base + L.off_bcur),
-                       (unsigned*)(base + L.off_bstart), (unsigned*)(base + L.off_bsum), (int*)(base + L.off_bu), (int*)(base + L.off_bv),
-                       (int*)(base + L.off_bi), (int*)(base + L.off_blen), (unsigned)L.bmax, h.di.sms, s);
+    unsigned* tiles = (unsigned*)(base + L.off_tiles);
+    int *cu = (int*)(base + L.off_cu), *cv = (int*)(base + L.off_cv), *ci = (int*)(base + L.off_ci);
+    if (bodies & 2) launch_tiles(ctl, h.kA, h.vA, h.kB, h.vB, tiles, cu, cv, ci, h.di.sms, s);
+    launch_queues(ctl, h.kA, h.vA, h.kB, h.vB, tiles, cu, cv, ci, n, out_idx, out_n, s);
+    if (!(bodies & 2)) return;
     {
         ProfScope p("sort", s);
         const int grid_sort = h.di.sms * h.di.occ_sort;
@@ -372,11 +368,9 @@ static void enqueue_large_part(const float* pts, long long n, int32_t* out_idx, 
     }
     {
         ProfScope p("hull_chains", s);
-        launch_chain(ctl, h.kB, h.vB, (const int*)(base + L.off_bu), (const int*)(base + L.off_bv),
-                     (const int*)(base + L.off_bi), (const int*)(base + L.off_blen), (int*)(base + L.off_cu),
-                     (int*)(base + L.off_cv), (int*)(base + L.off_ci), (int*)(base + L.off_clen),
-                     (int*)(base + L.off_counters), (int)L.ctcap, (int*)h.vA, (int*)h.kA, (int*)h.kB, (int*)h.vB,
-                     pts, n, out_idx, out_n, h.di.sms * h.di.occ_chain, s);
+        launch_chain(ctl, h.kB, h.vB, cu, cv, ci, (int*)(base + L.off_clen), (int*)(base + L.off_counters),
+                     (int)L.ctcap, (int*)h.vA, (int*)h.kA, (int*)h.kB, (int*)h.vB, pts, n, out_idx, out_n,
+                     h.di.sms * h.di.occ_chain, s);
     }
 }
 
@@ -386,13 +380,14 @@ static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, 
     const int st = hull_setup(pts, n, dev, owner, base, L, &h);
     if (st != CH_OK) return st;
     enqueue_filter_part(pts, n, out_idx, out_n, s, h, 0ull);
-    enqueue_large_part(pts, n, out_idx, out_n, s, base, L, h);
+    enqueue_large_part(pts, n, out_idx, out_n, s, base, L, h, 3);
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ECUDA;
 }
 
-// Captures the sequence on `cs` with the large-survivor part as the body of
-// a conditional (if) node whose condition the post pass raises; replays of
-// small-survivor calls then launch only the filter part.  False when any step
+// Captures the sequence on `cs` with the large-survivor part as the two bodies
+// of a conditional (switch) node whose value the post pass sets; replays of
+// small-survivor calls then launch only the filter part (the default value
+// names no body).  False when any step
 // of the capture fails (the caller then captures the plain sequence).
 static bool capture_conditional(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t cs,
                                 int dev, char* base, const Layout& L, cudaStream_t owner, cudaGraph_t* out) {
@@ -410,7 +405,7 @@ static bool capture_conditional(const float* pts, long long n, int32_t* out_idx,
         const cudaGraphEdgeData* edata = nullptr;
         size_t ndeps = 0;
         ok = cudaStreamGetCaptureInfo(cs, &stc, &id, &graph, &deps, &edata, &ndeps) == cudaSuccess && graph;
-        if (ok) ok = cudaGraphConditionalHandleCreate(&cond, graph, 0u, cudaGraphCondAssignDefault) == cudaSuccess;
+        if (ok) ok = cudaGraphConditionalHandleCreate(&cond, graph, 2u, cudaGraphCondAssignDefault) == cudaSuccess;
     }
     if (ok) {
         enqueue_filter_part(pts, n, out_idx, out_n, cs, h, (unsigned long long)cond);
@@ -425,19 +420,19 @@ static bool capture_conditional(const float* pts, long long n, int32_t* out_idx,
         if (ok) {
             np.type = cudaGraphNodeTypeConditional;
             np.conditional.handle = cond;
-            np.conditional.type = cudaGraphCondTypeIf;
-            np.conditional.size = 1;
+            np.conditional.type = cudaGraphCondTypeSwitch;
+            np.conditional.size = 2;
             ok = cudaGraphAddNode(&node, graph, deps, edata, ndeps, &np) == cudaSuccess;
         }
         if (ok) ok = cudaStreamUpdateCaptureDependencies(cs, &node, nullptr, 1, cudaStreamSetCaptureDependencies) ==
                      cudaSuccess;
         if (ok) ok = cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking) == cudaSuccess;
-        if (ok) {
-            cudaGraph_t body = np.conditional.phGraph_out[0];
+        for (int b = 0; ok && b < 2; ++b) {
+            cudaGraph_t body = np.conditional.phGraph_out[b];
             ok = cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
                  cudaSuccess;
             if (ok) {
-                enqueue_large_part(pts, n, out_idx, out_n, bs, base, L, h);
+                enqueue_large_part(pts, n, out_idx, out_n, bs, base, L, h, 1 << b);
                 cudaGraph_t tmp = nullptr;
                 ok = cudaStreamEndCapture(bs, &tmp) == cudaSuccess;
             }

@@ -1447,7 +1447,7 @@ __global__ void __launch_bounds__(T) bt_queue_chain(BArgs a) {
         queue_frame(qq, c->oct.vx[2 * qq], c->oct.vy[2 * qq], ulo, v);
         queue_frame(qq, c->oct.vx[(2 * qq + 2) & 7], c->oct.vy[(2 * qq + 2) & 7], uhi, v);
         qc_sort<T>(q, n, (int)ulo, (int)uhi);
-        unsigned long long *src = q.b, *dst = q.a;
+        unsigned long long *src = q.a, *dst = q.b;
         const int len = qc_eliminate<T>(src, dst, n, q.tmp);
         for (int j = tid; j < len; j += T) {
             const unsigned long long x = src[j];

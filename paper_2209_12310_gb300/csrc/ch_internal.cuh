@@ -38,8 +38,13 @@ constexpr int kChainThreads = 256;
 constexpr int kChainItems = 16;
 constexpr int kChainTile = kChainThreads * kChainItems;
 constexpr int kMergeSmemCap = 8192;           // chain points a global merge keeps on chip
-// Bucketed large-survivor path (bucket.cu): records per bucket on average,
-// chain vertices a bucket may keep, bucket chains per chain-kernel tile.
+// Large-survivor path of the single hull (queues.cu): records of a queue that
+// one block reduces to its chain, and the ways a call can take.
+constexpr int kQueueCap = 10240;
+enum Path { kPathNone = 0, kPathQueues, kPathTiles, kPathSort };
+// Bucketed large-survivor path of a batch (batched_large.cu): records per
+// bucket on average, chain vertices a bucket may keep, bucket chains per
+// chain-kernel tile.
 constexpr int kBkAvg = 256;
 constexpr int kBkNearHull = 64;   // records per bucket when a star polygon filtered them
 constexpr int kBkChain = 32;
@@ -48,11 +53,10 @@ constexpr int kBkGroup = kChainTile / kBkChain;
 // 7 cnt^(1/3) (at most one per 8 records).  The queue chain of cnt records
 // on a thin ring (the ring workload: width 64 at radius 2^23) has about
 // 54 cnt^(1/3) vertices, so a bucket holds about 8 of them and its chain
-// stays within kBkChain; a queue whose chains still overflow takes the
-// radix-sort path.  kBkMinQ bounds the floor (7 cnt^(1/3) - cnt / kBkAvg
+// stays within kBkChain; a set whose chains still overflow takes the
+// single-hull path.  kBkMinQ bounds the floor (7 cnt^(1/3) - cnt / kBkAvg
 // stays below 115), for the workspace bounds.
 constexpr int kBkMinQ = 256;
-constexpr int kBkCoarseMax = 4096;   // coarse bucket groups of the two-level partition at most
 
 __host__ __device__ __forceinline__ unsigned bk_buckets_for(unsigned cnt) {
     unsigned nb = (cnt + kBkAvg - 1) / kBkAvg;
@@ -121,21 +125,15 @@ struct Ctl {
     int done;                           // the hull has been written by a small-path block
     int records_ready;                  // sort records complete before the re-classify stage
     unsigned int blocks_done[4];        // last-arriver counters (sample, main, stage C, roots)
-    unsigned int tile_ctr[4];           // onesweep tile claim counters
+    unsigned int tile_ctr[4];           // onesweep tile claim counters (0 .. 2), tile_chain_kernel's (3)
     unsigned int digit_hist[kSortPasses][kDigits];   // sort fallback only (sort_hist_kernel)
     unsigned int rec_q[4];              // records per queue
-    unsigned int reg_start[4], reg_end[4];
-    unsigned int reg_tile_base[5];      // chain tiles of queue r: [base[r], base[r+1])
+    unsigned int reg_end[4];            // chain length of queue r (queue_kernel, bt_queue_chain)
     unsigned int counts4[4];            // survivors per queue (ch_filter)
     unsigned long long line_ep[8];      // end points of survivors on the 4 axis support lines
-    int bk_state;                       // large-survivor path: 0 unused, 1 buckets, 2 full sort
-    unsigned int bk_cursor;             // tiles of the second partition level
-    unsigned int bk_nb[4];              // buckets of queue r
-    unsigned int bk_base[5];            // first bucket of queue r
-    int bk_lo[4];                       // u of queue r's first chain point
-    float bk_scale[4];                  // buckets per unit of u in queue r
-    int bk_shift;                       // fine buckets per coarse group: 1 << bk_shift
-    unsigned int bk_next;               // next bucket for a bk_hull warp
+    int bk_state;                       // large-survivor path: 0 unused, 1 queues / tiles / buckets, 2 full sort
+    int path;                           // the single hull's large-survivor path (Path)
+    unsigned int q_tile[5];             // path tiles: tiles of queue r are [q_tile[r], q_tile[r + 1])
     int samp_ok;                        // oct_s holds this call's sample octagon
     int star_ok;                        // the star pass found dense data: the post pass builds the polygon
     int star_k;                         // the polygon's vertices (post pass)

@@ -49,7 +49,7 @@ __global__ void init_kernel(Ctl* ctl, int mode) {
         ctl->done = 0;
         ctl->records_ready = 0;
         ctl->bk_state = 0;
-        ctl->bk_cursor = 0u;
+        ctl->path = kPathNone;
         ctl->samp_ok = 0;
         ctl->star_ok = 0;
         ctl->star_k = 0;

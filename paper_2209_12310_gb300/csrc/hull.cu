@@ -32,12 +32,8 @@ namespace ch {
 
 // ---------------------------------------------------------------------------
 struct HullBufs {
-    const uint32_t* keys;   // sorted records (sort-based path)
+    const uint32_t* keys;   // sorted records
     const uint64_t* vals;
-    const int* bu;          // bucket chains (bucketed path): bucket b at [b*kBkChain, ...)
-    const int* bv;
-    const int* bi;
-    const int* blen;
     int* cu;                // chain storage: tile c at [c*kChainTile, ...)
     int* cv;
     int* ci;
@@ -72,24 +68,17 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(Ctl* ctl, HullBufs
         return;
     }
     const int tid = threadIdx.x;
-    // Bucketed input: the leaves are bucket chains, kBkGroup per tile; queue
-    // r owns buckets [bk_base[r], bk_base[r+1]).  Sorted input: queue r holds
-    // the top-pass digits [128 r, 128 (r + 1)), so its size is a sum of that
-    // histogram.
-    const bool bk = *(volatile int*)&ctl->bk_state == 1;
+    // Queue r holds the top-pass digits [128 r, 128 (r + 1)), so its size is a
+    // sum of that histogram.
     if (tid < 4) s_qn[tid] = 0u;
     __syncthreads();
-    if (bk) {
-        if (tid < 4) s_qn[tid] = ctl->bk_base[tid + 1] - ctl->bk_base[tid];
-    } else {
-        for (int d = tid; d < kDigits; d += blockDim.x) {
-            const unsigned c = ctl->digit_hist[kSortPasses - 1][d];
-            if (c) atomicAdd(&s_qn[d >> (kDigitBits - 2)], c);
-        }
+    for (int d = tid; d < kDigits; d += blockDim.x) {
+        const unsigned c = ctl->digit_hist[kSortPasses - 1][d];
+        if (c) atomicAdd(&s_qn[d >> (kDigitBits - 2)], c);
     }
     __syncthreads();
     if (tid == 0) {
-        const unsigned per = bk ? (unsigned)kBkGroup : (unsigned)kChainTile;
+        const unsigned per = (unsigned)kChainTile;
         unsigned q = 0, tb = 0;
         for (int r = 0; r < 4; ++r) {
             s_q0[r] = q;
@@ -103,8 +92,8 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(Ctl* ctl, HullBufs
     __syncthreads();
     const unsigned total_tiles = s_tb[4];
     const unsigned nrec = ctl->count;
-    const int seg = bk ? kBkChain : kChainItems;           // shared-memory slot per leaf chain
-    const int nseg = bk ? kBkGroup : kChainThreads;        // leaf chains per tile
+    const int seg = kChainItems;      // shared-memory slot per leaf chain
+    const int nseg = kChainThreads;   // leaf chains per tile
 
     for (unsigned c = blockIdx.x; c < total_tiles; c += gridDim.x) {
         CH_MG_DECL
@@ -114,20 +103,9 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(Ctl* ctl, HullBufs
         const unsigned ct = s_tb[r + 1] - rb;
         const unsigned t_local = c - rb;
         const unsigned q0 = s_q0[r], q1 = s_q0[r + 1];
-        const unsigned ts = q0 + t_local * (bk ? (unsigned)kBkGroup : (unsigned)kChainTile);
-        const unsigned te = min(q1, ts + (bk ? (unsigned)kBkGroup : (unsigned)kChainTile));
+        const unsigned ts = q0 + t_local * (unsigned)kChainTile;
+        const unsigned te = min(q1, ts + (unsigned)kChainTile);
 
-        if (bk) {
-            // 1') the tile's bucket chains (buckets ts .. te): their slots are
-            // contiguous, so the whole block copies them with coalesced loads
-            s_len[tid] = (tid < kBkGroup && ts + tid < te) ? __ldcg(hb.blen + ts + tid) : 0;
-            const size_t o0 = (size_t)ts * kBkChain;
-            for (unsigned e = tid; e < (te - ts) * kBkChain; e += blockDim.x) {
-                su[e] = __ldcg(hb.bu + o0 + e);
-                sv[e] = __ldcg(hb.bv + o0 + e);
-                si[e] = __ldcg(hb.bi + o0 + e);
-            }
-        } else {
         // 1) run reduction + per-thread chain (records [ts + 16 tid, +16)).
         {
             const int sbase = tid * kChainItems;
@@ -154,7 +132,6 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(Ctl* ctl, HullBufs
                 ++sp;
             }
             s_len[tid] = sp;
-        }
         }
         __syncthreads();
         CH_MG(0);
@@ -217,11 +194,10 @@ namespace ch {
 
 size_t chain_smem_bytes() { return (size_t)3 * kMergeSmemCap * sizeof(int); }
 
-void launch_chain(Ctl* ctl, const uint32_t* keys, const uint64_t* vals, const int* bu, const int* bv,
-                  const int* bi, const int* blen, int* cu, int* cv, int* ci, int* clen, int* counters, int ctcap,
-                  int* vbuf, int* kbuf, int* xbuf, int* ybuf, const float* pts, long long n, int32_t* out_idx,
-                  int64_t* out_n, int grid, cudaStream_t s) {
-    HullBufs hb{keys, vals, bu, bv, bi, blen, cu, cv, ci, clen, counters, ctcap, vbuf, kbuf, xbuf, ybuf, pts, n,
+void launch_chain(Ctl* ctl, const uint32_t* keys, const uint64_t* vals, int* cu, int* cv, int* ci, int* clen,
+                  int* counters, int ctcap, int* vbuf, int* kbuf, int* xbuf, int* ybuf, const float* pts, long long n,
+                  int32_t* out_idx, int64_t* out_n, int grid, cudaStream_t s) {
+    HullBufs hb{keys, vals, cu, cv, ci, clen, counters, ctcap, vbuf, kbuf, xbuf, ybuf, pts, n,
                 out_idx, out_n};
     chain_kernel<<<grid, kChainThreads, chain_smem_bytes(), s>>>(ctl, hb);
 }

@@ -28,14 +28,17 @@ void launch_sort_hist(const uint32_t* keys, Ctl* ctl, int grid, cudaStream_t s);
 void launch_sort_pass(const uint32_t* kin, const uint64_t* vin, uint32_t* kout, uint64_t* vout,
                       Ctl* ctl, unsigned long long* status, int pass, int grid, cudaStream_t s);
 
-void launch_chain(Ctl* ctl, const uint32_t* keys, const uint64_t* vals, const int* bu, const int* bv,
-                  const int* bi, const int* blen, int* cu, int* cv, int* ci, int* clen, int* counters, int ctcap,
-                  int* vbuf, int* kbuf, int* xbuf, int* ybuf, const float* pts, long long n, int32_t* out_idx,
-                  int64_t* out_n, int grid, cudaStream_t s);
-void launch_bucket_pass(Ctl* ctl, uint32_t* kA, uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned* bcount,
-                        unsigned* bcur, unsigned* bstart, unsigned* bsum, int* bu, int* bv, int* bi, int* blen,
-                        unsigned bmax, int sms, cudaStream_t s);
-cudaError_t configure_bucket_kernels();
+void launch_chain(Ctl* ctl, const uint32_t* keys, const uint64_t* vals, int* cu, int* cv, int* ci, int* clen,
+                  int* counters, int ctcap, int* vbuf, int* kbuf, int* xbuf, int* ybuf, const float* pts, long long n,
+                  int32_t* out_idx, int64_t* out_n, int grid, cudaStream_t s);
+// The large-survivor paths without a sort (queues.cu); tiles: tiles_bytes() of
+// the workspace, its first kPtGroups words zero at rest.
+void launch_tiles(Ctl* ctl, uint32_t* kA, uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned* tiles, int* cu, int* cv,
+                  int* ci, int sms, cudaStream_t s);
+void launch_queues(Ctl* ctl, const uint32_t* kA, const uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned* tiles,
+                   int* cu, int* cv, int* ci, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s);
+size_t tiles_bytes();
+cudaError_t configure_queue_kernels();
 size_t chain_smem_bytes();
 cudaError_t configure_hull_kernels();
 cudaError_t configure_filter_kernels();

@@ -6,7 +6,7 @@
 // records (queue | u, v | index).  The block that finishes last adds the
 // records of the support-line end points and, when the records are few,
 // computes the hull itself (quickhull rounds over the queues), so the
-// sort-based path that follows finds ctl->done set and exits at once.
+// large-survivor path that follows finds ctl->done set and exits at once.
 #include "ch_internal.cuh"
 #include "hullcore.cuh"
 #include "launch.h"
@@ -131,12 +131,23 @@ __device__ __forceinline__ void flush_queue_counts(QueueTally& tally, Ctl* ctl) 
     if (threadIdx.x < 4 && s_q[threadIdx.x]) atomicAdd(&ctl->rec_q[threadIdx.x], s_q[threadIdx.x]);
 }
 
-// The block that finished last: support-line records, then with at most
-// kMidCap records the hull (quickhull rounds, else the sort-based mid_hull).
-// Every other record is already in keys/vals and in the per-queue counts.
+// The block that finished last: support-line records, then the hull of few
+// records (at most kMidCap: quickhull rounds, else the sort-based mid_hull), or
+// the path of the large-survivor part.  On dense data (two-pass mode, or more
+// than a quarter of the points kept) the records are near the hull, mostly
+// vertices, and past kNearHullRec of them they would outgrow
+// the quickhull rounds' vertex capacity: the queues then, a block each (one
+// million points of a ring: 27,265 records, 13,024 vertices: queue_kernel takes
+// the place of a partition into buckets, a warp's quickhull per bucket and a
+// radix sort when their chains overflow).  The sort takes what neither a
+// block nor the tiles are for: a queue too large for a block among few
+// records in all.  Every other record is already in keys/vals and in the
+// per-queue counts.
+constexpr unsigned kNearHullRec = 512;
+
 __device__ void post_last_block(const float* __restrict__ pts, long long n, Ctl* ctl, const Octagon& o,
                                 uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n, char* dyn,
-                                unsigned long long cond) {
+                                bool dense, unsigned long long cond) {
     __shared__ unsigned long long s_lep[8];
     __shared__ uint64_t s_lval[8];
     __shared__ unsigned s_lkey[8];
@@ -161,14 +172,24 @@ __device__ void post_last_block(const float* __restrict__ pts, long long n, Ctl*
     }
     __syncthreads();
     const unsigned total = s_total;
-    const bool small = total <= (unsigned)kMidCap;
+    const bool near_hull = dense || 4ll * total > n;
+    const bool small = total <= (near_hull ? kNearHullRec : (unsigned)kMidCap);
     if (tid < 8 && s_lpos[tid] >= 0) {
         keys[s_lpos[tid]] = s_lkey[tid];
         vals[s_lpos[tid]] = s_lval[tid];
         if (!small) atomicAdd(&ctl->rec_q[s_lkey[tid] >> kKeyBits], 1u);
     }
     if (!small) {   // the large-survivor path follows
-        if (cond && tid == 0) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, 1u);
+        __syncthreads();
+        if (tid == 0) {
+            unsigned most = 0u;
+            for (int r = 0; r < 4; ++r) most = max(most, *(volatile unsigned*)&ctl->rec_q[r]);
+            const int path = most <= (unsigned)kQueueCap ? kPathQueues
+                             : *(volatile int*)&ctl->star_final || total > 4u * (unsigned)kQueueCap ? kPathTiles : kPathSort;
+            ctl->path = path;
+            ctl->bk_state = path == kPathSort ? 2 : 1;
+            if (cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, path == kPathQueues ? 0u : 1u);
+        }
         return;
     }
     __syncthreads();      // also makes this block's line records visible to it
@@ -204,10 +225,10 @@ constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 // Points of dense data that the star polygon's radius test leaves undecided,
 // queued per warp and taken 32 at a time through the exact tests, so that a
 // few such points do not hold a whole warp in the slow path.
-constexpr int kQueueCap = 96;   // < 32 waiting + 64 added per step
+constexpr int kWarpQueueCap = 96;   // < 32 waiting + 64 added per step
 struct WarpQueue {
-    int x[kQueueCap], y[kQueueCap];
-    unsigned idx[kQueueCap];
+    int x[kWarpQueueCap], y[kWarpQueueCap];
+    unsigned idx[kWarpQueueCap];
 };
 
 // Dynamic shared memory while points are classified: the star polygon, the
@@ -397,7 +418,7 @@ __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __re
     CH_TL(ctl, 6, 0);
     if (s_star)   // every block has built its polygon: clear the bins for the next call
         for (int b = tid; b < kStarBins; b += blockDim.x) star_bins[b] = 0ull;
-    post_last_block(pts, n, ctl, s_o, keys, vals, out_idx, out_n, dyn, cond);
+    post_last_block(pts, n, ctl, s_o, keys, vals, out_idx, out_n, dyn, s_mode == 1, cond);
     CH_TL(ctl, 6, 1);
 }
 

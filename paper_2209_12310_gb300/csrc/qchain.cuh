@@ -50,19 +50,23 @@ struct QcSmem {
     int big;
 };
 
-// Order by (u, v), then by the lowest index.
+// Order by (u, v), then by the lowest index, then by slot (a record can occur
+// twice: the two ends of a support line with one survivor).
 __device__ __forceinline__ bool qc_less(unsigned long long x, unsigned long long y, const int* si) {
     const unsigned long long kx = x >> kQcPosBits, ky = y >> kQcPosBits;
     if (kx != ky) return kx < ky;
-    return x != kQcPad && y != kQcPad && si[qc_pos(x)] < si[qc_pos(y)];
+    if (x == kQcPad || y == kQcPad) return false;
+    const int ix = si[qc_pos(x)], iy = si[qc_pos(y)];
+    return ix != iy ? ix < iy : x < y;
 }
 
-// The n points of q.a (u in [lo, hi]) in order, into q.b.  Whole block of T
-// threads.  Buckets of equal width in u hold about two points each, and a
-// thread sorts a bucket by insertion; when some bucket holds more than
-// kQcBucket (points crowded in u), the whole array goes through a bitonic
-// sort instead.
-constexpr unsigned kQcBucket = 32;
+// The n points of q.a (u in [lo, hi]) in order, in place.  Whole block of T
+// threads.  Buckets of equal width in u hold about two points each; every point
+// counts the points of its bucket before it (independent loads, where an
+// insertion sort per bucket is a chain of them: records that a polygon leaves
+// can crowd a few buckets by the hundred).  When some bucket holds more than
+// kQcBucket, the whole array goes through a bitonic sort instead.
+constexpr unsigned kQcBucket = 512;
 
 template <int T, class Q>
 __device__ void qc_sort(Q& q, int n, int lo, int hi) {
@@ -105,8 +109,6 @@ __device__ void qc_sort(Q& q, int n, int lo, int hi) {
                 }
                 __syncthreads();
             }
-        for (int j = tid; j < n; j += T) q.b[j] = s[j];   // the points are all in a again: n <= CAP
-        __syncthreads();
         return;
     }
     for (int b = b0; b < b1; ++b) {
@@ -120,18 +122,13 @@ __device__ void qc_sort(Q& q, int n, int lo, int hi) {
         q.b[atomicAdd(&q.cnt[bucket(w)], 1u)] = w;
     }
     __syncthreads();
-    for (int b = tid; b < nb; b += T) {   // cnt[b] is now the end of bucket b
+    for (int j = tid; j < n; j += T) {
+        const unsigned long long w = q.b[j];
+        const int b = bucket(w);   // cnt[b] is now the end of bucket b
         const int s = b ? (int)q.cnt[b - 1] : 0, e = (int)q.cnt[b];
-        for (int i = s + 1; i < e; ++i) {
-            const unsigned long long w = q.b[i];
-            int j = i;
-            for (; j > s; --j) {
-                const unsigned long long x = q.b[j - 1];
-                if (!qc_less(w, x, q.si)) break;
-                q.b[j] = x;
-            }
-            q.b[j] = w;
-        }
+        int r = s;
+        for (int i = s; i < e; ++i) r += qc_less(q.b[i], w, q.si) ? 1 : 0;
+        q.a[r] = w;
     }
     __syncthreads();
 }

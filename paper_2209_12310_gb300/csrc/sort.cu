@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kSortThreads) onesweep_kernel(
 }
 
 // Digit histograms of the records for the three passes (the sort-based
-// fallback only: the bucketed path needs none and leaves bk_state == 1).
+// path only: the others need none and leave bk_state == 1).
 __global__ void __launch_bounds__(kSortThreads) sort_hist_kernel(const uint32_t* __restrict__ keys, Ctl* ctl) {
     __shared__ unsigned s_h[kSortPasses][kDigits];
     if (*(volatile int*)&ctl->done || read_status(ctl) != CH_OK || *(volatile int*)&ctl->bk_state == 1) return;

@@ -1,7 +1,8 @@
 """Hulls of dense sets, queue by queue (the block sort by u and the elimination
-rounds): bit-exact with the oracle at the edges of the kernel's shapes, and on
-inputs that take its other branches (crowded buckets, long chains that hide
-each other, duplicates, a queue over the largest shape)."""
+rounds), batched and single: bit-exact with the oracle at the edges of the
+kernels' shapes, and on inputs that take their other branches (crowded buckets,
+long chains that hide each other, duplicates, a queue over the largest shape,
+tiles of u ranges, a tile over its block's capacity)."""
 import numpy as np
 import pytest
 
@@ -67,3 +68,23 @@ def test_dense_sets_queue_by_queue(lib, name):
     got = lib.hull_batched(pts, off)
     for i, s in enumerate(sets):
         np.testing.assert_array_equal(got[i].cpu().numpy(), oracle.hull(s), err_msg=str(i))
+
+
+SINGLE = dict(CASES)
+SINGLE.update({
+    "tiles": lambda: [W.ring(8_000_001, 4), W.distorted(20_000_003, 5)],
+    "tiles without a polygon": lambda: [_shuffled([_arc(4095)] * 12, 6), _shuffled([_columns(4000)] * 2, 7)],
+    "a tile in pieces": lambda: [_shuffled([_arc(100)] * 4000, 8)],
+})
+
+
+@pytest.mark.parametrize("name", list(SINGLE))
+def test_single_hull_queue_by_queue(lib, name):
+    for i, s in enumerate(SINGLE[name]()):
+        pts = torch.from_numpy(s).cuda()
+        want = oracle.hull(s)
+        out_idx = torch.empty(s.shape[0], dtype=torch.int32, device="cuda")
+        out_n = torch.empty(1, dtype=torch.int64, device="cuda")
+        for _ in range(3):   # launched, captured, replayed
+            got = lib.hull(pts, out_idx=out_idx, out_n=out_n)
+            np.testing.assert_array_equal(got.cpu().numpy(), want, err_msg=str(i))
