@@ -116,7 +116,8 @@ int ch_hull_batched(const float* pts, const int64_t* offsets, int32_t k,
  * (current device) did per set, for measurement and tests: for set i,
  *   out[4 i]      records handed to the hull stage (the filter's survivors,
  *                 the chain end points included),
- *   out[4 i + 1]  vertices of the star polygon that filtered the set (0 when
+ *   out[4 i + 1]  vertices of the star polygon that filtered the set, those in
+ *                 its reflex dents (dropped before use) included (0 when
  *                 none: a sparse set, a set under 16384 points, or a polygon
  *                 that failed its checks),
  *   out[4 i + 2]  the set's status (CH_OK or a negative ch_status),
@@ -250,13 +251,15 @@ int ch_reserve(int64_t n, int32_t k, void* stream);
  *           discard against the sample's polygon),
  *   out[1]  sort records handed to the hull stage (the chain end points
  *           included): the survivors of the filter,
- *   out[2]  0 when one streaming pass did the extremes and the filter, 1 when
- *           a second pass classified every point,
+ *   out[2]  0 when the fused streaming pass did the extremes and the octagon
+ *           filter; 1 when a second pass did the filter (small inputs, and
+ *           dense data without a star polygon) or a star polygon did (out[5]),
  *   out[3]  hull stage: 0 finished by one block (few records), 1 bucketed
  *           chains, 2 the radix-sort fallback,
  *   out[4]  the call's status (CH_OK or the negative code it reported),
- *   out[5]  vertices of the star polygon that filtered dense data (0 when
- *           the call built none)
+ *   out[5]  vertices of the star polygon that filtered dense data, those in
+ *           its reflex dents (dropped before use) included (0 when the call
+ *           built none)
  * and returns how many counters exist (6).  Synchronises the stream.
  * CH_EINVAL when no hull ran on that stream (or out is NULL).
  */

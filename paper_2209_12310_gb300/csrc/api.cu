@@ -18,7 +18,7 @@ namespace ch {
 // Device information (SM count, resident blocks per SM of every kernel).
 struct DevInfo {
     int sms = 0;
-    int occ_main = 1, occ_post = 1, occ_lab = 1, occ_sort = 1, occ_chain = 1;
+    int occ_main = 1, occ_post = 1, occ_lab = 1, occ_sort = 1;
 };
 
 static std::mutex g_mu;
@@ -33,17 +33,14 @@ static int device_info(int dev, DevInfo* out) {
     if (configure_hull_kernels() != cudaSuccess) return CH_ECUDA;
     if (configure_filter_kernels() != cudaSuccess) return CH_ECUDA;
     if (configure_post_kernel() != cudaSuccess) return CH_ECUDA;
-    if (configure_queue_kernels() != cudaSuccess) return CH_ECUDA;
-    if (configure_star_kernel() != cudaSuccess) return CH_ECUDA;
+    if (configure_large_kernel() != cudaSuccess) return CH_ECUDA;
     if (occupancy_filter(&di.occ_main, &di.occ_lab) != cudaSuccess) return CH_ECUDA;
     if (occupancy_post(&di.occ_post) != cudaSuccess) return CH_ECUDA;
     if (occupancy_sort(&di.occ_sort) != cudaSuccess) return CH_ECUDA;
-    if (occupancy_chain(&di.occ_chain) != cudaSuccess) return CH_ECUDA;
     di.occ_main = std::max(1, di.occ_main);
     di.occ_post = std::max(1, di.occ_post);
     di.occ_lab = std::max(1, di.occ_lab);
     di.occ_sort = std::max(1, di.occ_sort);
-    di.occ_chain = std::max(1, di.occ_chain);
     g_dev[dev] = di;
     *out = di;
     return CH_OK;
@@ -70,9 +67,10 @@ Layout make_layout(long long n) {
     L.off_ctl = take(sizeof(Ctl));
     L.off_status = take(8 * (size_t)kDigits * L.sort_tiles);
     L.off_counters = take(4 * (size_t)kMaxLevels * L.ctcap);
-    L.off_star_bins = take(star_bins_bytes());   // the star and post passes leave them at zero
-    L.off_tiles = take(tiles_bytes());           // tile_hist_kernel leaves its counters at zero
+    L.off_star_bins = take(star_bins_bytes());   // dense_kernel leaves them at zero
+    L.off_tiles = take(tiles_bytes());           // large_kernel leaves its counters at zero
     L.zero_bytes = o;
+    L.off_star_poly = take(star_poly_bytes());
     L.off_kA = take(4 * (size_t)L.cap);
     L.off_kB = take(4 * (size_t)L.cap);
     L.off_vA = take(8 * (size_t)L.cap);
@@ -92,10 +90,6 @@ struct Workspace {
     // staging for the host-buffer entry point
     char* stage = nullptr;
     size_t stage_bytes = 0;
-    // the star pass's branch: a stream of its own, forked from and joined
-    // back into the caller's stream by two events
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
 static std::map<std::pair<int, cudaStream_t>, Workspace> g_ws;
@@ -109,7 +103,6 @@ static int grow_workspace(Workspace& ws, long long n, cudaStream_t s, int dev) {
     const Layout L = make_layout(want);
     if (ws.base) {
         cudaStreamSynchronize(s);
-        if (ws.side) cudaStreamSynchronize(ws.side);
         cudaFree(ws.base);
         ws.base = nullptr;
         ws.bytes = 0;
@@ -142,12 +135,8 @@ int get_workspace(int dev, cudaStream_t s, long long n, char** base, Layout* L) 
 
 static void free_workspace(Workspace& w, cudaStream_t s) {
     cudaStreamSynchronize(s);
-    if (w.side) cudaStreamSynchronize(w.side);
     if (w.base) cudaFree(w.base);
     if (w.stage) cudaFree(w.stage);
-    if (w.ev_fork) cudaEventDestroy(w.ev_fork);
-    if (w.ev_join) cudaEventDestroy(w.ev_join);
-    if (w.side) cudaStreamDestroy(w.side);
     w = Workspace();
 }
 
@@ -160,32 +149,6 @@ void release_stream_workspace(int dev, cudaStream_t s) {
     drop_graphs(dev, s);
     free_workspace(it->second, s);
     g_ws.erase(it);
-}
-
-// The star pass's stream and events of (dev, s), created on first use;
-// false when they cannot be (the hull then runs without the star pass).
-static bool get_side(int dev, cudaStream_t s, cudaStream_t* side, cudaEvent_t* fork, cudaEvent_t* join) {
-    std::lock_guard<std::mutex> lk(g_mu);
-    Workspace& ws = g_ws[std::make_pair(dev, s)];
-    if (!ws.side) {
-        cudaStream_t st = nullptr;
-        cudaEvent_t a = nullptr, b = nullptr;
-        if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&a, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&b, cudaEventDisableTiming) != cudaSuccess) {
-            if (st) cudaStreamDestroy(st);
-            if (a) cudaEventDestroy(a);
-            cudaGetLastError();
-            return false;
-        }
-        ws.side = st;
-        ws.ev_fork = a;
-        ws.ev_join = b;
-    }
-    *side = ws.side;
-    *fork = ws.ev_fork;
-    *join = ws.ev_join;
-    return true;
 }
 
 static int get_stage(int dev, cudaStream_t s, size_t bytes, char** out) {
@@ -267,192 +230,72 @@ static void prof_drain() {
 }
 
 // ---------------------------------------------------------------------------
-// The launch sequence of one hull (n >= 1) on an allocated workspace, in two
-// parts: the filter (init .. post), after which small survivor sets are done,
-// and the large-survivor path (queues, tiles, the sort).  `cond`, when
-// non-zero, is a graph condition the post pass sets when the second part has
-// work (see the CUDA-graph cache below).
-struct HullLaunch {
+// The launch sequence of one hull (n >= 1) on an allocated workspace: one chain
+// of kernels, each of which returns at once when the call does not need it (the
+// dense part on sparse data, the main pass on dense data, the large-survivor
+// paths not taken).  What a call may need beyond the sparse path is packed in
+// three cooperative kernels with grid barriers inside: an empty launch costs
+// about 2 us, and a conditional graph node about 7 (measured on 65,537 points:
+// 50 us a call with one such node, 57 with two).
+static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s,
+                               int dev, char* base, const Layout& L) {
     DevInfo di;
-    Ctl* ctl;
-    uint32_t *kA, *kB;
-    uint64_t *vA, *vB;
-    int head;
-    long long ntiles;
-    // the star pass (dense data): its branch and its buffers; side is null
-    // when the input is too small for it
-    cudaStream_t side;
-    cudaEvent_t ev_fork, ev_join;
-    void* star_bins;
-};
-
-// Inputs below this many warp tiles skip the star pass.
-constexpr long long kStarMinTiles = 256;
-
-// owner: the caller's stream, whose workspace (and star branch) the launches use.
-static int hull_setup(const float* pts, long long n, int dev, cudaStream_t owner, char* base, const Layout& L,
-                      HullLaunch* h) {
-    int st = device_info(dev, &h->di);
+    const int st = device_info(dev, &di);
     if (st != CH_OK) return st;
-    h->ctl = (Ctl*)(base + L.off_ctl);
-    h->kA = (uint32_t*)(base + L.off_kA);
-    h->kB = (uint32_t*)(base + L.off_kB);
-    h->vA = (uint64_t*)(base + L.off_vA);
-    h->vB = (uint64_t*)(base + L.off_vB);
-    h->head = (((uintptr_t)pts & 15u) != 0u && n > 0) ? 1 : 0;
-    h->ntiles = (n - h->head) / kWarpTilePts;
-    h->star_bins = base + L.off_star_bins;
-    h->side = nullptr;
-    h->ev_fork = h->ev_join = nullptr;
-    if (h->ntiles >= kStarMinTiles && !get_side(dev, owner, &h->side, &h->ev_fork, &h->ev_join)) h->side = nullptr;
-    return CH_OK;
-}
-
-static void enqueue_filter_part(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s,
-                                const HullLaunch& h, unsigned long long cond) {
-    const long long samples = sample_tiles_host(h.ntiles);
+    Ctl* ctl = (Ctl*)(base + L.off_ctl);
+    uint32_t *kA = (uint32_t*)(base + L.off_kA), *kB = (uint32_t*)(base + L.off_kB);
+    uint64_t *vA = (uint64_t*)(base + L.off_vA), *vB = (uint64_t*)(base + L.off_vB);
+    const int head = ((uintptr_t)pts & 15u) != 0u ? 1 : 0;
+    const long long ntiles = (n - head) / kWarpTilePts;
+    const long long samples = sample_tiles_host(ntiles);
     const int grid_sample = (int)std::max<long long>(1, std::min<long long>(256, (samples + 7) / 8));
-    // Raw survivors of the fused pass live in the B buffers until the post
-    // pass has turned them into sort records in the A buffers.
-    uint64_t* raw_xy = h.vB;
-    uint32_t* raw_idx = h.kB;
+    // Raw survivors live in the B buffers until the post pass has turned them
+    // into sort records in the A buffers.
     const unsigned switch_at = (unsigned)std::max<long long>(1 << 16, n >> 5);
-    { ProfScope p("init", s); launch_init(h.ctl, 0, s); }
-    { ProfScope p("sample", s); launch_sample(pts, n, h.head, h.ntiles, h.ctl, grid_sample, s); }
-    // The star pass needs only the sample octagon: it runs on its own branch
-    // beside the main pass, and the post pass waits for both.  The main pass
-    // is enqueued first, so that its blocks are placed before the star pass's.
-    const bool star = h.side != nullptr;
-    if (star) cudaEventRecord(h.ev_fork, s);
-    {
+    const bool dense = ntiles >= kStarMinTiles;   // large enough for a star polygon
+    // Inputs that stay in L2 take two passes: the extremes, then the filter
+    // against their octagon.  Larger ones take one, with a sample's octagon.
+    const bool two_pass = n <= kTwoPassMax;
+    if (two_pass) {
+        { ProfScope p("init", s); launch_init(ctl, 1, s); }
         ProfScope p("main_filter", s);
-        launch_main(pts, n, h.head, h.ntiles, h.ctl, raw_xy, raw_idx, switch_at, h.kA, h.vA,
-                    h.di.sms * h.di.occ_main, s);
+        launch_main(pts, n, head, ntiles, ctl, nullptr, nullptr, switch_at, kA, vA, 1, di.sms * di.occ_main, s);
+    } else {
+        ProfScope p("sample", s);
+        launch_sample(pts, n, head, ntiles, ctl, dense ? switch_at : 0xFFFFFFFFu, grid_sample, s);
     }
-    if (star) {
-        cudaStreamWaitEvent(h.side, h.ev_fork, 0);
-        {
-            ProfScope p("star", h.side);
-            launch_star(pts, n, h.head, h.ntiles, h.ctl, h.star_bins, h.di.sms, h.side);
-        }
-        cudaEventRecord(h.ev_join, h.side);
-        cudaStreamWaitEvent(s, h.ev_join, 0);
+    if (dense) {
+        ProfScope p("dense_filter", s);
+        launch_dense(pts, n, head, ntiles, ctl, base + L.off_star_bins, base + L.off_star_poly, vB, kB, kA, vA, di.sms,
+                     s);
+    }
+    if (!two_pass) {
+        ProfScope p("main_filter", s);
+        launch_main(pts, n, head, ntiles, ctl, vB, kB, switch_at, kA, vA, 0, di.sms * di.occ_main, s);
     }
     {
         ProfScope p("post", s);
-        launch_post(pts, n, h.head, h.ntiles, h.ctl, raw_xy, raw_idx, h.kA, h.vA, out_idx, out_n,
-                    star ? h.star_bins : nullptr, cond, h.di.sms * h.di.occ_post, s);
+        launch_post(pts, n, head, ntiles, ctl, vB, kB, kA, vA, out_idx, out_n, di.sms * di.occ_post, s);
     }
-}
-
-// The large-survivor part of a call: the queues that fit a block each (bodies
-// & 1), the tiled queues and the sort (bodies & 2).  Each kernel returns at once
-// when the call took another path; a captured graph holds the two bodies apart
-// and runs the one that the post pass chose.
-static void enqueue_large_part(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s,
-                               char* base, const Layout& L, const HullLaunch& h, int bodies) {
-    Ctl* ctl = h.ctl;
-    unsigned long long* status = (unsigned long long*)(base + L.off_status);
     unsigned* tiles = (unsigned*)(base + L.off_tiles);
     int *cu = (int*)(base + L.off_cu), *cv = (int*)(base + L.off_cv), *ci = (int*)(base + L.off_ci);
-    if (bodies & 2) launch_tiles(ctl, h.kA, h.vA, h.kB, h.vB, tiles, cu, cv, ci, h.di.sms, s);
-    launch_queues(ctl, h.kA, h.vA, h.kB, h.vB, tiles, cu, cv, ci, n, out_idx, out_n, s);
-    if (!(bodies & 2)) return;
+    const bool large = n + 16 > kQueueCap;   // else every queue fits a block
     {
+        ProfScope p("large", s);
+        launch_large(ctl, kA, vA, kB, vB, tiles, cu, cv, ci, n, out_idx, out_n, large ? di.sms : 4, s);
+    }
+    if (large) {
         ProfScope p("sort", s);
-        const int grid_sort = h.di.sms * h.di.occ_sort;
-        launch_sort_hist(h.kA, ctl, h.di.sms, s);
-        launch_sort_pass(h.kA, h.vA, h.kB, h.vB, ctl, status, 0, grid_sort, s);
-        launch_sort_pass(h.kB, h.vB, h.kA, h.vA, ctl, status, 1, grid_sort, s);
-        launch_sort_pass(h.kA, h.vA, h.kB, h.vB, ctl, status, 2, grid_sort, s);
+        launch_sort(ctl, kA, vA, kB, vB, (unsigned long long*)(base + L.off_status), cu, cv, ci,
+                    (int*)(base + L.off_clen), (int*)(base + L.off_counters), (int)L.ctcap, pts, n, out_idx, out_n,
+                    di.sms * di.occ_sort, s);
     }
-    {
-        ProfScope p("hull_chains", s);
-        launch_chain(ctl, h.kB, h.vB, cu, cv, ci, (int*)(base + L.off_clen), (int*)(base + L.off_counters),
-                     (int)L.ctcap, (int*)h.vA, (int*)h.kA, (int*)h.kB, (int*)h.vB, pts, n, out_idx, out_n,
-                     h.di.sms * h.di.occ_chain, s);
-    }
-}
-
-static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s,
-                               int dev, char* base, const Layout& L, cudaStream_t owner) {
-    HullLaunch h;
-    const int st = hull_setup(pts, n, dev, owner, base, L, &h);
-    if (st != CH_OK) return st;
-    enqueue_filter_part(pts, n, out_idx, out_n, s, h, 0ull);
-    enqueue_large_part(pts, n, out_idx, out_n, s, base, L, h, 3);
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ECUDA;
-}
-
-// Captures the sequence on `cs` with the large-survivor part as the two bodies
-// of a conditional (switch) node whose value the post pass sets; replays of
-// small-survivor calls then launch only the filter part (the default value
-// names no body).  False when any step
-// of the capture fails (the caller then captures the plain sequence).
-static bool capture_conditional(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t cs,
-                                int dev, char* base, const Layout& L, cudaStream_t owner, cudaGraph_t* out) {
-    HullLaunch h;
-    if (hull_setup(pts, n, dev, owner, base, L, &h) != CH_OK) return false;
-    if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
-    bool ok = true;
-    cudaGraph_t graph = nullptr;
-    cudaGraphConditionalHandle cond = 0;
-    cudaStream_t bs = nullptr;
-    {
-        cudaStreamCaptureStatus stc;
-        unsigned long long id = 0;
-        const cudaGraphNode_t* deps = nullptr;
-        const cudaGraphEdgeData* edata = nullptr;
-        size_t ndeps = 0;
-        ok = cudaStreamGetCaptureInfo(cs, &stc, &id, &graph, &deps, &edata, &ndeps) == cudaSuccess && graph;
-        if (ok) ok = cudaGraphConditionalHandleCreate(&cond, graph, 2u, cudaGraphCondAssignDefault) == cudaSuccess;
-    }
-    if (ok) {
-        enqueue_filter_part(pts, n, out_idx, out_n, cs, h, (unsigned long long)cond);
-        cudaStreamCaptureStatus stc;
-        unsigned long long id = 0;
-        const cudaGraphNode_t* deps = nullptr;
-        const cudaGraphEdgeData* edata = nullptr;
-        size_t ndeps = 0;
-        ok = cudaStreamGetCaptureInfo(cs, &stc, &id, &graph, &deps, &edata, &ndeps) == cudaSuccess;
-        cudaGraphNode_t node = nullptr;
-        cudaGraphNodeParams np = {};
-        if (ok) {
-            np.type = cudaGraphNodeTypeConditional;
-            np.conditional.handle = cond;
-            np.conditional.type = cudaGraphCondTypeSwitch;
-            np.conditional.size = 2;
-            ok = cudaGraphAddNode(&node, graph, deps, edata, ndeps, &np) == cudaSuccess;
-        }
-        if (ok) ok = cudaStreamUpdateCaptureDependencies(cs, &node, nullptr, 1, cudaStreamSetCaptureDependencies) ==
-                     cudaSuccess;
-        if (ok) ok = cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking) == cudaSuccess;
-        for (int b = 0; ok && b < 2; ++b) {
-            cudaGraph_t body = np.conditional.phGraph_out[b];
-            ok = cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
-                 cudaSuccess;
-            if (ok) {
-                enqueue_large_part(pts, n, out_idx, out_n, bs, base, L, h, 1 << b);
-                cudaGraph_t tmp = nullptr;
-                ok = cudaStreamEndCapture(bs, &tmp) == cudaSuccess;
-            }
-        }
-    }
-    cudaGraph_t g = nullptr;
-    const bool ended = cudaStreamEndCapture(cs, &g) == cudaSuccess;
-    if (bs) cudaStreamDestroy(bs);
-    if (!ok || !ended || !g) {
-        if (g) cudaGraphDestroy(g);
-        cudaGetLastError();
-        return false;
-    }
-    *out = g;
-    return true;
 }
 
 // ---------------------------------------------------------------------------
 // CUDA-graph cache.  A call repeated with the same (device, stream, points,
-// n, outputs, workspace) replays one captured graph instead of ~10 separate
+// n, outputs, workspace) replays one captured graph instead of separate
 // launches.  The first call of a key runs directly; the second captures the
 // sequence on a private stream and instantiates it; later ones replay it.
 // Disabled while profiling (per-kernel events) and when the caller's stream
@@ -507,7 +350,7 @@ int enqueue_hull_nograph(const float* pts, long long n, int32_t* out_idx, int64_
     Layout L;
     const int st = get_workspace(dev, s, n, &base, &L);
     if (st != CH_OK) return st;
-    return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L, s);
+    return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L);
 }
 
 int enqueue_hull(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s, int dev) {
@@ -521,7 +364,7 @@ int enqueue_hull(const float* pts, long long n, int32_t* out_idx, int64_t* out_n
     if (st != CH_OK) return st;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (g_prof || cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
-        return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L, s);
+        return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L);
     const GraphKey key{dev, s, pts, n, out_idx, out_n, base};
     cudaGraphExec_t exec = nullptr;
     {
@@ -529,30 +372,27 @@ int enqueue_hull(const float* pts, long long n, int32_t* out_idx, int64_t* out_n
         GraphEntry& e = g_graphs[key];
         e.last_use = ++g_graph_clock;
         if (e.exec) exec = e.exec;
-        else if (e.seen++ == 0) return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L, s);
+        else if (e.seen++ == 0) return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L);
     }
     if (exec) return cudaGraphLaunch(exec, s) == cudaSuccess ? CH_OK : CH_ECUDA;
     // Second call of this key: capture on a private stream, then replay.
     cudaStream_t cs = nullptr;
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
-        return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L, s);
+        return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L);
     }
     cudaGraph_t graph = nullptr;
-    bool ok = capture_conditional(pts, n, out_idx, out_n, cs, dev, base, L, s, &graph);
-    if (!ok) {   // plain capture of the whole sequence
-        ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (ok) {
-            st = enqueue_hull_direct(pts, n, out_idx, out_n, cs, dev, base, L, s);
-            ok = cudaStreamEndCapture(cs, &graph) == cudaSuccess && st == CH_OK && graph;
-        }
+    bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+        st = enqueue_hull_direct(pts, n, out_idx, out_n, cs, dev, base, L);
+        ok = cudaStreamEndCapture(cs, &graph) == cudaSuccess && st == CH_OK && graph;
     }
     if (ok) ok = cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
     if (graph) cudaGraphDestroy(graph);
     cudaStreamDestroy(cs);
     if (!ok) {
         cudaGetLastError();
-        return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L, s);
+        return enqueue_hull_direct(pts, n, out_idx, out_n, s, dev, base, L);
     }
     {
         std::lock_guard<std::mutex> lk(g_graph_mu);
@@ -619,7 +459,7 @@ int ch_filter(const float* pts, int64_t n, int32_t* out_ext8, uint8_t* out_label
     { ProfScope p("init", s); launch_init(ctl, 1, s); }
     {
         ProfScope p("main_filter", s);
-        launch_main(pts, n, head, ntiles, ctl, nullptr, nullptr, 0xFFFFFFFFu, kA, vA, di.sms * di.occ_main, s);
+        launch_main(pts, n, head, ntiles, ctl, nullptr, nullptr, 0xFFFFFFFFu, kA, vA, 0, di.sms * di.occ_main, s);
     }
     if (out_labels || out_counts4) {
         ProfScope p("labels", s);
@@ -691,7 +531,7 @@ int ch_hull_counters(void* stream, int64_t* out, int cap) {
     const int64_t v[] = {
         (int64_t)c.count_raw,
         (int64_t)c.count,
-        (int64_t)c.mode,
+        (int64_t)(c.mode || c.star_final),
         (int64_t)(c.bk_state == 2 ? 2 : c.bk_state == 1 ? 1 : 0),
         (int64_t)c.status,
         (int64_t)(c.star_final ? c.star_k : 0),

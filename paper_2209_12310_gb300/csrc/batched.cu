@@ -791,14 +791,13 @@ __global__ void __launch_bounds__(kBStarBinThreads) bt_star_bin(BArgs a) {
 // set without one keeps star_k = 0 and is filtered by its octagon alone.
 constexpr int kBStarThreads = 512;
 constexpr size_t kBStarAOff = (sizeof(StarPoly) + 15) / 16 * 16;
-constexpr size_t kBStarSmem = kBStarAOff + (sizeof(int2) + sizeof(unsigned short)) * kStarBins;
+constexpr size_t kBStarSmem = kBStarAOff + sizeof(unsigned long long) * kStarBins;
 static_assert(sizeof(StarPoly) % 16 == 0, "the polygon is copied in 16-byte words");
 
 __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_build(BArgs a) {
     extern __shared__ __align__(16) char dyn[];
     StarPoly& P = *reinterpret_cast<StarPoly*>(dyn);
-    int2* va = reinterpret_cast<int2*>(dyn + kBStarAOff);
-    unsigned short* ba = reinterpret_cast<unsigned short*>(dyn + kBStarAOff + sizeof(int2) * kStarBins);
+    unsigned long long* work = reinterpret_cast<unsigned long long*>(dyn + kBStarAOff);
     __shared__ int s_set;
     const int tid = threadIdx.x;
     const unsigned listed = a.star_ctr[0];
@@ -814,7 +813,7 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_build(BArgs a) {
         const long long base = a.offsets[i], ni = a.offsets[i + 1] - base;
         const int slot = a.star_slot[i];
         const int K = star_finish<kBStarThreads>(a.star_bins + (size_t)slot * kStarBins, a.pts + 2 * base, ni,
-                                                 c->star_cx, c->star_cy, va, ba, P, c);
+                                                 c->star_cx, c->star_cy, work, P, c);
         if (K) {
             const int4* src = reinterpret_cast<const int4*>(&P);
             int4* dst = reinterpret_cast<int4*>(a.star_polys + slot);
@@ -969,7 +968,7 @@ __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
         }
         __syncthreads();
         const int cx = c->star_cx, cy = c->star_cy;
-        const long long r0 = P.rmin;
+        const float fcx = (float)cx, fcy = (float)cy, tmin = P.tmin;
         const float2* p2 = reinterpret_cast<const float2*>(a.pts) + base;
         unsigned cnt = 0u, qn = 0u;
         unsigned nq[4] = {0u, 0u, 0u, 0u};
@@ -991,12 +990,8 @@ __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
                 const long long j = s0 + u * kBDenseThreads + tid;
                 bool need = false;
                 if (j < hi) {
-                    const long long px = __float2int_rn(cur[u].x) - cx, py = __float2int_rn(cur[u].y) - cy;
-                    const long long d2 = px * px + py * py;
-                    if (d2 >= r0 * r0) {
-                        const long long rr = P.rin[star_bin((int)px, (int)py)];
-                        need = d2 >= rr * rr;
-                    }
+                    const float dx = cur[u].x - fcx, dy = cur[u].y - fcy;   // exact
+                    need = star_d2(dx, dy) >= tmin && !star_inside_fast(dx, dy, star_bin(dx, dy), P);
                 }
                 const unsigned bal = __ballot_sync(0xFFFFFFFFu, need);
                 if (need) {   // queued
@@ -1059,8 +1054,6 @@ __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
 // next step in flight while it works on the current one.
 constexpr int kBRefineU = 8;                    // records per lane and step
 constexpr unsigned kBRefineHuge = 1u << 16;     // records of the sets taken first
-static_assert(sizeof(unsigned long long) * kStarBins <= (sizeof(int2) + sizeof(unsigned short)) * kStarBins,
-              "the bins fit in work area A");
 
 // One step of a warp: records [r, r + 32 kBRefineU) of a range ending at hi,
 // record r + 32 u + lane in slot u.
@@ -1083,9 +1076,7 @@ __device__ __forceinline__ void bt_record_xy(uint32_t k, uint64_t v, int& X, int
 __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_refine(BArgs a) {
     extern __shared__ __align__(16) char dyn[];
     StarPoly& P = *reinterpret_cast<StarPoly*>(dyn);
-    unsigned long long* bins = reinterpret_cast<unsigned long long*>(dyn + kBStarAOff);
-    int2* va = reinterpret_cast<int2*>(dyn + kBStarAOff);
-    unsigned short* ba = reinterpret_cast<unsigned short*>(dyn + kBStarAOff + sizeof(int2) * kStarBins);
+    unsigned long long* bins = reinterpret_cast<unsigned long long*>(dyn + kBStarAOff);   // star_finish's work area too
     constexpr int kWarps = kBStarThreads / 32;
     constexpr unsigned kStep = 32u * kBRefineU;
     __shared__ unsigned s_kept, s_q[4];
@@ -1144,7 +1135,7 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_refine(BArgs a) {
         }
         __syncthreads();
         // 2. the polygon
-        const int K = star_finish<kBStarThreads, true>(bins, a.pts + 2 * base, ni, cx, cy, va, ba, P, c);
+        const int K = star_finish<kBStarThreads, true>(bins, a.pts + 2 * base, ni, cx, cy, bins, P, c);
         if (K == 0) {
             __syncthreads();
             continue;

@@ -67,10 +67,15 @@ __host__ __device__ __forceinline__ unsigned bk_buckets_for(unsigned cnt) {
     return nb > 0u ? nb : 1u;
 }
 constexpr int kSampleTiles = 1024;            // warp tiles read by the sample pass (512k points)
-// Star polygon of dense data (star.cu): angular bins around the sample
+// Star polygon of dense data (star.cuh, dense_kernel): angular bins around the sample
 // octagon's centre, extra warp tiles read when the sample is dense.
 constexpr int kStarBins = 8192;
 constexpr int kStarExtraTiles = 2048;
+constexpr long long kStarMinTiles = 128;      // inputs below this many warp tiles skip the star pass
+// Inputs of at most this many points stay in L2 between two passes, so the
+// extremes come first and no sample is needed (the fused pass saves reads of
+// HBM at the price of one more kernel in the chain).
+constexpr long long kTwoPassMax = 1 << 22;
 constexpr int kMaxLevels = 32;
 
 // Warp tiles read by the sample pass: about 1/32 of the input, at most
@@ -125,6 +130,7 @@ struct Ctl {
     int done;                           // the hull has been written by a small-path block
     int records_ready;                  // sort records complete before the re-classify stage
     unsigned int blocks_done[4];        // last-arriver counters (sample, main, stage C, roots)
+    unsigned int barrier[3];            // grid barriers (dense_kernel, large_kernel, sort_kernel)
     unsigned int tile_ctr[4];           // onesweep tile claim counters (0 .. 2), tile_chain_kernel's (3)
     unsigned int digit_hist[kSortPasses][kDigits];   // sort fallback only (sort_hist_kernel)
     unsigned int rec_q[4];              // records per queue
@@ -135,12 +141,12 @@ struct Ctl {
     int path;                           // the single hull's large-survivor path (Path)
     unsigned int q_tile[5];             // path tiles: tiles of queue r are [q_tile[r], q_tile[r + 1])
     int samp_ok;                        // oct_s holds this call's sample octagon
-    int star_ok;                        // the star pass found dense data: the post pass builds the polygon
-    int star_k;                         // the polygon's vertices (post pass)
-    int star_final;                     // the post pass built and accepted the polygon
+    int samp_dense;                     // dense data (oct_s: an octagon of input points): the star pass bins points
+    int oct_ready;                      // the octagon of the true extremes and the end-point records stand
+    int star_ok;                        // batched: the set is listed for a star polygon
+    int star_k;                         // the polygon's vertices, the dropped ones included
+    int star_final;                     // a polygon was built and accepted
     int star_cx, star_cy;               // its centre (vertices are stored relative to it)
-    unsigned int star_pts, star_out;    // points the star pass read / found outside the sample octagon
-    unsigned int star_done;             // last-arriver counter of the star pass
     Octagon oct;                        // octagon of the true extremes
     Octagon oct_s;                      // octagon of a sample's extremes
 #if defined(CH_TRACE) || defined(CH_TIMELINE)
@@ -190,6 +196,12 @@ __device__ __forceinline__ unsigned long long l2_evict_first() {
     return pol;
 }
 
+__device__ __forceinline__ unsigned long long l2_evict_normal() {
+    unsigned long long pol;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+
 __device__ __forceinline__ float4 ld_stream_f4(const float4* p, unsigned long long pol) {
     float4 r;
     asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
@@ -233,6 +245,30 @@ __device__ __forceinline__ bool spin_give_up(unsigned& spins, Ctl* ctl) {
     }
     __nanosleep(64);
     return false;
+}
+
+// Grid-wide barrier of a cooperative launch (all its blocks are resident): the
+// k-th (k = 1, 2, ...) use of the counter, which starts at zero.  Every wait is
+// bounded: false when it gave up (status CH_ETIMEOUT), and the kernel returns.
+// Whole block.
+__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned k, Ctl* ctl) {
+    __shared__ int s_ok;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned target = k * gridDim.x;
+        unsigned spins = 0u;
+        s_ok = 1;
+        atomicAdd(counter, 1u);
+        while (*(volatile unsigned*)counter < target)
+            if (spin_give_up(spins, ctl)) {
+                s_ok = 0;
+                break;
+            }
+        __threadfence();
+    }
+    __syncthreads();
+    return s_ok != 0;
 }
 
 __device__ __forceinline__ int read_status(const Ctl* ctl) {

@@ -1,7 +1,8 @@
 // filter.cu -- the filtering stage of GPU heaphull (Alg. 2, GPUfilter) on sm_103a.
 //
 // Kernels (in launch order):
-//   init_kernel     reset the per-call control block.
+//   init_kernel     reset the per-call control block (ch_filter; ch_hull's sample
+//                   pass does it).
 //   sample_kernel   extremes of an evenly spaced sample of warp tiles; its last
 //                   block builds the sample octagon (vertices are input points).
 //   main_kernel     findExtremes (Alg. 2; Sec. 3) over every point: all 8
@@ -17,6 +18,10 @@
 //                   stops filtering and the second pass does it (two-pass mode).
 //                   Its last block builds the octagon of the true extremes
 //                   and the records of the chain end points.
+//   dense_kernel    the main pass on dense data (an earlier pass's verdict):
+//                   the star polygon (star.cuh), then one streaming read that
+//                   validates the coordinates and drops the points strictly
+//                   inside the polygon; the extremes are among the others.
 //   (post.cu)       the classification of the survivors and the hull.
 //   labels_kernel   ch_filter: the label array Q of Alg. 2 (paper rule).
 #include "ch_internal.cuh"
@@ -24,6 +29,7 @@
 #include "launch.h"
 #include "extremes.cuh"
 #include "octagon.cuh"
+#include "star.cuh"
 #include "tma.cuh"
 
 #include <climits>
@@ -31,14 +37,22 @@
 namespace ch {
 
 // ---------------------------------------------------------------------------
-__global__ void init_kernel(Ctl* ctl, int mode) {
+// Resets the per-call control block (one block).  The fields that the sample
+// pass itself gathers in (samp_packed, blocks_done[0]) are at rest between
+// calls: its last block leaves them at zero.
+__device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
     const int t = threadIdx.x;
     if (t < 8) {
         ctl->ext_packed[t] = 0ull;
-        ctl->samp_packed[t] = 0ull;
         ctl->line_ep[t] = (t & 1) ? 0ull : ~0ull;   // even: minimum slot, odd: maximum slot
     }
-    if (t < 4) { ctl->tile_ctr[t] = 0u; ctl->counts4[t] = 0u; ctl->blocks_done[t] = 0u; ctl->rec_q[t] = 0u; }
+    if (t < 4) {
+        ctl->tile_ctr[t] = 0u;
+        ctl->counts4[t] = 0u;
+        ctl->rec_q[t] = 0u;
+        if (t) ctl->blocks_done[t] = 0u;
+        if (t < 3) ctl->barrier[t] = 0u;
+    }
     if (t == 0) {
         ctl->status = CH_OK;
         ctl->abort = 0;
@@ -51,23 +65,20 @@ __global__ void init_kernel(Ctl* ctl, int mode) {
         ctl->bk_state = 0;
         ctl->path = kPathNone;
         ctl->samp_ok = 0;
+        ctl->samp_dense = 0;
+        ctl->oct_ready = 0;
         ctl->star_ok = 0;
         ctl->star_k = 0;
         ctl->star_final = 0;
-        ctl->star_pts = 0u;
-        ctl->star_out = 0u;
-        ctl->star_done = 0u;
     }
     unsigned* h = &ctl->digit_hist[0][0];
     for (int i = t; i < kSortPasses * kDigits; i += blockDim.x) h[i] = 0u;
 #if defined(CH_TRACE) || defined(CH_TIMELINE)
     if (t < 14) { ctl->tl[t][0] = ~0ull; ctl->tl[t][1] = 0ull; }
-    __syncthreads();
-    CH_TL(ctl, 0, 0);
-    CH_TL(ctl, 0, 1);
 #endif
 }
 
+__global__ void init_kernel(Ctl* ctl, int mode) { reset_ctl(ctl, mode); }
 
 // ---------------------------------------------------------------------------
 // Sample pass: packed (key, other coordinate) maxima per direction; the other
@@ -80,14 +91,55 @@ __device__ __forceinline__ unsigned long long samp_pack(int d, int X, int Y) {
     return ((unsigned long long)hk << 32) | aux;
 }
 
+// Density test of the block that built the octagon o (256 threads): kDensePts
+// points spread over nspread warp tiles (tile(k), k < nspread); true when the
+// share of them outside o would give the main pass more raw survivors than it
+// gives up at (switch_at).  The points are loaded before the octagon is built,
+// so that their latency is hidden.
+constexpr int kDensePts = 2048;
+struct DenseProbe {
+    float2 p[kDensePts / 256];
+    template <class Tile>
+    __device__ __forceinline__ void load(const float4* p4, long long nspread, Tile tile) {
+#pragma unroll
+        for (int j = 0; j < kDensePts / 256; ++j) {
+            const long long k = (long long)(j * 256 + threadIdx.x) * nspread / kDensePts;
+            p[j] = __ldcg(reinterpret_cast<const float2*>(p4 + tile(k) * kWarpTileF4) +
+                          (37 * threadIdx.x + 64 * j) % kWarpTilePts);
+        }
+    }
+    __device__ __forceinline__ bool dense(const Octagon& o, long long n, unsigned switch_at) const {
+        __shared__ unsigned s_out;
+        __shared__ float s_e[24];
+        if (threadIdx.x < 8) {
+            s_e[3 * threadIdx.x] = o.oct[threadIdx.x].A;
+            s_e[3 * threadIdx.x + 1] = o.oct[threadIdx.x].B;
+            s_e[3 * threadIdx.x + 2] = o.oct[threadIdx.x].C;
+        }
+        if (threadIdx.x == 0) s_out = 0u;
+        __syncthreads();
+        unsigned out = 0u;
+#pragma unroll
+        for (int j = 0; j < kDensePts / 256; ++j)
+            out += in_inner(o, __float2int_rn(p[j].x), __float2int_rn(p[j].y)) || pt_in_sample(p[j].x, p[j].y, s_e)
+                       ? 0u
+                       : 1u;
+        out = __reduce_add_sync(0xFFFFFFFFu, out);
+        if ((threadIdx.x & 31) == 0 && out) atomicAdd(&s_out, out);
+        __syncthreads();
+        return (long long)s_out * n > (long long)kDensePts * switch_at;
+    }
+};
+
 __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ pts, long long n, int head,
-                                                     long long ntiles, Ctl* ctl) {
+                                                     long long ntiles, Ctl* ctl, unsigned switch_at) {
     __shared__ unsigned long long s_red[8][8];
     __shared__ Octagon s_o;
     __shared__ int s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long gwarp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    if (blockIdx.x == 0) reset_ctl(ctl, 0);   // for the kernels that follow, and for this one's last block
     CH_TL(ctl, 1, 0);
     unsigned long long best[8];
 #pragma unroll
@@ -136,11 +188,15 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ p
     CH_TRACE_MARK();
     __shared__ int s_v[2][8];
     __shared__ int s_ok;
+    const bool test = ntiles >= kStarMinTiles;
+    DenseProbe probe;
+    if (test) probe.load(p4, nsamp, [&](long long k) { return k * ntiles / nsamp; });
     if (threadIdx.x == 0) s_ok = nsamp > 0;
     __syncthreads();
     if (threadIdx.x < 8) {
         const int d = threadIdx.x;
         const unsigned long long p = *(volatile unsigned long long*)&ctl->samp_packed[d];
+        ctl->samp_packed[d] = 0ull;   // at rest again
         if (p == 0ull) atomicAnd(&s_ok, 0);
         const unsigned hk = (unsigned)(p >> 32), aux = (unsigned)p;
         const int key = dir_is_max(d) ? (int)hk : (int)(0xFFFFFFFFu - hk);
@@ -169,8 +225,16 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ p
         return;
     }
     copy_octagon(&ctl->oct_s, &s_o);
+    // Dense data (points near a circle) goes to the star pass and dense_kernel
+    // from the start; the main pass would find out by writing switch_at raw
+    // survivors, and all points would be read again.
+    const bool dense = test && !s_o.discard_none && probe.dense(s_o, n, switch_at);
     __syncthreads();
     if (threadIdx.x == 0) {
+        if (dense) {
+            ctl->samp_dense = 1;
+            ctl->mode = 1;
+        }
         __threadfence();
         ctl->samp_ok = 1;
     }
@@ -374,7 +438,7 @@ constexpr size_t kMainSmemBytes = (size_t)8 * kStages * kWarpTileF4 * sizeof(flo
 __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ pts, long long n, int head,
                                                       long long ntiles, Ctl* ctl, uint64_t* raw_xy,
                                                       uint32_t* raw_idx, unsigned switch_at, uint32_t* keys,
-                                                      uint64_t* vals) {
+                                                      uint64_t* vals, int two_pass) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ int s_inner[8];
     __shared__ float s_edge[24];
@@ -387,6 +451,7 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
     const long long gwarp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     CH_TL(ctl, 3, 0);
+    if (!two_pass && *(volatile int*)&ctl->samp_dense && *(volatile int*)&ctl->star_final) return;   // dense_kernel's
     if (threadIdx.x == 0) s_mode = *(volatile int*)&ctl->mode;   // one read: uniform per block
     if (threadIdx.x < 4) {
         s_inner[threadIdx.x] = ctl->oct_s.in_lo[threadIdx.x];
@@ -403,8 +468,8 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
     unsigned wcnt = 0u;
     Track tr;
     track_init(tr);
-    // Scalar ranges (warp 0): the unaligned head point first and the ragged
-    // tail last, so every lane visits tile codes in increasing order.
+    // Scalar ranges: the unaligned head point first and the ragged tail last,
+    // so every lane visits tile codes in increasing order.
     auto scalar_range = [&](long long lo_i, long long hi_i, unsigned code) {
         int tk[8];
         bool any = false;
@@ -430,7 +495,7 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
     // Warp tiles t = gwarp + k * nwarps stream through a double-buffered
     // shared-memory ring filled by bulk asynchronous copies (TMA).
     WarpStream ws{reinterpret_cast<float4*>(dsm) + warp * kStages * kWarpTileF4, s_bar[warp],
-                  reinterpret_cast<const float4*>(pts + 2 * head), gwarp, nwarps, ntiles, lane};
+                  reinterpret_cast<const float4*>(pts + 2 * head), gwarp, nwarps, ntiles, lane, two_pass != 0};
     ws.start();
     for (long long k = 0;; ++k) {
         const long long t = gwarp + k * nwarps;
@@ -500,8 +565,10 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
         }
         ws.release(k);
     }
-    if (gwarp == 0 && head + ntiles * kWarpTilePts < n)
-        scalar_range(head + ntiles * kWarpTilePts, n, (unsigned)(ntiles + 1));
+    // the ragged tail, 32 points per warp from the last warp down (one warp
+    // taking all of it is a chain of up to 16 dependent loads)
+    const long long tail = head + ntiles * kWarpTilePts + 32 * (nwarps - 1 - gwarp);
+    if (tail < n) scalar_range(tail, min(n, tail + 32), (unsigned)(ntiles + 1));
     flush_raw(wbuf, wcnt, ctl, raw_xy, raw_idx);
 
     const bool err = tr.bad || (tr.orv >> kCoordBits) != 0u;
@@ -531,9 +598,320 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
     CH_TRACE_DECL
     CH_TRACE_MARK();
     if (__syncthreads_or(read_status(ctl) != CH_OK)) return;
-    finalize_block(pts, n, head, ctl, *reinterpret_cast<Octagon*>(dsm), keys, vals);
+    // A call without a sample pass (two_pass) finds out here whether the data
+    // are dense, against the octagon of the true extremes.
+    const bool test = two_pass && ntiles >= kStarMinTiles;
+    DenseProbe probe;
+    if (test)
+        probe.load(reinterpret_cast<const float4*>(pts + 2 * head), kDensePts / 4,
+                   [&](long long k) { return k * ntiles / (kDensePts / 4); });
+    Octagon& o = *reinterpret_cast<Octagon*>(dsm);
+    finalize_block(pts, n, head, ctl, o, keys, vals);
+    if (test && read_status(ctl) == CH_OK && !o.discard_none && probe.dense(o, n, switch_at)) {
+        copy_octagon(&ctl->oct_s, &o);
+        if (threadIdx.x == 0) {
+            ctl->samp_dense = 1;
+            ctl->oct_ready = 1;
+        }
+    }
     CH_TRACE_PRINT("finalize");
     CH_TL(ctl, 4, 1);
+}
+
+// ---------------------------------------------------------------------------
+// The main pass on dense data (points near a circle, Table V), one cooperative
+// launch of one block per SM:
+//   1. the angular bins of the star polygon (star.cuh): the sample pass's
+//      tiles (still in L2) and kStarExtraTiles more, spread over the input.
+//      Every point outside oct_s goes to its angular bin around that octagon's
+//      centre c, where a 64-bit atomicMax keeps the point farthest from c (its
+//      squared distance, truncated, above its index); a point first reads its
+//      bin and issues the atomic only if it beats it;
+//   2. one block makes the polygon of the bins' points (star_finish) and clears
+//      the bins;
+//   3. one streaming read of all points.  A point closer to c than its bin's
+//      radius bound is strictly inside the polygon; the others wait in a
+//      per-warp queue and go 32 at a time through the exact wedge test; what
+//      that leaves are the raw survivors, classified by the post pass.  A point
+//      strictly inside the polygon is interior to the hull, so it reaches no
+//      extreme: the 8 extremes are tracked over the raw survivors alone.  Every
+//      coordinate is validated.
+// Without a polygon (its checks failed) the main pass and the post pass read
+// all points.  Before, the main pass's full tracking (143 us on 1e8 points)
+// ran beside 1, every block of the post pass did 2 (90 us) and the post pass 3
+// with integer distances (400 us).
+// Warp tile of the star pass's k-th read: the sample pass's tiles first, then
+// the extra tiles, half a stride away from an even spread.
+__device__ __forceinline__ long long star_tile(long long k, long long nsamp, long long nextra, long long ntiles) {
+    if (k < nsamp) return k * ntiles / nsamp;
+    const long long e = k - nsamp;
+    return ((2 * e + 1) * ntiles) / (2 * nextra);
+}
+
+// One warp tile: bins the points outside the sample octagon.
+__device__ __forceinline__ void star_tile_pass(const float4* __restrict__ p4, long long t, int head, const int* s_in,
+                                               const float* s_edge, int cx, int cy, unsigned long long* bins,
+                                               unsigned long long pol) {
+    const int lane = threadIdx.x & 31;
+    const float4* base = p4 + t * kWarpTileF4 + lane;
+    constexpr int kHalf = kLoadsPerLane / 2;   // half a tile's loads in flight keeps the registers low
+#pragma unroll 1
+    for (int j0 = 0; j0 < kLoadsPerLane; j0 += kHalf) {
+        float4 v[kHalf];
+#pragma unroll
+        for (int j = 0; j < kHalf; ++j) v[j] = ld_stream_f4(base + (j0 + j) * 32, pol);
+        // the keys of the points outside the sample octagon, then one load of
+        // each point's bin: only a point that beats the bin's current value
+        // issues the atomicMax (after a bin's first few points that is rare,
+        // so far fewer atomics meet at each bin)
+        unsigned long long key[2 * kHalf];
+        int bin[2 * kHalf];
+#pragma unroll
+        for (int j = 0; j < kHalf; ++j) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float x = h ? v[j].z : v[j].x, y = h ? v[j].w : v[j].y;
+                const int X = __float2int_rn(x), Y = __float2int_rn(y);
+                const bool out = !pt_in_inner(X, Y, s_in) && !pt_in_sample(x, y, s_edge);
+                const int dx = X - cx, dy = Y - cy;
+                const unsigned long long d2 = (unsigned long long)((long long)dx * dx + (long long)dy * dy);
+                const unsigned idx = (unsigned)(head + t * kWarpTilePts + 2 * ((j0 + j) * 32 + lane) + h);
+                key[2 * j + h] = out ? ((d2 >> 17) << 32) | idx : 0ull;
+                bin[2 * j + h] = star_bin(dx, dy);
+            }
+        }
+        unsigned long long cur[2 * kHalf];
+#pragma unroll
+        for (int i = 0; i < 2 * kHalf; ++i) cur[i] = key[i] ? __ldcg(bins + bin[i]) : ~0ull;
+#pragma unroll
+        for (int i = 0; i < 2 * kHalf; ++i)
+            if (key[i] > cur[i]) atomicMax(&bins[bin[i]], key[i]);
+    }
+}
+
+constexpr int kDenseThreads = 512;
+constexpr int kDenseQueue = 96;   // < 32 waiting + 64 added per step
+struct DenseWarp {
+    RawBuf raw;
+    float x[kDenseQueue], y[kDenseQueue];
+    unsigned idx[kDenseQueue];
+    unsigned cnt;                 // raw survivors staged
+    int best[8];                  // the warp's extreme keys so far and the
+    unsigned code[8];             // first tile where each occurred
+};
+constexpr size_t kDenseWarpOff = (sizeof(StarPoly) + 15) / 16 * 16;
+constexpr size_t kDenseSmemBytes = kDenseWarpOff + (kDenseThreads / 32) * sizeof(DenseWarp);
+static_assert((kDenseThreads / 32) * sizeof(DenseWarp) >= sizeof(unsigned long long) * kStarBins, "star_finish's work area");
+static_assert(sizeof(StarPoly) % 16 == 0, "the polygon is copied in 16-byte words");
+
+// Warp-collective, out of line: the queued points [first, first + count),
+// count <= 32.
+__device__ __noinline__ void dense_drain(const StarPoly& P, int cx, int cy, DenseWarp& w, unsigned first,
+                                         unsigned count, int head, Ctl* ctl, uint64_t* raw_xy, uint32_t* raw_idx) {
+    const int lane = threadIdx.x & 31;
+    const bool valid = (unsigned)lane < count;
+    const float x = valid ? w.x[first + lane] : 0.0f, y = valid ? w.y[first + lane] : 0.0f;
+    const unsigned idx = valid ? w.idx[first + lane] : 0u;
+    const int X = __float2int_rn(x), Y = __float2int_rn(y);
+    const bool keep = valid && !star_inside_exact(X - cx, Y - cy, star_bin(x - (float)cx, y - (float)cy), P);
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
+    if (!bal) return;
+    // tile code as in extremes.cuh: 0 = head, t + 1 = body tile t or the tail
+    const unsigned code = idx < (unsigned)head ? 0u : (idx - (unsigned)head) / (unsigned)kWarpTilePts + 1u;
+    bool better = false;
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {
+        const int key = dir_key(d, X, Y), b = w.best[d];
+        better |= dir_is_max(d) ? key > b : key < b;
+        better |= key == b && code < w.code[d];
+    }
+    if (__any_sync(0xFFFFFFFFu, keep && better)) {
+        __syncwarp();
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            const unsigned key = (unsigned)dir_key(d, X, Y);
+            const unsigned m = dir_is_max(d) ? __reduce_max_sync(0xFFFFFFFFu, keep ? key : 0u)
+                                             : __reduce_min_sync(0xFFFFFFFFu, keep ? key : 0xFFFFFFFFu);
+            const unsigned c = __reduce_min_sync(0xFFFFFFFFu, keep && key == m ? code : 0xFFFFFFFFu);
+            if (lane == 0) {
+                const int b = w.best[d];
+                const bool up = dir_is_max(d) ? (int)m > b : (int)m < b;
+                if (up || ((int)m == b && c < w.code[d])) {
+                    w.best[d] = (int)m;
+                    w.code[d] = c;
+                }
+            }
+        }
+    }
+    unsigned cnt = w.cnt;
+    if (cnt + (unsigned)__popc(bal) > (unsigned)kWarpBuf) flush_raw(w.raw, cnt, ctl, raw_xy, raw_idx);
+    if (keep) {
+        const unsigned pos = cnt + __popc(bal & lanemask_lt());
+        w.raw.xy[pos] = ((unsigned long long)(unsigned)X << 32) | (unsigned)Y;
+        w.raw.idx[pos] = idx;
+    }
+    __syncwarp();
+    if (lane == 0) w.cnt = cnt + (unsigned)__popc(bal);
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __restrict__ pts, long long n, int head,
+                                                                 long long ntiles, Ctl* ctl, unsigned long long* bins,
+                                                                 StarPoly* poly, uint64_t* raw_xy, uint32_t* raw_idx,
+                                                                 uint32_t* keys, uint64_t* vals) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ unsigned long long s_red[kDenseThreads / 32][8];
+    __shared__ int s_flag, s_in[8];
+    __shared__ float s_edge[24];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kWarps = kDenseThreads / 32;
+    if (tid == 0) s_flag = *(volatile int*)&ctl->samp_dense && read_status(ctl) == CH_OK;
+    __syncthreads();
+    if (!s_flag) return;
+    const Octagon& os = ctl->oct_s;
+    const int cx = (os.vx[W] + os.vx[E]) / 2, cy = (os.vy[S] + os.vy[N]) / 2;
+    const float4* p4 = reinterpret_cast<const float4*>(pts + 2 * head);
+    const unsigned long long pol = l2_evict_first();
+    {   // 1. bins
+        if (tid < 4) {
+            s_in[tid] = os.in_lo[tid];
+            s_in[4 + tid] = os.in_hi[tid];
+        }
+        if (tid < 8) {
+            s_edge[3 * tid] = os.oct[tid].A;
+            s_edge[3 * tid + 1] = os.oct[tid].B;
+            s_edge[3 * tid + 2] = os.oct[tid].C;
+        }
+        __syncthreads();
+        const long long nsamp = sample_tiles(ntiles);
+        const long long nextra = ntiles < kStarExtraTiles ? ntiles : kStarExtraTiles;
+        // tile k belongs to block k % grid, warp (k / grid) % kWarps
+        for (long long k = blockIdx.x + (long long)gridDim.x * warp; k < nsamp + nextra;
+             k += (long long)gridDim.x * kWarps)
+            star_tile_pass(p4, star_tile(k, nsamp, nextra, ntiles), head, s_in, s_edge, cx, cy, bins, pol);
+        CH_TL(ctl, 7, 1);
+        if (!grid_barrier(&ctl->barrier[0], 1u, ctl)) return;
+    }
+    const StarPoly& P = *reinterpret_cast<const StarPoly*>(dsm);
+    if (blockIdx.x == 0) {   // 2. polygon
+        StarPoly& M = *reinterpret_cast<StarPoly*>(dsm);
+        const int K = star_finish<kDenseThreads>(bins, pts, n, cx, cy,
+                                                 reinterpret_cast<unsigned long long*>(dsm + kDenseWarpOff), M, ctl);
+        __syncthreads();
+        if (K)
+            for (int j = tid; j < (int)(sizeof(StarPoly) / 16); j += kDenseThreads)
+                reinterpret_cast<int4*>(poly)[j] = reinterpret_cast<const int4*>(dsm)[j];
+        for (int b = tid; b < kStarBins; b += kDenseThreads) bins[b] = 0ull;   // at rest again
+        if (tid == 0) {
+            ctl->star_k = K;
+            ctl->star_cx = cx;
+            ctl->star_cy = cy;
+            ctl->star_final = K ? 1 : 0;
+        }
+        CH_TL(ctl, 8, 1);
+    }
+    if (!grid_barrier(&ctl->barrier[0], 2u, ctl)) return;
+    if (!*(volatile int*)&ctl->star_final) return;
+    // 3. the filter
+    if (blockIdx.x != 0) {
+        const int4* src = reinterpret_cast<const int4*>(poly);
+        int4* dst = reinterpret_cast<int4*>(dsm);
+        for (int j = tid; j < (int)(sizeof(StarPoly) / 16); j += kDenseThreads) dst[j] = __ldcg(src + j);
+    }
+    DenseWarp& w = reinterpret_cast<DenseWarp*>(dsm + kDenseWarpOff)[warp];
+    if (lane == 0) w.cnt = 0u;
+    if (lane < 8) {
+        w.best[lane] = dir_is_max(lane) ? INT_MIN : INT_MAX;
+        w.code[lane] = 0u;
+    }
+    __syncthreads();
+    const float fcx = (float)cx, fcy = (float)cy;
+    const long long first = ((long long)blockIdx.x * kDenseThreads + tid) >> 5;
+    const long long stride = ((long long)gridDim.x * kDenseThreads) >> 5;
+    const unsigned lt = lanemask_lt();
+    unsigned qn = 0u;   // points queued (warp-uniform)
+    bool bad = false;
+    float lowest = 0.0f, highest = 0.0f;
+    // x is an integer or at least 2^23 in magnitude when adding and taking
+    // away 2^24 leaves it alone (NaN does not); with the range check this is
+    // convert_pt's validity without integer conversions
+    auto check = [&](float x, float y) {
+        bad |= __fadd_rn(__fadd_rn(x, -16777216.0f), 16777216.0f) != x;
+        bad |= __fadd_rn(__fadd_rn(y, -16777216.0f), 16777216.0f) != y;
+        asm("min.f32 %0, %0, %1, %2;" : "+f"(lowest) : "f"(x), "f"(y));
+        asm("max.f32 %0, %0, %1, %2;" : "+f"(highest) : "f"(x), "f"(y));
+    };
+    float4 v[kLoadsPerLane];
+#pragma unroll
+    for (int j = 0; j < kLoadsPerLane; ++j)
+        if (first < ntiles) v[j] = ld_stream_f4(p4 + first * kWarpTileF4 + j * 32 + lane, pol);
+#pragma unroll 1
+    for (long long t = first; t < ntiles; t += stride) {
+        const bool more = t + stride < ntiles;
+        const float4* next = p4 + (t + stride) * kWarpTileF4 + lane;
+        const unsigned i0 = (unsigned)head + (unsigned)t * kWarpTilePts + 2u * lane;   // n < 2^31
+#pragma unroll
+        for (int j = 0; j < kLoadsPerLane; ++j) {
+            const float4 p = v[j];
+            if (more) v[j] = ld_stream_f4(next + j * 32, pol);
+            check(p.x, p.y);
+            check(p.z, p.w);
+            const float dx0 = p.x - fcx, dy0 = p.y - fcy, dx1 = p.z - fcx, dy1 = p.w - fcy;   // exact
+            const bool q0 = !star_inside_fast(dx0, dy0, star_bin(dx0, dy0), P);
+            const bool q1 = !star_inside_fast(dx1, dy1, star_bin(dx1, dy1), P);
+            const unsigned m0 = __ballot_sync(0xFFFFFFFFu, q0), m1 = __ballot_sync(0xFFFFFFFFu, q1);
+            if (m0 | m1) {
+                if (q0) {
+                    const unsigned pos = qn + __popc(m0 & lt);
+                    w.x[pos] = p.x; w.y[pos] = p.y; w.idx[pos] = i0 + 64u * j;
+                }
+                if (q1) {
+                    const unsigned pos = qn + __popc(m0) + __popc(m1 & lt);
+                    w.x[pos] = p.z; w.y[pos] = p.w; w.idx[pos] = i0 + 64u * j + 1u;
+                }
+                qn += __popc(m0) + __popc(m1);
+                __syncwarp();
+                while (qn >= 32u) {
+                    qn -= 32u;
+                    dense_drain(P, cx, cy, w, qn, 32u, head, ctl, raw_xy, raw_idx);
+                }
+            }
+        }
+    }
+    if (qn) dense_drain(P, cx, cy, w, 0u, qn, head, ctl, raw_xy, raw_idx);
+    // the unaligned head point, and the ragged tail by 32 points per warp
+    const long long tail = head + ntiles * kWarpTilePts + 32 * (stride - 1 - first);
+    const long long ranges[2][2] = {{0, first == 0 ? head : 0}, {tail, min(n, tail + 32)}};
+    for (int rg = 0; rg < 2; ++rg) {
+        const long long i = ranges[rg][0] + lane, cnt = ranges[rg][1] - ranges[rg][0];
+        if (cnt <= 0) continue;
+        __syncwarp();
+        if (lane < cnt) {
+            w.x[lane] = pts[2 * i];
+            w.y[lane] = pts[2 * i + 1];
+            w.idx[lane] = (unsigned)i;
+            check(w.x[lane], w.y[lane]);
+        }
+        __syncwarp();
+        dense_drain(P, cx, cy, w, 0u, (unsigned)cnt, head, ctl, raw_xy, raw_idx);
+    }
+    bad |= lowest < 0.0f || highest >= (float)kCoordLimit;
+    if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) set_status(ctl, CH_ERANGE);
+    unsigned cnt = w.cnt;
+    flush_raw(w.raw, cnt, ctl, raw_xy, raw_idx);
+    if (lane < 8) s_red[warp][lane] = pack_best(lane, w.best[lane], w.code[lane]);
+    __syncthreads();
+    if (tid < 8) {
+        unsigned long long m = 0ull;
+        for (int k = 0; k < kDenseThreads / 32; ++k) m = s_red[k][tid] > m ? s_red[k][tid] : m;
+        if (m) atomicMax(&ctl->ext_packed[tid], m);
+    }
+    CH_TL(ctl, 3, 1);
+    if (!last_block(&ctl->blocks_done[1], &s_flag)) return;
+    if (__syncthreads_or(read_status(ctl) != CH_OK)) return;
+    if (tid == 0) ctl->mode = 0;   // the post pass classifies the raw survivors
+    __syncthreads();
+    if (!*(volatile int*)&ctl->oct_ready) finalize_block(pts, n, head, ctl, *reinterpret_cast<Octagon*>(dsm), keys, vals);
 }
 
 // ---------------------------------------------------------------------------
@@ -654,14 +1032,26 @@ __global__ void filter_output_kernel(const Ctl* ctl, long long n, int32_t* out_e
 // Host launchers
 void launch_init(Ctl* ctl, int mode, cudaStream_t s) { init_kernel<<<1, 256, 0, s>>>(ctl, mode); }
 
-void launch_sample(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, int grid, cudaStream_t s) {
-    sample_kernel<<<grid, 256, 0, s>>>(pts, n, head, ntiles, ctl);
+void launch_sample(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, unsigned switch_at, int grid,
+                   cudaStream_t s) {
+    sample_kernel<<<grid, 256, 0, s>>>(pts, n, head, ntiles, ctl, switch_at);
 }
 
 void launch_main(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, uint64_t* raw_xy,
-                 uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int grid, cudaStream_t s) {
-    main_kernel<<<grid, 256, kMainSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, switch_at, keys, vals);
+                 uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass, int grid,
+                 cudaStream_t s) {
+    main_kernel<<<grid, 256, kMainSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, switch_at, keys, vals,
+                                                  two_pass);
 }
+
+void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, void* bins, void* poly,
+                  uint64_t* raw_xy, uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int sms, cudaStream_t s) {
+    launch_grid(dense_kernel, sms, kDenseThreads, kDenseSmemBytes, s, pts, n, head, ntiles, ctl,
+                (unsigned long long*)bins, (StarPoly*)poly, raw_xy, raw_idx, keys, vals);
+}
+
+size_t star_bins_bytes() { return sizeof(unsigned long long) * kStarBins; }
+size_t star_poly_bytes() { return sizeof(StarPoly); }
 
 void launch_labels(const float* pts, long long n, Ctl* ctl, uint8_t* labels, int grid, cudaStream_t s) {
     if (((uintptr_t)pts & 15u) == 0u && ((uintptr_t)labels & 3u) == 0u) {
@@ -681,6 +1071,8 @@ long long sample_tiles_host(long long ntiles) { return sample_tiles(ntiles); }
 
 cudaError_t configure_filter_kernels() {
     cudaError_t e = cudaFuncSetAttribute(main_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMainSmemBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSmemBytes);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(labels_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kLabStreamSmemBytes);

@@ -11,7 +11,7 @@ namespace ch {
 struct Layout {
     size_t off_ctl, off_kA, off_kB, off_vA, off_vB, off_status, zero_bytes;
     size_t off_cu, off_cv, off_ci, off_clen, off_counters;
-    size_t off_tiles, off_star_bins, total;
+    size_t off_tiles, off_star_bins, off_star_poly, total;
     long long cap, sort_tiles, ctcap;
 };
 

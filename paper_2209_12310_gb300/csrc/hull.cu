@@ -1,11 +1,13 @@
-// hull.cu -- hull of the sorted survivors on the device.
+// hull.cu -- the large-survivor path by sort: the radix sort (sort.cuh) and the
+// hull of the sorted survivors, in one cooperative launch.
 //
 // The paper ends with "for i = 1..4: CH <- CH U hull(Q_i, n_i)" (Alg. 1): one
 // hull per queue, joined.  Here every queue r is a chain from quad vertex r
 // to quad vertex r+1 that is strictly monotone in the queue-frame coordinate u
 // (see queue_frame), and its hull chain is Andrew's lower chain (Table I) in
 // the (u, v) frame:
-//   chain_kernel   queue boundaries from the top-digit histogram; per tile
+//   sort_kernel    the digit histograms, the three passes; then queue
+//                  boundaries from the top-digit histogram; per tile
 //                  of 4096 records: keep the minimum-(v, index)
 //                  record of every run of equal u (only it can be a vertex),
 //                  build per-thread chains, merge them pairwise in shared
@@ -15,6 +17,7 @@
 //                  the block completing the fourth queue root joins the
 //                  chains (stitch_core: collinear junction vertices dropped,
 //                  degenerate cases, rotation to the lex-smallest vertex).
+// As one kernel the path costs a call that does not take it one empty launch.
 //
 // Merging two chains A, B (all u of A below all u of B): a_k (k > 0) stays iff
 // every b in B is strictly left of a_{k-1} -> a_k; b_l (l < |B|-1) stays iff
@@ -25,6 +28,7 @@
 #include "hullcore.cuh"
 #include "launch.h"
 #include "merge.cuh"
+#include "sort.cuh"
 
 #include <climits>
 
@@ -50,7 +54,10 @@ struct HullBufs {
     int64_t* out_n;
 };
 
-__global__ void __launch_bounds__(kChainThreads) chain_kernel(Ctl* ctl, HullBufs hb) {
+static_assert(kSortThreads == kChainThreads, "one block shape");
+
+__global__ void __launch_bounds__(kChainThreads) sort_kernel(Ctl* ctl, uint32_t* kA, uint64_t* vA, uint32_t* kB,
+                                                             uint64_t* vB, unsigned long long* status, HullBufs hb) {
     extern __shared__ int smem[];
     int* su = smem;
     int* sv = su + kMergeSmemCap;
@@ -62,9 +69,21 @@ __global__ void __launch_bounds__(kChainThreads) chain_kernel(Ctl* ctl, HullBufs
     __shared__ int s_mv[kChainThreads / 2][3];   // per pair: destination, source, count
 
     if (*(volatile int*)&ctl->done) return;
-    const int st0 = read_status(ctl);
-    if (st0 != CH_OK) {   // a sort pass gave up (timed-out wait): report it
-        if (blockIdx.x == 0 && threadIdx.x == 0) *hb.out_n = st0;
+    bool go = read_status(ctl) == CH_OK;
+    if (go) {
+        if (*(volatile int*)&ctl->bk_state != 2) return;
+        SortSmem& sm = *reinterpret_cast<SortSmem*>(smem);
+        sort_hist(reinterpret_cast<unsigned(*)[kDigits]>(smem), kA, ctl);
+        go = grid_barrier(&ctl->barrier[2], 1u, ctl);
+        if (go) onesweep(sm, kA, vA, kB, vB, ctl, status, 0);
+        go = go && grid_barrier(&ctl->barrier[2], 2u, ctl);
+        if (go) onesweep(sm, kB, vB, kA, vA, ctl, status, 1);
+        go = go && grid_barrier(&ctl->barrier[2], 3u, ctl);
+        if (go) onesweep(sm, kA, vA, kB, vB, ctl, status, 2);
+        go = go && grid_barrier(&ctl->barrier[2], 4u, ctl);
+    }
+    if (__syncthreads_or(!go || read_status(ctl) != CH_OK)) {   // a wait gave up: report it
+        if (threadIdx.x == 0) *hb.out_n = read_status(ctl);
         return;
     }
     const int tid = threadIdx.x;
@@ -194,22 +213,22 @@ namespace ch {
 
 size_t chain_smem_bytes() { return (size_t)3 * kMergeSmemCap * sizeof(int); }
 
-void launch_chain(Ctl* ctl, const uint32_t* keys, const uint64_t* vals, int* cu, int* cv, int* ci, int* clen,
-                  int* counters, int ctcap, int* vbuf, int* kbuf, int* xbuf, int* ybuf, const float* pts, long long n,
-                  int32_t* out_idx, int64_t* out_n, int grid, cudaStream_t s) {
-    HullBufs hb{keys, vals, cu, cv, ci, clen, counters, ctcap, vbuf, kbuf, xbuf, ybuf, pts, n,
-                out_idx, out_n};
-    chain_kernel<<<grid, kChainThreads, chain_smem_bytes(), s>>>(ctl, hb);
+void launch_sort(Ctl* ctl, uint32_t* kA, uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned long long* status, int* cu,
+                 int* cv, int* ci, int* clen, int* counters, int ctcap, const float* pts, long long n, int32_t* out_idx,
+                 int64_t* out_n, int grid, cudaStream_t s) {
+    // the A buffers are free once the records are sorted into B, and B once
+    // its chains are built: the stitch's scratch
+    const HullBufs hb{kB, vB, cu, cv, ci, clen, counters, ctcap, (int*)vA, (int*)kA, (int*)kB, (int*)vB, pts, n, out_idx,
+                      out_n};
+    launch_grid(sort_kernel, grid, kChainThreads, chain_smem_bytes(), s, ctl, kA, vA, kB, vB, status, hb);
 }
 
 cudaError_t configure_hull_kernels() {
-    return cudaFuncSetAttribute(chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)chain_smem_bytes());
+    return cudaFuncSetAttribute(sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem_bytes());
 }
 
-
-cudaError_t occupancy_chain(int* b) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(b, chain_kernel, kChainThreads, chain_smem_bytes());
+cudaError_t occupancy_sort(int* b) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(b, sort_kernel, kChainThreads, chain_smem_bytes());
 }
 
 }  // namespace ch

@@ -12,7 +12,6 @@
 #include "launch.h"
 #include "octagon.cuh"
 #include "records.cuh"
-#include "star.cuh"
 
 #include <climits>
 
@@ -67,26 +66,16 @@ __device__ __forceinline__ void post_stage(int r, int X, int Y, unsigned idx, co
     __syncwarp();
 }
 
-// The star polygon in shared memory (null when this call has none) and its
-// centre; points strictly inside it are dropped before the octagon test.
-struct StarView {
-    const StarPoly* P;
-    int cx, cy;
-    __device__ __forceinline__ bool inside(int X, int Y) const {
-        return P != nullptr && star_inside(X - cx, Y - cy, *P);
-    }
-};
-
 // Warp-collective: classifies one point per lane (valid = false for none) and
 // stages it; folds the tally (one add per lane and call).
-__device__ __forceinline__ void post_point(bool valid, float x, float y, unsigned idx, const Octagon& o,
-                                           const StarView& sv, RecBuf& b, unsigned& cnt, Ctl* ctl, uint32_t* keys,
-                                           uint64_t* vals, QueueTally& tally) {
+__device__ __forceinline__ void post_point(bool valid, float x, float y, unsigned idx, const Octagon& o, RecBuf& b,
+                                           unsigned& cnt, Ctl* ctl, uint32_t* keys, uint64_t* vals,
+                                           QueueTally& tally) {
     int r = -1, X = 0, Y = 0;
     if (valid) {
         X = __float2int_rn(x);
         Y = __float2int_rn(y);
-        if (!sv.inside(X, Y)) r = classify_hull(x, y, o);
+        r = classify_hull(x, y, o);
     }
     post_stage(r, X, Y, idx, o, b, cnt, ctl, keys, vals, tally);
     tally.fold();
@@ -133,8 +122,8 @@ __device__ __forceinline__ void flush_queue_counts(QueueTally& tally, Ctl* ctl) 
 
 // The block that finished last: support-line records, then the hull of few
 // records (at most kMidCap: quickhull rounds, else the sort-based mid_hull), or
-// the path of the large-survivor part.  On dense data (two-pass mode, or more
-// than a quarter of the points kept) the records are near the hull, mostly
+// the path of the large-survivor part.  On dense data (an earlier pass's
+// verdict, or more than a quarter of the points kept) the records are near the hull, mostly
 // vertices, and past kNearHullRec of them they would outgrow
 // the quickhull rounds' vertex capacity: the queues then, a block each (one
 // million points of a ring: 27,265 records, 13,024 vertices: queue_kernel takes
@@ -147,7 +136,7 @@ constexpr unsigned kNearHullRec = 512;
 
 __device__ void post_last_block(const float* __restrict__ pts, long long n, Ctl* ctl, const Octagon& o,
                                 uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n, char* dyn,
-                                bool dense, unsigned long long cond) {
+                                bool dense) {
     __shared__ unsigned long long s_lep[8];
     __shared__ uint64_t s_lval[8];
     __shared__ unsigned s_lkey[8];
@@ -188,7 +177,6 @@ __device__ void post_last_block(const float* __restrict__ pts, long long n, Ctl*
                              : *(volatile int*)&ctl->star_final || total > 4u * (unsigned)kQueueCap ? kPathTiles : kPathSort;
             ctl->path = path;
             ctl->bk_state = path == kPathSort ? 2 : 1;
-            if (cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, path == kPathQueues ? 0u : 1u);
         }
         return;
     }
@@ -222,48 +210,18 @@ __device__ void post_last_block(const float* __restrict__ pts, long long n, Ctl*
 
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 
-// Points of dense data that the star polygon's radius test leaves undecided,
-// queued per warp and taken 32 at a time through the exact tests, so that a
-// few such points do not hold a whole warp in the slow path.
-constexpr int kWarpQueueCap = 96;   // < 32 waiting + 64 added per step
-struct WarpQueue {
-    int x[kWarpQueueCap], y[kWarpQueueCap];
-    unsigned idx[kWarpQueueCap];
-};
-
-// Dynamic shared memory while points are classified: the star polygon, the
-// warps' record buffers, the warps' queues.  The polygon is finished first,
-// with the region from the record buffers on as its work area A; afterwards
-// the last block's hull reuses all of it.
-constexpr size_t kRecBufOff = (sizeof(StarPoly) + 15) / 16 * 16;
-constexpr size_t kQueueOff = kRecBufOff + (size_t)(kPostThreads / 32) * sizeof(RecBuf);
-constexpr size_t kClassifyBytes = kQueueOff + (size_t)(kPostThreads / 32) * sizeof(WarpQueue);
-constexpr size_t kWorkABytes = (sizeof(int2) + sizeof(unsigned short)) * kStarBins;
+// Dynamic shared memory: the warps' record buffers while points are
+// classified; the last block's hull reuses it.
 constexpr size_t kPostSmemBytes =
-    cmax(cmax(kMidSmemBytes, sizeof(QhSmem)), cmax(kClassifyBytes, kRecBufOff + kWorkABytes));
-
-// Warp-collective: the exact star test and the octagon classification of one
-// queued point per lane (valid = false for none), then staging.
-__device__ __forceinline__ void post_queued(bool valid, int X, int Y, unsigned idx, const Octagon& o,
-                                            const StarView& sv, RecBuf& b, unsigned& cnt, Ctl* ctl, uint32_t* keys,
-                                            uint64_t* vals, QueueTally& tally) {
-    int r = -1;
-    if (valid) {
-        const int px = X - sv.cx, py = Y - sv.cy;
-        if (!star_inside_exact(px, py, star_bin(px, py), *sv.P)) r = classify_hull((float)X, (float)Y, o);
-    }
-    post_stage(r, X, Y, idx, o, b, cnt, ctl, keys, vals, tally);
-}
+    cmax(cmax(kMidSmemBytes, sizeof(QhSmem)), (kPostThreads / 32) * sizeof(RecBuf));
 
 __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __restrict__ pts, long long n, int head,
                                                                long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
                                                                const uint32_t* raw_idx, uint32_t* keys,
-                                                               uint64_t* vals, int32_t* out_idx, int64_t* out_n,
-                                                               unsigned long long* star_bins,
-                                                               unsigned long long cond) {
+                                                               uint64_t* vals, int32_t* out_idx, int64_t* out_n) {
     extern __shared__ __align__(16) char dyn[];
     __shared__ Octagon s_o;
-    __shared__ int s_flag, s_mode, s_star, s_scx, s_scy;
+    __shared__ int s_flag, s_mode, s_dense;
     __shared__ unsigned s_nraw;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     CH_TL(ctl, 5, 0);
@@ -271,34 +229,16 @@ __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __re
         s_flag = read_status(ctl);
         s_mode = *(volatile int*)&ctl->mode;
         s_nraw = *(volatile unsigned*)&ctl->count_raw;
-        s_star = star_bins != nullptr && *(volatile int*)&ctl->star_ok;
-        s_scx = ctl->star_cx;
-        s_scy = ctl->star_cy;
+        // (small inputs take two passes whatever the data)
+        s_dense = *(volatile int*)&ctl->samp_dense || (s_mode == 1 && n > kTwoPassMax);
     }
     copy_octagon(&s_o, &ctl->oct);
     __syncthreads();
     if (s_flag != CH_OK) {   // data error or timeout of an earlier stage
         if (blockIdx.x == 0 && tid == 0) { *out_n = s_flag; ctl->done = 1; }
-        if (blockIdx.x == 0 && s_star)   // leave the star bins clear for the next call
-            for (int b = tid; b < kStarBins; b += blockDim.x) star_bins[b] = 0ull;
         return;
     }
-    StarView sv{nullptr, s_scx, s_scy};
-    if (s_star) {   // the star pass gathered a vertex list: finish the polygon here
-        StarPoly* P = reinterpret_cast<StarPoly*>(dyn);
-        int2* va = reinterpret_cast<int2*>(dyn + kRecBufOff);
-        unsigned short* ba = reinterpret_cast<unsigned short*>(dyn + kRecBufOff + sizeof(int2) * kStarBins);
-        CH_TL(ctl, 8, 0);
-        const int k = star_finish<kPostThreads>(star_bins, pts, n, s_scx, s_scy, va, ba, *P, ctl);
-        if (k) sv.P = P;
-        CH_TL(ctl, 8, 1);
-        if (blockIdx.x == 0 && tid == 0) {
-            ctl->star_final = k ? 1 : 0;
-            ctl->star_k = k;
-        }
-        __syncthreads();
-    }
-    RecBuf& rb = reinterpret_cast<RecBuf*>(dyn + kRecBufOff)[warp];
+    RecBuf& rb = reinterpret_cast<RecBuf*>(dyn)[warp];
     unsigned rc = 0u;
     QueueTally tally;
     if (s_mode == 1) {   // two-pass mode: every point
@@ -318,8 +258,6 @@ __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __re
             return (st % kLoadsPerLane == kLoadsPerLane - 1) ? st + sstep - (kLoadsPerLane - 1) : st + 1;
         };
         unsigned s = gwarp * kLoadsPerLane, sl = s;   // sl: the step of the newest load
-        WarpQueue& wq = reinterpret_cast<WarpQueue*>(dyn + kQueueOff)[warp];
-        unsigned qn = 0u;   // points waiting in wq (warp-uniform)
         float4 q[kAhead];
 #pragma unroll
         for (int a = 0; a < kAhead; ++a) {
@@ -337,78 +275,42 @@ __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __re
                                 2u * lane;
             const int X0 = __float2int_rn(v.x), Y0 = __float2int_rn(v.y);
             const int X1 = __float2int_rn(v.z), Y1 = __float2int_rn(v.w);
-            if (sv.P) {
-                // most points of dense data are inside the star polygon's
-                // radius bound of their bin; the rest wait in the queue
-                const int px0 = X0 - sv.cx, py0 = Y0 - sv.cy, px1 = X1 - sv.cx, py1 = Y1 - sv.cy;
-                const bool d0 = star_inside_fast(px0, py0, star_bin(px0, py0), *sv.P);
-                const bool d1 = star_inside_fast(px1, py1, star_bin(px1, py1), *sv.P);
-                const unsigned m0 = __ballot_sync(0xFFFFFFFFu, !d0), m1 = __ballot_sync(0xFFFFFFFFu, !d1);
-                if (m0 | m1) {
-                    const unsigned lt = lanemask_lt();
-                    if (!d0) {
-                        const unsigned pos = qn + __popc(m0 & lt);
-                        wq.x[pos] = X0; wq.y[pos] = Y0; wq.idx[pos] = i0;
-                    }
-                    if (!d1) {
-                        const unsigned pos = qn + __popc(m0) + __popc(m1 & lt);
-                        wq.x[pos] = X1; wq.y[pos] = Y1; wq.idx[pos] = i0 + 1u;
-                    }
-                    qn += __popc(m0) + __popc(m1);
-                    __syncwarp();
-                    while (qn >= 32u) {
-                        qn -= 32u;
-                        const int X = wq.x[qn + lane], Y = wq.y[qn + lane];
-                        const unsigned id = wq.idx[qn + lane];
-                        __syncwarp();
-                        post_queued(true, X, Y, id, s_o, sv, rb, rc, ctl, keys, vals, tally);
-                    }
-                }
-            } else {
-                int r0 = classify_hull_fast(v.x, v.y, X0, Y0, s_o);
-                int r1 = classify_hull_fast(v.z, v.w, X1, Y1, s_o);
-                if (r0 == kUndecided) r0 = classify_hull_slow(v.x, v.y, &s_o);
-                if (r1 == kUndecided) r1 = classify_hull_slow(v.z, v.w, &s_o);
-                post_stage(r0, X0, Y0, i0, s_o, rb, rc, ctl, keys, vals, tally);
-                post_stage(r1, X1, Y1, i0 + 1u, s_o, rb, rc, ctl, keys, vals, tally);
-            }
+            int r0 = classify_hull_fast(v.x, v.y, X0, Y0, s_o);
+            int r1 = classify_hull_fast(v.z, v.w, X1, Y1, s_o);
+            if (r0 == kUndecided) r0 = classify_hull_slow(v.x, v.y, &s_o);
+            if (r1 == kUndecided) r1 = classify_hull_slow(v.z, v.w, &s_o);
+            post_stage(r0, X0, Y0, i0, s_o, rb, rc, ctl, keys, vals, tally);
+            post_stage(r1, X1, Y1, i0 + 1u, s_o, rb, rc, ctl, keys, vals, tally);
             if (s % kLoadsPerLane == kLoadsPerLane - 1) tally.fold();   // at most 2 kLoadsPerLane adds
             s = next_step(s);
         }
-        if (qn) {   // the queue's remainder
-            const bool valid = (unsigned)lane < qn;
-            const int X = valid ? wq.x[lane] : 0, Y = valid ? wq.y[lane] : 0;
-            const unsigned id = valid ? wq.idx[lane] : 0u;
-            __syncwarp();
-            post_queued(valid, X, Y, id, s_o, sv, rb, rc, ctl, keys, vals, tally);
-            tally.fold();
-        }
-        if (gwarp == 0) {   // the unaligned head point and the ragged tail
-            const long long ranges[2][2] = {{0, head}, {head + ntiles * kWarpTilePts, n}};
-            for (int rg = 0; rg < 2; ++rg)
-                for (long long b = ranges[rg][0]; b < ranges[rg][1]; b += 32) {
-                    const long long i = b + lane;
-                    const bool valid = i < ranges[rg][1];
-                    float x = 0.0f, y = 0.0f;
-                    if (valid) { x = pts[2 * i]; y = pts[2 * i + 1]; }
-                    post_point(valid, x, y, (unsigned)i, s_o, sv, rb, rc, ctl, keys, vals, tally);
-                }
+        // the unaligned head point, and the ragged tail by 32 points per warp
+        const long long tail = head + ntiles * kWarpTilePts + 32ll * (nwarps - 1u - gwarp);
+        const long long ranges[2][2] = {{0, gwarp == 0 ? head : 0}, {tail, min(n, tail + 32)}};
+        for (int rg = 0; rg < 2; ++rg) {
+            if (ranges[rg][0] >= ranges[rg][1]) continue;
+            const long long i = ranges[rg][0] + lane;
+            const bool valid = i < ranges[rg][1];
+            float x = 0.0f, y = 0.0f;
+            if (valid) { x = pts[2 * i]; y = pts[2 * i + 1]; }
+            post_point(valid, x, y, (unsigned)i, s_o, rb, rc, ctl, keys, vals, tally);
         }
     } else {   // fused mode: the raw survivors of the main pass
+        // the next point's loads in flight while one is classified
         const unsigned nraw = s_nraw;
         const unsigned stride = gridDim.x * blockDim.x;
-        for (unsigned b = blockIdx.x * blockDim.x + warp * 32; b < nraw; b += stride) {
-            const unsigned i = b + lane;
+        unsigned i = blockIdx.x * blockDim.x + warp * 32 + lane;
+        unsigned long long nxy = i < nraw ? __ldcs(raw_xy + i) : 0ull;
+        unsigned nidx = i < nraw ? __ldcs(raw_idx + i) : 0u;
+        for (; i - lane < nraw; i += stride) {
             const bool valid = i < nraw;
-            float x = 0.0f, y = 0.0f;
-            unsigned idx = 0u;
-            if (valid) {
-                const unsigned long long xy = raw_xy[i];
-                x = (float)(unsigned)(xy >> 32);
-                y = (float)(unsigned)(xy & 0xFFFFFFFFull);
-                idx = raw_idx[i];
+            const float x = (float)(unsigned)(nxy >> 32), y = (float)(unsigned)(nxy & 0xFFFFFFFFull);
+            const unsigned idx = nidx;
+            if (i + stride < nraw) {
+                nxy = __ldcs(raw_xy + i + stride);
+                nidx = __ldcs(raw_idx + i + stride);
             }
-            post_point(valid, x, y, idx, s_o, sv, rb, rc, ctl, keys, vals, tally);
+            post_point(valid, x, y, idx, s_o, rb, rc, ctl, keys, vals, tally);
         }
     }
     rec_flush_block(rb, rc, ctl, keys, vals);
@@ -416,18 +318,16 @@ __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __re
     CH_TL(ctl, 5, 1);
     if (!last_block(&ctl->blocks_done[2], &s_flag)) return;
     CH_TL(ctl, 6, 0);
-    if (s_star)   // every block has built its polygon: clear the bins for the next call
-        for (int b = tid; b < kStarBins; b += blockDim.x) star_bins[b] = 0ull;
-    post_last_block(pts, n, ctl, s_o, keys, vals, out_idx, out_n, dyn, s_mode == 1, cond);
+    post_last_block(pts, n, ctl, s_o, keys, vals, out_idx, out_n, dyn, s_dense != 0);
     CH_TL(ctl, 6, 1);
 }
 
 // ---------------------------------------------------------------------------
 void launch_post(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
                  const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n,
-                 void* star_bins, unsigned long long cond, int grid, cudaStream_t s) {
-    post_kernel<<<grid, kPostThreads, kPostSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, keys, vals,
-                                                          out_idx, out_n, (unsigned long long*)star_bins, cond);
+                 int grid, cudaStream_t s) {
+    post_kernel<<<grid, kPostThreads, kPostSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, keys, vals, out_idx,
+                                                          out_n);
 }
 
 cudaError_t configure_post_kernel() {

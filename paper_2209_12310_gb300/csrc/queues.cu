@@ -2,20 +2,19 @@
 //
 // The post pass leaves the records in no order, counted per queue, and picks
 // one of three ways (post_last_block):
-//   queues  every queue fits one block: queue_kernel, a block per queue, sorts
-//           the queue by u and reduces it to its lower chain in shared memory
-//           (qchain.cuh);
-//   tiles   the u range of each queue is cut into tiles of about kTileTarget
-//           records: tile_hist_kernel counts the records of kQGroups equal u
-//           ranges per queue and its last block joins neighbouring ranges into
-//           tiles; tile_part_kernel moves the records into their tiles' ranges
-//           (partition.cuh); tile_chain_kernel reduces each tile to its lower
-//           chain by the same block sort and elimination; queue_kernel then
-//           reduces each queue's tile chains, joined in u order, to its chain;
-//   sort    the radix sort and the merge tree (sort.cu, hull.cu), also when
+//   queues  every queue fits one block: a block per queue sorts the queue by u
+//           and reduces it to its lower chain in shared memory (qchain.cuh);
+//   tiles   the u range of each queue is cut into tiles of some thousand
+//           records, which a block each reduces the same way, and a block per
+//           queue reduces its tiles' chains, joined in u order, to its chain;
+//   sort    the radix sort and the merge tree (sort.cuh, hull.cu), also when
 //           a tile's or a queue's chain outgrows shared memory.
 // The lower chain of a set of points equals the lower chain of the chains of
 // any partition of it into u ranges, joined in u order.
+//
+// large_kernel is one cooperative launch for the first two ways: the phases of
+// the tiles (count, cut, move, reduce) meet at grid barriers.  As one kernel it
+// costs a call that needs none of it one empty launch.
 #include "ch_internal.cuh"
 #include "host.h"
 #include "hullcore.cuh"
@@ -26,10 +25,11 @@
 namespace ch {
 
 constexpr int kQGroups = 1024;          // equal u ranges of a queue
-constexpr unsigned kTileTarget = 1280;  // records of a tile on average: half of what its block holds
-constexpr int kTileThreads = 256;
-constexpr int kQueueThreads = 1024;
-using QcTile = QcSmem<2560, 1024>;
+// Records of a tile on average: as many tiles as blocks, or twice, three times
+// ... as many while a tile would have more than kTileMost (the density of near-
+// hull records varies by a quarter around its average along a queue).
+constexpr unsigned kTileMost = 6000;
+constexpr int kLargeThreads = 1024;
 using QcQueue = QcSmem<kQueueCap, 4096>;
 static_assert(4 * kQGroups == kPtGroups, "groups of the four queues; as many tiles at most");
 
@@ -58,88 +58,102 @@ __device__ __forceinline__ unsigned q_group(const QMap& m, uint32_t key) {
     return (unsigned)(r * kQGroups + max(0, min(kQGroups - 1, g)));
 }
 
-// The call takes path p and no earlier stage failed.
-__device__ __forceinline__ bool on_path(Ctl* ctl, int p) {
-    return *(volatile int*)&ctl->path == p && *(volatile int*)&ctl->bk_state == 1 && read_status(ctl) == CH_OK;
-}
+struct LargeArgs {
+    Ctl* ctl;
+    const uint32_t* keys;    // the records
+    const uint64_t* vals;
+    uint32_t* kB;            // the records by tile; then scratch and
+    uint64_t* vB;            // the queues' chains (u, v)
+    unsigned *ghist, *gtile, *tbeg, *tcur;   // kPtGroups each
+    int* tlen;
+    int *cu, *cv, *ci;       // the tiles' chains; then (cu) the queues' chains (index)
+    long long n;
+    int32_t* out_idx;
+    int64_t* out_n;
+};
 
-// Records per group; the block that finishes last cuts the tiles: gtile maps a
-// group to its tile, tile t's records go to [tbeg[t], tbeg[t + 1]).
-__global__ void __launch_bounds__(kPtThreads, 1) tile_hist_kernel(Ctl* ctl, const uint32_t* keys, unsigned* ghist,
-                                                                  unsigned* gtile, unsigned* tbeg, unsigned* tcur) {
-    __shared__ unsigned s_h[kPtGroups];   // records per group; then per tile
-    __shared__ unsigned s_beg[kPtGroups];
-    __shared__ unsigned s_q0[5], s_tb[5];
-    __shared__ QMap s_m;
-    __shared__ int s_go, s_last, s_tmp[33];
+// Records per group (shared-memory counts, then one atomic per group that
+// occurs).
+struct TileHistSmem {
+    unsigned h[kPtGroups];     // records per group; in the cut, per tile
+    unsigned beg[kPtGroups];
+    unsigned q0[5], tb[5];
+    int tmp[33];
+};
+
+__device__ void tile_hist(const LargeArgs& a, TileHistSmem& sm, const QMap& m) {
     const int tid = threadIdx.x;
-    if (tid == 0) s_go = on_path(ctl, kPathTiles);
+    for (int g = tid; g < kPtGroups; g += kLargeThreads) sm.h[g] = 0u;
     __syncthreads();
-    if (!s_go) return;
-    q_map(ctl->oct, s_m);
-    for (int g = tid; g < kPtGroups; g += kPtThreads) s_h[g] = 0u;
-    __syncthreads();
-    const unsigned n = ctl->count;
-    const unsigned stride = gridDim.x * kPtThreads;
+    const unsigned n = a.ctl->count;
+    const unsigned stride = gridDim.x * kLargeThreads;
     constexpr int kU = 4;
-    for (unsigned i0 = blockIdx.x * kPtThreads + tid; i0 < n; i0 += stride * kU) {
+    for (unsigned i0 = blockIdx.x * kLargeThreads + tid; i0 < n; i0 += stride * kU) {
         uint32_t k[kU];
 #pragma unroll
         for (int j = 0; j < kU; ++j)
-            if (i0 + j * stride < n) k[j] = __ldcs(keys + i0 + j * stride);
+            if (i0 + j * stride < n) k[j] = __ldcg(a.keys + i0 + j * stride);
 #pragma unroll
         for (int j = 0; j < kU; ++j)
-            if (i0 + j * stride < n) atomicAdd(&s_h[q_group(s_m, k[j])], 1u);
+            if (i0 + j * stride < n) atomicAdd(&sm.h[q_group(m, k[j])], 1u);
     }
     __syncthreads();
-    for (int g = tid; g < kPtGroups; g += kPtThreads)
-        if (s_h[g]) atomicAdd(&ghist[g], s_h[g]);
-    if (!last_block(&ctl->blocks_done[2], &s_last)) return;
-    __syncthreads();
-    constexpr int kE = kPtGroups / kPtThreads;   // groups per thread, all of one queue
+    for (int g = tid; g < kPtGroups; g += kLargeThreads)
+        if (sm.h[g]) atomicAdd(&a.ghist[g], sm.h[g]);
+}
+
+// One block cuts the tiles: gtile maps a group to its tile, tile t's records go
+// to tbeg[t] on.
+__device__ void tile_cut(const LargeArgs& a, TileHistSmem& sm) {
+    const int tid = threadIdx.x;
+    Ctl* ctl = a.ctl;
+    constexpr int kE = kPtGroups / kLargeThreads;   // groups per thread, all of one queue
     unsigned c[kE], sum = 0u;
 #pragma unroll
     for (int e = 0; e < kE; ++e) {
-        c[e] = __ldcg(ghist + tid * kE + e);
-        ghist[tid * kE + e] = 0u;   // at rest again
+        c[e] = __ldcg(a.ghist + tid * kE + e);
+        a.ghist[tid * kE + e] = 0u;   // at rest again
         sum += c[e];
     }
     int tot;
-    unsigned run = (unsigned)block_excl_scan((int)sum, s_tmp, &tot);
-    if (tid % (kQGroups / kE) == 0) s_q0[tid / (kQGroups / kE)] = run;
-    if (tid == 0) s_q0[4] = (unsigned)tot;
-    for (int t = tid; t < kPtGroups; t += kPtThreads) {
-        s_h[t] = 0u;
-        s_beg[t] = 0xFFFFFFFFu;
+    unsigned run = (unsigned)block_excl_scan((int)sum, sm.tmp, &tot);
+    if (tid % (kQGroups / kE) == 0) sm.q0[tid / (kQGroups / kE)] = run;
+    if (tid == 0) sm.q0[4] = (unsigned)tot;
+    for (int t = tid; t < kPtGroups; t += kLargeThreads) {
+        sm.h[t] = 0u;
+        sm.beg[t] = 0xFFFFFFFFu;
     }
     __syncthreads();
-    const unsigned target = max(kTileTarget, n / (unsigned)(kPtGroups - 96));   // at most kPtGroups - 92 tiles
+    const unsigned n = (unsigned)tot;
+    const unsigned rounds = (n + gridDim.x * kTileMost - 1) / (gridDim.x * kTileMost);
+    // at most kPtGroups - 92 tiles (more records: larger tiles, in pieces)
+    const unsigned target = max(n / (gridDim.x * rounds) + 1u, n / (unsigned)(kPtGroups - 96) + 1u);
     if (tid == 0) {
         unsigned t = 0u;
         for (int r = 0; r < 4; ++r) {
-            s_tb[r] = t;
-            t += (s_q0[r + 1] - s_q0[r]) / target + 1u;
+            sm.tb[r] = t;
+            t += (sm.q0[r + 1] - sm.q0[r]) / target + 1u;
         }
-        s_tb[4] = t;
-        for (int r = 0; r < 5; ++r) ctl->q_tile[r] = s_tb[r];
+        sm.tb[4] = t;
+        for (int r = 0; r < 5; ++r) ctl->q_tile[r] = sm.tb[r];
     }
     __syncthreads();
     const int r = tid / (kQGroups / kE);
 #pragma unroll
     for (int e = 0; e < kE; ++e) {
-        const unsigned t = s_tb[r] + (run - s_q0[r]) / target;
-        gtile[tid * kE + e] = t;
+        const unsigned t = sm.tb[r] + (run - sm.q0[r]) / target;
+        a.gtile[tid * kE + e] = t;
         if (c[e]) {
-            atomicMin(&s_beg[t], run);
-            atomicAdd(&s_h[t], c[e]);
+            atomicMin(&sm.beg[t], run);
+            atomicAdd(&sm.h[t], c[e]);
         }
         run += c[e];
     }
     __syncthreads();
-    for (unsigned t = tid; t < s_tb[4]; t += kPtThreads) {
-        const unsigned b = s_h[t] ? s_beg[t] : 0u;   // a tile that a large group skipped is empty
-        tbeg[t] = b;
-        tcur[t] = b;
+    for (unsigned t = tid; t < sm.tb[4]; t += kLargeThreads) {
+        const unsigned b = sm.h[t] ? sm.beg[t] : 0u;   // a tile that a large group skipped is empty
+        a.tbeg[t] = b;
+        a.tcur[t] = b;
     }
 }
 
@@ -149,55 +163,36 @@ struct TilePartSmem {
     unsigned short gtile[kPtGroups];
 };
 
-__global__ void __launch_bounds__(kPtThreads, 1) tile_part_kernel(Ctl* ctl, const uint32_t* kin, const uint64_t* vin,
-                                                                  const unsigned* gtile, unsigned* tcur,
-                                                                  uint32_t* kout, uint64_t* vout) {
-    extern __shared__ __align__(16) unsigned char s_dyn[];
-    TilePartSmem& sm = *reinterpret_cast<TilePartSmem*>(s_dyn);
-    __shared__ QMap s_m;
-    __shared__ int s_go;
+__device__ void tile_part(const LargeArgs& a, TilePartSmem& sm, const QMap& m) {
+    static_assert(kLargeThreads == kPtThreads, "partition block");
     const int tid = threadIdx.x;
-    if (tid == 0) s_go = on_path(ctl, kPathTiles);
+    for (int g = tid; g < kPtGroups; g += kPtThreads) sm.gtile[g] = (unsigned short)__ldcg(a.gtile + g);
     __syncthreads();
-    if (!s_go) return;
-    q_map(ctl->oct, s_m);
-    for (int g = tid; g < kPtGroups; g += kPtThreads) sm.gtile[g] = (unsigned short)gtile[g];
-    __syncthreads();
-    const unsigned n = ctl->count, nt = ctl->q_tile[4];
+    const unsigned n = a.ctl->count, nt = *(volatile unsigned*)&a.ctl->q_tile[4];
     for (unsigned i0 = blockIdx.x * kPtTile; i0 < n; i0 += gridDim.x * kPtTile)
         partition_tile(
-            sm.p, kin, vin, i0, min((unsigned)kPtTile, n - i0), nt,
-            [&](uint32_t key) { return (unsigned)sm.gtile[q_group(s_m, key)]; },
-            [&](unsigned g, unsigned cnt) { return atomicAdd(&tcur[g], cnt); }, kout, vout);
+            sm.p, a.keys, a.vals, i0, min((unsigned)kPtTile, n - i0), nt,
+            [&](uint32_t key) { return (unsigned)sm.gtile[q_group(m, key)]; },
+            [&](unsigned g, unsigned cnt) { return atomicAdd(&a.tcur[g], cnt); }, a.kB, a.vB);
 }
 
-// Each tile's lower chain, to [tbeg[t], tbeg[t] + tlen[t]) of cu / cv / ci
+// The tiles' lower chains, to [tbeg[t], tbeg[t] + tlen[t]) of cu / cv / ci
 // (u, v, index).  A tile with more records than the block holds goes in
 // pieces, the chain so far taken along with each; when that chain fills the
 // block, the call goes to the sort.
-__global__ void __launch_bounds__(kTileThreads) tile_chain_kernel(Ctl* ctl, const uint32_t* keys, const uint64_t* vals,
-                                                                  const unsigned* tbeg, const unsigned* tend, int* cu,
-                                                                  int* cv, int* ci, int* tlen) {
-    extern __shared__ __align__(16) unsigned char s_dyn[];
-    QcTile& q = *reinterpret_cast<QcTile*>(s_dyn);
-    __shared__ int s_go;
-    __shared__ unsigned s_tile, s_nt;
+__device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
+    __shared__ unsigned s_tile;
     const int tid = threadIdx.x;
-    constexpr int kCap = QcTile::kCap, kCarry = kCap * 3 / 4, kPer = kCap / kTileThreads;
-    static_assert(kCap % kTileThreads == 0, "carried points per thread");
-    if (tid == 0) {
-        s_go = on_path(ctl, kPathTiles);
-        s_nt = ctl->q_tile[4];
-    }
-    __syncthreads();
-    if (!s_go) return;
+    constexpr int T = kLargeThreads, kCap = QcQueue::kCap, kCarry = kCap * 3 / 4, kPer = kCap / T;
+    static_assert(kCap % T == 0, "carried points per thread");
+    const unsigned nt = *(volatile unsigned*)&a.ctl->q_tile[4];
     for (;;) {
         __syncthreads();
-        if (tid == 0) s_tile = atomicAdd(&ctl->tile_ctr[3], 1u);   // the sort's passes use 0 .. 2
+        if (tid == 0) s_tile = atomicAdd(&a.ctl->tile_ctr[3], 1u);
         __syncthreads();
         const unsigned t = s_tile;
-        if (t >= s_nt) return;
-        const unsigned beg = tbeg[t], cnt = tend[t] - beg;
+        if (t >= nt) return;
+        const unsigned beg = __ldcg(a.tbeg + t), cnt = __ldcg(a.tcur + t) - beg;
         unsigned long long *src = q.a, *dst = q.b;
         int len = 0;
         for (unsigned c0 = 0; c0 < cnt;) {
@@ -207,14 +202,14 @@ __global__ void __launch_bounds__(kTileThreads) tile_chain_kernel(Ctl* ctl, cons
                 int id[kPer];
 #pragma unroll
                 for (int e = 0; e < kPer; ++e) {
-                    const int j = e * kTileThreads + tid;
+                    const int j = e * T + tid;
                     w[e] = j < len ? src[j] : 0ull;
                     id[e] = j < len ? q.si[qc_pos(w[e])] : 0;
                 }
                 __syncthreads();
 #pragma unroll
                 for (int e = 0; e < kPer; ++e) {
-                    const int j = e * kTileThreads + tid;
+                    const int j = e * T + tid;
                     if (j < len) {
                         q.a[j] = qc_pack((unsigned)qc_u(w[e]), (unsigned)qc_v(w[e]), (unsigned)j);
                         q.si[j] = id[e];
@@ -222,39 +217,39 @@ __global__ void __launch_bounds__(kTileThreads) tile_chain_kernel(Ctl* ctl, cons
                 }
             }
 #pragma unroll 5
-            for (int j = tid; j < take; j += kTileThreads) {
-                const uint32_t k = __ldcs(keys + beg + c0 + j);
-                const uint64_t w = __ldcs(vals + beg + c0 + j);
+            for (int j = tid; j < take; j += T) {
+                const uint32_t k = __ldcg(a.kB + beg + c0 + j);
+                const uint64_t w = __ldcg(a.vB + beg + c0 + j);
                 q.a[len + j] = qc_pack(k & kKeyMask, (unsigned)(w >> 31), (unsigned)(len + j));
                 q.si[len + j] = (int)(w & 0x7FFFFFFFull);
             }
             __syncthreads();
             // the buckets span the points' own range, which is the tile's
             int lo = INT_MAX, hi = INT_MIN;
-            for (int j = tid; j < len + take; j += kTileThreads) {
+            for (int j = tid; j < len + take; j += T) {
                 lo = min(lo, qc_u(q.a[j]));
                 hi = max(hi, qc_u(q.a[j]));
             }
             lo = block_reduce<int>(lo, [](int x, int y) { return min(x, y); }, q.tmp);
             hi = block_reduce<int>(hi, [](int x, int y) { return max(x, y); }, q.tmp);
-            qc_sort<kTileThreads>(q, len + take, lo, hi);
+            qc_sort<T>(q, len + take, lo, hi);
             src = q.a;
             dst = q.b;
-            len = qc_eliminate<kTileThreads>(src, dst, len + take, q.tmp);
+            len = qc_eliminate<T>(src, dst, len + take, q.tmp);
             c0 += (unsigned)take;
             if (len > kCarry && c0 < cnt) {   // no room for the rest
-                if (tid == 0) ctl->bk_state = 2;
+                if (tid == 0) a.ctl->bk_state = 2;
                 len = 0;
                 break;
             }
         }
-        for (int j = tid; j < len; j += kTileThreads) {
+        for (int j = tid; j < len; j += T) {
             const unsigned long long w = src[j];
-            cu[beg + j] = qc_u(w);
-            cv[beg + j] = qc_v(w);
-            ci[beg + j] = q.si[qc_pos(w)];
+            a.cu[beg + j] = qc_u(w);
+            a.cv[beg + j] = qc_v(w);
+            a.ci[beg + j] = q.si[qc_pos(w)];
         }
-        if (tid == 0) tlen[t] = len;
+        if (tid == 0) a.tlen[t] = len;
     }
 }
 
@@ -266,30 +261,54 @@ struct QcJoin {
     unsigned off[kPtGroups];   // tile chains' places in the queue
     int tmp[33];
 };
-constexpr size_t kQueueSmem = sizeof(QcJoin) > sizeof(QcQueue) ? sizeof(QcJoin) : sizeof(QcQueue);
-static_assert(kQueueSmem <= 226 * 1024 && QcJoin::kCap < (1 << kQcPosBits), "one block's shared memory");
+constexpr size_t large_max(size_t x, size_t y) { return x > y ? x : y; }
+constexpr size_t kLargeSmem = large_max(large_max(sizeof(QcJoin), sizeof(QcQueue)),
+                                        large_max(sizeof(TileHistSmem), sizeof(TilePartSmem)));
+static_assert(kLargeSmem <= 226 * 1024 && QcJoin::kCap < (1 << kQcPosBits), "one block's shared memory");
 
-// Block q: queue q's chain from its records (path queues) or its tiles' chains
-// (path tiles), left at the queue's records' place in (vout, iout); the block
-// that finishes last joins the four.
-__global__ void __launch_bounds__(kQueueThreads, 1) queue_kernel(Ctl* ctl, const uint32_t* keys, const uint64_t* vals,
-                                                                 const unsigned* tbeg, const int* tlen, const int* cu,
-                                                                 const int* cv, const int* ci, uint64_t* vout,
-                                                                 int* iout, unsigned* scratch, long long n,
-                                                                 int32_t* out_idx, int64_t* out_n) {
+// Blocks 0 .. 3 end with a queue each: its chain from its records (path queues)
+// or from its tiles' chains (path tiles), left at the queue's records' place in
+// vB (u, v) and cu (index; each queue's own tiles' chains lie there, consumed by
+// then); the block that finishes last joins the four.
+__global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ QMap s_m;
     __shared__ int s_path, s_n, s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, qq = blockIdx.x;
-    constexpr int T = kQueueThreads;
+    constexpr int T = kLargeThreads;
+    Ctl* ctl = a.ctl;
     if (tid == 0) {
-        s_path = on_path(ctl, kPathQueues) ? kPathQueues : on_path(ctl, kPathTiles) ? kPathTiles : 0;
+        s_path = *(volatile int*)&ctl->bk_state == 1 && read_status(ctl) == CH_OK ? *(volatile int*)&ctl->path
+                                                                                  : kPathNone;
         s_n = 0;
     }
     __syncthreads();
     const int path = s_path;
-    if (!path) return;
+    if (path != kPathTiles && (path != kPathQueues || qq >= 4)) return;
     q_map(ctl->oct, s_m);
+    __syncthreads();
+    if (path == kPathTiles) {
+        tile_hist(a, *reinterpret_cast<TileHistSmem*>(s_dyn), s_m);
+        bool go = grid_barrier(&ctl->barrier[1], 1u, ctl);
+        if (go && qq == 0) tile_cut(a, *reinterpret_cast<TileHistSmem*>(s_dyn));
+        go = go && grid_barrier(&ctl->barrier[1], 2u, ctl);
+        if (go) tile_part(a, *reinterpret_cast<TilePartSmem*>(s_dyn), s_m);
+        go = go && grid_barrier(&ctl->barrier[1], 3u, ctl);
+        if (go) tile_chains(a, *reinterpret_cast<QcQueue*>(s_dyn));
+        go = go && grid_barrier(&ctl->barrier[1], 4u, ctl);
+        if (!go && tid == 0) *a.out_n = CH_ETIMEOUT;
+        if (!go || qq >= 4 || *(volatile int*)&ctl->bk_state != 1) return;
+    }
+    const uint32_t* keys = a.keys;
+    const uint64_t* vals = a.vals;
+    const unsigned* tbeg = a.tbeg;
+    const int *tlen = a.tlen, *cu = a.cu, *cv = a.cv, *ci = a.ci;
+    uint64_t* vout = a.vB;
+    int* iout = a.cu;
+    unsigned* scratch = a.kB;
+    const long long n = a.n;
+    int32_t* out_idx = a.out_idx;
+    int64_t* out_n = a.out_n;
     unsigned pre[5];   // records of the queues before each queue
     pre[0] = 0u;
 #pragma unroll
@@ -338,7 +357,7 @@ __global__ void __launch_bounds__(kQueueThreads, 1) queue_kernel(Ctl* ctl, const
         }
     } else {
         QcJoin& q = *reinterpret_cast<QcJoin*>(s_dyn);
-        const unsigned t0 = ctl->q_tile[qq], nt = ctl->q_tile[qq + 1] - t0;
+        const unsigned t0 = *(volatile unsigned*)&ctl->q_tile[qq], nt = *(volatile unsigned*)&ctl->q_tile[qq + 1] - t0;
         constexpr int kE = kPtGroups / T;
         unsigned c[kE], sum = 0u;
 #pragma unroll
@@ -358,7 +377,7 @@ __global__ void __launch_bounds__(kQueueThreads, 1) queue_kernel(Ctl* ctl, const
         ok = tot <= QcJoin::kCap;
         if (ok) {
             for (unsigned t = warp; t < nt; t += T / 32) {
-                const unsigned o = q.off[t], l = (unsigned)__ldcg(tlen + t0 + t), b = tbeg[t0 + t];
+                const unsigned o = q.off[t], l = (unsigned)__ldcg(tlen + t0 + t), b = __ldcg(tbeg + t0 + t);
                 for (unsigned j = lane; j < l; j += 32) {
                     q.a[o + j] = qc_pack((unsigned)__ldcg(cu + b + j), (unsigned)__ldcg(cv + b + j), o + j);
                     scratch[pre[qq] + o + j] = (unsigned)__ldcg(ci + b + j);
@@ -415,41 +434,17 @@ __global__ void __launch_bounds__(kQueueThreads, 1) queue_kernel(Ctl* ctl, const
 }
 
 // ---------------------------------------------------------------------------
-void launch_tiles(Ctl* ctl, uint32_t* kA, uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned* tiles, int* cu, int* cv,
-                  int* ci, int sms, cudaStream_t s) {
-    unsigned *ghist = tiles, *gtile = ghist + kPtGroups, *tbeg = gtile + kPtGroups, *tcur = tbeg + kPtGroups;
-    int* tlen = (int*)(tcur + kPtGroups);
-    { ProfScope p("bk_hist", s); tile_hist_kernel<<<sms, kPtThreads, 0, s>>>(ctl, kA, ghist, gtile, tbeg, tcur); }
-    {
-        ProfScope p("bk_part1", s);
-        tile_part_kernel<<<sms, kPtThreads, sizeof(TilePartSmem), s>>>(ctl, kA, vA, gtile, tcur, kB, vB);
-    }
-    {
-        ProfScope p("bk_hull", s);
-        tile_chain_kernel<<<4 * sms, kTileThreads, sizeof(QcTile), s>>>(ctl, kB, vB, tbeg, tcur, cu, cv, ci, tlen);
-    }
+void launch_large(Ctl* ctl, const uint32_t* kA, const uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned* tiles, int* cu,
+                  int* cv, int* ci, long long n, int32_t* out_idx, int64_t* out_n, int grid, cudaStream_t s) {
+    const LargeArgs a{ctl, kA, vA, kB, vB, tiles, tiles + kPtGroups, tiles + 2 * kPtGroups, tiles + 3 * kPtGroups,
+                      (int*)(tiles + 4 * kPtGroups), cu, cv, ci, n, out_idx, out_n};
+    launch_grid(large_kernel, grid, kLargeThreads, kLargeSmem, s, a);
 }
 
 size_t tiles_bytes() { return sizeof(unsigned) * 5 * (size_t)kPtGroups; }
 
-void launch_queues(Ctl* ctl, const uint32_t* kA, const uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned* tiles,
-                   int* cu, int* cv, int* ci, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s) {
-    ProfScope p("queues", s);
-    unsigned* tbeg = tiles + 2 * kPtGroups;
-    // the tile chains are consumed into shared memory and kB before the
-    // queue's chain is written to vB and cu (each queue to its own records'
-    // place, where only its own tiles' chains lie)
-    queue_kernel<<<4, kQueueThreads, kQueueSmem, s>>>(ctl, kA, vA, tbeg, (const int*)(tbeg + 2 * kPtGroups), cu, cv,
-                                                      ci, vB, cu, kB, n, out_idx, out_n);
-}
-
-cudaError_t configure_queue_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(tile_part_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(TilePartSmem));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(tile_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(QcTile));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(queue_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQueueSmem);
+cudaError_t configure_large_kernel() {
+    return cudaFuncSetAttribute(large_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLargeSmem);
 }
 
 }  // namespace ch

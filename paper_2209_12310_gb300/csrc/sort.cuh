@@ -1,4 +1,4 @@
-// sort.cu -- stable LSD radix sort of the survivor records by (queue, u).
+// sort.cuh -- stable LSD radix sort of the survivor records by (queue, u).
 //
 // The paper keeps the survivors of each queue semi-ordered in a priority
 // queue (a heap, Sec. 1.2, "partial ordering") and builds each queue's hull
@@ -8,15 +8,17 @@
 // pass ranks a 4096-record tile in shared memory, publishes its per-digit
 // counts, resolves its global offsets by decoupled look-back over the
 // preceding tiles, and scatters.  The digit histograms of all three passes
-// come from one counting pass over the records (sort_hist_kernel) before the
-// first scatter; the post pass keeps only per-queue counts.
+// come from one counting pass over the records (sort_hist) before the first
+// scatter; the post pass keeps only per-queue counts.  These are phases of
+// sort_kernel (hull.cu), with grid barriers between them.
 //
 // Look-back waits are bounded (kSpinLimit polls with back-off); a wait that
 // gives up raises CH_ETIMEOUT and the abort flag, after which every other
 // wait gives up too.  Tiles are claimed in order through an atomic counter, so
 // a tile only ever waits for tiles whose blocks are already running.
+#pragma once
+
 #include "ch_internal.cuh"
-#include "launch.h"
 
 namespace ch {
 
@@ -35,7 +37,7 @@ __device__ __forceinline__ unsigned long long ld_volatile(const unsigned long lo
 }
 
 // Exclusive scan of 2 values per thread over a 256-thread block.
-__device__ __forceinline__ unsigned block_excl_scan(unsigned x, unsigned* s_warp) {
+__device__ __forceinline__ unsigned sort_excl_scan(unsigned x, unsigned* s_warp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned incl = x;
 #pragma unroll
@@ -51,16 +53,21 @@ __device__ __forceinline__ unsigned block_excl_scan(unsigned x, unsigned* s_warp
     return off + incl - x;
 }
 
-__global__ void __launch_bounds__(kSortThreads) onesweep_kernel(
-    const uint32_t* __restrict__ kin, const uint64_t* __restrict__ vin, uint32_t* __restrict__ kout,
-    uint64_t* __restrict__ vout, Ctl* ctl, unsigned long long* status, int pass) {
-    __shared__ unsigned s_base[kDigits];
-    __shared__ unsigned s_excl[kDigits];
-    __shared__ unsigned short s_wcnt[kSortThreads / 32][kDigits];
-    __shared__ unsigned s_warp[kSortThreads / 32];
-    __shared__ unsigned s_tile;
+struct SortSmem {
+    unsigned base[kDigits];
+    unsigned excl[kDigits];
+    unsigned short wcnt[kSortThreads / 32][kDigits];
+    unsigned warp[kSortThreads / 32];
+    unsigned tile;
+};
 
-    if (*(volatile int*)&ctl->done || read_status(ctl) != CH_OK || *(volatile int*)&ctl->bk_state == 1) return;
+__device__ void onesweep(SortSmem& sm, const uint32_t* kin, const uint64_t* vin, uint32_t* kout, uint64_t* vout, Ctl* ctl,
+                         unsigned long long* status, int pass) {
+    unsigned(&s_base)[kDigits] = sm.base;
+    unsigned(&s_excl)[kDigits] = sm.excl;
+    unsigned short(&s_wcnt)[kSortThreads / 32][kDigits] = sm.wcnt;
+    unsigned(&s_warp)[kSortThreads / 32] = sm.warp;
+    unsigned& s_tile = sm.tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned count = ctl->count;
     const unsigned ntiles = (count + kSortTile - 1) / kSortTile;
@@ -78,7 +85,7 @@ __global__ void __launch_bounds__(kSortThreads) onesweep_kernel(
         if (!have_base) {   // global digit offsets of this pass (once per block)
             const unsigned a = ctl->digit_hist[pass][2 * threadIdx.x];
             const unsigned b = ctl->digit_hist[pass][2 * threadIdx.x + 1];
-            const unsigned ex = block_excl_scan(a + b, s_warp);
+            const unsigned ex = sort_excl_scan(a + b, s_warp);
             s_base[2 * threadIdx.x] = ex;
             s_base[2 * threadIdx.x + 1] = ex + a;
             have_base = true;
@@ -171,11 +178,8 @@ __global__ void __launch_bounds__(kSortThreads) onesweep_kernel(
     }
 }
 
-// Digit histograms of the records for the three passes (the sort-based
-// path only: the others need none and leave bk_state == 1).
-__global__ void __launch_bounds__(kSortThreads) sort_hist_kernel(const uint32_t* __restrict__ keys, Ctl* ctl) {
-    __shared__ unsigned s_h[kSortPasses][kDigits];
-    if (*(volatile int*)&ctl->done || read_status(ctl) != CH_OK || *(volatile int*)&ctl->bk_state == 1) return;
+// Digit histograms of the records for the three passes.
+__device__ void sort_hist(unsigned (*s_h)[kDigits], const uint32_t* keys, Ctl* ctl) {
     for (int i = threadIdx.x; i < kSortPasses * kDigits; i += blockDim.x) (&s_h[0][0])[i] = 0u;
     __syncthreads();
     const unsigned count = ctl->count;
@@ -189,20 +193,6 @@ __global__ void __launch_bounds__(kSortThreads) sort_hist_kernel(const uint32_t*
         const unsigned c = (&s_h[0][0])[i];
         if (c) atomicAdd(&(&ctl->digit_hist[0][0])[i], c);
     }
-}
-
-void launch_sort_hist(const uint32_t* keys, Ctl* ctl, int grid, cudaStream_t s) {
-    sort_hist_kernel<<<grid, kSortThreads, 0, s>>>(keys, ctl);
-}
-
-void launch_sort_pass(const uint32_t* kin, const uint64_t* vin, uint32_t* kout, uint64_t* vout,
-                      Ctl* ctl, unsigned long long* status, int pass, int grid, cudaStream_t s) {
-    onesweep_kernel<<<grid, kSortThreads, 0, s>>>(kin, vin, kout, vout, ctl, status, pass);
-}
-
-
-cudaError_t occupancy_sort(int* b) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(b, onesweep_kernel, kSortThreads, 0);
 }
 
 }  // namespace ch

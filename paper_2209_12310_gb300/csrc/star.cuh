@@ -5,10 +5,9 @@
 // every point.  A polygon with thousands of vertices that are input points
 // hugs the hull far closer.  It is built from a sample: around a centre c,
 // the sample is split into kStarBins angular bins and each bin keeps its point
-// farthest from c (star.cu); every post-pass block then builds the polygon
-// in shared memory (star_finish): it gathers the bins' points, drops some
-// reflex vertices, which only enlarges the polygon, checks it exactly, and
-// builds the lookup tables of the point tests.
+// farthest from c (dense_kernel); one block then builds the polygon (star_finish):
+// it gathers the bins' points, drops reflex vertices, which only enlarges the
+// polygon, checks it exactly, and builds the lookup tables of the point tests.
 //
 // Why dropping points strictly inside it is exact: every vertex is an input
 // point, and the polygon is star-shaped around c with every wedge
@@ -24,36 +23,44 @@
 
 namespace ch {
 
-// The finished polygon (shared memory of a post-pass block):
+// The finished polygon:
 //   v    vertices relative to c (|.| < 2^24: every orientation is exact in
 //        int64), counter-clockwise, the first two repeated after the last;
 //   tbl  per bin, the last vertex whose bin comes before it (K - 1 if none);
-//   rin  per bin, an integer radius no larger than the distance from c to
-//        the line of any edge whose wedge meets the bin or its two
-//        neighbours on either side: a point of the bin closer to c than that
-//        is strictly inside (0 when no bound was found);
-//   rmin the smallest line radius of all edges: a point closer to c than
-//        that is strictly inside, whatever its bin (it lies in some wedge,
-//        on the inner side of that wedge's edge line).
+//   thr  per bin, a bound on the squared distance from c as floats compute it:
+//        let r be an integer radius no larger than the distance from c to the
+//        line of any edge whose wedge meets the bin or its two neighbours on
+//        either side; a point of the bin closer to c than r is strictly inside.
+//        thr is r^2 less 5 parts in 2^24, rounded down, and star_d2 is at most
+//        2 parts in 2^24 below d^2: star_d2 < thr proves d < r.  (0 when no
+//        bound was found.)
+//   tmin the same for the smallest line radius of all edges: a point closer
+//        to c than that is strictly inside, whatever its bin (it lies in some
+//        wedge, on the inner side of that wedge's edge line).
 struct StarPoly {
     int2 v[kStarBins + 2];
     unsigned short tbl[kStarBins];
-    unsigned rin[kStarBins];
-    unsigned rmin;
+    float thr[kStarBins];
+    float tmin;
     unsigned pad[3];
 };
 
-// Angular bin of an offset (dx, dy) from c: a pseudo-angle in [0, 4) that
-// grows with the angle (|dy| / (|dx| + |dy|) per quadrant), scaled to
-// kStarBins bins.  Float rounding may move a point near a bin boundary to the
-// neighbouring bin; no test relies on the bin being right to within one bin.
-__device__ __forceinline__ int star_bin(int dx, int dy) {
-    const float fx = (float)dx, fy = (float)dy;   // exact: |d| < 2^24
-    const float ax = fabsf(fx), ay = fabsf(fy), s = ax + ay;
-    const float t = s > 0.0f ? __fdividef(ay, s) : 0.0f;
-    const float a = fx >= 0.0f ? (fy >= 0.0f ? t : 4.0f - t) : (fy >= 0.0f ? 2.0f - t : 2.0f + t);
-    return (int)(a * (float)(kStarBins / 4)) & (kStarBins - 1);
+// Angular bin of an offset (dx, dy) from c (integers below 2^24, exact as
+// floats): a pseudo-angle in [0, 4) that grows with the angle (1 - dx / (|dx| +
+// |dy|) above, 3 + dx / (|dx| + |dy|) below), scaled to kStarBins bins and
+// rounded to the nearest (adding 2^23 leaves the integer in the low bits).
+// Float rounding may move a point near a bin boundary to the neighbouring
+// bin; no test relies on the bin being right to within one bin.
+__device__ __forceinline__ int star_bin(float dx, float dy) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fabsf(dx) + fabsf(dy)));
+    const float w = copysignf(fmaf(dx, r, 1.0f), dy);
+    return __float_as_int(fmaf(w, -(float)(kStarBins / 4), 8388608.0f + (float)(kStarBins / 2))) & (kStarBins - 1);
 }
+__device__ __forceinline__ int star_bin(int dx, int dy) { return star_bin((float)dx, (float)dy); }
+
+// Squared distance in floats: two roundings, at most 2 parts in 2^24 low.
+__device__ __forceinline__ float star_d2(float dx, float dy) { return fmaf(dx, dx, dy * dy); }
 
 // orient(c, v, p) for v, p given relative to c.
 __device__ __forceinline__ long long star_orient_c(int2 v, int px, int py) {
@@ -76,36 +83,52 @@ __device__ __forceinline__ bool star_inside_exact(int px, int py, int b, const S
     return spoke_ok && side > 0;
 }
 
-// Fast test, exact in int64: true when p = c + (px, py) lies closer to c than
-// its bin's radius bound, hence strictly inside; false says nothing.
-__device__ __forceinline__ bool star_inside_fast(int px, int py, int b, const StarPoly& P) {
-    const long long r = (long long)P.rin[b];
-    return (long long)px * px + (long long)py * py < r * r;
+// Fast test: true when p = c + (dx, dy) lies closer to c than its bin's
+// radius bound, hence strictly inside; false says nothing.
+__device__ __forceinline__ bool star_inside_fast(float dx, float dy, int b, const StarPoly& P) {
+    return star_d2(dx, dy) < P.thr[b];
 }
 
 // Full test: the bin's radius bound, then the exact wedge test.
 __device__ __forceinline__ bool star_inside(int px, int py, const StarPoly& P) {
     const int b = star_bin(px, py);
-    return star_inside_fast(px, py, b, P) || star_inside_exact(px, py, b, P);
+    return star_inside_fast((float)px, (float)py, b, P) || star_inside_exact(px, py, b, P);
 }
 
 // The largest integer r with r^2 <= o^2 / l2: the distance from c to an edge
 // line with orient(c, A, B) = o and |B - A|^2 = l2 (0 < o < 2^50,
-// 0 < l2 < 2^52; the distance is below 2^25), rounded down.  A float
-// estimate (four roundings of 2^-24 each: off by less than 8) less 8 is
-// raised step by step while (r + 1)^2 l2 <= o^2 holds in exact 128-bit
-// arithmetic.  Every loop is bounded; leaving one early only lowers the
-// result, and 0 means no bound.
+// 0 < l2 < 2^52; the distance is below 2^25), rounded down.  A float estimate
+// (four roundings of 2^-24 each: off by less than 8) takes one Newton step on
+// the exact 128-bit residual, then single steps while they improve it.  Every
+// loop is bounded; leaving one early only lowers the result, and 0 means no
+// bound.
 __device__ __forceinline__ unsigned star_line_radius(long long o, long long l2) {
     typedef unsigned __int128 u128;
     const unsigned long long ul = (unsigned long long)l2;
     const u128 oo = (u128)(unsigned long long)o * (unsigned long long)o;
-    const float rf = (float)o / sqrtf((float)l2);
-    unsigned long long r = rf > 8.0f ? (unsigned long long)rf - 8ull : 0ull;
-    for (int it = 0; it < 8 && r > 0ull && (u128)(r * r) * ul > oo; ++it) --r;
+    const float root = sqrtf((float)l2);
+    const float rf = (float)o / root;
+    if (rf < 16.0f) return 0u;   // too close to c to be of use
+    unsigned long long r = (unsigned long long)rf;
+    {
+        // residual / (2 r l2), below 10 in magnitude
+        const u128 rr = (u128)(r * r) * ul;
+        const bool over = rr > oo;
+        const u128 e = over ? rr - oo : oo - rr;
+        const float ef = fmaf(__ull2float_rn((unsigned long long)(e >> 64)), 18446744073709551616.0f,
+                              __ull2float_rn((unsigned long long)e));
+        const float step = ef / (2.0f * rf * (float)l2);
+        r = over ? r - (unsigned long long)ceilf(step) : r + (unsigned long long)floorf(step);
+    }
+    for (int it = 0; it < 4 && (u128)(r * r) * ul > oo; ++it) --r;
     if ((u128)(r * r) * ul > oo) return 0u;
-    for (int it = 0; it < 24 && (u128)((r + 1ull) * (r + 1ull)) * ul <= oo; ++it) ++r;
+    for (int it = 0; it < 4 && (u128)((r + 1ull) * (r + 1ull)) * ul <= oo; ++it) ++r;
     return (unsigned)r;
+}
+
+// Bound on star_d2 for radius r (see StarPoly).
+__device__ __forceinline__ float star_threshold(unsigned r) {
+    return __fmul_rd(__ull2float_rd((unsigned long long)r * r), 1.0f - 5.0f / 16777216.0f);
 }
 
 // Block-wide exclusive scan of one count per thread (warp shuffles, then the
@@ -135,50 +158,105 @@ __device__ __forceinline__ int star_scan(int c, unsigned* s, int* total) {
     return (int)(before + incl - (unsigned)c);
 }
 
-constexpr int kStarSweeps = 4;   // reflex-removal sweeps (alternately even and odd positions)
+// A vertex under construction: (dx, dy) relative to c, biased by 2^24 (25 bits
+// each), and its bin (13 bits).
+static_assert(kStarBins == 1 << 13, "a vertex's bin has 13 bits");
+__device__ __forceinline__ unsigned long long star_pack(int dx, int dy, int b) {
+    return ((unsigned long long)(unsigned)(dx + kCoordLimit) << 38) |
+           ((unsigned long long)(unsigned)(dy + kCoordLimit) << 13) | (unsigned)b;
+}
+__device__ __forceinline__ int2 star_xy(unsigned long long w) {
+    return make_int2((int)(w >> 38) - kCoordLimit, (int)((w >> 13) & 0x1FFFFFFull) - kCoordLimit);
+}
 
-// Builds the polygon in shared memory, all T threads of the block, from the
-// star pass's bins (bins[b]: the packed farthest point of bin b, or 0) around
-// c = (cx, cy): work area A (va, ba) and the polygon P, whose first bytes
-// double as work area B (vb, bb).  Returns the polygon's vertex count (the
-// same in every thread) when it passed its checks and P is ready, else 0;
-// leaves the bins as they are.  With kSharedBins the bins are in this
-// block's shared memory, and they may share their bytes with work area A:
-// every bin is read before the first write to A.
+// Drops the reflex and flat vertices of the polygon of the n points in src
+// (counter-clockwise around c, cyclic), until a round drops none or kStarRounds
+// rounds are done; returns the vertices left, src points at them.  A vertex m
+// between a and z goes when orient(a, m, z) <= 0 and a and z turn by less than
+// pi around c: it then lies in the hull of c, a and z, whatever becomes of a
+// and z.  So every thread takes a run of consecutive vertices, with the vertex
+// before and the one after it as fixed context, through Andrew's scan, and the
+// runs that are left are packed together and cut at other places in the next
+// round (qc_eliminate's rounds, cyclic).  Dropping such vertices only enlarges
+// the polygon, towards the hull of its points.  Whole block of T threads.
+constexpr int kStarRounds = 12;
+
+template <int T>
+__device__ int star_eliminate(unsigned long long*& src, unsigned long long*& dst, int n, unsigned* s_scan,
+                              int* s_tot) {
+    const int tid = threadIdx.x;
+    for (int round = 0; round < kStarRounds && n > 3; ++round) {
+        const int c = max(5, (n + T - 2) / (T - 1)) | 1;
+        const int shift = (round & 1) ? c / 2 : 0;
+        const int l0 = tid * c - shift;
+        const int lo = max(0, min(n, l0)), hi = max(0, min(n, l0 + c));
+        const bool some = lo < hi;
+        const int2 left = star_xy(some ? src[lo > 0 ? lo - 1 : n - 1] : 0ull);
+        const int2 right = star_xy(some ? src[hi < n ? hi : 0] : 0ull);
+        __syncthreads();   // every context is read before the runs are rewritten
+        int2 top = left, sec = left;
+        int cnt = 0;   // vertices kept: src[lo .. lo + cnt)
+        auto pop_before = [&](int2 w) {
+            while (cnt > 0) {
+                const long long turn =
+                    (long long)(top.x - sec.x) * (w.y - sec.y) - (long long)(top.y - sec.y) * (w.x - sec.x);
+                if (turn > 0 || star_orient_c(sec, w.x, w.y) <= 0) break;
+                --cnt;
+                top = sec;
+                sec = cnt >= 2 ? star_xy(src[lo + cnt - 2]) : left;
+            }
+        };
+        for (int j = lo; j < hi; ++j) {
+            const unsigned long long w = src[j];
+            const int2 p = star_xy(w);
+            pop_before(p);
+            src[lo + cnt] = w;
+            ++cnt;
+            sec = top;
+            top = p;
+        }
+        if (some) pop_before(right);
+        const int off = star_scan<T>(cnt, s_scan, s_tot);
+        const int tot = *s_tot;
+        __syncthreads();   // read by all before the next scan writes it
+        if (tot == n) break;
+        for (int j = 0; j < cnt; ++j) dst[off + j] = src[lo + j];
+        __syncthreads();
+        unsigned long long* t = src;
+        src = dst;
+        dst = t;
+        n = tot;
+    }
+    return n;
+}
+
+// Builds the polygon in P, all T threads of the block, from the star pass's
+// bins (bins[b]: the packed farthest point of bin b, or 0) around c = (cx, cy);
+// work: kStarBins words of shared memory, P too is in shared memory (its first
+// kStarBins words double as the second work area).  Returns the number of
+// points it was made of (the same in every thread) when it passed its checks
+// and P is ready, else 0; leaves the bins as they are.  With kSharedBins the bins are in
+// this block's shared memory and may share their bytes with work: every bin is
+// read before the first write to it.
 //
 // Gather: each non-empty bin's point is re-read from the input by its index
 // (so every vertex is an input point of this call, whatever the bins held)
 // and kept if it is a valid coordinate and falls in that bin again; the kept
-// points, in bin order, are the vertices.
-//
-// Sweeps: a vertex at an even (then odd) position is dropped when it is
-// reflex or flat, orient(V_j-1, V_j, V_j+1) <= 0, and its neighbours still
-// turn by less than pi around c, orient(c, V_j-1, V_j+1) > 0; same-parity
-// vertices are never neighbours (with K odd, the last vertex sits out the
-// even sweeps), so every drop sees its neighbours unchanged.  Dropping a
-// reflex vertex adds the triangle (V_j-1, V_j, V_j+1) to the polygon.
-//
-// Threads own contiguous chunks of the vertex list (the compaction keeps the
-// order); each lane walks its chunk from a different start, so that the
-// lanes of a warp touch different shared-memory banks.
+// points, in bin order, are the vertices.  Then star_eliminate, and the checks.
 template <int T, bool kSharedBins = false>
-__device__ int star_finish(const unsigned long long* bins, const float* __restrict__ pts, long long n,
-                            int cx, int cy, int2* va, unsigned short* ba, StarPoly& P, Ctl* ctl) {
+__device__ int star_finish(const unsigned long long* bins, const float* __restrict__ pts, long long n, int cx, int cy,
+                           unsigned long long* work, StarPoly& P, Ctl* ctl) {
     (void)ctl;   // debug timeline only
     static_assert(T % 32 == 0 && T >= 256 && T <= 1024, "block size");
     constexpr int kPer = kStarBins / T;   // bins per thread: at most 32
-    static_assert(sizeof(StarPoly) >= sizeof(int2) * kStarBins + sizeof(unsigned short) * kStarBins,
-                  "work area B fits in the polygon");
-    int2* vb = P.v;
-    unsigned short* bb = reinterpret_cast<unsigned short*>(reinterpret_cast<char*>(P.v) +
-                                                           sizeof(int2) * kStarBins);
+    static_assert(kPer <= 16, "gather registers");
+    static_assert(sizeof(P.v) >= sizeof(unsigned long long) * kStarBins, "the second work area fits in the vertices");
     __shared__ unsigned s_scan[T / 32];
-    __shared__ int s_K, s_bad, s_cross;
-    const int t = threadIdx.x, lane = t & 31;
+    __shared__ int s_K, s_bad, s_cross, s_last[T / 32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (t == 0) { s_bad = 0; s_cross = 0; }
     // 1. gather: bins [t kPer, (t + 1) kPer); all their keys, then all their
     // points, in flight at once
-    static_assert(kPer <= 16, "gather registers");
     unsigned kept = 0u;
     int2 d[kPer];
     {
@@ -202,72 +280,31 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
             if (valid && star_bin(X - cx, Y - cy) == b) kept |= 1u << i;
         }
     }
+    unsigned long long *src = work, *dst = reinterpret_cast<unsigned long long*>(P.v);
     {
         const int off = star_scan<T>(__popc(kept), s_scan, &s_K);
 #pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            if (!((kept >> i) & 1u)) continue;
-            const int o = off + __popc(kept & ((1u << i) - 1u));
-            va[o] = d[i];
-            ba[o] = (unsigned short)(t * kPer + i);
-        }
+        for (int i = 0; i < kPer; ++i)
+            if ((kept >> i) & 1u)
+                src[off + __popc(kept & ((1u << i) - 1u))] = star_pack(d[i].x, d[i].y, t * kPer + i);
     }
     __syncthreads();
     CH_TL(ctl, 9, 1);
-    if (s_K < 3) return 0;
-    // 2. sweeps, A -> B -> A ...
-    int2* src = va; int2* dst = vb;
-    unsigned short* bsrc = ba; unsigned short* bdst = bb;
-    int idle = 0;   // consecutive sweeps that dropped nothing
-    for (int sweep = 0; sweep < kStarSweeps && idle < 2; ++sweep) {
-        const int k = s_K;
-        if (k <= 3) break;
-        const int par = sweep & 1;
-        const int chunk = (k + T - 1) / T;   // <= kPer
-        const int lo = min(k, t * chunk), hi = min(k, lo + chunk), len = hi - lo;
-        const int rot = len > 0 ? lane % len : 0;
-        unsigned keep = 0u;
-        for (int i = 0; i < len; ++i) {
-            int jj = i + rot;
-            if (jj >= len) jj -= len;
-            const int j = lo + jj;
-            bool drop = (j & 1) == par && !((k & 1) && j == k - 1);
-            if (drop) {
-                const int2 a = src[j == 0 ? k - 1 : j - 1], m = src[j], z = src[j + 1 == k ? 0 : j + 1];
-                const long long turn = (long long)(m.x - a.x) * (z.y - a.y) - (long long)(m.y - a.y) * (z.x - a.x);
-                drop = turn <= 0 && star_orient_c(a, z.x, z.y) > 0;
-            }
-            if (!drop) keep |= 1u << jj;
-        }
-        __syncthreads();   // every read of s_K and src of this sweep is done
-        const int off = star_scan<T>(__popc(keep), s_scan, &s_K);
-        idle = s_K == k ? idle + 1 : 0;
-        for (int i = 0; i < len; ++i) {
-            int jj = i + rot;
-            if (jj >= len) jj -= len;
-            if (!((keep >> jj) & 1u)) continue;
-            const int o = off + __popc(keep & ((1u << jj) - 1u));
-            dst[o] = src[lo + jj];
-            bdst[o] = bsrc[lo + jj];
-        }
-        __syncthreads();
-        int2* tv = src; src = dst; dst = tv;
-        unsigned short* tb = bsrc; bsrc = bdst; bdst = tb;
-    }
+    const int K0 = s_K;
+    __syncthreads();
+    if (K0 < 3) return 0;
+    // 2. reflex vertices
+    const int K = star_eliminate<T>(src, dst, K0, s_scan, &s_K);
     CH_TL(ctl, 10, 1);
-    int K = s_K;
-    if (src != va) {   // the list must sit in A before P is written over B
-        for (int i = t; i < K; i += T) {
-            va[i] = vb[i];
-            ba[i] = bb[i];
-        }
+    if (src != work) {   // the list must sit in work before P is written over it
+        for (int i = t; i < K; i += T) work[i] = src[i];
         __syncthreads();
     }
     // 3. checks: every wedge turns counter-clockwise by less than pi, and
     // exactly one edge crosses the ray from c along +x (the wedges wind once)
     int bad = 0, cross = 0;
     for (int j = t; j < K; j += T) {
-        const int2 a = va[j], b = va[j + 1 == K ? 0 : j + 1];
+        const int2 a = star_xy(work[j]), b = star_xy(work[j + 1 == K ? 0 : j + 1]);
         bad |= star_orient_c(a, b.x, b.y) <= 0;
         cross += (a.y < 0 && b.y >= 0) ? 1 : 0;
     }
@@ -276,22 +313,47 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
     __syncthreads();
     const bool ok = K >= 3 && !s_bad && s_cross == 1;
     if (!ok) return 0;
-    // 4. the polygon: vertices, the bin table, then the radius bounds
-    for (int j = t; j < K + 2; j += T) P.v[j] = va[j < K ? j : j - K];
-    for (int j = t; j < K; j += T) {
-        const int b0 = ba[j];
-        const int b1 = j + 1 < K ? (int)ba[j + 1] : (int)ba[0] + kStarBins;
-        for (int b = b0 + 1; b <= b1; ++b) P.tbl[b & (kStarBins - 1)] = (unsigned short)j;
+    // 4. the polygon: vertices; the bin table by a running maximum over the
+    // bins' vertices (thr holds them meanwhile, no vertex as -1)
+    int* mark = reinterpret_cast<int*>(P.thr);
+    for (int j = t; j < K + 2; j += T) P.v[j] = star_xy(work[j < K ? j : j - K]);
+    for (int b = t; b < kStarBins; b += T) mark[b] = -1;
+    __syncthreads();
+    for (int j = t; j < K; j += T) mark[(int)(work[j] & (kStarBins - 1))] = j;
+    __syncthreads();
+    {
+        int m[kPer], best = -1;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            m[i] = mark[t * kPer + i];
+            best = max(best, m[i]);
+        }
+        int incl = best;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl = max(incl, u);
+        }
+        if (lane == 31) s_last[warp] = incl;
+        int run = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+        if (lane == 0) run = -1;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) run = max(run, s_last[w]);
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            P.tbl[t * kPer + i] = (unsigned short)(run < 0 ? K - 1 : run);
+            run = max(run, m[i]);
+        }
     }
     __syncthreads();
     CH_TL(ctl, 11, 1);
-    // each edge's line radius (work area A is free again), then per bin the
-    // smallest over the edges whose wedges can hold its points: from the last
-    // vertex before bin b - 2 to the first vertex from bin b + 2 on
-    unsigned* er = reinterpret_cast<unsigned*>(va);
-    if (t == 0) P.rmin = 0xFFFFFFFFu;
+    // each edge's line radius (work is free again), then per bin the smallest
+    // over the edges whose wedges can hold its points: from the last vertex
+    // before bin b - 2 to the first vertex from bin b + 2 on
+    unsigned* er = reinterpret_cast<unsigned*>(work);
+    if (t == 0) s_K = 0x7FFFFFFF;
     __syncthreads();
-    unsigned emin = 0xFFFFFFFFu;
+    unsigned emin = 0x7FFFFFFFu;
     for (int e = t; e < K; e += T) {
         const int2 a = P.v[e], c2 = P.v[e + 1];
         const long long o = (long long)a.x * c2.y - (long long)a.y * c2.x;   // > 0 (checked above)
@@ -300,7 +362,7 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
         emin = min(emin, er[e]);
     }
     emin = __reduce_min_sync(0xFFFFFFFFu, emin);
-    if (lane == 0 && emin != 0xFFFFFFFFu) atomicMin(&P.rmin, emin);
+    if (lane == 0) atomicMin(&s_K, (int)emin);
     __syncthreads();
     CH_TL(ctl, 12, 1);
     for (int b = t; b < kStarBins; b += T) {
@@ -314,10 +376,11 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
             m = min(m, er[e]);
             ++steps;
         }
-        P.rin[b] = e == last ? m : 0u;   // a window longer than 8 edges gets no bound
+        P.thr[b] = star_threshold(e == last ? m : 0u);   // a window longer than 8 edges gets no bound
     }
+    if (t == 0) P.tmin = star_threshold((unsigned)s_K);
     __syncthreads();
-    return K;
+    return K0;
 }
 
 }  // namespace ch

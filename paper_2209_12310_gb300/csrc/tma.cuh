@@ -78,6 +78,7 @@ struct WarpStreamT {
     const float4* src;            // 16-byte aligned body of the point array
     long long first, stride, ntiles;
     int lane;
+    bool keep = false;            // leave the data in L2 for a later pass (else evicted first)
 
     __device__ __forceinline__ void issue(long long k) {
         const long long t = first + k * stride;
@@ -85,7 +86,7 @@ struct WarpStreamT {
             const int s = (int)(k % kStages);
             fence_proxy_async();
             mbar_expect_tx(&bar[s], kF4 * 16);
-            tma_load(ring + s * kF4, src + t * kF4, kF4 * 16, &bar[s], l2_evict_first());
+            tma_load(ring + s * kF4, src + t * kF4, kF4 * 16, &bar[s], keep ? l2_evict_normal() : l2_evict_first());
         }
     }
     __device__ __forceinline__ void start() {

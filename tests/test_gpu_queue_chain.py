@@ -73,6 +73,7 @@ def test_dense_sets_queue_by_queue(lib, name):
 SINGLE = dict(CASES)
 SINGLE.update({
     "tiles": lambda: [W.ring(8_000_001, 4), W.distorted(20_000_003, 5)],
+    "the dense pass's smallest inputs": lambda: [W.ring(n, n) for n in (65_535, 65_537, 66_000, 70_001, 131_073)],
     "tiles without a polygon": lambda: [_shuffled([_arc(4095)] * 12, 6), _shuffled([_columns(4000)] * 2, 7)],
     "a tile in pieces": lambda: [_shuffled([_arc(100)] * 4000, 8)],
 })
@@ -88,3 +89,15 @@ def test_single_hull_queue_by_queue(lib, name):
         for _ in range(3):   # launched, captured, replayed
             got = lib.hull(pts, out_idx=out_idx, out_n=out_n)
             np.testing.assert_array_equal(got.cpu().numpy(), want, err_msg=str(i))
+
+
+@pytest.mark.parametrize("bad", [-1.0, 0.5, float(1 << 24), float("nan"), float("inf")])
+@pytest.mark.parametrize("at", [0, 150_000, 200_001])
+def test_dense_data_with_a_bad_coordinate(lib, bad, at):
+    pts = W.ring(200_002, 9)
+    pts[at, at & 1] = bad
+    with pytest.raises(lib.CHError) as e:
+        lib.hull(torch.from_numpy(pts).cuda())
+    assert e.value.status == lib.CH_ERANGE
+    good = W.ring(200_002, 10)   # the star pass's bins are clear again
+    np.testing.assert_array_equal(lib.hull(torch.from_numpy(good).cuda()).cpu().numpy(), oracle.hull(good))
