@@ -62,15 +62,18 @@ Layout make_layout(long long n) {
         return r;
     };
     // zeroed at allocation: the control block, the sort's look-back status
-    // words, the merge tree's arrival counters, the star bins and the tile
+    // words, the merge tree's arrival counters and the tile
     // counters (each kernel leaves them in that state for the next call)
     L.off_ctl = take(sizeof(Ctl));
     L.off_status = take(8 * (size_t)kDigits * L.sort_tiles);
     L.off_counters = take(4 * (size_t)kMaxLevels * L.ctcap);
-    L.off_star_bins = take(star_bins_bytes());   // dense_kernel leaves them at zero
     L.off_tiles = take(tiles_bytes());           // large_kernel leaves its counters at zero
     L.zero_bytes = o;
-    L.off_star_poly = take(star_poly_bytes());
+    // inputs that dense_kernel can take (device-independent: at most kStarBlocks
+    // blocks of it run)
+    const bool star = n / kWarpTilePts >= kStarMinTiles;
+    L.off_star_poly = take(star ? star_poly_bytes() : 0);
+    L.off_star_bins = take(star ? star_bins_bytes(kStarBlocks) : 0);
     L.off_kA = take(4 * (size_t)L.cap);
     L.off_kB = take(4 * (size_t)L.cap);
     L.off_vA = take(8 * (size_t)L.cap);
@@ -266,8 +269,8 @@ static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, 
     }
     if (dense) {
         ProfScope p("dense_filter", s);
-        launch_dense(pts, n, head, ntiles, ctl, base + L.off_star_bins, base + L.off_star_poly, vB, kB, kA, vA, di.sms,
-                     s);
+        launch_dense(pts, n, head, ntiles, ctl, base + L.off_star_bins, base + L.off_star_poly, vB, kB, kA, vA,
+                     std::min(di.sms, kStarBlocks), s);
     }
     if (!two_pass) {
         ProfScope p("main_filter", s);
@@ -543,15 +546,15 @@ int ch_hull_counters(void* stream, int64_t* out, int cap) {
 
 #if defined(CH_TRACE) || defined(CH_TIMELINE)
 // Debug builds: the phase timeline of the most recent call on the first
-// workspace (%globaltimer ns; 14 phases, first start and last end of each).
-int ch_trace_timeline(unsigned long long* out28) {
+// workspace (%globaltimer ns; 24 phases, first start and last end of each).
+int ch_trace_timeline(unsigned long long* out48) {
     std::lock_guard<std::mutex> lk(g_mu);
     if (g_ws.empty() || !g_ws.begin()->second.base) return CH_EINVAL;
     Ctl c;
     if (cudaMemcpy(&c, g_ws.begin()->second.base, sizeof(Ctl), cudaMemcpyDeviceToHost) != cudaSuccess) return CH_ECUDA;
-    for (int i = 0; i < 14; ++i) {
-        out28[2 * i] = c.tl[i][0];
-        out28[2 * i + 1] = c.tl[i][1];
+    for (int i = 0; i < 24; ++i) {
+        out48[2 * i] = c.tl[i][0];
+        out48[2 * i + 1] = c.tl[i][1];
     }
     return CH_OK;
 }

@@ -67,10 +67,9 @@ __host__ __device__ __forceinline__ unsigned bk_buckets_for(unsigned cnt) {
     return nb > 0u ? nb : 1u;
 }
 constexpr int kSampleTiles = 1024;            // warp tiles read by the sample pass (512k points)
-// Star polygon of dense data (star.cuh, dense_kernel): angular bins around the sample
-// octagon's centre, extra warp tiles read when the sample is dense.
+// Star polygon of dense data (star.cuh): angular bins around a centre.
 constexpr int kStarBins = 8192;
-constexpr int kStarExtraTiles = 2048;
+constexpr int kStarBlocks = 160;              // blocks of dense_kernel at most
 constexpr long long kStarMinTiles = 128;      // inputs below this many warp tiles skip the star pass
 // Inputs of at most this many points stay in L2 between two passes, so the
 // extremes come first and no sample is needed (the fused pass saves reads of
@@ -145,12 +144,13 @@ struct Ctl {
     int oct_ready;                      // the octagon of the true extremes and the end-point records stand
     int star_ok;                        // batched: the set is listed for a star polygon
     int star_k;                         // the polygon's vertices, the dropped ones included
+    int star_edges;                     // dense_kernel: the polygon's vertices in use (0: none)
     int star_final;                     // a polygon was built and accepted
     int star_cx, star_cy;               // its centre (vertices are stored relative to it)
     Octagon oct;                        // octagon of the true extremes
     Octagon oct_s;                      // octagon of a sample's extremes
 #if defined(CH_TRACE) || defined(CH_TIMELINE)
-    unsigned long long tl[14][2];       // debug builds: first start / last end per phase (%globaltimer)
+    unsigned long long tl[24][2];       // debug builds: first start / last end per phase (%globaltimer)
 #endif
 };
 

@@ -74,7 +74,7 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
     unsigned* h = &ctl->digit_hist[0][0];
     for (int i = t; i < kSortPasses * kDigits; i += blockDim.x) h[i] = 0u;
 #if defined(CH_TRACE) || defined(CH_TIMELINE)
-    if (t < 14) { ctl->tl[t][0] = ~0ull; ctl->tl[t][1] = 0ull; }
+    if (t < 24) { ctl->tl[t][0] = ~0ull; ctl->tl[t][1] = 0ull; }
 #endif
 }
 
@@ -621,14 +621,16 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
 // ---------------------------------------------------------------------------
 // The main pass on dense data (points near a circle, Table V), one cooperative
 // launch of one block per SM:
-//   1. the angular bins of the star polygon (star.cuh): the sample pass's
-//      tiles (still in L2) and kStarExtraTiles more, spread over the input.
-//      Every point outside oct_s goes to its angular bin around that octagon's
-//      centre c, where a 64-bit atomicMax keeps the point farthest from c (its
-//      squared distance, truncated, above its index); a point first reads its
-//      bin and issues the atomic only if it beats it;
-//   2. one block makes the polygon of the bins' points (star_finish) and clears
-//      the bins;
+//   1. the angular bins of the star polygon (star.cuh), per block in shared
+//      memory: a warp tile per warp, spread over the input.  Every point
+//      outside oct_s goes to its angular bin around that octagon's centre c,
+//      where an atomicMax keeps the point farthest from c (its squared
+//      distance, truncated, above its index), unless its key is no larger than
+//      the bin's already.  (Bins shared by all blocks in L2 took 37 us: most of
+//      the first points of every block met there as atomics.)
+//   2. every block merges its share of the bins and re-reads their points, one
+//      block makes the polygon of them (star_polygon), every block finds its
+//      share of the bins' radius bounds;
 //   3. one streaming read of all points.  A point closer to c than its bin's
 //      radius bound is strictly inside the polygon; the others wait in a
 //      per-warp queue and go 32 at a time through the exact wedge test; what
@@ -640,15 +642,7 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
 // all points.  Before, the main pass's full tracking (143 us on 1e8 points)
 // ran beside 1, every block of the post pass did 2 (90 us) and the post pass 3
 // with integer distances (400 us).
-// Warp tile of the star pass's k-th read: the sample pass's tiles first, then
-// the extra tiles, half a stride away from an even spread.
-__device__ __forceinline__ long long star_tile(long long k, long long nsamp, long long nextra, long long ntiles) {
-    if (k < nsamp) return k * ntiles / nsamp;
-    const long long e = k - nsamp;
-    return ((2 * e + 1) * ntiles) / (2 * nextra);
-}
-
-// One warp tile: bins the points outside the sample octagon.
+// One warp tile: bins (in shared memory) the points outside the octagon.
 __device__ __forceinline__ void star_tile_pass(const float4* __restrict__ p4, long long t, int head, const int* s_in,
                                                const float* s_edge, int cx, int cy, unsigned long long* bins,
                                                unsigned long long pol) {
@@ -660,49 +654,77 @@ __device__ __forceinline__ void star_tile_pass(const float4* __restrict__ p4, lo
         float4 v[kHalf];
 #pragma unroll
         for (int j = 0; j < kHalf; ++j) v[j] = ld_stream_f4(base + (j0 + j) * 32, pol);
-        // the keys of the points outside the sample octagon, then one load of
-        // each point's bin: only a point that beats the bin's current value
-        // issues the atomicMax (after a bin's first few points that is rare,
-        // so far fewer atomics meet at each bin)
-        unsigned long long key[2 * kHalf];
-        int bin[2 * kHalf];
 #pragma unroll
         for (int j = 0; j < kHalf; ++j) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const float x = h ? v[j].z : v[j].x, y = h ? v[j].w : v[j].y;
                 const int X = __float2int_rn(x), Y = __float2int_rn(y);
-                const bool out = !pt_in_inner(X, Y, s_in) && !pt_in_sample(x, y, s_edge);
+                if (pt_in_inner(X, Y, s_in) || pt_in_sample(x, y, s_edge)) continue;
                 const int dx = X - cx, dy = Y - cy;
                 const unsigned long long d2 = (unsigned long long)((long long)dx * dx + (long long)dy * dy);
                 const unsigned idx = (unsigned)(head + t * kWarpTilePts + 2 * ((j0 + j) * 32 + lane) + h);
-                key[2 * j + h] = out ? ((d2 >> 17) << 32) | idx : 0ull;
-                bin[2 * j + h] = star_bin(dx, dy);
+                const unsigned long long key = ((d2 >> 17) << 32) | idx;
+                unsigned long long* bin = bins + star_bin(dx, dy);
+                if (key > *(volatile unsigned long long*)bin) atomicMax(bin, key);
             }
         }
-        unsigned long long cur[2 * kHalf];
-#pragma unroll
-        for (int i = 0; i < 2 * kHalf; ++i) cur[i] = key[i] ? __ldcg(bins + bin[i]) : ~0ull;
-#pragma unroll
-        for (int i = 0; i < 2 * kHalf; ++i)
-            if (key[i] > cur[i]) atomicMax(&bins[bin[i]], key[i]);
     }
 }
 
-constexpr int kDenseThreads = 512;
-constexpr int kDenseQueue = 96;   // < 32 waiting + 64 added per step
+constexpr int kDenseThreads = 1024;
+constexpr int kDenseF4 = kWarpTileF4 / 2;   // float4 of a warp's ring tile: 32 warps' rings fit
+constexpr int kDenseQueue = 64;   // < 32 waiting + 32 added per step
+constexpr int kDenseBuf = 64;     // raw survivors staged per warp
 struct DenseWarp {
-    RawBuf raw;
-    float x[kDenseQueue], y[kDenseQueue];
+    unsigned long long xy[kDenseBuf];
+    unsigned raw_idx[kDenseBuf];
+    float2 p[kDenseQueue];
     unsigned idx[kDenseQueue];
     unsigned cnt;                 // raw survivors staged
     int best[8];                  // the warp's extreme keys so far and the
     unsigned code[8];             // first tile where each occurred
 };
-constexpr size_t kDenseWarpOff = (sizeof(StarPoly) + 15) / 16 * 16;
-constexpr size_t kDenseSmemBytes = kDenseWarpOff + (kDenseThreads / 32) * sizeof(DenseWarp);
-static_assert((kDenseThreads / 32) * sizeof(DenseWarp) >= sizeof(unsigned long long) * kStarBins, "star_finish's work area");
-static_assert(sizeof(StarPoly) % 16 == 0, "the polygon is copied in 16-byte words");
+// Shared memory: the radius bounds, the warps' buffers, their rings of tiles;
+// first of all, in the block that makes it, the polygon and star_polygon's work
+// area.  The exact tests read the polygon from L2: few points take them.
+constexpr size_t kDenseWarpOff = sizeof(float) * kStarBins;
+constexpr size_t kDenseRingOff = (kDenseWarpOff + (kDenseThreads / 32) * sizeof(DenseWarp) + 127) / 128 * 128;
+constexpr size_t kDenseWorkOff = (sizeof(StarPoly) + 15) / 16 * 16;
+constexpr size_t kDenseStream = kDenseRingOff + (size_t)(kDenseThreads / 32) * kStages * kDenseF4 * sizeof(float4);
+constexpr size_t kDenseBuild = kDenseWorkOff + sizeof(unsigned long long) * kStarBins;
+constexpr size_t kDenseSmemBytes = kDenseStream > kDenseBuild ? kDenseStream : kDenseBuild;
+static_assert(kDenseSmemBytes <= 224 * 1024 && sizeof(StarPoly) % 16 == 0, "one block's shared memory");
+
+__device__ __forceinline__ void dense_flush(DenseWarp& w, unsigned cnt, Ctl* ctl, uint64_t* raw_xy, uint32_t* raw_idx) {
+    const int lane = threadIdx.x & 31;
+    if (cnt == 0u) return;
+    unsigned base = 0u;
+    if (lane == 0) base = atomicAdd(&ctl->count_raw, cnt);
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    for (unsigned i = lane; i < cnt; i += 32) {
+        raw_xy[base + i] = w.xy[i];
+        raw_idx[base + i] = w.raw_idx[i];
+    }
+    __syncwarp();
+}
+
+// Packed pairs of floats (x, y).
+__device__ __forceinline__ unsigned long long f2_pack(float x, float y) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 
 // Warp-collective, out of line: the queued points [first, first + count),
 // count <= 32.
@@ -710,10 +732,10 @@ __device__ __noinline__ void dense_drain(const StarPoly& P, int cx, int cy, Dens
                                          unsigned count, int head, Ctl* ctl, uint64_t* raw_xy, uint32_t* raw_idx) {
     const int lane = threadIdx.x & 31;
     const bool valid = (unsigned)lane < count;
-    const float x = valid ? w.x[first + lane] : 0.0f, y = valid ? w.y[first + lane] : 0.0f;
+    const float2 p = valid ? w.p[first + lane] : make_float2(0.0f, 0.0f);
     const unsigned idx = valid ? w.idx[first + lane] : 0u;
-    const int X = __float2int_rn(x), Y = __float2int_rn(y);
-    const bool keep = valid && !star_inside_exact(X - cx, Y - cy, star_bin(x - (float)cx, y - (float)cy), P);
+    const int X = __float2int_rn(p.x), Y = __float2int_rn(p.y);
+    const bool keep = valid && !star_inside_exact(X - cx, Y - cy, star_bin(p.x - (float)cx, p.y - (float)cy), P);
     const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
     if (!bal) return;
     // tile code as in extremes.cuh: 0 = head, t + 1 = body tile t or the tail
@@ -744,11 +766,14 @@ __device__ __noinline__ void dense_drain(const StarPoly& P, int cx, int cy, Dens
         }
     }
     unsigned cnt = w.cnt;
-    if (cnt + (unsigned)__popc(bal) > (unsigned)kWarpBuf) flush_raw(w.raw, cnt, ctl, raw_xy, raw_idx);
+    if (cnt + (unsigned)__popc(bal) > (unsigned)kDenseBuf) {
+        dense_flush(w, cnt, ctl, raw_xy, raw_idx);
+        cnt = 0u;
+    }
     if (keep) {
         const unsigned pos = cnt + __popc(bal & lanemask_lt());
-        w.raw.xy[pos] = ((unsigned long long)(unsigned)X << 32) | (unsigned)Y;
-        w.raw.idx[pos] = idx;
+        w.xy[pos] = ((unsigned long long)(unsigned)X << 32) | (unsigned)Y;
+        w.raw_idx[pos] = idx;
     }
     __syncwarp();
     if (lane == 0) w.cnt = cnt + (unsigned)__popc(bal);
@@ -761,7 +786,9 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
                                                                  uint32_t* keys, uint64_t* vals) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ unsigned long long s_red[kDenseThreads / 32][8];
-    __shared__ int s_flag, s_in[8];
+    __shared__ unsigned long long s_bar[kDenseThreads / 32][kStages];
+    __shared__ int s_flag, s_in[8], s_K0;
+    __shared__ unsigned s_scan[kDenseThreads / 32];
     __shared__ float s_edge[24];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kWarps = kDenseThreads / 32;
@@ -771,7 +798,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
     const Octagon& os = ctl->oct_s;
     const int cx = (os.vx[W] + os.vx[E]) / 2, cy = (os.vy[S] + os.vy[N]) / 2;
     const float4* p4 = reinterpret_cast<const float4*>(pts + 2 * head);
-    const unsigned long long pol = l2_evict_first();
+    unsigned long long* merged = bins + (size_t)gridDim.x * kStarBins;
     {   // 1. bins
         if (tid < 4) {
             s_in[tid] = os.in_lo[tid];
@@ -783,41 +810,100 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
             s_edge[3 * tid + 2] = os.oct[tid].C;
         }
         __syncthreads();
-        const long long nsamp = sample_tiles(ntiles);
-        const long long nextra = ntiles < kStarExtraTiles ? ntiles : kStarExtraTiles;
-        // tile k belongs to block k % grid, warp (k / grid) % kWarps
-        for (long long k = blockIdx.x + (long long)gridDim.x * warp; k < nsamp + nextra;
-             k += (long long)gridDim.x * kWarps)
-            star_tile_pass(p4, star_tile(k, nsamp, nextra, ntiles), head, s_in, s_edge, cx, cy, bins, pol);
+        unsigned long long* mine = reinterpret_cast<unsigned long long*>(dsm);
+        for (int b = tid; b < kStarBins; b += kDenseThreads) mine[b] = 0ull;
+        __syncthreads();
+        const long long nt = min(ntiles, (long long)gridDim.x * kWarps), k = blockIdx.x + (long long)gridDim.x * warp;
+        if (k < nt)
+            star_tile_pass(p4, ((2 * k + 1) * ntiles) / (2 * nt), head, s_in, s_edge, cx, cy, mine, l2_evict_first());
+        __syncthreads();
+        for (int b = tid; b < kStarBins; b += kDenseThreads) bins[(size_t)blockIdx.x * kStarBins + b] = mine[b];
         CH_TL(ctl, 7, 1);
         if (!grid_barrier(&ctl->barrier[0], 1u, ctl)) return;
     }
-    const StarPoly& P = *reinterpret_cast<const StarPoly*>(dsm);
-    if (blockIdx.x == 0) {   // 2. polygon
+    // 2. polygon: every block merges some bins and re-reads their points, one block makes the polygon of them, every block finds
+    // some bins' radius bounds
+    {
+        // 64 consecutive bins at a time, 16 threads each over the blocks' bins
+        constexpr int kSlots = 64, kGroups = kDenseThreads / kSlots;
+        unsigned long long* part = reinterpret_cast<unsigned long long*>(dsm);
+        const int slot = tid % kSlots, grp = tid / kSlots;
+        for (int b0 = (int)blockIdx.x * kSlots; b0 < kStarBins; b0 += (int)gridDim.x * kSlots) {
+            unsigned long long key = 0ull;
+            for (int g = grp; g < (int)gridDim.x; g += kGroups) {
+                const unsigned long long x = __ldcg(bins + (size_t)g * kStarBins + b0 + slot);
+                key = x > key ? x : key;
+            }
+            part[tid] = key;
+            __syncthreads();
+            if (tid < kSlots) {
+#pragma unroll
+                for (int g = 1; g < kGroups; ++g) key = part[g * kSlots + tid] > key ? part[g * kSlots + tid] : key;
+                merged[b0 + tid] = star_vertex(key, star_point(key, pts, n), b0 + tid, cx, cy);
+            }
+            __syncthreads();
+        }
+    }
+    CH_TL(ctl, 14, 1);
+    if (!grid_barrier(&ctl->barrier[0], 2u, ctl)) return;
+    if (blockIdx.x == 0) {
         StarPoly& M = *reinterpret_cast<StarPoly*>(dsm);
-        const int K = star_finish<kDenseThreads>(bins, pts, n, cx, cy,
-                                                 reinterpret_cast<unsigned long long*>(dsm + kDenseWarpOff), M, ctl);
+        unsigned long long* work = reinterpret_cast<unsigned long long*>(dsm + kDenseWorkOff);
+        constexpr int kPer = kStarBins / kDenseThreads;
+        unsigned long long v[kPer];
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            v[i] = __ldcg(merged + tid * kPer + i);
+            c += v[i] != 0ull;
+        }
+        int o = star_scan<kDenseThreads>(c, s_scan, &s_K0);
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+            if (v[i]) work[o++] = v[i];
         __syncthreads();
-        if (K)
-            for (int j = tid; j < (int)(sizeof(StarPoly) / 16); j += kDenseThreads)
-                reinterpret_cast<int4*>(poly)[j] = reinterpret_cast<const int4*>(dsm)[j];
-        for (int b = tid; b < kStarBins; b += kDenseThreads) bins[b] = 0ull;   // at rest again
+        CH_TL(ctl, 9, 1);
+        const int K0 = s_K0;
+        const int K = star_polygon<kDenseThreads>(work, K0, M, ctl);
+        __syncthreads();
+        for (int j = tid; K && j < K + 2; j += kDenseThreads) poly->v[j] = M.v[j];
+        for (int j = tid; K && j < kStarBins; j += kDenseThreads) poly->tbl[j] = M.tbl[j];
         if (tid == 0) {
-            ctl->star_k = K;
+            ctl->star_k = K ? K0 : 0;
+            ctl->star_edges = K;
             ctl->star_cx = cx;
             ctl->star_cy = cy;
             ctl->star_final = K ? 1 : 0;
         }
         CH_TL(ctl, 8, 1);
     }
-    if (!grid_barrier(&ctl->barrier[0], 2u, ctl)) return;
-    if (!*(volatile int*)&ctl->star_final) return;
-    // 3. the filter
-    if (blockIdx.x != 0) {
-        const int4* src = reinterpret_cast<const int4*>(poly);
-        int4* dst = reinterpret_cast<int4*>(dsm);
-        for (int j = tid; j < (int)(sizeof(StarPoly) / 16); j += kDenseThreads) dst[j] = __ldcg(src + j);
+    if (!grid_barrier(&ctl->barrier[0], 3u, ctl)) return;
+    const int K = *(volatile int*)&ctl->star_edges;
+    if (!K) return;
+    {   // kStarWindow threads per bin, an edge of its window each
+        constexpr int kSlots = kDenseThreads / kStarWindow;
+        const int k = tid % kStarWindow;
+        for (int b0 = (int)blockIdx.x; b0 < kStarBins; b0 += (int)gridDim.x * kSlots) {
+            const int b = b0 + tid / kStarWindow * (int)gridDim.x;
+            const bool some = b < kStarBins;
+            int first, count;
+            star_window(poly->tbl, K, some ? b : 0, first, count);
+            unsigned r = 0xFFFFFFFFu;
+            if (k < count && count <= kStarWindow) {
+                const int e = first + k < K ? first + k : first + k - K;
+                r = star_edge_radius(poly->v[e], poly->v[e + 1]);
+            }
+#pragma unroll
+            for (int d = kStarWindow / 2; d; d >>= 1) r = min(r, __shfl_xor_sync(0xFFFFFFFFu, r, d));
+            if (some && k == 0) poly->thr[b] = star_threshold(count <= kStarWindow ? r : 0u);
+        }
     }
+    if (!grid_barrier(&ctl->barrier[0], 4u, ctl)) return;
+    CH_TL(ctl, 12, 1);
+    // 3. the filter
+    float* thr = reinterpret_cast<float*>(dsm);
+    for (int j = tid; j < kStarBins / 4; j += kDenseThreads)
+        reinterpret_cast<float4*>(thr)[j] = __ldcg(reinterpret_cast<const float4*>(poly->thr) + j);
     DenseWarp& w = reinterpret_cast<DenseWarp*>(dsm + kDenseWarpOff)[warp];
     if (lane == 0) w.cnt = 0u;
     if (lane < 8) {
@@ -825,60 +911,67 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
         w.code[lane] = 0u;
     }
     __syncthreads();
-    const float fcx = (float)cx, fcy = (float)cy;
+    CH_TL(ctl, 3, 0);
     const long long first = ((long long)blockIdx.x * kDenseThreads + tid) >> 5;
     const long long stride = ((long long)gridDim.x * kDenseThreads) >> 5;
-    const unsigned lt = lanemask_lt();
     unsigned qn = 0u;   // points queued (warp-uniform)
-    bool bad = false;
+    unsigned bad = 0u;  // bits of the differences that a valid coordinate leaves at zero
     float lowest = 0.0f, highest = 0.0f;
-    // x is an integer or at least 2^23 in magnitude when adding and taking
-    // away 2^24 leaves it alone (NaN does not); with the range check this is
-    // convert_pt's validity without integer conversions
-    auto check = [&](float x, float y) {
-        bad |= __fadd_rn(__fadd_rn(x, -16777216.0f), 16777216.0f) != x;
-        bad |= __fadd_rn(__fadd_rn(y, -16777216.0f), 16777216.0f) != y;
+    const unsigned long long away = f2_pack(-16777216.0f, -16777216.0f), back = f2_pack(16777216.0f, 16777216.0f);
+    const unsigned long long minus_c = f2_pack(-(float)cx, -(float)cy);
+    // Checks a point and tells whether the radius bound settles it.  A
+    // coordinate is an integer, or at least 2^23 in magnitude, when adding and
+    // taking away 2^24 leaves it alone (an infinity or NaN does not); with the
+    // range check this is convert_pt's validity without integer conversions.
+    auto undecided = [&](float x, float y) __attribute__((always_inline)) {
+        const unsigned long long p = f2_pack(x, y);
+        const float2 r = f2_unpack(f2_add(f2_add(p, away), back));
+        bad |= __float_as_uint(__fsub_rn(r.x, x)) | __float_as_uint(__fsub_rn(r.y, y));
         asm("min.f32 %0, %0, %1, %2;" : "+f"(lowest) : "f"(x), "f"(y));
         asm("max.f32 %0, %0, %1, %2;" : "+f"(highest) : "f"(x), "f"(y));
+        const float2 d = f2_unpack(f2_add(p, minus_c));   // exact
+        return !(star_d2(d.x, d.y) < thr[star_bin(d.x, d.y)]);
     };
-    float4 v[kLoadsPerLane];
+    const long long nt = ntiles * (kWarpTileF4 / kDenseF4);
+    WarpStreamT<kDenseF4> ws{reinterpret_cast<float4*>(dsm + kDenseRingOff) + warp * kStages * kDenseF4, s_bar[warp], p4,
+                             first, stride, nt, lane};
+    ws.start();
+    for (long long k = 0;; ++k) {
+        const long long t = first + k * stride;
+        if (t >= nt) break;
+        const float4* cur = ws.acquire(k, ctl);
+        if (!cur) {   // a copy never completed: status is CH_ETIMEOUT
+            ws.drain(k);
+            break;
+        }
+        unsigned mask = 0u;   // the lane's undecided points: bit 2 j + half
 #pragma unroll
-    for (int j = 0; j < kLoadsPerLane; ++j)
-        if (first < ntiles) v[j] = ld_stream_f4(p4 + first * kWarpTileF4 + j * 32 + lane, pol);
-#pragma unroll 1
-    for (long long t = first; t < ntiles; t += stride) {
-        const bool more = t + stride < ntiles;
-        const float4* next = p4 + (t + stride) * kWarpTileF4 + lane;
-        const unsigned i0 = (unsigned)head + (unsigned)t * kWarpTilePts + 2u * lane;   // n < 2^31
-#pragma unroll
-        for (int j = 0; j < kLoadsPerLane; ++j) {
-            const float4 p = v[j];
-            if (more) v[j] = ld_stream_f4(next + j * 32, pol);
-            check(p.x, p.y);
-            check(p.z, p.w);
-            const float dx0 = p.x - fcx, dy0 = p.y - fcy, dx1 = p.z - fcx, dy1 = p.w - fcy;   // exact
-            const bool q0 = !star_inside_fast(dx0, dy0, star_bin(dx0, dy0), P);
-            const bool q1 = !star_inside_fast(dx1, dy1, star_bin(dx1, dy1), P);
-            const unsigned m0 = __ballot_sync(0xFFFFFFFFu, q0), m1 = __ballot_sync(0xFFFFFFFFu, q1);
-            if (m0 | m1) {
-                if (q0) {
-                    const unsigned pos = qn + __popc(m0 & lt);
-                    w.x[pos] = p.x; w.y[pos] = p.y; w.idx[pos] = i0 + 64u * j;
-                }
-                if (q1) {
-                    const unsigned pos = qn + __popc(m0) + __popc(m1 & lt);
-                    w.x[pos] = p.z; w.y[pos] = p.w; w.idx[pos] = i0 + 64u * j + 1u;
-                }
-                qn += __popc(m0) + __popc(m1);
-                __syncwarp();
-                while (qn >= 32u) {
-                    qn -= 32u;
-                    dense_drain(P, cx, cy, w, qn, 32u, head, ctl, raw_xy, raw_idx);
-                }
+        for (int j = 0; j < kDenseF4 / 32; ++j) {
+            const float4 p = cur[j * 32 + lane];
+            if (undecided(p.x, p.y)) mask |= 1u << (2 * j);
+            if (undecided(p.z, p.w)) mask |= 2u << (2 * j);
+        }
+        // queued, a point per lane and step (few lanes have more than one or
+        // two of 8); full rounds of 32 go through the exact test
+        const float2* cur2 = reinterpret_cast<const float2*>(cur);
+        for (unsigned bal; (bal = __ballot_sync(0xFFFFFFFFu, mask != 0u)) != 0u;) {
+            if (mask) {
+                const int s = __ffs((int)mask) - 1, f2 = 64 * (s >> 1) + 2 * lane + (s & 1);
+                mask &= mask - 1u;
+                const unsigned pos = qn + __popc(bal & lanemask_lt());
+                w.p[pos] = cur2[f2];
+                w.idx[pos] = (unsigned)(head + t * (2 * kDenseF4)) + (unsigned)f2;
+            }
+            qn += __popc(bal);
+            __syncwarp();
+            if (qn >= 32u) {
+                qn -= 32u;
+                dense_drain(*poly, cx, cy, w, qn, 32u, head, ctl, raw_xy, raw_idx);
             }
         }
+        ws.release(k);
     }
-    if (qn) dense_drain(P, cx, cy, w, 0u, qn, head, ctl, raw_xy, raw_idx);
+    if (qn) dense_drain(*poly, cx, cy, w, 0u, qn, head, ctl, raw_xy, raw_idx);
     // the unaligned head point, and the ragged tail by 32 points per warp
     const long long tail = head + ntiles * kWarpTilePts + 32 * (stride - 1 - first);
     const long long ranges[2][2] = {{0, first == 0 ? head : 0}, {tail, min(n, tail + 32)}};
@@ -887,18 +980,16 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
         if (cnt <= 0) continue;
         __syncwarp();
         if (lane < cnt) {
-            w.x[lane] = pts[2 * i];
-            w.y[lane] = pts[2 * i + 1];
+            w.p[lane] = reinterpret_cast<const float2*>(pts)[i];
             w.idx[lane] = (unsigned)i;
-            check(w.x[lane], w.y[lane]);
+            undecided(w.p[lane].x, w.p[lane].y);   // the checks
         }
         __syncwarp();
-        dense_drain(P, cx, cy, w, 0u, (unsigned)cnt, head, ctl, raw_xy, raw_idx);
+        dense_drain(*poly, cx, cy, w, 0u, (unsigned)cnt, head, ctl, raw_xy, raw_idx);
     }
-    bad |= lowest < 0.0f || highest >= (float)kCoordLimit;
-    if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) set_status(ctl, CH_ERANGE);
-    unsigned cnt = w.cnt;
-    flush_raw(w.raw, cnt, ctl, raw_xy, raw_idx);
+    const bool err = bad != 0u || lowest < 0.0f || highest >= (float)kCoordLimit;
+    if (__any_sync(0xFFFFFFFFu, err) && lane == 0) set_status(ctl, CH_ERANGE);
+    dense_flush(w, w.cnt, ctl, raw_xy, raw_idx);
     if (lane < 8) s_red[warp][lane] = pack_best(lane, w.best[lane], w.code[lane]);
     __syncthreads();
     if (tid < 8) {
@@ -1050,7 +1141,7 @@ void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl
                 (unsigned long long*)bins, (StarPoly*)poly, raw_xy, raw_idx, keys, vals);
 }
 
-size_t star_bins_bytes() { return sizeof(unsigned long long) * kStarBins; }
+size_t star_bins_bytes(int sms) { return sizeof(unsigned long long) * kStarBins * ((size_t)sms + 1); }
 size_t star_poly_bytes() { return sizeof(StarPoly); }
 
 void launch_labels(const float* pts, long long n, Ctl* ctl, uint8_t* labels, int grid, cudaStream_t s) {

@@ -102,6 +102,8 @@ static __device__ int merge_smem_seq(int* su, int* sv, int* si, int sa, int la, 
     return is + 1 + n;
 }
 
+// Every warp reduces (scans) the warps' values itself, by shuffles: at most 32
+// warps, a power of two of them for the reduction.
 template <typename T, typename Op>
 __device__ __forceinline__ T block_reduce(T v, Op op, T* s_tmp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -110,13 +112,13 @@ __device__ __forceinline__ T block_reduce(T v, Op op, T* s_tmp) {
     __syncthreads();
     if (lane == 0) s_tmp[warp] = v;
     __syncthreads();
-    T r = s_tmp[0];
-    for (int w = 1; w < nw; ++w) r = op(r, s_tmp[w]);
-    __syncthreads();
+    T r = s_tmp[lane & (nw - 1)];
+    for (int o = nw >> 1; o; o >>= 1) r = op(r, __shfl_xor_sync(0xFFFFFFFFu, r, o));
     return r;
 }
 
-// Exclusive block scan of one int per thread; *total receives the sum.
+// Exclusive block scan of one int per thread; *total receives the sum.  The
+// next use of s_tmp is behind its own first barrier.
 __device__ __forceinline__ int block_excl_scan(int x, int* s_tmp, int* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
     int incl = x;
@@ -128,14 +130,15 @@ __device__ __forceinline__ int block_excl_scan(int x, int* s_tmp, int* total) {
     __syncthreads();
     if (lane == 31) s_tmp[warp] = incl;
     __syncthreads();
-    int off = 0, tot = 0;
-    for (int w = 0; w < nw; ++w) {
-        if (w < warp) off += s_tmp[w];
-        tot += s_tmp[w];
+    int sums = lane < nw ? s_tmp[lane] : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xFFFFFFFFu, sums, o);
+        if (lane >= o) sums += t;
     }
-    __syncthreads();
-    *total = tot;
-    return off + incl - x;
+    *total = __shfl_sync(0xFFFFFFFFu, sums, 31);
+    const int before = __shfl_sync(0xFFFFFFFFu, sums, (warp + 31) & 31);
+    return (warp ? before : 0) + incl - x;
 }
 
 __device__ __forceinline__ void pt_xy(const float* pts, int i, long long& x, long long& y) {

@@ -40,7 +40,7 @@ void launch_post(const float* pts, long long n, int head, long long ntiles, Ctl*
                  const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n,
                  int grid, cudaStream_t s);
 void launch_labels(const float* pts, long long n, Ctl* ctl, uint8_t* labels, int grid, cudaStream_t s);
-size_t star_bins_bytes();
+size_t star_bins_bytes(int sms);   // a block's bins each, and the merged ones
 size_t star_poly_bytes();
 void launch_filter_output(const Ctl* ctl, long long n, int32_t* out_ext8, int64_t* out_counts4, cudaStream_t s);
 

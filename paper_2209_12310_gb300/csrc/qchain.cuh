@@ -133,13 +133,6 @@ __device__ void qc_sort(Q& q, int n, int lo, int hi) {
     __syncthreads();
 }
 
-__device__ __forceinline__ long long qc_cross(unsigned long long o, unsigned long long a, unsigned long long b) {
-    return cross_uv(qc_u(o), qc_v(o), qc_u(a), qc_v(a), qc_u(b), qc_v(b));
-}
-__device__ __forceinline__ bool qc_same_u(unsigned long long a, unsigned long long b) {
-    return ((a ^ b) >> (kKeyBits + kQcPosBits)) == 0ull;
-}
-
 // The lower chain of the n >= 1 points in src, ordered by (u, v, index):
 // returns its length; src points at it (the two buffers change roles).  Of
 // points of equal u only the first can be a vertex: the others are skipped
@@ -160,36 +153,39 @@ __device__ int qc_eliminate(unsigned long long*& src, unsigned long long*& dst, 
         const long long l0 = (long long)tid * c - shift;
         const int lo = (int)max(0ll, min((long long)n, l0)), hi = (int)max(0ll, min((long long)n, l0 + c));
         const bool some = lo < hi, ctx = some && lo > 0, after = some && hi < n;
-        const unsigned long long left = ctx ? src[lo - 1] : 0ull;
-        unsigned long long top = left, sec = 0ull;
-        const unsigned long long right = after ? src[hi] : 0ull;
+        const unsigned long long left = ctx ? src[lo - 1] : 0ull, right = after ? src[hi] : 0ull;
         __syncthreads();   // every context is read before the runs are rewritten
-        int cnt = 0;                // points kept: src[lo .. lo + cnt)
-        const int below = ctx ? 1 : 0;   // the context is the stack's bottom
-        int depth = below;
-        auto pop_above = [&](unsigned long long w) {
-            while (depth >= 2 && qc_cross(sec, top, w) <= 0) {
-                --depth;
+        // the stack: the context if there is one, then src[lo .. lo + cnt), the
+        // points kept; its top (tu, tv) and the edge that leads there (eu, ev)
+        // stay in registers
+        int cnt = 0;
+        const int below = ctx ? 1 : 0;
+        int tu = ctx ? qc_u(left) : -1, tv = qc_v(left), eu = 0, ev = 0;
+        auto pop_before = [&](int u, int v) {
+            while (cnt + below >= 2 && (long long)eu * (v - tv) <= (long long)ev * (u - tu)) {
                 --cnt;
-                top = sec;
-                // the element below the new top
-                if (depth >= 2) {
-                    const int e = depth - 2 - below;
-                    sec = e >= 0 ? src[lo + e] : left;
+                tu -= eu;
+                tv -= ev;
+                if (cnt + below >= 2) {   // the edge that leads to the new top
+                    const unsigned long long w = cnt >= 2 ? src[lo + cnt - 2] : left;
+                    eu = tu - qc_u(w);
+                    ev = tv - qc_v(w);
                 }
             }
         };
         for (int j = lo; j < hi; ++j) {
             const unsigned long long w = src[j];
-            if (depth > 0 && qc_same_u(top, w)) continue;
-            pop_above(w);
+            const int u = qc_u(w), v = qc_v(w);
+            if (u == tu) continue;
+            pop_before(u, v);
             src[lo + cnt] = w;
             ++cnt;
-            ++depth;
-            sec = top;
-            top = w;
+            eu = u - tu;
+            ev = v - tv;
+            tu = u;
+            tv = v;
         }
-        if (after && !qc_same_u(top, right)) pop_above(right);
+        if (after && qc_u(right) != tu) pop_before(qc_u(right), qc_v(right));
         int tot;
         const int off = block_excl_scan(cnt, s_tmp, &tot);
         if (tot == n) return n;   // nothing removed: convex

@@ -285,16 +285,21 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
     __syncthreads();
     const int path = s_path;
     if (path != kPathTiles && (path != kPathQueues || qq >= 4)) return;
+    CH_TL(ctl, 13, 0);
     q_map(ctl->oct, s_m);
     __syncthreads();
     if (path == kPathTiles) {
         tile_hist(a, *reinterpret_cast<TileHistSmem*>(s_dyn), s_m);
+        CH_TL(ctl, 15, 1);
         bool go = grid_barrier(&ctl->barrier[1], 1u, ctl);
         if (go && qq == 0) tile_cut(a, *reinterpret_cast<TileHistSmem*>(s_dyn));
         go = go && grid_barrier(&ctl->barrier[1], 2u, ctl);
+        CH_TL(ctl, 16, 1);
         if (go) tile_part(a, *reinterpret_cast<TilePartSmem*>(s_dyn), s_m);
+        CH_TL(ctl, 17, 1);
         go = go && grid_barrier(&ctl->barrier[1], 3u, ctl);
         if (go) tile_chains(a, *reinterpret_cast<QcQueue*>(s_dyn));
+        CH_TL(ctl, 18, 1);
         go = go && grid_barrier(&ctl->barrier[1], 4u, ctl);
         if (!go && tid == 0) *a.out_n = CH_ETIMEOUT;
         if (!go || qq >= 4 || *(volatile int*)&ctl->bk_state != 1) return;
@@ -346,8 +351,10 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
             }
         }
         __syncthreads();
+        CH_TL(ctl, 19, 1);
         const int cnt = min(s_n, QcQueue::kCap);   // rec_q[qq], the two end points among them
         qc_sort<T>(q, cnt, s_m.lo[qq], s_m.hi[qq]);
+        CH_TL(ctl, 20, 1);
         src = q.a;
         dst = q.b;
         len = qc_eliminate<T>(src, dst, cnt, q.tmp);
@@ -384,6 +391,7 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
                 }
             }
             __syncthreads();
+            CH_TL(ctl, 19, 1);
             src = q.a;
             dst = q.b;
             len = qc_eliminate<T>(src, dst, tot, q.tmp);
@@ -393,6 +401,7 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
             }
         }
     }
+    CH_TL(ctl, 21, 1);
     if (tid == 0) {
         ctl->reg_end[qq] = ok ? (unsigned)len : 0u;
         if (!ok) ctl->bk_state = 2;   // the sort takes over (its input is untouched)
@@ -407,6 +416,7 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
     }
     __syncthreads();
     if (!s_last) return;
+    CH_TL(ctl, 22, 1);
     int off[5];
     off[0] = 0;
     for (int r = 0; r < 4; ++r) off[r + 1] = off[r] + max((int)__ldcg(&ctl->reg_end[r]) - 1, 0);
@@ -431,6 +441,7 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
         stitch_cycle(X, Y, V, off[4], tmp, ctl, n, out_idx, out_n);
     }
     if (tid == 0) ctl->done = 1;
+    CH_TL(ctl, 13, 1);
 }
 
 // ---------------------------------------------------------------------------

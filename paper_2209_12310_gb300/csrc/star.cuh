@@ -29,8 +29,8 @@ namespace ch {
 //   tbl  per bin, the last vertex whose bin comes before it (K - 1 if none);
 //   thr  per bin, a bound on the squared distance from c as floats compute it:
 //        let r be an integer radius no larger than the distance from c to the
-//        line of any edge whose wedge meets the bin or its two neighbours on
-//        either side; a point of the bin closer to c than r is strictly inside.
+//        line of any edge whose wedge can hold points of the bin (star_window);
+//        a point of the bin closer to c than r is strictly inside.
 //        thr is r^2 less 5 parts in 2^24, rounded down, and star_d2 is at most
 //        2 parts in 2^24 below d^2: star_d2 < thr proves d < r.  (0 when no
 //        bound was found.)
@@ -146,16 +146,16 @@ __device__ __forceinline__ int star_scan(int c, unsigned* s, int* total) {
     }
     if (lane == 31) s[warp] = incl;
     __syncthreads();
-    unsigned before = 0u, all = 0u;
+    unsigned sums = lane < kWarps ? s[lane] : 0u;   // every warp scans the warps' totals
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        const unsigned x = s[w];
-        before += w < warp ? x : 0u;
-        all += x;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned u = __shfl_up_sync(0xFFFFFFFFu, sums, o);
+        if (lane >= o) sums += u;
     }
-    if (threadIdx.x == 0) *total = (int)all;
+    if (threadIdx.x == 31) *total = (int)sums;
+    const unsigned before = __shfl_sync(0xFFFFFFFFu, sums, (warp + 31) & 31);
     __syncthreads();
-    return (int)(before + incl - (unsigned)c);
+    return (int)((warp ? before : 0u) + incl - (unsigned)c);
 }
 
 // A vertex under construction: (dx, dy) relative to c, biased by 2^24 (25 bits
@@ -230,78 +230,45 @@ __device__ int star_eliminate(unsigned long long*& src, unsigned long long*& dst
     return n;
 }
 
-// Builds the polygon in P, all T threads of the block, from the star pass's
-// bins (bins[b]: the packed farthest point of bin b, or 0) around c = (cx, cy);
-// work: kStarBins words of shared memory, P too is in shared memory (its first
-// kStarBins words double as the second work area).  Returns the number of
-// points it was made of (the same in every thread) when it passed its checks
-// and P is ready, else 0; leaves the bins as they are.  With kSharedBins the bins are in
-// this block's shared memory and may share their bytes with work: every bin is
-// read before the first write to it.
-//
-// Gather: each non-empty bin's point is re-read from the input by its index
-// (so every vertex is an input point of this call, whatever the bins held)
-// and kept if it is a valid coordinate and falls in that bin again; the kept
-// points, in bin order, are the vertices.  Then star_eliminate, and the checks.
-template <int T, bool kSharedBins = false>
-__device__ int star_finish(const unsigned long long* bins, const float* __restrict__ pts, long long n, int cx, int cy,
-                           unsigned long long* work, StarPoly& P, Ctl* ctl) {
+// The vertex of bin b: its packed farthest point's index (key, 0 for an empty
+// bin) names a point of the input; that point, if it is a valid coordinate and
+// falls in that bin again (so every vertex is an input point of this call,
+// whatever the bins held), as a word of star_pack, else 0 (no word of a vertex).
+__device__ __forceinline__ unsigned long long star_vertex(unsigned long long key, float2 p, int b, int cx, int cy) {
+    const int X = __float2int_rn(p.x), Y = __float2int_rn(p.y);
+    const bool valid = key != 0ull && __int2float_rn(X) == p.x && __int2float_rn(Y) == p.y &&
+                       ((unsigned)(X | Y) >> kCoordBits) == 0u;
+    return valid && star_bin(X - cx, Y - cy) == b ? star_pack(X - cx, Y - cy, b) : 0ull;
+}
+__device__ __forceinline__ float2 star_point(unsigned long long key, const float* __restrict__ pts, long long n) {
+    const long long idx = (long long)(unsigned)key;
+    return key != 0ull && idx < n ? __ldcg(reinterpret_cast<const float2*>(pts) + idx) : make_float2(-1.0f, -1.0f);
+}
+
+// The polygon of the K0 vertices in work (shared memory, in bin order), all T
+// threads of the block: star_eliminate, the checks, then v and tbl of P (shared
+// memory; its first kStarBins words double as the second work area).  Returns
+// its vertices (the same in every thread), or 0 when the checks fail.
+template <int T>
+__device__ int star_polygon(unsigned long long* work, int K0, StarPoly& P, Ctl* ctl) {
     (void)ctl;   // debug timeline only
-    static_assert(T % 32 == 0 && T >= 256 && T <= 1024, "block size");
-    constexpr int kPer = kStarBins / T;   // bins per thread: at most 32
-    static_assert(kPer <= 16, "gather registers");
+    constexpr int kPer = kStarBins / T;
     static_assert(sizeof(P.v) >= sizeof(unsigned long long) * kStarBins, "the second work area fits in the vertices");
     __shared__ unsigned s_scan[T / 32];
     __shared__ int s_K, s_bad, s_cross, s_last[T / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (t == 0) { s_bad = 0; s_cross = 0; }
-    // 1. gather: bins [t kPer, (t + 1) kPer); all their keys, then all their
-    // points, in flight at once
-    unsigned kept = 0u;
-    int2 d[kPer];
-    {
-        unsigned long long key[kPer];
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) key[i] = kSharedBins ? bins[t * kPer + i] : __ldcg(bins + t * kPer + i);
-        float2 p[kPer];
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const long long idx = (long long)(unsigned)key[i];
-            p[i] = (key[i] != 0ull && idx < n) ? __ldcg(reinterpret_cast<const float2*>(pts) + idx)
-                                               : make_float2(-1.0f, -1.0f);
-        }
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const int b = t * kPer + i;
-            const int X = __float2int_rn(p[i].x), Y = __float2int_rn(p[i].y);
-            const bool valid = key[i] != 0ull && __int2float_rn(X) == p[i].x && __int2float_rn(Y) == p[i].y &&
-                               ((unsigned)(X | Y) >> kCoordBits) == 0u;
-            d[i] = make_int2(X - cx, Y - cy);
-            if (valid && star_bin(X - cx, Y - cy) == b) kept |= 1u << i;
-        }
-    }
-    unsigned long long *src = work, *dst = reinterpret_cast<unsigned long long*>(P.v);
-    {
-        const int off = star_scan<T>(__popc(kept), s_scan, &s_K);
-#pragma unroll
-        for (int i = 0; i < kPer; ++i)
-            if ((kept >> i) & 1u)
-                src[off + __popc(kept & ((1u << i) - 1u))] = star_pack(d[i].x, d[i].y, t * kPer + i);
-    }
-    __syncthreads();
-    CH_TL(ctl, 9, 1);
-    const int K0 = s_K;
     __syncthreads();
     if (K0 < 3) return 0;
-    // 2. reflex vertices
+    unsigned long long *src = work, *dst = reinterpret_cast<unsigned long long*>(P.v);
     const int K = star_eliminate<T>(src, dst, K0, s_scan, &s_K);
     CH_TL(ctl, 10, 1);
     if (src != work) {   // the list must sit in work before P is written over it
         for (int i = t; i < K; i += T) work[i] = src[i];
         __syncthreads();
     }
-    // 3. checks: every wedge turns counter-clockwise by less than pi, and
-    // exactly one edge crosses the ray from c along +x (the wedges wind once)
+    // every wedge turns counter-clockwise by less than pi, and exactly one edge
+    // crosses the ray from c along +x (the wedges wind once)
     int bad = 0, cross = 0;
     for (int j = t; j < K; j += T) {
         const int2 a = star_xy(work[j]), b = star_xy(work[j + 1 == K ? 0 : j + 1]);
@@ -313,8 +280,8 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
     __syncthreads();
     const bool ok = K >= 3 && !s_bad && s_cross == 1;
     if (!ok) return 0;
-    // 4. the polygon: vertices; the bin table by a running maximum over the
-    // bins' vertices (thr holds them meanwhile, no vertex as -1)
+    // the vertices; the bin table by a running maximum over the bins' vertices
+    // (thr holds them meanwhile, no vertex as -1)
     int* mark = reinterpret_cast<int*>(P.thr);
     for (int j = t; j < K + 2; j += T) P.v[j] = star_xy(work[j < K ? j : j - K]);
     for (int b = t; b < kStarBins; b += T) mark[b] = -1;
@@ -347,38 +314,93 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
     }
     __syncthreads();
     CH_TL(ctl, 11, 1);
-    // each edge's line radius (work is free again), then per bin the smallest
-    // over the edges whose wedges can hold its points: from the last vertex
-    // before bin b - 2 to the first vertex from bin b + 2 on
-    unsigned* er = reinterpret_cast<unsigned*>(work);
-    if (t == 0) s_K = 0x7FFFFFFF;
+    return K;
+}
+
+// The line radius of edge (a, c2), vertices relative to c turning counter-clockwise.
+__device__ __forceinline__ unsigned star_edge_radius(int2 a, int2 c2) {
+    const long long o = (long long)a.x * c2.y - (long long)a.y * c2.x;   // > 0 (checked)
+    const long long dx = (long long)c2.x - a.x, dy = (long long)c2.y - a.y;
+    return star_line_radius(o, dx * dx + dy * dy);
+}
+
+// The edges whose wedges can hold points of bin b of a polygon of K vertices:
+// [first, first + count), cyclic.  A point's or a vertex's computed bin is off
+// by far less than a bin at its boundaries, so the last vertex before bin b - 1
+// and the first one from bin b + 2 on enclose the bin.
+constexpr int kStarWindow = 8;   // edges of a bin's window at most; a longer one gets no bound
+template <class Tbl>
+__device__ __forceinline__ void star_window(Tbl tbl, int K, int b, int& first, int& count) {
+    first = (int)tbl[(b - 1) & (kStarBins - 1)];
+    int last = (int)tbl[(b + 2) & (kStarBins - 1)];   // the edge from the last vertex before bin b + 2
+    count = (last >= first ? last - first : last - first + K) + 1;
+}
+
+// Builds the whole polygon in P (shared memory), all T threads of one block,
+// from bins (bins[b]: the packed farthest point of bin b, or 0) around c = (cx,
+// cy); work: kStarBins words of shared memory.  Returns the number of points it
+// was made of (the same in every thread) when it passed its checks and P is
+// ready, else 0; leaves the bins as they are.  With kSharedBins the bins are in
+// this block's shared memory and may share their bytes with work: every bin is
+// read before the first write to it.
+template <int T, bool kSharedBins = false>
+__device__ int star_finish(const unsigned long long* bins, const float* __restrict__ pts, long long n, int cx, int cy,
+                           unsigned long long* work, StarPoly& P, Ctl* ctl) {
+    static_assert(T % 32 == 0 && T >= 256 && T <= 1024, "block size");
+    constexpr int kPer = kStarBins / T;   // bins per thread: at most 32
+    static_assert(kPer <= 16, "gather registers");
+    __shared__ unsigned s_scan2[T / 32];
+    __shared__ int s_K0, s_min;
+    const int t = threadIdx.x, lane = t & 31;
+    // bins [t kPer, (t + 1) kPer): all their keys, then all their points, in
+    // flight at once
+    unsigned kept = 0u;
+    unsigned long long w[kPer];
+    {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) w[i] = kSharedBins ? bins[t * kPer + i] : __ldcg(bins + t * kPer + i);
+        float2 p[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) p[i] = star_point(w[i], pts, n);
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            w[i] = star_vertex(w[i], p[i], t * kPer + i, cx, cy);
+            if (w[i]) kept |= 1u << i;
+        }
+    }
+    const int off = star_scan<T>(__popc(kept), s_scan2, &s_K0);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+        if ((kept >> i) & 1u) work[off + __popc(kept & ((1u << i) - 1u))] = w[i];
     __syncthreads();
+    CH_TL(ctl, 9, 1);
+    const int K0 = s_K0;
+    if (t == 0) s_min = 0x7FFFFFFF;
+    const int K = star_polygon<T>(work, K0, P, ctl);
+    if (!K) return 0;
+    // each edge's line radius (work is free again), then per bin the smallest
+    // of its window
+    unsigned* er = reinterpret_cast<unsigned*>(work);
     unsigned emin = 0x7FFFFFFFu;
     for (int e = t; e < K; e += T) {
-        const int2 a = P.v[e], c2 = P.v[e + 1];
-        const long long o = (long long)a.x * c2.y - (long long)a.y * c2.x;   // > 0 (checked above)
-        const long long dx = (long long)c2.x - a.x, dy = (long long)c2.y - a.y;
-        er[e] = star_line_radius(o, dx * dx + dy * dy);
+        er[e] = star_edge_radius(P.v[e], P.v[e + 1]);
         emin = min(emin, er[e]);
     }
     emin = __reduce_min_sync(0xFFFFFFFFu, emin);
-    if (lane == 0) atomicMin(&s_K, (int)emin);
+    if (lane == 0) atomicMin(&s_min, (int)emin);
     __syncthreads();
     CH_TL(ctl, 12, 1);
     for (int b = t; b < kStarBins; b += T) {
-        int e = P.tbl[(b - 2) & (kStarBins - 1)];
-        int last = P.tbl[(b + 2) & (kStarBins - 1)] + 1;
-        if (last == K) last = 0;
-        unsigned m = er[e];
-        int steps = 0;
-        while (e != last && steps < 8) {
-            e = e + 1 == K ? 0 : e + 1;
-            m = min(m, er[e]);
-            ++steps;
+        int first, count;
+        star_window(P.tbl, K, b, first, count);
+        unsigned m = 0u;
+        if (count <= kStarWindow) {
+            m = er[first];
+            for (int k = 1; k < count; ++k) m = min(m, er[first + k < K ? first + k : first + k - K]);
         }
-        P.thr[b] = star_threshold(e == last ? m : 0u);   // a window longer than 8 edges gets no bound
+        P.thr[b] = star_threshold(m);
     }
-    if (t == 0) P.tmin = star_threshold((unsigned)s_K);
+    if (t == 0) P.tmin = star_threshold((unsigned)s_min);
     __syncthreads();
     return K0;
 }
