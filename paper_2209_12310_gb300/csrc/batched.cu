@@ -89,13 +89,15 @@ struct BArgs {
     long long nwt;            // warp tiles of the streamed body
     int head;                 // points before the body's first 16-byte boundary (0 or 1)
     int wtile;                // points per warp tile (32 x points per lane)
+    int fchunk;               // warp tiles that a warp of bt_filter takes at a time
     int* star_slot;           // k: the set's star slot, or -1
     unsigned long long* star_bins;   // kStarBins per slot (zeroed before every batch)
     StarPoly* star_polys;     // one per slot
     unsigned* star_ctr;       // work lists: [0] dense sets listed, [1] taken by bt_star_build;
                               // [2] / [3] sets for bt_star_refine from the front / back, [4] taken;
                               // [5] sets for bt_hull, [6] taken; [7] bt_dense's units, [8] taken;
-                              // [9] / [10] sets for bt_queue_chain from the front / back, [11] / [12] queues taken
+                              // [9] / [10] sets for bt_queue_chain from the front / back, [11] / [12] queues taken;
+                              // [13] bt_filter's chunks taken; [14] sets for the bucketed path
     int* star_list;           // k entries
     unsigned* unit_base;      // k entries: first bt_dense unit of each listed set
     int* refine_list;         // k entries
@@ -128,6 +130,7 @@ __global__ void __launch_bounds__(256) bt_init(BArgs a) {
         c->done = 0;
         c->bk_state = 0;
         c->star_ok = 0;
+        c->skip = 0;
         c->star_k = 0;
         c->star_cx = 0;
         c->star_cy = 0;
@@ -350,6 +353,7 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
         if (tid == 0) {
             a.out_n[i] = ni == 0 ? 0 : s_st;
             c->done = 1;
+            c->skip = 1;
         }
         return;
     }
@@ -366,10 +370,16 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
         lo = max(lo, base);
         hi = min(hi, base + ni);
         long long first = LLONG_MAX;
-#pragma unroll 4
-        for (long long j = lo + lane; j < hi; j += 32) {
-            const float2 p = __ldg(reinterpret_cast<const float2*>(a.pts) + j);
-            if (j < first && dir_key(d, __float2int_rn(p.x), __float2int_rn(p.y)) == best) first = j;
+        for (long long j0 = lo + lane; j0 < hi; j0 += 32 * 16) {   // 16 points of the lane in flight
+            float2 p[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u)
+                if (j0 + 32 * u < hi) p[u] = __ldg(reinterpret_cast<const float2*>(a.pts) + j0 + 32 * u);
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+                const long long j = j0 + 32 * u;
+                if (j < hi && j < first && dir_key(d, __float2int_rn(p[u].x), __float2int_rn(p[u].y)) == best) first = j;
+            }
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
@@ -393,6 +403,7 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
             set_status(c, CH_ECUDA);
             a.out_n[i] = CH_ECUDA;
             c->done = 1;
+            c->skip = 1;
         }
         return;
     }
@@ -429,10 +440,13 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
         __syncthreads();
         const long long step = ni / kBDenseSample;   // >= 1: ni >= kBStarMinPts
         unsigned out = 0u;
-        for (int j = tid; j < kBDenseSample; j += kBOctThreads) {
-            const float2 p = __ldg(reinterpret_cast<const float2*>(a.pts) + base + j * step);
-            out += in_inner(s_o, __float2int_rn(p.x), __float2int_rn(p.y)) ? 0u : 1u;
-        }
+        float2 p[kBDenseSample / kBOctThreads];
+#pragma unroll
+        for (int u = 0; u < kBDenseSample / kBOctThreads; ++u)
+            p[u] = __ldg(reinterpret_cast<const float2*>(a.pts) + base + (tid + u * kBOctThreads) * step);
+#pragma unroll
+        for (int u = 0; u < kBDenseSample / kBOctThreads; ++u)
+            out += in_inner(s_o, __float2int_rn(p[u].x), __float2int_rn(p[u].y)) ? 0u : 1u;
         out = __reduce_add_sync(0xFFFFFFFFu, out);
         if (lane == 0 && out) atomicAdd(&s_out, out);
         __syncthreads();
@@ -447,15 +461,18 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
 
 // ---------------------------------------------------------------------------
 // The filter of the sets without a star polygon, streamed (the loop of
-// Alg. 1/2): the warp tiles and block chunks of bt_extremes.  A warp keeps
+// Alg. 1/2): the warp tiles of bt_extremes, which the warps take in chunks from
+// a counter (the sets with a polygon, bt_dense's, are passed over, so the work
+// is uneven along the batch) and stream through their rings.  A warp keeps
 // the octagon of its current set in shared memory.  Per point: the octagon's
-// inner region drops it (a whole lane's points at once when their key
-// extremes lie in the region); the points it leaves wait in a per-warp queue
-// and go 32 at a time through the hull-rule classification, and the kept
-// ones become records of their queue, staged per warp and written to the
-// set's region with one atomic per batch.  Survivors on a support line of
-// the octagon reduce to the lines' end points (reduce_on_line).  The sets
-// with a star polygon are bt_dense's: their tiles are streamed and skipped.
+// inner region drops it, eight float instructions on the keys x, y, x + y and
+// x - y scaled to the region (BtInner); the points it leaves wait in a per-warp
+// queue and go 32 at a time through the hull-rule classification, and the kept
+// ones become records of their queue, staged per warp and written to the set's
+// region with one atomic per batch.  Survivors on a support line of the octagon
+// reduce to the lines' end points (reduce_on_line).  (Integer keys folded per
+// lane and a second look at failing lanes' points took 39 warp instructions
+// per 32 points, ncu, and every tile was copied: 0.94 ms on the 4096-set batch.)
 constexpr int kBtWarpRecs = 128;
 constexpr int kBtQueue = 64;   // < 32 waiting + 32 added per step
 struct BtWarpSmem {
@@ -464,7 +481,6 @@ struct BtWarpSmem {
     uint32_t key[kBtWarpRecs];
     float qx[kBtQueue], qy[kBtQueue];   // points waiting for the exact tests
     unsigned qi[kBtQueue];
-    unsigned char lanes[32];         // lanes whose tile the inner region did not settle
     Ctl* c;                          // the warp's set: control block, record region,
     long long rb;
     unsigned cnt;                    // records staged,
@@ -479,6 +495,33 @@ struct BtWarpSet {
     long long base = 0;
     bool skip = true;              // empty, failed, or bt_dense's: nothing to classify
     unsigned qn = 0u;              // points queued
+};
+
+// The inner region of an octagon as four scaled keys: a point is inside when
+// |key * scale + offset| <= 1 for x, y, x + y and x - y.  The region is taken 8
+// units smaller on each side (16 for x + y) than the octagon's: the three
+// roundings of a scaled key are below 2^-23 (|key| + |centre|), 4 units (8 and
+// 2 for the sum), so a point that passes is inside.
+struct BtInner {
+    float sx, ox, sy, oy, ss, os, sd, od;
+    __device__ __forceinline__ void axis(int lo, int hi, float margin, float& s, float& o) const {
+        const float h = 0.5f * (float)(hi - lo) - margin;
+        const bool some = lo <= hi && h > 0.0f;
+        s = some ? 1.0f / h : 0.0f;
+        o = some ? -0.5f * ((float)lo + (float)hi) * s : 2.0f;
+    }
+    __device__ __forceinline__ void set(const Octagon& o) {
+        axis(o.in_lo[0], o.in_hi[0], 8.0f, sx, ox);
+        axis(o.in_lo[1], o.in_hi[1], 8.0f, sy, oy);
+        axis(o.in_lo[2], o.in_hi[2], 16.0f, ss, os);
+        axis(o.in_lo[3] - kCoordLimit, o.in_hi[3] - kCoordLimit, 8.0f, sd, od);
+    }
+    __device__ __forceinline__ bool outside(float x, float y) const {
+        float m;
+        asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(fmaf(x, sx, ox)), "f"(fmaf(y, sy, oy)), "f"(fmaf(x + y, ss, os)));
+        asm("max.abs.f32 %0, %1, %2, %2;" : "=f"(m) : "f"(m), "f"(fmaf(x - y, sd, od)));
+        return m > 1.0f;
+    }
 };
 
 __device__ __forceinline__ void bt_flush_recs(BtWarpSmem& m, uint32_t* keys, uint64_t* vals) {
@@ -585,10 +628,9 @@ __device__ __forceinline__ void bt_warp_set(const BArgs& a, int q, BtWarpSet& w,
     Ctl* c = a.ctl + q;
     w.set = q;
     w.base = a.offsets[q];
-    const int slot = a.star_slot[q];
     // empty and failed sets (bt_octagon's verdict), and the sets with a star
     // polygon, which bt_dense filters
-    w.skip = *(volatile int*)&c->done != 0 || (slot >= 0 && c->star_k > 0);
+    w.skip = c->skip != 0;
     if (lane == 0) {
         m.c = c;
         m.rb = region_base(a, q);
@@ -624,162 +666,203 @@ __device__ void bt_filter_global(const BArgs& a, long long lo, long long hi, BtW
     }
 }
 
+// A warp's place in the batch: its chunk's next tile t (below end), and the set
+// s that holds the tile's first point.
+template <int P>
+struct BtCursor {
+    static constexpr long long kPts = 32ll * P;
+    long long t = 0, end = 0;
+    int s = 0;
+    bool skip = false;   // of set s
+    // The next tile with a point to classify, in (t, end, s); false when the
+    // batch is done.  Tiles wholly inside a set to skip are passed over.
+    __device__ __forceinline__ bool next(const BArgs& a) {
+        const int lane = threadIdx.x & 31;
+        for (;;) {
+            if (t >= end) {
+                unsigned g = 0u;
+                if (lane == 0) g = atomicAdd(&a.star_ctr[13], 1u);
+                t = (long long)__shfl_sync(0xFFFFFFFFu, g, 0) * a.fchunk;
+                if (t >= a.nwt) return false;
+                end = min(a.nwt, t + a.fchunk);
+                s = bt_find_set(a, a.head + t * kPts);
+                skip = __ldcg(&a.ctl[s].skip) != 0;
+            }
+            const long long p0 = a.head + t * kPts;
+            if (__ldg(a.offsets + s + 1) <= p0) {
+                do ++s;
+                while (__ldg(a.offsets + s + 1) <= p0);
+                skip = __ldcg(&a.ctl[s].skip) != 0;
+            }
+            if (!skip) return true;
+            const long long past = (__ldg(a.offsets + s + 1) - a.head) / kPts;   // first tile not wholly before the set's end
+            if (past <= t) return true;   // the tile meets the next set
+            t = min(end, past);
+        }
+    }
+};
+
 template <int T, int P>
-__global__ void __launch_bounds__(T, 1) bt_filter(BArgs a) {
+__global__ void __launch_bounds__(T, T <= 256 ? 2 : 1) bt_filter(BArgs a) {
     constexpr int kWarps = T / 32, kF4 = 16 * P;
     constexpr long long kPts = 32ll * P;
+    static_assert(P <= 32 && kStages == 2, "a mask bit per point of a lane; two tiles in flight");
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ unsigned long long s_bar[kWarps][kStages];
     __shared__ BtWarpSmem s_w[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     BtWarpSmem& m = s_w[warp];
     BtWarpSet w;
-    const long long nwt = a.nwt;
-    const long long per = (nwt + gridDim.x - 1) / gridDim.x;
-    const long long c0 = min(nwt, (long long)blockIdx.x * per), c1 = min(nwt, c0 + per);
+    BtInner in;
     if (blockIdx.x == 0 && warp == 0) {
         bt_filter_global(a, 0, a.head, w, m);
-        bt_filter_global(a, a.head + nwt * kPts, a.total, w, m);
+        bt_filter_global(a, a.head + a.nwt * kPts, a.total, w, m);
+        bt_warp_done(a, m, w);
     }
-    if (c0 + warp < c1) {
-        WarpStreamT<kF4> ws{reinterpret_cast<float4*>(dsm) + warp * kStages * kF4, s_bar[warp],
-                            reinterpret_cast<const float4*>(a.pts + 2 * a.head), c0 + warp, kWarps, c1, lane};
-        int s = bt_find_set(a, a.head + (c0 + warp) * kPts);
-        ws.start();
-        for (long long k = 0;; ++k) {
-            const long long t = c0 + warp + k * kWarps;
-            if (t >= c1) break;
-            const long long p0 = a.head + t * kPts;
-            while (__ldg(a.offsets + s + 1) <= p0) ++s;
-            const float4* cur = ws.acquire(k, a.ctl + s);
-            if (!cur) {   // a copy never completed: every set of the rest of the chunk fails
-                ws.drain(k);
-                const long long pend = a.head + c1 * kPts;
-                for (int q = s + lane; q < a.k && __ldg(a.offsets + q) < pend; q += 32)
+    const float4* body = reinterpret_cast<const float4*>(a.pts + 2 * a.head);
+    WarpRing<kF4> ring{reinterpret_cast<float4*>(dsm) + warp * kStages * kF4, s_bar[warp], lane};
+    ring.init();
+    BtCursor<P> cur;              // runs ahead of the tile at hand
+    long long t0 = -1, t1 = -1, e0 = 0, e1 = 0;   // the tiles in flight, their chunks' ends
+    int s0 = 0, s1 = 0;                           // and their first points' sets
+    auto advance = [&](long long& t, long long& e, int& s) {
+        t = -1;
+        if (!cur.next(a)) return;
+        t = cur.t++;
+        e = cur.end;
+        s = cur.s;
+        ring.issue(body + t * kF4);
+    };
+    advance(t0, e0, s0);
+    if (t0 >= 0) advance(t1, e1, s1);
+    while (t0 >= 0) {
+        const float4* tile = ring.acquire(a.ctl + s0);
+        if (!tile) {   // a copy never completed: every set of the rest of the chunks in hand fails
+            ring.drain();
+            for (int f = 0; f < 2; ++f) {
+                const long long t = f ? t1 : t0, pend = a.head + (f ? e1 : e0) * kPts;
+                if (t < 0) continue;
+                for (int q = (f ? s1 : s0) + lane; q < a.k && __ldg(a.offsets + q) < pend; q += 32)
                     set_status(a.ctl + q, CH_ETIMEOUT);
-                break;
             }
-            const float2* cur2 = reinterpret_cast<const float2*>(cur);
-            if (__ldg(a.offsets + s + 1) >= p0 + kPts) {   // inside set s
-                if (s != w.set) bt_warp_set(a, s, w, m);
-                if (!w.skip) {
-                    const Octagon& so = m.o;
-                    int tk[8];
-#pragma unroll
-                    for (int j = 0; j < P / 2; ++j) {
-                        const float4 v = cur[j * 32 + lane];
-                        tile_keys2(tk, __float2int_rn(v.x), __float2int_rn(v.y), __float2int_rn(v.z),
-                                   __float2int_rn(v.w), j == 0);
-                    }
-                    const bool inside = tk[W] >= so.in_lo[0] && tk[E] <= so.in_hi[0] && tk[S] >= so.in_lo[1] &&
-                                        tk[N] <= so.in_hi[1] && tk[SW] >= so.in_lo[2] && tk[NE] <= so.in_hi[2] &&
-                                        tk[NW] >= so.in_lo[3] && tk[SE] <= so.in_hi[3];
-                    // The points of the lanes whose tile failed are spread over
-                    // the warp, 32 at a time (slot s: failing lane of rank
-                    // s / P, its point s % P, in float4 (s % P) / 2, half s % 2).
-                    // A point outside the inner region waits for the
-                    // classification.
-                    const unsigned fail = __ballot_sync(0xFFFFFFFFu, !inside);
-                    if (fail) {
-                        if (!inside) m.lanes[__popc(fail & lanemask_lt())] = (unsigned char)lane;
-                        __syncwarp();
-                        const unsigned slots = (unsigned)P * (unsigned)__popc(fail);
-#pragma unroll 1
-                        for (unsigned s0 = 0; s0 < slots; s0 += 32u) {
-                            const unsigned sl = s0 + (unsigned)lane;
-                            bool need = false;
-                            float x = 0.0f, y = 0.0f;
-                            unsigned li = 0u;
-                            if (sl < slots) {
-                                const int ln = m.lanes[sl / P], j = (int)(sl % P);
-                                const int f2 = 2 * ((j >> 1) * 32 + ln) + (j & 1);
-                                const float2 p = cur2[f2];
-                                x = p.x;
-                                y = p.y;
-                                li = (unsigned)(p0 - w.base) + (unsigned)f2;
-                                need = !in_inner(so, __float2int_rn(x), __float2int_rn(y));
-                            }
-                            bt_queue_push(a, w, m, need, x, y, li);
-                        }
-                        __syncwarp();
-                    }
-                }
-            } else {   // the tile meets a set boundary: set by set
-                for (int q = s; q < a.k; ++q) {
-                    const long long qb = __ldg(a.offsets + q), qe = __ldg(a.offsets + q + 1);
-                    if (qb >= p0 + kPts) break;
-                    if (qe <= p0) continue;
-                    if (q != w.set) bt_warp_set(a, q, w, m);
-                    if (w.skip) continue;
-#pragma unroll 1
-                    for (int j = 0; j < P; ++j) {
-                        const long long i = p0 + 2 * ((j >> 1) * 32 + lane) + (j & 1);
-                        const float2 p = cur2[2 * ((j >> 1) * 32 + lane) + (j & 1)];
-                        bt_classify32(a.keys, a.vals, m, i >= qb && i < qe, p.x, p.y, (unsigned)(i - qb));
-                    }
-                }
-            }
-            ws.release(k);
+            if (w.set >= 0 && lane == 0) set_status(a.ctl + w.set, CH_ETIMEOUT);
+            break;
         }
+        const long long p0 = a.head + t0 * kPts;
+        const float2* tile2 = reinterpret_cast<const float2*>(tile);
+        if (__ldg(a.offsets + s0 + 1) >= p0 + kPts) {   // inside set s0
+            if (s0 != w.set) {
+                bt_warp_set(a, s0, w, m);
+                in.set(m.o);
+            }
+            unsigned mask = 0u;   // the lane's points outside the inner region
+#pragma unroll
+            for (int j = 0; j < P / 2; ++j) {
+                const float4 v = tile[j * 32 + lane];
+                if (in.outside(v.x, v.y)) mask |= 1u << (2 * j);
+                if (in.outside(v.z, v.w)) mask |= 2u << (2 * j);
+            }
+            const unsigned li0 = (unsigned)(p0 - w.base);
+            while (__any_sync(0xFFFFFFFFu, mask != 0u)) {   // a point per lane and step
+                const int b = __ffs((int)mask) - 1, f2 = 64 * (b >> 1) + 2 * lane + (b & 1);
+                const float2 p = mask ? tile2[f2] : make_float2(0.0f, 0.0f);
+                bt_queue_push(a, w, m, mask != 0u, p.x, p.y, li0 + (unsigned)f2);
+                mask &= mask - 1u;
+            }
+        } else {   // the tile meets a set boundary: set by set
+            for (int q = s0; q < a.k; ++q) {
+                const long long qb = __ldg(a.offsets + q), qe = __ldg(a.offsets + q + 1);
+                if (qb >= p0 + kPts) break;
+                if (qe <= p0) continue;
+                if (q != w.set) {
+                    bt_warp_set(a, q, w, m);
+                    in.set(m.o);
+                }
+                if (w.skip) continue;
+#pragma unroll 1
+                for (int j = 0; j < P; ++j) {
+                    const long long i = p0 + 2 * ((j >> 1) * 32 + lane) + (j & 1);
+                    const float2 p = tile2[2 * ((j >> 1) * 32 + lane) + (j & 1)];
+                    const bool mine = i >= qb && i < qe;
+                    bt_queue_push(a, w, m, mine && in.outside(p.x, p.y), p.x, p.y, (unsigned)(i - qb));
+                }
+            }
+        }
+        ring.release();
+        t0 = t1;
+        e0 = e1;
+        s0 = s1;
+        if (t0 >= 0) advance(t1, e1, s1);
     }
     bt_warp_done(a, m, w);
 }
 
 // ---------------------------------------------------------------------------
-// Bins of the dense sets (bt_octagon's list).  Chunk ch of the work is run
-// ch % kBStarParts of listed set ch / kBStarParts: the points
-// [base + part * (n / kBStarParts), + min(n / kBStarParts, kBStarRun)).
-// Every point outside the octagon's inner region goes to its angular bin
-// around the set's centre, where a 64-bit atomicMax keeps the point farthest
-// from the centre, packed (squared distance >> 17, local index); a point
-// reads its bin first and issues the atomic only when it beats it.
-constexpr int kBStarBinThreads = 256;
+// Bins of the dense sets (bt_octagon's list): kBStarParts evenly spread runs
+// of a set's points, [r (n / kBStarParts), + min(n / kBStarParts, kBStarRun)).
+// Every point outside the octagon's inner region goes to its angular bin around
+// the set's centre, where an atomicMax keeps the point farthest from the centre,
+// packed (squared distance >> 17, local index); a point reads its bin first and
+// issues the atomic only when it beats it.  A block bins in shared memory and
+// writes its bins out once (bins in L2 took 0.49 ms on the 4096-set batch, most
+// of it waiting for them); with few sets listed, several blocks share a set's
+// runs and meet in the set's bins.
+constexpr int kBStarBinThreads = 512;
 constexpr int kBStarBinU = 8;   // points per thread in flight
+constexpr size_t kBStarBinSmem = sizeof(unsigned long long) * kStarBins;
 
 __global__ void __launch_bounds__(kBStarBinThreads) bt_star_bin(BArgs a) {
+    extern __shared__ __align__(16) unsigned long long mine[];
     const int tid = threadIdx.x;
-    const unsigned nchunks = a.star_ctr[0] * (unsigned)kBStarParts;
-    for (unsigned ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int i = a.star_list[ch / kBStarParts];
-        const int part = (int)(ch % kBStarParts);
+    const unsigned listed = a.star_ctr[0];
+    if (listed == 0u) return;
+    int parts = kBStarParts;   // blocks per set: the runs shared out while blocks are idle
+    while (parts > 1 && (unsigned)parts * listed > gridDim.x) parts >>= 1;
+    for (unsigned w = blockIdx.x; w < listed * (unsigned)parts; w += gridDim.x) {
+        const int i = a.star_list[w / (unsigned)parts];
+        const int part = (int)(w % (unsigned)parts);
         const Ctl* c = a.ctl + i;
         const long long base = a.offsets[i], ni = a.offsets[i + 1] - base;
         const long long step = ni / kBStarParts;
-        const long long lo = (long long)part * step;   // local index of the run
         const int len = (int)min(step, (long long)kBStarRun);
         const int cx = c->star_cx, cy = c->star_cy;
         const int xl = c->oct.in_lo[0], yl = c->oct.in_lo[1], sl = c->oct.in_lo[2], dl = c->oct.in_lo[3];
         const int xh = c->oct.in_hi[0], yh = c->oct.in_hi[1], sh = c->oct.in_hi[2], dh = c->oct.in_hi[3];
-        unsigned long long* bins = a.star_bins + (size_t)a.star_slot[i] * kStarBins;
-        const float2* p2 = reinterpret_cast<const float2*>(a.pts) + base + lo;
-        for (int j0 = 0; j0 < len; j0 += kBStarBinThreads * kBStarBinU) {
-            float2 p[kBStarBinU];
+        for (int b = tid; b < kStarBins; b += kBStarBinThreads) mine[b] = 0ull;
+        __syncthreads();
+        for (int r = part; r < kBStarParts; r += parts) {
+            const long long lo = (long long)r * step;   // local index of the run
+            const float2* p2 = reinterpret_cast<const float2*>(a.pts) + base + lo;
+            for (int j0 = 0; j0 < len; j0 += kBStarBinThreads * kBStarBinU) {
+                float2 p[kBStarBinU];
 #pragma unroll
-            for (int u = 0; u < kBStarBinU; ++u) {
-                const int j = j0 + u * kBStarBinThreads + tid;
-                p[u] = j < len ? __ldcs(p2 + j) : make_float2(-1.0f, -1.0f);
+                for (int u = 0; u < kBStarBinU; ++u) {
+                    const int j = j0 + u * kBStarBinThreads + tid;
+                    p[u] = j < len ? __ldg(p2 + j) : make_float2(-1.0f, -1.0f);
+                }
+#pragma unroll
+                for (int u = 0; u < kBStarBinU; ++u) {
+                    const int X = __float2int_rn(p[u].x), Y = __float2int_rn(p[u].y);
+                    const int S = X + Y, D = X - Y + kCoordLimit;
+                    const bool inner =
+                        X >= xl && X <= xh && Y >= yl && Y <= yh && S >= sl && S <= sh && D >= dl && D <= dh;
+                    if (inner || ((unsigned)(X | Y) >> kCoordBits) != 0u) continue;   // or past the run's end
+                    const int dx = X - cx, dy = Y - cy;
+                    const unsigned long long d2 = (unsigned long long)((long long)dx * dx + (long long)dy * dy);
+                    const long long li = lo + j0 + u * kBStarBinThreads + tid;
+                    const unsigned long long key = ((d2 >> 17) << 32) | (unsigned long long)li;
+                    unsigned long long* bin = mine + star_bin(dx, dy);
+                    if (key > *(volatile unsigned long long*)bin) atomicMax(bin, key);
+                }
             }
-            unsigned long long key[kBStarBinU];
-            int bin[kBStarBinU];
-#pragma unroll
-            for (int u = 0; u < kBStarBinU; ++u) {
-                const int X = __float2int_rn(p[u].x), Y = __float2int_rn(p[u].y);
-                const int S = X + Y, D = X - Y + kCoordLimit;
-                const bool inner = X >= xl && X <= xh && Y >= yl && Y <= yh && S >= sl && S <= sh && D >= dl && D <= dh;
-                const bool ok = ((unsigned)(X | Y) >> kCoordBits) == 0u && !inner;   // the set's points are valid
-                const int dx = X - cx, dy = Y - cy;
-                const unsigned long long d2 = (unsigned long long)((long long)dx * dx + (long long)dy * dy);
-                const long long li = lo + j0 + u * kBStarBinThreads + tid;
-                key[u] = ok ? ((d2 >> 17) << 32) | (unsigned long long)li : 0ull;
-                bin[u] = star_bin(dx, dy);
-            }
-            unsigned long long cur[kBStarBinU];
-#pragma unroll
-            for (int u = 0; u < kBStarBinU; ++u) cur[u] = key[u] ? __ldcg(bins + bin[u]) : ~0ull;
-#pragma unroll
-            for (int u = 0; u < kBStarBinU; ++u)
-                if (key[u] > cur[u]) atomicMax(&bins[bin[u]], key[u]);
         }
+        __syncthreads();
+        unsigned long long* bins = a.star_bins + (size_t)a.star_slot[i] * kStarBins;
+        for (int b = tid; b < kStarBins; b += kBStarBinThreads) {
+            if (parts == 1) bins[b] = mine[b];
+            else if (mine[b]) atomicMax(&bins[b], mine[b]);
+        }
+        __syncthreads();
     }
 }
 
@@ -819,7 +902,10 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_build(BArgs a) {
             int4* dst = reinterpret_cast<int4*>(a.star_polys + slot);
             for (int j = tid; j < (int)(sizeof(StarPoly) / 16); j += kBStarThreads) dst[j] = src[j];
         }
-        if (tid == 0) c->star_k = K;
+        if (tid == 0) {
+            c->star_k = K;
+            c->skip = K > 0;   // bt_dense's
+        }
         __syncthreads();
     }
 }
@@ -829,28 +915,31 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_build(BArgs a) {
 // bt_filter leaves to this kernel: the single hull's dense post pass per
 // set.  Work units are runs of up to kBDenseRun points of a set
 // (bt_dense_plan numbers them); a block takes units one at a time, copies the
-// set's polygon (all of it, 112 KB, mostly from L2) and octagon into shared
-// memory, and streams the run's points with the loads of its next step in
-// flight: a point closer to the centre than the polygon's inscribed radius,
-// or than its bin's radius bound, is strictly inside the polygon; the others
-// wait in a per-warp queue and go 32 at a time through the exact wedge test
-// and the hull-rule classification; kept points become records of their
-// queue, staged per warp and written to the set's region with one atomic per
-// batch.
-constexpr int kBDenseThreads = 512;
+// set's radius bounds and octagon into shared memory, and streams the run's
+// points through its warps' rings: a point closer to the centre than its
+// bin's radius bound is strictly inside the polygon; the others wait in a
+// per-warp queue and go 32 at a time through the exact wedge test (the polygon
+// read from L2) and the hull-rule classification; kept points become records
+// of their queue, staged per warp and written to the set's region with one
+// atomic per batch.  (With 64-bit distances and a ballot per 32 points it
+// executed 92 warp instructions per 32 points, ncu, and took 0.80 ms on the
+// 4096-set batch.)
+constexpr int kBDenseThreads = 1024;
 constexpr int kBDenseRun = 1 << 18;    // points of a work unit
-constexpr int kBDenseU = 8;            // points per thread and step
-constexpr int kBDenseRecs = 256;       // records staged per warp
-constexpr int kBDenseQueue = 32 * kBDenseU + 32;   // < 32 waiting + a step's points
+constexpr int kBDenseF4 = 128;         // float4 of a warp's ring tile
+constexpr int kBDenseRecs = 64;        // records staged per warp
+constexpr int kBDenseQueue = 64;       // < 32 waiting + 32 added per step
 struct BtDenseWarp {
     uint64_t val[kBDenseRecs];
     uint32_t key[kBDenseRecs];
-    float qx[kBDenseQueue], qy[kBDenseQueue];
+    float2 q[kBDenseQueue];
     unsigned qi[kBDenseQueue];
+    unsigned cnt, nq[4];               // records staged, records per queue of the unit
 };
-constexpr size_t kBDenseWarpOff = (sizeof(StarPoly) + sizeof(Octagon) + 15) / 16 * 16;
-constexpr size_t kBDenseSmem = kBDenseWarpOff + (kBDenseThreads / 32) * sizeof(BtDenseWarp);
-static_assert(kBDenseSmem <= 227 * 1024, "one block's shared memory");
+constexpr size_t kBDenseWarpOff = sizeof(float) * kStarBins;
+constexpr size_t kBDenseRingOff = (kBDenseWarpOff + (kBDenseThreads / 32) * sizeof(BtDenseWarp) + 127) / 128 * 128;
+constexpr size_t kBDenseSmem = kBDenseRingOff + (size_t)(kBDenseThreads / 32) * kStages * kBDenseF4 * sizeof(float4);
+static_assert(kBDenseSmem <= 225 * 1024, "one block's shared memory");
 
 // Work units of the sets with a polygon: unit_base[j] = first unit of listed
 // set j (one block of 1024 threads; star_ctr[7] = total units).
@@ -884,35 +973,50 @@ __global__ void __launch_bounds__(1024) bt_dense_plan(BArgs a) {
     if (tid == 1023) a.star_ctr[7] = s_part[1023];
 }
 
-// Warp-collective: the exact tests of one queued point per lane (valid =
-// false for none) and the staging of the kept ones.
-__device__ __forceinline__ void bt_dense_exact(const BArgs& a, const StarPoly& P, const Octagon& so, Ctl* c,
-                                               long long rb, int cx, int cy, BtDenseWarp& wb, unsigned& cnt,
-                                               unsigned (&nq)[4], bool valid, float x, float y, unsigned li) {
+// A unit's set, in shared memory.
+struct BtDenseSet {
+    Ctl* c;
+    uint32_t* keys;       // the set's record region
+    uint64_t* vals;
+    const StarPoly* P;
+    int cx, cy;
+    Octagon o;
+};
+
+__device__ __forceinline__ void bt_dense_flush(const BtDenseSet& m, BtDenseWarp& wb, unsigned cnt) {
     const int lane = threadIdx.x & 31;
-    int r = -1, X = 0, Y = 0;
-    if (valid) {
-        X = __float2int_rn(x);
-        Y = __float2int_rn(y);
-        const int px = X - cx, py = Y - cy;
-        if (!star_inside_exact(px, py, star_bin(px, py), P)) r = classify_hull(x, y, so);
+    unsigned base = 0u;
+    if (lane == 0) base = atomicAdd(&m.c->count, cnt);
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    for (unsigned j = lane; j < cnt; j += 32) {
+        m.keys[base + j] = wb.key[j];
+        m.vals[base + j] = wb.val[j];
     }
+    __syncwarp();
+}
+
+// Warp-collective, out of line: the exact tests of the queued points [first,
+// first + count), count <= 32, and the staging of the kept ones.
+__device__ __noinline__ void bt_dense_drain(const BtDenseSet& m, BtDenseWarp& wb, unsigned first, unsigned count) {
+    const int lane = threadIdx.x & 31, cx = m.cx, cy = m.cy;
+    const Octagon& so = m.o;
+    const bool valid = (unsigned)lane < count;
+    const float2 p = valid ? wb.q[first + lane] : make_float2(0.0f, 0.0f);
+    const unsigned li = valid ? wb.qi[first + lane] : 0u;
+    const int X = __float2int_rn(p.x), Y = __float2int_rn(p.y);
+    int r = -1;
+    if (valid && !star_inside_exact(X - cx, Y - cy, star_bin(X - cx, Y - cy), *m.P)) r = classify_hull(p.x, p.y, so);
     bool keep = r >= 0;
     if (!__any_sync(0xFFFFFFFFu, keep)) return;
-    if (reduce_on_line(so, keep, X, Y, li, c)) keep = false;
+    if (reduce_on_line(so, keep, X, Y, li, m.c)) keep = false;
     const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
     if (!bal) return;
+    unsigned nq[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) nq[q] += (unsigned)__popc(__ballot_sync(0xFFFFFFFFu, keep && r == q));
+    for (int q = 0; q < 4; ++q) nq[q] = (unsigned)__popc(__ballot_sync(0xFFFFFFFFu, keep && r == q));
+    unsigned cnt = wb.cnt;
     if (cnt + (unsigned)__popc(bal) > (unsigned)kBDenseRecs) {   // write the staged records out
-        unsigned base = 0u;
-        if (lane == 0) base = atomicAdd(&c->count, cnt);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        for (unsigned j = lane; j < cnt; j += 32) {
-            a.keys[rb + base + j] = wb.key[j];
-            a.vals[rb + base + j] = wb.val[j];
-        }
-        __syncwarp();
+        bt_dense_flush(m, wb, cnt);
         cnt = 0u;
     }
     if (keep) {
@@ -922,17 +1026,25 @@ __device__ __forceinline__ void bt_dense_exact(const BArgs& a, const StarPoly& P
         wb.key[pos] = make_key(r, u);
         wb.val[pos] = make_val(v, li);
     }
-    cnt += (unsigned)__popc(bal);
+    __syncwarp();
+    if (lane == 0) {
+        wb.cnt = cnt + (unsigned)__popc(bal);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) wb.nq[q] += nq[q];
+    }
     __syncwarp();
 }
 
 __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
-    extern __shared__ __align__(16) char dyn[];
-    StarPoly& P = *reinterpret_cast<StarPoly*>(dyn);
-    Octagon& so = *reinterpret_cast<Octagon*>(dyn + sizeof(StarPoly));
+    extern __shared__ __align__(128) char dyn[];
+    __shared__ unsigned long long s_bar[kBDenseThreads / 32][kStages];
+    float* thr = reinterpret_cast<float*>(dyn);
+    __shared__ BtDenseSet m;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kWarps = kBDenseThreads / 32, kPts = 2 * kBDenseF4;
     BtDenseWarp& wb = reinterpret_cast<BtDenseWarp*>(dyn + kBDenseWarpOff)[warp];
-    constexpr int kStep = kBDenseThreads * kBDenseU;
+    WarpRing<kBDenseF4> ring{reinterpret_cast<float4*>(dyn + kBDenseRingOff) + warp * kStages * kBDenseF4, s_bar[warp], lane};
+    ring.init();
     __shared__ int s_set, s_part;
     const unsigned nunits = a.star_ctr[7];
     const int listed = (int)a.star_ctr[0];
@@ -960,80 +1072,84 @@ __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
         const long long base = a.offsets[i], ni = a.offsets[i + 1] - base;
         const long long rb = region_base(a, i);
         const long long lo = (long long)s_part * kBDenseRun, hi = min(ni, lo + kBDenseRun);
-        {   // the polygon and the octagon into shared memory
-            const int4* src = reinterpret_cast<const int4*>(a.star_polys + a.star_slot[i]);
-            int4* dst = reinterpret_cast<int4*>(&P);
-            for (int j = tid; j < (int)(sizeof(StarPoly) / 16); j += kBDenseThreads) dst[j] = __ldcg(src + j);
-            copy_octagon(&so, &c->oct);
+        const StarPoly& P = a.star_polys[a.star_slot[i]];
+        for (int j = tid; j < kStarBins / 4; j += kBDenseThreads)
+            reinterpret_cast<float4*>(thr)[j] = __ldcg(reinterpret_cast<const float4*>(P.thr) + j);
+        copy_octagon(&m.o, &c->oct);
+        if (tid == 0) {
+            m.c = c;
+            m.keys = a.keys + rb;
+            m.vals = a.vals + rb;
+            m.P = &P;
+            m.cx = c->star_cx;
+            m.cy = c->star_cy;
         }
-        __syncthreads();
-        const int cx = c->star_cx, cy = c->star_cy;
-        const float fcx = (float)cx, fcy = (float)cy, tmin = P.tmin;
+        if (lane == 0) wb.cnt = 0u;
+        if (lane < 4) wb.nq[lane] = 0u;
+        const float fcx = (float)c->star_cx, fcy = (float)c->star_cy;
         const float2* p2 = reinterpret_cast<const float2*>(a.pts) + base;
-        unsigned cnt = 0u, qn = 0u;
-        unsigned nq[4] = {0u, 0u, 0u, 0u};
-        float2 cur[kBDenseU];
-#pragma unroll
-        for (int u = 0; u < kBDenseU; ++u) {
-            const long long j = lo + u * kBDenseThreads + tid;
-            cur[u] = j < hi ? __ldcs(p2 + j) : make_float2(0.0f, 0.0f);
-        }
-        for (long long s0 = lo; s0 < hi; s0 += kStep) {
-            float2 nxt[kBDenseU];
-#pragma unroll
-            for (int u = 0; u < kBDenseU; ++u) {
-                const long long j = s0 + kStep + u * kBDenseThreads + tid;
-                nxt[u] = j < hi ? __ldcs(p2 + j) : make_float2(0.0f, 0.0f);
+        // the 16-byte aligned body of the run in tiles of kPts points
+        const int odd = (reinterpret_cast<uintptr_t>(p2 + lo) & 15u) != 0u ? 1 : 0;
+        const float4* body = reinterpret_cast<const float4*>(p2 + lo + odd);
+        const int nt = (int)((hi - lo - odd) / kPts);
+        for (int t = warp; t < nt && t < kStages * kWarps; t += kWarps) ring.issue(body + (size_t)t * kBDenseF4);
+        __syncthreads();
+        unsigned qn = 0u;
+        for (int t = warp; t < nt; t += kWarps) {
+            const float4* cur = ring.acquire(c);
+            if (!cur) {   // a copy never completed: the set fails
+                ring.drain();
+                if (lane == 0) set_status(c, CH_ETIMEOUT);
+                break;
             }
+            unsigned mask = 0u;   // the lane's points that the radius bounds leave
 #pragma unroll
-            for (int u = 0; u < kBDenseU; ++u) {
-                const long long j = s0 + u * kBDenseThreads + tid;
-                bool need = false;
-                if (j < hi) {
-                    const float dx = cur[u].x - fcx, dy = cur[u].y - fcy;   // exact
-                    need = star_d2(dx, dy) >= tmin && !star_inside_fast(dx, dy, star_bin(dx, dy), P);
-                }
-                const unsigned bal = __ballot_sync(0xFFFFFFFFu, need);
-                if (need) {   // queued
+            for (int j = 0; j < kBDenseF4 / 32; ++j) {
+                const float4 p = cur[j * 32 + lane];
+                const float dx0 = p.x - fcx, dy0 = p.y - fcy, dx1 = p.z - fcx, dy1 = p.w - fcy;   // exact
+                if (!(star_d2(dx0, dy0) < thr[star_bin(dx0, dy0)])) mask |= 1u << (2 * j);
+                if (!(star_d2(dx1, dy1) < thr[star_bin(dx1, dy1)])) mask |= 2u << (2 * j);
+            }
+            // queued, a point per lane and step; full rounds of 32 go through
+            // the exact tests
+            const float2* cur2 = reinterpret_cast<const float2*>(cur);
+            for (unsigned bal; (bal = __ballot_sync(0xFFFFFFFFu, mask != 0u)) != 0u;) {
+                if (mask) {
+                    const int s = __ffs((int)mask) - 1, f2 = 64 * (s >> 1) + 2 * lane + (s & 1);
+                    mask &= mask - 1u;
                     const unsigned pos = qn + (unsigned)__popc(bal & lanemask_lt());
-                    wb.qx[pos] = cur[u].x;
-                    wb.qy[pos] = cur[u].y;
-                    wb.qi[pos] = (unsigned)j;
+                    wb.q[pos] = cur2[f2];
+                    wb.qi[pos] = (unsigned)(lo + odd) + (unsigned)(t * kPts + f2);
                 }
                 qn += (unsigned)__popc(bal);
-            }
-            __syncwarp();
-            while (qn >= 32u) {   // full rounds of 32 through the exact tests
-                qn -= 32u;
-                const float qx = wb.qx[qn + lane], qy = wb.qy[qn + lane];
-                const unsigned qi = wb.qi[qn + lane];
                 __syncwarp();
-                bt_dense_exact(a, P, so, c, rb, cx, cy, wb, cnt, nq, true, qx, qy, qi);
+                if (qn >= 32u) {
+                    qn -= 32u;
+                    bt_dense_drain(m, wb, qn, 32u);
+                }
             }
-#pragma unroll
-            for (int u = 0; u < kBDenseU; ++u) cur[u] = nxt[u];
+            ring.release();
+            const int next = t + kStages * kWarps;
+            if (next < nt) ring.issue(body + (size_t)next * kBDenseF4);
         }
-        if (qn) {   // the queue's remainder
-            const bool valid = (unsigned)lane < qn;
-            const float qx = valid ? wb.qx[lane] : 0.0f, qy = valid ? wb.qy[lane] : 0.0f;
-            const unsigned qi = valid ? wb.qi[lane] : 0u;
+        if (qn) bt_dense_drain(m, wb, 0u, qn);
+        // the point before the body, and the ragged end by 32 points per warp
+        const long long tail = lo + odd + (long long)nt * kPts + 32 * (kWarps - 1 - warp);
+        const long long ranges[2][2] = {{lo, warp == 0 ? lo + odd : lo}, {tail, min(hi, tail + 32)}};
+        for (int rg = 0; rg < 2; ++rg) {
+            const long long cnt = ranges[rg][1] - ranges[rg][0];
+            if (cnt <= 0) continue;
             __syncwarp();
-            bt_dense_exact(a, P, so, c, rb, cx, cy, wb, cnt, nq, valid, qx, qy, qi);
-        }
-        if (cnt) {
-            unsigned b0 = 0u;
-            if (lane == 0) b0 = atomicAdd(&c->count, cnt);
-            b0 = __shfl_sync(0xFFFFFFFFu, b0, 0);
-            for (unsigned j = lane; j < cnt; j += 32) {
-                a.keys[rb + b0 + j] = wb.key[j];
-                a.vals[rb + b0 + j] = wb.val[j];
+            if (lane < cnt) {
+                wb.q[lane] = __ldcs(p2 + ranges[rg][0] + lane);
+                wb.qi[lane] = (unsigned)(ranges[rg][0] + lane);
             }
+            __syncwarp();
+            bt_dense_drain(m, wb, 0u, (unsigned)cnt);
         }
-        if (lane == 0)
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (nq[q]) atomicAdd(&c->counts4[q], nq[q]);
-        __syncthreads();   // the polygon's shared memory is reloaded by the next unit
+        if (wb.cnt) bt_dense_flush(m, wb, wb.cnt);
+        if (lane < 4 && wb.nq[lane]) atomicAdd(&c->counts4[lane], wb.nq[lane]);
+        __syncthreads();   // the bounds' shared memory is reloaded by the next unit
     }
 }
 
@@ -1403,7 +1519,10 @@ __global__ void __launch_bounds__(T) bt_queue_chain(BArgs a) {
             fits = fits && cr <= (unsigned)Q::kCap;
         }
         if (!fits) {
-            if (tid == 0 && qq == 0) a.big[i] = 1;
+            if (tid == 0 && qq == 0) {
+                a.big[i] = 1;
+                atomicAdd(&a.star_ctr[14], 1u);
+            }
             __syncthreads();
             continue;
         }
@@ -1666,7 +1785,9 @@ static int bt_configure(int dev, BtDevice* out) {
     d.name = prop.name;
     if (cudaFuncSetAttribute(bt_hull, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBHullSmem) != cudaSuccess)
         return CH_ECUDA;
-    if (cudaFuncSetAttribute(bt_star_build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBStarSmem) !=
+    if (cudaFuncSetAttribute(bt_star_bin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBStarBinSmem) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(bt_star_build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBStarSmem) !=
             cudaSuccess ||
         cudaFuncSetAttribute(bt_star_refine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBStarSmem) !=
             cudaSuccess ||
@@ -1831,7 +1952,7 @@ static int bt_enqueue_tiles(const BtCall& c, cudaStream_t s) {
     { ProfScope p("batched_octagon", s); bt_octagon<<<a.k, kBOctThreads, 0, s>>>(a); }
     {
         ProfScope p("batched_star", s);
-        bt_star_bin<<<c.sms * 8, kBStarBinThreads, 0, s>>>(a);
+        bt_star_bin<<<c.sms * 3, kBStarBinThreads, kBStarBinSmem, s>>>(a);
         bt_star_build<<<c.sms, kBStarThreads, kBStarSmem, s>>>(a);
     }
     {
@@ -1936,6 +2057,8 @@ static void bt_set_shape(BtCall& c, const BtDevice& d, int shape) {
     c.shape = shape;
     c.a.wtile = 32 * sh.per;
     c.a.nwt = (c.a.total - c.a.head) / c.a.wtile;
+    const long long warps = (long long)d.sms * d.occ[shape][1] * (sh.threads / 32);
+    c.a.fchunk = (int)std::max(1ll, std::min(16ll, c.a.nwt / (8 * warps)));   // at least 8 chunks a warp
     c.grid_e = (int)std::max(1ll, std::min(c.a.nwt, (long long)d.sms * d.occ[shape][0]));
     c.grid_f = (int)std::max(1ll, std::min(c.a.nwt, (long long)d.sms * d.occ[shape][1]));
 }
@@ -2106,6 +2229,7 @@ int hull_batched_impl(const float* pts, const int64_t* offsets, int32_t k, int32
     b.rt_base = (unsigned*)(base + L.rt_base);
     b.rt_map = (int*)(base + L.rmap);
     b.totals = (unsigned*)(base + L.totals);
+    b.nbig = a.star_ctr + 14;
     b.bcount = (unsigned*)(base + L.bcount);
     b.bcur = (unsigned*)(base + L.bcur);
     b.bstart = (unsigned*)(base + L.bstart);

@@ -59,6 +59,10 @@ __device__ unsigned block_prefix_inplace(unsigned* a, int n, unsigned* s_part, i
 __global__ void __launch_bounds__(1024) btl_prep(BLArgs a) {
     __shared__ unsigned s_part[1024];
     const int tid = threadIdx.x;
+    if (*a.nbig == 0u) {   // nothing for this path: the launches that follow return at once
+        if (tid < 4) a.totals[tid] = tid == 3 ? 1u : 0u;
+        return;
+    }
     const int nseg = 4 * a.k;
     for (int sg = tid; sg < nseg; sg += 1024) {
         const int i = sg >> 2, q = sg & 3;

@@ -17,7 +17,8 @@ struct BLArgs {
     Ctl* ctl;                      // k control blocks (batched)
     uint32_t* keys;                // batched records: set i at offsets[i] + 16 i
     uint64_t* vals;
-    const unsigned char* big;      // k: the set's records exceed one block
+    const unsigned char* big;      // k: 1 when a queue of the set exceeds one block
+    const unsigned* nbig;          // how many such sets there are
     int32_t* out_idx;
     int64_t* out_n;
     // per segment (set, queue): 4k (+1 for the prefixes)

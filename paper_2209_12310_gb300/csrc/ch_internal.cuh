@@ -139,10 +139,10 @@ struct Ctl {
     int bk_state;                       // large-survivor path: 0 unused, 1 queues / tiles / buckets, 2 full sort
     int path;                           // the single hull's large-survivor path (Path)
     unsigned int q_tile[5];             // path tiles: tiles of queue r are [q_tile[r], q_tile[r + 1])
-    int samp_ok;                        // oct_s holds this call's sample octagon
     int samp_dense;                     // dense data (oct_s: an octagon of input points): the star pass bins points
     int oct_ready;                      // the octagon of the true extremes and the end-point records stand
     int star_ok;                        // batched: the set is listed for a star polygon
+    int skip;                           // batched: nothing for bt_filter (empty, failed, or bt_dense's)
     int star_k;                         // the polygon's vertices, the dropped ones included
     int star_edges;                     // dense_kernel: the polygon's vertices in use (0: none)
     int star_final;                     // a polygon was built and accepted

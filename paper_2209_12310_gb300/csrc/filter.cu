@@ -64,7 +64,6 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
         ctl->records_ready = 0;
         ctl->bk_state = 0;
         ctl->path = kPathNone;
-        ctl->samp_ok = 0;
         ctl->samp_dense = 0;
         ctl->oct_ready = 0;
         ctl->star_ok = 0;
@@ -230,13 +229,9 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ p
     // survivors, and all points would be read again.
     const bool dense = test && !s_o.discard_none && probe.dense(s_o, n, switch_at);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        if (dense) {
-            ctl->samp_dense = 1;
-            ctl->mode = 1;
-        }
-        __threadfence();
-        ctl->samp_ok = 1;
+    if (threadIdx.x == 0 && dense) {
+        ctl->samp_dense = 1;
+        ctl->mode = 1;
     }
     CH_TRACE_MARK();
     CH_TL(ctl, 2, 1);

@@ -182,15 +182,18 @@ __device__ __forceinline__ bool inner_fits(const Octagon& o, const int lo[4], co
 // Fills every field of o (in shared memory) from the 8 vertices.  The whole
 // block calls it (all threads, same arguments; blockDim.x >= 64).  Threads
 // 0..7 build the edges, 8..11 the quadrilateral; with with_inner, the block
-// then searches the inner region's scale t/1024: rounds of a 4-way search in
-// which each of up to 3 candidate scales has its 64 (corner, edge) exact
-// tests done by 64 threads at once.  Only scales whose test passed are kept,
-// so the region is verified whatever the search finds.  Without with_inner
+// then searches the inner region's scale t/1024: each (corner, edge) pair's edge
+// function is linear in t, so 64 threads find the scale where it turns negative,
+// and the smallest of those and the two scales below it have their 64 exact
+// tests done at once (rounds of a 4-way search, 5 of them in general, were most
+// of this function's 8 us).  Should none pass, the 4-way search takes over.
+// Only scales whose test passed are kept, so the region is verified whatever
+// the search finds.  Without with_inner
 // the inner region is empty (every test takes the exact path).
 static __device__ void setup_octagon_block(Octagon& o, const int vx[8], const int vy[8], const int ext[8],
                                            bool with_inner) {
     __shared__ long long s_area[8];
-    __shared__ int s_lo, s_hi, s_bad[3];
+    __shared__ int s_lo, s_hi, s_est, s_bad[3];
     const int tid = (int)threadIdx.x;
     if (tid < 8) {
         const int j = (tid + 1) & 7;
@@ -206,6 +209,8 @@ static __device__ void setup_octagon_block(Octagon& o, const int vx[8], const in
     if (tid == 0) {
         s_lo = 0;      // the largest scale verified so far (0: none)
         s_hi = 1025;   // a scale known not to fit
+        s_est = 1024;
+        s_bad[0] = s_bad[1] = s_bad[2] = 0;
     }
     __syncthreads();
     long long area2 = 0;
@@ -222,23 +227,46 @@ static __device__ void setup_octagon_block(Octagon& o, const int vx[8], const in
         const int j = tid >> 6, k = (tid >> 3) & 7, e = tid & 7;
         const int nc = blockDim.x >= 192 ? 3 : 1, sh = blockDim.x >= 192 ? 2 : 1;
         const Edge ed = o.oct[e];
+        auto fails = [&](int t) {   // scale t, corner k, edge e
+            int bl[4], bh[4];
+            inner_bounds(lo0, hi0, t, bl, bh);
+            bool bad = bl[0] > bh[0] || bl[1] > bh[1] || bl[2] > bh[2] || bl[3] > bh[3];
+            if (!bad && (ed.dx | ed.dy) != 0) {
+                long long px, py;
+                inner_corner(bl, bh, k, px, py);
+                bad = edge_exact(ed, px, py) < 0;
+            }
+            return bad;
+        };
+        if (tid < 64) {
+            long long px, py;
+            inner_corner(lo0, hi0, k, px, py);
+            const float f1 = (float)edge_exact(ed, px, py);
+            const float f0 = (float)edge_exact(ed, ((long long)lo0[0] + hi0[0]) / 2, ((long long)lo0[1] + hi0[1]) / 2);
+            const int est = f1 < 0.0f ? max(0, (int)(1024.0f * f0 / (f0 - f1))) : 1024;
+            const int least = __reduce_min_sync(0xFFFFFFFFu, est);
+            if ((tid & 31) == 0) atomicMin(&s_est, least);
+        }
+        __syncthreads();
+        const int est = s_est;
+        if (j < nc && est - j > 0 && fails(est - j)) s_bad[j] = 1;
+        __syncthreads();
+        if (tid == 0) {
+            s_hi = max(1, est - nc + 1);
+            for (int c = nc - 1; c >= 0; --c)
+                if (est - c > 0 && !s_bad[c]) {
+                    s_lo = est - c;
+                    s_hi = s_lo + 1;
+                }
+        }
+        __syncthreads();
         for (int round = 0; round < 12; ++round) {
             const int lo = s_lo, hi = s_hi;
             if (hi - lo <= 1) break;
             if (tid < 3) s_bad[tid] = 0;
             __syncthreads();
             const int t = lo + (((hi - lo) * (j + 1)) >> sh);
-            if (j < nc && t > lo && t < hi) {
-                int bl[4], bh[4];
-                inner_bounds(lo0, hi0, t, bl, bh);
-                bool bad = bl[0] > bh[0] || bl[1] > bh[1] || bl[2] > bh[2] || bl[3] > bh[3];
-                if (!bad && (ed.dx | ed.dy) != 0) {
-                    long long px, py;
-                    inner_corner(bl, bh, k, px, py);
-                    bad = edge_exact(ed, px, py) < 0;
-                }
-                if (bad) s_bad[j] = 1;
-            }
+            if (j < nc && t > lo && t < hi && fails(t)) s_bad[j] = 1;
             __syncthreads();
             if (tid == 0) {   // the largest passing candidate; the next failing one above it
                 int nlo = lo, nhi = hi;

@@ -34,15 +34,10 @@ namespace ch {
 //        thr is r^2 less 5 parts in 2^24, rounded down, and star_d2 is at most
 //        2 parts in 2^24 below d^2: star_d2 < thr proves d < r.  (0 when no
 //        bound was found.)
-//   tmin the same for the smallest line radius of all edges: a point closer
-//        to c than that is strictly inside, whatever its bin (it lies in some
-//        wedge, on the inner side of that wedge's edge line).
 struct StarPoly {
     int2 v[kStarBins + 2];
     unsigned short tbl[kStarBins];
     float thr[kStarBins];
-    float tmin;
-    unsigned pad[3];
 };
 
 // Angular bin of an offset (dx, dy) from c (integers below 2^24, exact as
@@ -350,8 +345,8 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
     constexpr int kPer = kStarBins / T;   // bins per thread: at most 32
     static_assert(kPer <= 16, "gather registers");
     __shared__ unsigned s_scan2[T / 32];
-    __shared__ int s_K0, s_min;
-    const int t = threadIdx.x, lane = t & 31;
+    __shared__ int s_K0;
+    const int t = threadIdx.x;
     // bins [t kPer, (t + 1) kPer): all their keys, then all their points, in
     // flight at once
     unsigned kept = 0u;
@@ -375,19 +370,12 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
     __syncthreads();
     CH_TL(ctl, 9, 1);
     const int K0 = s_K0;
-    if (t == 0) s_min = 0x7FFFFFFF;
     const int K = star_polygon<T>(work, K0, P, ctl);
     if (!K) return 0;
     // each edge's line radius (work is free again), then per bin the smallest
     // of its window
     unsigned* er = reinterpret_cast<unsigned*>(work);
-    unsigned emin = 0x7FFFFFFFu;
-    for (int e = t; e < K; e += T) {
-        er[e] = star_edge_radius(P.v[e], P.v[e + 1]);
-        emin = min(emin, er[e]);
-    }
-    emin = __reduce_min_sync(0xFFFFFFFFu, emin);
-    if (lane == 0) atomicMin(&s_min, (int)emin);
+    for (int e = t; e < K; e += T) er[e] = star_edge_radius(P.v[e], P.v[e + 1]);
     __syncthreads();
     CH_TL(ctl, 12, 1);
     for (int b = t; b < kStarBins; b += T) {
@@ -400,7 +388,6 @@ __device__ int star_finish(const unsigned long long* bins, const float* __restri
         }
         P.thr[b] = star_threshold(m);
     }
-    if (t == 0) P.tmin = star_threshold((unsigned)s_min);
     __syncthreads();
     return K0;
 }

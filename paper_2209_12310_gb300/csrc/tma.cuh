@@ -126,4 +126,50 @@ struct WarpStreamT {
 
 using WarpStream = WarpStreamT<kWarpTileF4>;
 
+// A warp's ring of kStages tiles of kF4 float4 whose sources the caller names
+// one by one (any order, any number of streams in turn): init() once, then
+// issue(src) at most kStages ahead of acquire() / release().
+template <int kF4>
+struct WarpRing {
+    float4* ring;                 // kStages * kF4 float4 of shared memory
+    unsigned long long* bar;      // kStages barriers
+    int lane;
+    unsigned issued = 0u, taken = 0u;
+
+    __device__ __forceinline__ void init() {
+        if (lane == 0) {
+            for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], 1);
+            fence_barrier_init();
+        }
+        __syncwarp();
+    }
+    __device__ __forceinline__ void issue(const float4* src) {
+        if (lane == 0) {
+            const unsigned s = issued % kStages;
+            fence_proxy_async();
+            mbar_expect_tx(&bar[s], kF4 * 16);
+            tma_load(ring + s * kF4, src, kF4 * 16, &bar[s], l2_evict_first());
+        }
+        ++issued;
+    }
+    // Waits for the oldest tile not taken yet; nullptr when the wait gave up.
+    __device__ __forceinline__ const float4* acquire(Ctl* ctl) {
+        const unsigned s = taken % kStages;
+        if (!mbar_wait(&bar[s], (taken / kStages) & 1u, ctl)) return nullptr;
+        return ring + s * kF4;
+    }
+    // Every lane is done reading the tile: its stage can be issued again.
+    __device__ __forceinline__ void release() {
+        __syncwarp();
+        ++taken;
+    }
+    // After an abandoned wait: waits (bounded) for the copies still in flight.
+    __device__ __forceinline__ void drain() {
+        for (; taken != issued; ++taken)
+            for (unsigned i = 0; i < kSpinLimit; ++i)
+                if (mbar_try_wait(&bar[taken % kStages], (taken / kStages) & 1u)) break;
+        __syncwarp();
+    }
+};
+
 }  // namespace ch
