@@ -89,7 +89,8 @@ struct BArgs {
     long long nwt;            // warp tiles of the streamed body
     int head;                 // points before the body's first 16-byte boundary (0 or 1)
     int wtile;                // points per warp tile (32 x points per lane)
-    int fchunk;               // warp tiles that a warp of bt_filter takes at a time
+    int fchunk;               // warp tiles that a warp of bt_filter takes at a time, while
+    unsigned fbig;            // chunk < fbig; one tile each after that
     int* star_slot;           // k: the set's star slot, or -1
     unsigned long long* star_bins;   // kStarBins per slot (zeroed before every batch)
     StarPoly* star_polys;     // one per slot
@@ -97,9 +98,11 @@ struct BArgs {
                               // [2] / [3] sets for bt_star_refine from the front / back, [4] taken;
                               // [5] sets for bt_hull, [6] taken; [7] bt_dense's units, [8] taken;
                               // [9] / [10] sets for bt_queue_chain from the front / back, [11] / [12] queues taken;
-                              // [13] bt_filter's chunks taken; [14] sets for the bucketed path
+                              // [13] bt_filter's chunks taken; [14] sets for the bucketed path;
+                              // [15] points of a bt_dense unit
     int* star_list;           // k entries
     unsigned* unit_base;      // k entries: first bt_dense unit of each listed set
+    int* unit_map;            // the listed set of each unit (k + total / kBDenseRunMin entries at most)
     int* refine_list;         // k entries
     int* hull_list;           // k entries
     int* q_list;              // k entries: sets for bt_queue_chain, the small ones from the front, the large from the back
@@ -476,25 +479,19 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
 constexpr int kBtWarpRecs = 128;
 constexpr int kBtQueue = 64;   // < 32 waiting + 32 added per step
 struct BtWarpSmem {
-    Octagon o;                       // the warp's set's octagon
+    OctEdges e;                      // the edge functions of the warp's set's octagon
+    Octagon o;                       // the octagon
     uint64_t val[kBtWarpRecs];       // records staged
     uint32_t key[kBtWarpRecs];
     float qx[kBtQueue], qy[kBtQueue];   // points waiting for the exact tests
     unsigned qi[kBtQueue];
     Ctl* c;                          // the warp's set: control block, record region,
-    long long rb;
+    long long rb, base;              // first point,
+    int set;                         // its number (-1: none),
+    int skip;                        // empty, failed, or bt_dense's: nothing to classify
+    unsigned qn;                     // points queued,
     unsigned cnt;                    // records staged,
     unsigned nq[4];                  // records per queue
-};
-
-// A warp's current set: what the streaming loop reads stays in registers
-// (warp-uniform); what the classification needs is in the warp's shared
-// memory.
-struct BtWarpSet {
-    int set = -1;
-    long long base = 0;
-    bool skip = true;              // empty, failed, or bt_dense's: nothing to classify
-    unsigned qn = 0u;              // points queued
 };
 
 // The inner region of an octagon as four scaled keys: a point is inside when
@@ -551,7 +548,8 @@ __device__ __noinline__ void bt_classify32(uint32_t* keys, uint64_t* vals, BtWar
     if (valid) {
         X = __float2int_rn(x);
         Y = __float2int_rn(y);
-        r = classify_hull(x, y, so);
+        r = classify_edges(x, y, m.e);
+        if (r == kUndecided) r = classify_hull_slow(x, y, &so);
     }
     bool keep = r >= 0;
     if (!__any_sync(0xFFFFFFFFu, keep)) return;
@@ -579,83 +577,89 @@ __device__ __noinline__ void bt_classify32(uint32_t* keys, uint64_t* vals, BtWar
     __syncwarp();
 }
 
-// Warp-collective: queues the lanes' points with need = true; full rounds of
-// 32 go through bt_classify32.
-__device__ __forceinline__ void bt_queue_push(const BArgs& a, BtWarpSet& w, BtWarpSmem& m, bool need, float x, float y,
+// Warp-collective: queues the lanes' points with need = true, qn of them
+// waiting already; full rounds of 32 go through bt_classify32.
+__device__ __forceinline__ void bt_queue_push(const BArgs& a, unsigned& qn, BtWarpSmem& m, bool need, float x, float y,
                                               unsigned li) {
     const int lane = threadIdx.x & 31;
     const unsigned bal = __ballot_sync(0xFFFFFFFFu, need);
     if (!bal) return;
     if (need) {
-        const unsigned pos = w.qn + (unsigned)__popc(bal & lanemask_lt());
+        const unsigned pos = qn + (unsigned)__popc(bal & lanemask_lt());
         m.qx[pos] = x;
         m.qy[pos] = y;
         m.qi[pos] = li;
     }
-    w.qn += (unsigned)__popc(bal);
+    qn += (unsigned)__popc(bal);
     __syncwarp();
-    while (w.qn >= 32u) {
-        w.qn -= 32u;
-        const float qx = m.qx[w.qn + lane], qy = m.qy[w.qn + lane];
-        const unsigned qi = m.qi[w.qn + lane];
+    if (qn >= 32u) {
+        qn -= 32u;
+        const float qx = m.qx[qn + lane], qy = m.qy[qn + lane];
+        const unsigned qi = m.qi[qn + lane];
         __syncwarp();
         bt_classify32(a.keys, a.vals, m, true, qx, qy, qi);
     }
 }
 
 // Warp-collective: finishes the warp's set (queue, records, queue counts).
-__device__ __forceinline__ void bt_warp_done(const BArgs& a, BtWarpSmem& m, BtWarpSet& w) {
+__device__ __noinline__ void bt_warp_done(const BArgs& a, BtWarpSmem& m) {
     const int lane = threadIdx.x & 31;
-    if (w.set < 0) return;
-    if (w.qn) {
-        const bool valid = (unsigned)lane < w.qn;
+    if (m.set < 0) return;
+    const unsigned qn = m.qn;
+    if (qn) {
+        const bool valid = (unsigned)lane < qn;
         const float qx = valid ? m.qx[lane] : 0.0f, qy = valid ? m.qy[lane] : 0.0f;
         const unsigned qi = valid ? m.qi[lane] : 0u;
         __syncwarp();
-        w.qn = 0u;
         bt_classify32(a.keys, a.vals, m, valid, qx, qy, qi);
     }
     bt_flush_recs(m, a.keys, a.vals);
     if (lane < 4 && m.nq[lane]) atomicAdd(&m.c->counts4[lane], m.nq[lane]);
-    w.set = -1;
+    __syncwarp();
+    if (lane == 0) {
+        m.set = -1;
+        m.qn = 0u;
+    }
+    __syncwarp();
 }
 
 // Warp-collective: makes set q the warp's set (the previous one finished).
-__device__ __forceinline__ void bt_warp_set(const BArgs& a, int q, BtWarpSet& w, BtWarpSmem& m) {
+__device__ __noinline__ void bt_warp_set(const BArgs& a, int q, BtWarpSmem& m) {
     const int lane = threadIdx.x & 31;
-    bt_warp_done(a, m, w);
-    __syncwarp();
+    bt_warp_done(a, m);
     Ctl* c = a.ctl + q;
-    w.set = q;
-    w.base = a.offsets[q];
     // empty and failed sets (bt_octagon's verdict), and the sets with a star
     // polygon, which bt_dense filters
-    w.skip = c->skip != 0;
+    const int skip = c->skip;
     if (lane == 0) {
         m.c = c;
         m.rb = region_base(a, q);
+        m.base = a.offsets[q];
+        m.set = q;
+        m.skip = skip;
         m.cnt = 0u;
     }
     if (lane < 4) m.nq[lane] = 0u;
-    if (!w.skip) {
+    if (!skip) {
         const int* src = reinterpret_cast<const int*>(&c->oct);
         int* dst = reinterpret_cast<int*>(&m.o);
         for (int j = lane; j < (int)(sizeof(Octagon) / 4); j += 32) dst[j] = src[j];
+        m.e.set(c->oct, lane);
     }
     __syncwarp();
 }
 
 // Points [lo, hi) of the batch read from global memory, set by set from the
 // set holding lo (head and tail).
-__device__ void bt_filter_global(const BArgs& a, long long lo, long long hi, BtWarpSet& w, BtWarpSmem& m) {
+__device__ __noinline__ void bt_filter_global(const BArgs& a, long long lo, long long hi, BtWarpSmem& m) {
     const int lane = threadIdx.x & 31;
     if (lo >= hi) return;
     for (int q = bt_find_set(a, lo); q < a.k; ++q) {
         const long long qb = a.offsets[q], qe = a.offsets[q + 1];
         if (qb >= hi) break;
         if (qe <= lo) continue;
-        bt_warp_set(a, q, w, m);
-        if (w.skip) continue;
+        bt_warp_set(a, q, m);
+        if (m.skip) continue;
         const long long e = min(hi, qe);
         for (long long j0 = max(lo, qb); j0 < e; j0 += 32) {
             const long long j = j0 + lane;
@@ -666,44 +670,76 @@ __device__ void bt_filter_global(const BArgs& a, long long lo, long long hi, BtW
     }
 }
 
+// A tile that meets a set boundary (its points from p0 on), set by set from
+// set s on.
+template <int P>
+__device__ __noinline__ void bt_filter_straddle(const BArgs& a, const float2* tile2, long long p0, int s, BtWarpSmem& m) {
+    const int lane = threadIdx.x & 31;
+    constexpr long long kPts = 32ll * P;
+    for (int q = s; q < a.k; ++q) {
+        const long long qb = __ldg(a.offsets + q), qe = __ldg(a.offsets + q + 1);
+        if (qb >= p0 + kPts) break;
+        if (qe <= p0) continue;
+        if (q != m.set) bt_warp_set(a, q, m);
+        if (m.skip) continue;
+        BtInner in;
+        in.set(m.o);
+        unsigned qn = m.qn;
+#pragma unroll 1
+        for (int j = 0; j < P; ++j) {
+            const int f2 = 2 * ((j >> 1) * 32 + lane) + (j & 1);
+            const long long i = p0 + f2;
+            const float2 p = tile2[f2];
+            bt_queue_push(a, qn, m, i >= qb && i < qe && in.outside(p.x, p.y), p.x, p.y, (unsigned)(i - qb));
+        }
+        __syncwarp();
+        if (lane == 0) m.qn = qn;
+        __syncwarp();
+    }
+}
+
 // A warp's place in the batch: its chunk's next tile t (below end), and the set
 // s that holds the tile's first point.
 template <int P>
 struct BtCursor {
     static constexpr long long kPts = 32ll * P;
-    long long t = 0, end = 0;
+    unsigned t = 0u, end = 0u;
     int s = 0;
     bool skip = false;   // of set s
-    // The next tile with a point to classify, in (t, end, s); false when the
-    // batch is done.  Tiles wholly inside a set to skip are passed over.
+    // Moves t to the next tile with a point to classify; false when the batch
+    // is done.  Tiles wholly inside a set to skip are passed over.
     __device__ __forceinline__ bool next(const BArgs& a) {
         const int lane = threadIdx.x & 31;
+        const unsigned nwt = (unsigned)a.nwt;   // below 2^32 (checked on the host)
         for (;;) {
             if (t >= end) {
                 unsigned g = 0u;
                 if (lane == 0) g = atomicAdd(&a.star_ctr[13], 1u);
-                t = (long long)__shfl_sync(0xFFFFFFFFu, g, 0) * a.fchunk;
-                if (t >= a.nwt) return false;
-                end = min(a.nwt, t + a.fchunk);
+                g = __shfl_sync(0xFFFFFFFFu, g, 0);
+                const unsigned big = a.fbig * (unsigned)a.fchunk;
+                if (g >= a.fbig && g - a.fbig >= nwt - big) return false;
+                t = g < a.fbig ? g * (unsigned)a.fchunk : big + (g - a.fbig);
+                end = g < a.fbig ? t + (unsigned)a.fchunk : t + 1u;
                 s = bt_find_set(a, a.head + t * kPts);
                 skip = __ldcg(&a.ctl[s].skip) != 0;
             }
             const long long p0 = a.head + t * kPts;
-            if (__ldg(a.offsets + s + 1) <= p0) {
-                do ++s;
-                while (__ldg(a.offsets + s + 1) <= p0);
+            long long past = __ldg(a.offsets + s + 1);
+            if (past <= p0) {
+                do past = __ldg(a.offsets + ++s + 1);
+                while (past <= p0);
                 skip = __ldcg(&a.ctl[s].skip) != 0;
             }
             if (!skip) return true;
-            const long long past = (__ldg(a.offsets + s + 1) - a.head) / kPts;   // first tile not wholly before the set's end
-            if (past <= t) return true;   // the tile meets the next set
-            t = min(end, past);
+            past = (past - a.head) / kPts;   // the first tile not wholly before the set's end
+            if (past <= (long long)t) return true;   // the tile meets the next set
+            t = (unsigned)min((long long)end, past);
         }
     }
 };
 
 template <int T, int P>
-__global__ void __launch_bounds__(T, T <= 256 ? 2 : 1) bt_filter(BArgs a) {
+__global__ void __launch_bounds__(T, 512 / T) bt_filter(const __grid_constant__ BArgs a) {
     constexpr int kWarps = T / 32, kF4 = 16 * P;
     constexpr long long kPts = 32ll * P;
     static_assert(P <= 32 && kStages == 2, "a mask bit per point of a lane; two tiles in flight");
@@ -712,48 +748,54 @@ __global__ void __launch_bounds__(T, T <= 256 ? 2 : 1) bt_filter(BArgs a) {
     __shared__ BtWarpSmem s_w[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     BtWarpSmem& m = s_w[warp];
-    BtWarpSet w;
-    BtInner in;
-    if (blockIdx.x == 0 && warp == 0) {
-        bt_filter_global(a, 0, a.head, w, m);
-        bt_filter_global(a, a.head + a.nwt * kPts, a.total, w, m);
-        bt_warp_done(a, m, w);
+    if (lane == 0) {
+        m.set = -1;
+        m.qn = 0u;
     }
-    const float4* body = reinterpret_cast<const float4*>(a.pts + 2 * a.head);
+    __syncwarp();
+    if (blockIdx.x == 0 && warp == 0) {
+        bt_filter_global(a, 0, a.head, m);
+        bt_filter_global(a, a.head + a.nwt * kPts, a.total, m);
+    }
     WarpRing<kF4> ring{reinterpret_cast<float4*>(dsm) + warp * kStages * kF4, s_bar[warp], lane};
     ring.init();
+    BtInner in;
+    int inset = -1;               // the set of `in`
     BtCursor<P> cur;              // runs ahead of the tile at hand
-    long long t0 = -1, t1 = -1, e0 = 0, e1 = 0;   // the tiles in flight, their chunks' ends
-    int s0 = 0, s1 = 0;                           // and their first points' sets
-    auto advance = [&](long long& t, long long& e, int& s) {
-        t = -1;
-        if (!cur.next(a)) return;
-        t = cur.t++;
-        e = cur.end;
-        s = cur.s;
-        ring.issue(body + t * kF4);
-    };
-    advance(t0, e0, s0);
-    if (t0 >= 0) advance(t1, e1, s1);
-    while (t0 >= 0) {
+    constexpr unsigned kNone = 0xFFFFFFFFu;
+    unsigned t0 = kNone, t1 = kNone;   // the tiles in flight
+    int s0 = 0, s1 = 0;                // their first points' sets
+    if (cur.next(a)) {
+        t0 = cur.t++;
+        s0 = cur.s;
+        ring.issue(reinterpret_cast<const float4*>(a.pts + 2 * a.head) + (size_t)t0 * kF4);
+    }
+    while (t0 != kNone) {
+        if (t1 == kNone && cur.next(a)) {   // the next tile, while this one is worked on
+            t1 = cur.t++;
+            s1 = cur.s;
+            ring.issue(reinterpret_cast<const float4*>(a.pts + 2 * a.head) + (size_t)t1 * kF4);
+        }
         const float4* tile = ring.acquire(a.ctl + s0);
         if (!tile) {   // a copy never completed: every set of the rest of the chunks in hand fails
             ring.drain();
             for (int f = 0; f < 2; ++f) {
-                const long long t = f ? t1 : t0, pend = a.head + (f ? e1 : e0) * kPts;
-                if (t < 0) continue;
+                const unsigned t = f ? t1 : t0;
+                if (t == kNone) continue;
+                const long long pend = a.head + ((long long)t + a.fchunk) * kPts;
                 for (int q = (f ? s1 : s0) + lane; q < a.k && __ldg(a.offsets + q) < pend; q += 32)
                     set_status(a.ctl + q, CH_ETIMEOUT);
             }
-            if (w.set >= 0 && lane == 0) set_status(a.ctl + w.set, CH_ETIMEOUT);
+            if (m.set >= 0 && lane == 0) set_status(a.ctl + m.set, CH_ETIMEOUT);
             break;
         }
         const long long p0 = a.head + t0 * kPts;
         const float2* tile2 = reinterpret_cast<const float2*>(tile);
         if (__ldg(a.offsets + s0 + 1) >= p0 + kPts) {   // inside set s0
-            if (s0 != w.set) {
-                bt_warp_set(a, s0, w, m);
+            if (s0 != inset) {
+                if (s0 != m.set) bt_warp_set(a, s0, m);
                 in.set(m.o);
+                inset = s0;
             }
             unsigned mask = 0u;   // the lane's points outside the inner region
 #pragma unroll
@@ -762,39 +804,28 @@ __global__ void __launch_bounds__(T, T <= 256 ? 2 : 1) bt_filter(BArgs a) {
                 if (in.outside(v.x, v.y)) mask |= 1u << (2 * j);
                 if (in.outside(v.z, v.w)) mask |= 2u << (2 * j);
             }
-            const unsigned li0 = (unsigned)(p0 - w.base);
-            while (__any_sync(0xFFFFFFFFu, mask != 0u)) {   // a point per lane and step
-                const int b = __ffs((int)mask) - 1, f2 = 64 * (b >> 1) + 2 * lane + (b & 1);
-                const float2 p = mask ? tile2[f2] : make_float2(0.0f, 0.0f);
-                bt_queue_push(a, w, m, mask != 0u, p.x, p.y, li0 + (unsigned)f2);
-                mask &= mask - 1u;
+            if (__any_sync(0xFFFFFFFFu, mask != 0u)) {
+                const unsigned li0 = (unsigned)(p0 - m.base);
+                unsigned qn = m.qn;
+                do {   // a point per lane and step
+                    const int b = __ffs((int)mask) - 1, f2 = 64 * (b >> 1) + 2 * lane + (b & 1);
+                    const float2 p = mask ? tile2[f2] : make_float2(0.0f, 0.0f);
+                    bt_queue_push(a, qn, m, mask != 0u, p.x, p.y, li0 + (unsigned)f2);
+                    mask &= mask - 1u;
+                } while (__any_sync(0xFFFFFFFFu, mask != 0u));
+                if (lane == 0) m.qn = qn;
+                __syncwarp();
             }
-        } else {   // the tile meets a set boundary: set by set
-            for (int q = s0; q < a.k; ++q) {
-                const long long qb = __ldg(a.offsets + q), qe = __ldg(a.offsets + q + 1);
-                if (qb >= p0 + kPts) break;
-                if (qe <= p0) continue;
-                if (q != w.set) {
-                    bt_warp_set(a, q, w, m);
-                    in.set(m.o);
-                }
-                if (w.skip) continue;
-#pragma unroll 1
-                for (int j = 0; j < P; ++j) {
-                    const long long i = p0 + 2 * ((j >> 1) * 32 + lane) + (j & 1);
-                    const float2 p = tile2[2 * ((j >> 1) * 32 + lane) + (j & 1)];
-                    const bool mine = i >= qb && i < qe;
-                    bt_queue_push(a, w, m, mine && in.outside(p.x, p.y), p.x, p.y, (unsigned)(i - qb));
-                }
-            }
+        } else {
+            bt_filter_straddle<P>(a, tile2, p0, s0, m);
+            inset = -1;
         }
         ring.release();
         t0 = t1;
-        e0 = e1;
         s0 = s1;
-        if (t0 >= 0) advance(t1, e1, s1);
+        t1 = kNone;
     }
-    bt_warp_done(a, m, w);
+    bt_warp_done(a, m);
 }
 
 // ---------------------------------------------------------------------------
@@ -877,7 +908,9 @@ constexpr size_t kBStarAOff = (sizeof(StarPoly) + 15) / 16 * 16;
 constexpr size_t kBStarSmem = kBStarAOff + sizeof(unsigned long long) * kStarBins;
 static_assert(sizeof(StarPoly) % 16 == 0, "the polygon is copied in 16-byte words");
 
-__global__ void __launch_bounds__(kBStarThreads, 1) bt_star_build(BArgs a) {
+constexpr int kBStarBuildThreads = 1024;
+
+__global__ void __launch_bounds__(kBStarBuildThreads, 1) bt_star_build(BArgs a) {
     extern __shared__ __align__(16) char dyn[];
     StarPoly& P = *reinterpret_cast<StarPoly*>(dyn);
     unsigned long long* work = reinterpret_cast<unsigned long long*>(dyn + kBStarAOff);
@@ -895,12 +928,12 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_build(BArgs a) {
         Ctl* c = a.ctl + i;
         const long long base = a.offsets[i], ni = a.offsets[i + 1] - base;
         const int slot = a.star_slot[i];
-        const int K = star_finish<kBStarThreads>(a.star_bins + (size_t)slot * kStarBins, a.pts + 2 * base, ni,
+        const int K = star_finish<kBStarBuildThreads>(a.star_bins + (size_t)slot * kStarBins, a.pts + 2 * base, ni,
                                                  c->star_cx, c->star_cy, work, P, c);
         if (K) {
             const int4* src = reinterpret_cast<const int4*>(&P);
             int4* dst = reinterpret_cast<int4*>(a.star_polys + slot);
-            for (int j = tid; j < (int)(sizeof(StarPoly) / 16); j += kBStarThreads) dst[j] = src[j];
+            for (int j = tid; j < (int)(sizeof(StarPoly) / 16); j += kBStarBuildThreads) dst[j] = src[j];
         }
         if (tid == 0) {
             c->star_k = K;
@@ -913,7 +946,7 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_build(BArgs a) {
 // ---------------------------------------------------------------------------
 // The filter of the sets with a star polygon (bt_star_build's), which
 // bt_filter leaves to this kernel: the single hull's dense post pass per
-// set.  Work units are runs of up to kBDenseRun points of a set
+// set.  Work units are runs of a set's points
 // (bt_dense_plan numbers them); a block takes units one at a time, copies the
 // set's radius bounds and octagon into shared memory, and streams the run's
 // points through its warps' rings: a point closer to the centre than its
@@ -924,8 +957,8 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_build(BArgs a) {
 // atomic per batch.  (With 64-bit distances and a ballot per 32 points it
 // executed 92 warp instructions per 32 points, ncu, and took 0.80 ms on the
 // 4096-set batch.)
-constexpr int kBDenseThreads = 1024;
-constexpr int kBDenseRun = 1 << 18;    // points of a work unit
+constexpr int kBDenseThreads = 768;    // 80 registers: 1024 threads spill, and the small L1 that is left misses
+constexpr int kBDenseRunMin = 1 << 14, kBDenseRunMax = 1 << 18;   // points of a work unit
 constexpr int kBDenseF4 = 128;         // float4 of a warp's ring tile
 constexpr int kBDenseRecs = 64;        // records staged per warp
 constexpr int kBDenseQueue = 64;       // < 32 waiting + 32 added per step
@@ -941,20 +974,37 @@ constexpr size_t kBDenseRingOff = (kBDenseWarpOff + (kBDenseThreads / 32) * size
 constexpr size_t kBDenseSmem = kBDenseRingOff + (size_t)(kBDenseThreads / 32) * kStages * kBDenseF4 * sizeof(float4);
 static_assert(kBDenseSmem <= 225 * 1024, "one block's shared memory");
 
-// Work units of the sets with a polygon: unit_base[j] = first unit of listed
-// set j (one block of 1024 threads; star_ctr[7] = total units).
-__global__ void __launch_bounds__(1024) bt_dense_plan(BArgs a) {
+// Work units of the sets with a polygon: runs of star_ctr[15] points, about four
+// units per block of bt_dense while they stay within kBDenseRunMin and
+// kBDenseRunMax (a few sets' points are spread over all blocks; a unit's
+// radius bounds are 32 KB against 2 MB of points at most).  unit_base[j] = first
+// unit of listed set j, unit_map the other way round (one block of 1024
+// threads; star_ctr[7] = total units).
+__global__ void __launch_bounds__(1024) bt_dense_plan(BArgs a, int blocks) {
     __shared__ unsigned s_part[1024];
+    __shared__ unsigned long long s_pts;
     const int tid = threadIdx.x;
     const int n = (int)a.star_ctr[0];
     const int per = (n + 1023) / 1024;
     const int lo = tid * per, hi = min(n, lo + per);
-    unsigned sum = 0u;
+    unsigned long long mine = 0ull;
+    if (tid == 0) s_pts = 0ull;
+    __syncthreads();
     for (int j = lo; j < hi; ++j) {
         const int i = a.star_list[j];
-        const long long ni = a.offsets[i + 1] - a.offsets[i];
-        sum += a.ctl[i].star_k > 0 ? (unsigned)((ni + kBDenseRun - 1) / kBDenseRun) : 0u;
+        if (a.ctl[i].star_k > 0) mine += (unsigned long long)(a.offsets[i + 1] - a.offsets[i]);
     }
+    if (mine) atomicAdd(&s_pts, mine);
+    __syncthreads();
+    const long long run_pts = max((long long)kBDenseRunMin,
+                                  min((long long)kBDenseRunMax, (long long)(s_pts / (4ull * (unsigned)blocks)) + 1));
+    if (tid == 0) a.star_ctr[15] = (unsigned)run_pts;
+    auto units_of = [&](int i) {
+        const long long ni = a.offsets[i + 1] - a.offsets[i];
+        return a.ctl[i].star_k > 0 ? (unsigned)((ni + run_pts - 1) / run_pts) : 0u;
+    };
+    unsigned sum = 0u;
+    for (int j = lo; j < hi; ++j) sum += units_of(a.star_list[j]);
     s_part[tid] = sum;
     __syncthreads();
     for (int o = 1; o < 1024; o <<= 1) {
@@ -965,10 +1015,10 @@ __global__ void __launch_bounds__(1024) bt_dense_plan(BArgs a) {
     }
     unsigned run = s_part[tid] - sum;
     for (int j = lo; j < hi; ++j) {
-        const int i = a.star_list[j];
-        const long long ni = a.offsets[i + 1] - a.offsets[i];
+        const unsigned units = units_of(a.star_list[j]);
         a.unit_base[j] = run;
-        run += a.ctl[i].star_k > 0 ? (unsigned)((ni + kBDenseRun - 1) / kBDenseRun) : 0u;
+        for (unsigned u = 0u; u < units; ++u) a.unit_map[run + u] = j;
+        run += units;
     }
     if (tid == 1023) a.star_ctr[7] = s_part[1023];
 }
@@ -979,7 +1029,10 @@ struct BtDenseSet {
     uint32_t* keys;       // the set's record region
     uint64_t* vals;
     const StarPoly* P;
+    const float2* pts;    // the run: the set's points lo .. hi - 1
+    int lo, hi;
     int cx, cy;
+    OctEdges e;
     Octagon o;
 };
 
@@ -1005,7 +1058,12 @@ __device__ __noinline__ void bt_dense_drain(const BtDenseSet& m, BtDenseWarp& wb
     const unsigned li = valid ? wb.qi[first + lane] : 0u;
     const int X = __float2int_rn(p.x), Y = __float2int_rn(p.y);
     int r = -1;
-    if (valid && !star_inside_exact(X - cx, Y - cy, star_bin(X - cx, Y - cy), *m.P)) r = classify_hull(p.x, p.y, so);
+    if (valid && !star_inside_exact(X - cx, Y - cy, star_bin(X - cx, Y - cy), *m.P)) {
+        // outside the polygon, hence nearly always outside the octagon: its
+        // queue alone (a point kept inside the octagon is one record more)
+        r = classify_quad(p.x, p.y, m.e);
+        if (r == kUndecided) r = classify_hull_slow(p.x, p.y, &so);
+    }
     bool keep = r >= 0;
     if (!__any_sync(0xFFFFFFFFu, keep)) return;
     if (reduce_on_line(so, keep, X, Y, li, m.c)) keep = false;
@@ -1035,7 +1093,7 @@ __device__ __noinline__ void bt_dense_drain(const BtDenseSet& m, BtDenseWarp& wb
     __syncwarp();
 }
 
-__global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
+__global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(const __grid_constant__ BArgs a) {
     extern __shared__ __align__(128) char dyn[];
     __shared__ unsigned long long s_bar[kBDenseThreads / 32][kStages];
     float* thr = reinterpret_cast<float*>(dyn);
@@ -1045,61 +1103,61 @@ __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
     BtDenseWarp& wb = reinterpret_cast<BtDenseWarp*>(dyn + kBDenseWarpOff)[warp];
     WarpRing<kBDenseF4> ring{reinterpret_cast<float4*>(dyn + kBDenseRingOff) + warp * kStages * kBDenseF4, s_bar[warp], lane};
     ring.init();
-    __shared__ int s_set, s_part;
+    // the block's unit (set, part) and, fetched meanwhile, its next one
+    __shared__ int s_set[2], s_part[2];
     const unsigned nunits = a.star_ctr[7];
-    const int listed = (int)a.star_ctr[0];
-    for (;;) {
-        if (tid == 0) {
-            const unsigned u = atomicAdd(&a.star_ctr[8], 1u);
-            int set = -1, part = 0;
-            if (u < nunits) {   // the last listed set whose first unit is at or before u
-                int l = 0, r = listed;
-                while (r - l > 1) {
-                    const int mid = (l + r) >> 1;
-                    if (a.unit_base[mid] <= u) l = mid;
-                    else r = mid;
-                }
-                set = a.star_list[l];
-                part = (int)(u - a.unit_base[l]);
-            }
-            s_set = set;
-            s_part = part;
+    auto fetch = [&](unsigned u, int slot) {
+        int set = -1, part = 0;
+        if (u < nunits) {
+            const int l = a.unit_map[u];
+            set = a.star_list[l];
+            part = (int)(u - a.unit_base[l]);
         }
+        s_set[slot] = set;
+        s_part[slot] = part;
+    };
+    if (tid == 0) fetch(blockIdx.x, 0);
+    for (int turn = 0;; turn ^= 1) {
         __syncthreads();
-        const int i = s_set;
+        const int i = s_set[turn];
         if (i < 0) return;
-        Ctl* c = a.ctl + i;
-        const long long base = a.offsets[i], ni = a.offsets[i + 1] - base;
-        const long long rb = region_base(a, i);
-        const long long lo = (long long)s_part * kBDenseRun, hi = min(ni, lo + kBDenseRun);
-        const StarPoly& P = a.star_polys[a.star_slot[i]];
-        for (int j = tid; j < kStarBins / 4; j += kBDenseThreads)
-            reinterpret_cast<float4*>(thr)[j] = __ldcg(reinterpret_cast<const float4*>(P.thr) + j);
-        copy_octagon(&m.o, &c->oct);
-        if (tid == 0) {
-            m.c = c;
-            m.keys = a.keys + rb;
-            m.vals = a.vals + rb;
-            m.P = &P;
-            m.cx = c->star_cx;
-            m.cy = c->star_cy;
+        if (tid == kBDenseThreads - 1) fetch(gridDim.x + atomicAdd(&a.star_ctr[8], 1u), turn ^ 1);
+        {
+            Ctl* c = a.ctl + i;
+            const StarPoly& P = a.star_polys[a.star_slot[i]];
+            for (int j = tid; j < kStarBins / 4; j += kBDenseThreads)
+                reinterpret_cast<float4*>(thr)[j] = __ldcg(reinterpret_cast<const float4*>(P.thr) + j);
+            copy_octagon(&m.o, &c->oct);
+            m.e.set(c->oct, tid);
+            if (tid == 0) {
+                const long long base = a.offsets[i], rb = region_base(a, i);
+                const int run = (int)a.star_ctr[15], lo = s_part[turn] * run;   // set sizes are below 2^31
+                m.c = c;
+                m.keys = a.keys + rb;
+                m.vals = a.vals + rb;
+                m.P = &P;
+                m.pts = reinterpret_cast<const float2*>(a.pts) + base;
+                m.lo = lo;
+                m.hi = (int)min(a.offsets[i + 1] - base, (long long)lo + run);
+                m.cx = c->star_cx;
+                m.cy = c->star_cy;
+            }
+            if (lane == 0) wb.cnt = 0u;
+            if (lane < 4) wb.nq[lane] = 0u;
         }
-        if (lane == 0) wb.cnt = 0u;
-        if (lane < 4) wb.nq[lane] = 0u;
-        const float fcx = (float)c->star_cx, fcy = (float)c->star_cy;
-        const float2* p2 = reinterpret_cast<const float2*>(a.pts) + base;
-        // the 16-byte aligned body of the run in tiles of kPts points
-        const int odd = (reinterpret_cast<uintptr_t>(p2 + lo) & 15u) != 0u ? 1 : 0;
-        const float4* body = reinterpret_cast<const float4*>(p2 + lo + odd);
-        const int nt = (int)((hi - lo - odd) / kPts);
-        for (int t = warp; t < nt && t < kStages * kWarps; t += kWarps) ring.issue(body + (size_t)t * kBDenseF4);
         __syncthreads();
+        const float fcx = (float)m.cx, fcy = (float)m.cy;
+        // the 16-byte aligned body of the run in tiles of kPts points
+        const int odd = (reinterpret_cast<uintptr_t>(m.pts + m.lo) & 15u) != 0u ? 1 : 0;
+        const float4* body = reinterpret_cast<const float4*>(m.pts + m.lo + odd);
+        const int nt = (m.hi - m.lo - odd) / kPts;
+        for (int t = warp; t < nt && t < kStages * kWarps; t += kWarps) ring.issue(body + (size_t)t * kBDenseF4);
         unsigned qn = 0u;
         for (int t = warp; t < nt; t += kWarps) {
-            const float4* cur = ring.acquire(c);
+            const float4* cur = ring.acquire(m.c);
             if (!cur) {   // a copy never completed: the set fails
                 ring.drain();
-                if (lane == 0) set_status(c, CH_ETIMEOUT);
+                if (lane == 0) set_status(m.c, CH_ETIMEOUT);
                 break;
             }
             unsigned mask = 0u;   // the lane's points that the radius bounds leave
@@ -1119,7 +1177,7 @@ __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
                     mask &= mask - 1u;
                     const unsigned pos = qn + (unsigned)__popc(bal & lanemask_lt());
                     wb.q[pos] = cur2[f2];
-                    wb.qi[pos] = (unsigned)(lo + odd) + (unsigned)(t * kPts + f2);
+                    wb.qi[pos] = (unsigned)(m.lo + odd + t * kPts + f2);
                 }
                 qn += (unsigned)__popc(bal);
                 __syncwarp();
@@ -1134,21 +1192,20 @@ __global__ void __launch_bounds__(kBDenseThreads, 1) bt_dense(BArgs a) {
         }
         if (qn) bt_dense_drain(m, wb, 0u, qn);
         // the point before the body, and the ragged end by 32 points per warp
-        const long long tail = lo + odd + (long long)nt * kPts + 32 * (kWarps - 1 - warp);
-        const long long ranges[2][2] = {{lo, warp == 0 ? lo + odd : lo}, {tail, min(hi, tail + 32)}};
         for (int rg = 0; rg < 2; ++rg) {
-            const long long cnt = ranges[rg][1] - ranges[rg][0];
+            const long long from = rg ? (long long)m.lo + odd + nt * kPts + 32 * (kWarps - 1 - warp) : m.lo;
+            const int cnt = rg ? (int)min(m.hi - from, 32ll) : (warp == 0 ? odd : 0);
             if (cnt <= 0) continue;
             __syncwarp();
             if (lane < cnt) {
-                wb.q[lane] = __ldcs(p2 + ranges[rg][0] + lane);
-                wb.qi[lane] = (unsigned)(ranges[rg][0] + lane);
+                wb.q[lane] = __ldcs(m.pts + from + lane);
+                wb.qi[lane] = (unsigned)(from + lane);
             }
             __syncwarp();
             bt_dense_drain(m, wb, 0u, (unsigned)cnt);
         }
         if (wb.cnt) bt_dense_flush(m, wb, wb.cnt);
-        if (lane < 4 && wb.nq[lane]) atomicAdd(&c->counts4[lane], wb.nq[lane]);
+        if (lane < 4 && wb.nq[lane]) atomicAdd(&m.c->counts4[lane], wb.nq[lane]);
         __syncthreads();   // the bounds' shared memory is reloaded by the next unit
     }
 }
@@ -1485,7 +1542,7 @@ __global__ void __launch_bounds__(kBHullThreads, 1) bt_hull(BArgs a) {
 // hull vertices) both shapes take 0.50 ms together; the bucketed path took
 // 3.4 ms (bucket chains 1.0, merges 2.1) after a second polygon (0.45 ms)
 // that the sets no longer need.
-constexpr int kBQGather = 4;   // records per thread in flight
+constexpr int kBQGather = 8;   // records per thread in flight
 
 template <class Q, int T, bool kLarge>
 __global__ void __launch_bounds__(T) bt_queue_chain(BArgs a) {
@@ -1615,7 +1672,7 @@ static std::map<std::pair<int, cudaStream_t>, BWork> g_bws;
 static size_t bt_align(size_t x) { return (x + 255) / 256 * 256; }
 
 struct BLayout {
-    size_t ctl, keys, vals, rmap, big, redo, star_ctr, star_list, refine_list, hull_list, q_list, unit_base, star_slot, star_bins, star_polys;
+    size_t ctl, keys, vals, rmap, big, redo, star_ctr, star_list, refine_list, hull_list, q_list, unit_base, unit_map, star_slot, star_bins, star_polys;
     size_t seg_nb, seg_bbase, seg_lo, seg_scale, seg_tbase, rt_base, totals;
     size_t bcount, bcur, bstart, blen, bu, bv, bi, kP, vP, cu, cv, ci, clen, ctmap, counters;
     size_t zero_from, zero_to;   // star bins and bucket counters: cleared before each batch
@@ -1647,6 +1704,7 @@ static BLayout bt_layout(long long total, int k, long long big_pts, long long bi
     L.redo = take((size_t)k);
     L.star_ctr = take(4 * 16);
     L.unit_base = take(sizeof(unsigned) * (size_t)k);
+    L.unit_map = take(sizeof(int) * ((size_t)k + (size_t)(total / kBDenseRunMin)));
     L.refine_list = take(sizeof(int) * (size_t)k);
     L.hull_list = take(sizeof(int) * (size_t)k);
     L.q_list = take(sizeof(int) * (size_t)k);
@@ -1951,13 +2009,16 @@ static int bt_enqueue_tiles(const BtCall& c, cudaStream_t s) {
     }
     { ProfScope p("batched_octagon", s); bt_octagon<<<a.k, kBOctThreads, 0, s>>>(a); }
     {
-        ProfScope p("batched_star", s);
+        ProfScope p("batched_star_bin", s);
         bt_star_bin<<<c.sms * 3, kBStarBinThreads, kBStarBinSmem, s>>>(a);
-        bt_star_build<<<c.sms, kBStarThreads, kBStarSmem, s>>>(a);
+    }
+    {
+        ProfScope p("batched_star", s);
+        bt_star_build<<<c.sms, kBStarBuildThreads, kBStarSmem, s>>>(a);
     }
     {
         ProfScope p("batched_dense", s);
-        bt_dense_plan<<<1, 1024, 0, s>>>(a);
+        bt_dense_plan<<<1, 1024, 0, s>>>(a, c.sms);
         bt_dense<<<c.sms, kBDenseThreads, kBDenseSmem, s>>>(a);
     }
     {
@@ -2058,7 +2119,11 @@ static void bt_set_shape(BtCall& c, const BtDevice& d, int shape) {
     c.a.wtile = 32 * sh.per;
     c.a.nwt = (c.a.total - c.a.head) / c.a.wtile;
     const long long warps = (long long)d.sms * d.occ[shape][1] * (sh.threads / 32);
-    c.a.fchunk = (int)std::max(1ll, std::min(16ll, c.a.nwt / (8 * warps)));   // at least 8 chunks a warp
+    // at least 8 chunks a warp; the last eighth of the batch tile by tile, so
+    // that no warp ends long after the others (a tile of a small dense set
+    // takes 20 times as long as a sparse one's)
+    c.a.fchunk = (int)std::max(1ll, std::min(16ll, c.a.nwt / (8 * warps)));
+    c.a.fbig = (unsigned)((c.a.nwt - c.a.nwt / 8) / c.a.fchunk);
     c.grid_e = (int)std::max(1ll, std::min(c.a.nwt, (long long)d.sms * d.occ[shape][0]));
     c.grid_f = (int)std::max(1ll, std::min(c.a.nwt, (long long)d.sms * d.occ[shape][1]));
 }
@@ -2208,6 +2273,7 @@ int hull_batched_impl(const float* pts, const int64_t* offsets, int32_t k, int32
     a.hull_list = (int*)(base + L.hull_list);
     a.q_list = (int*)(base + L.q_list);
     a.unit_base = (unsigned*)(base + L.unit_base);
+    a.unit_map = (int*)(base + L.unit_map);
     a.kP = (uint32_t*)(base + L.kP);
     a.vP = (uint64_t*)(base + L.vP);
     BLArgs& b = c.b;

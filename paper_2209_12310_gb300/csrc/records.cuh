@@ -47,6 +47,43 @@ __device__ __forceinline__ int classify_hull_fast(float x, float y, int X, int Y
     return in_inner(o, X, Y) ? -1 : sure ? r : kUndecided;
 }
 
+// An octagon's edge functions as float4 (A, B, C, -), for warps that classify
+// a point per lane: one 16-byte read per edge.
+struct alignas(16) OctEdges {
+    float4 oct[8], quad[4];
+    int discard_none;
+    int pad[3];
+    // threads 0 .. 12 fill it
+    __device__ __forceinline__ void set(const Octagon& o, int t) {
+        if (t < 8) oct[t] = make_float4(o.oct[t].A, o.oct[t].B, o.oct[t].C, 0.0f);
+        else if (t < 12) quad[t - 8] = make_float4(o.quad[t - 8].A, o.quad[t - 8].B, o.quad[t - 8].C, 0.0f);
+        else if (t == 12) discard_none = o.discard_none;
+    }
+};
+
+// The queue of a point known to be kept: the first quad edge it is surely right
+// of while surely left of those before; kUndecided when the float error bound
+// leaves that open (or it is right of none).
+__device__ __forceinline__ int classify_quad(float x, float y, const OctEdges& e) {
+    int r = kUndecided;
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+        const float v = fmaf(e.quad[k].x, x, fmaf(e.quad[k].y, y, e.quad[k].z));
+        r = v < -kEdgeTol ? k : v <= kEdgeTol ? (int)kUndecided : r;
+    }
+    return r;
+}
+
+// Hull rule from the edge functions: -1 when surely in the octagon, a queue when
+// surely outside it, else kUndecided (classify_hull_slow decides).
+__device__ __forceinline__ int classify_edges(float x, float y, const OctEdges& e) {
+    float m = kHugePositive;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m = fminf(m, fmaf(e.oct[k].x, x, fmaf(e.oct[k].y, y, e.oct[k].z)));
+    if (e.discard_none) return classify_quad(x, y, e);
+    return m > kEdgeTol ? -1 : m < -kEdgeTol ? classify_quad(x, y, e) : kUndecided;
+}
+
 // Records per queue, counted per lane: an 8-bit field per queue in `packed`,
 // folded into the 32-bit counts before any field can reach 256 (every 255
 // add() calls at most).
