@@ -459,14 +459,30 @@ int ch_filter(const float* pts, int64_t n, int32_t* out_ext8, uint8_t* out_label
     const long long ntiles = (n - head) / kWarpTilePts;
     uint32_t* kA = (uint32_t*)(base + L.off_kA);
     uint64_t* vA = (uint64_t*)(base + L.off_vA);
-    { ProfScope p("init", s); launch_init(ctl, 1, s); }
+    uint32_t* kB = (uint32_t*)(base + L.off_kB);
+    uint64_t* vB = (uint64_t*)(base + L.off_vB);
+    const bool lab = out_labels || out_counts4;
+    // One read of the points that labels those of a region inside a sample's
+    // octagon at once and leaves the others for labels_kernel; inputs that stay
+    // in L2, or want no labels: the extremes first.
+    const bool fused = lab && n > kFilterTwoPassMax;
+    const unsigned switch_at = fused ? (unsigned)(n >> 5) : 0xFFFFFFFFu;
+    if (fused) {
+        ProfScope p("sample", s);
+        const int grid = (int)std::min<long long>(256, (sample_tiles_host(ntiles) + 7) / 8);
+        launch_sample(pts, n, head, ntiles, ctl, switch_at, grid, s, 1);
+    } else {
+        ProfScope p("init", s);
+        launch_init(ctl, 1, s);
+    }
     {
         ProfScope p("main_filter", s);
-        launch_main(pts, n, head, ntiles, ctl, nullptr, nullptr, 0xFFFFFFFFu, kA, vA, 0, di.sms * di.occ_main, s);
+        launch_main_labels(pts, n, head, ntiles, ctl, vB, kB, switch_at, kA, vA, lab && !fused, out_labels,
+                           di.sms * di.occ_main, s);
     }
-    if (out_labels || out_counts4) {
+    if (lab) {
         ProfScope p("labels", s);
-        launch_labels(pts, n, ctl, out_labels, di.sms * di.occ_lab, s);
+        launch_labels(pts, n, head, ntiles, ctl, vB, kB, out_labels, di.sms * di.occ_lab, s);
     }
     launch_filter_output(ctl, n, out_ext8, out_counts4, s);
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ECUDA;

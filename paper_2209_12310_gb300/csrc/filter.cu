@@ -1,8 +1,8 @@
 // filter.cu -- the filtering stage of GPU heaphull (Alg. 2, GPUfilter) on sm_103a.
 //
 // Kernels (in launch order):
-//   init_kernel     reset the per-call control block (ch_filter; ch_hull's sample
-//                   pass does it).
+//   init_kernel     reset the per-call control block (calls with two reads; the
+//                   sample pass does it itself).
 //   sample_kernel   extremes of an evenly spaced sample of warp tiles; its last
 //                   block builds the sample octagon (vertices are input points).
 //   main_kernel     findExtremes (Alg. 2; Sec. 3) over every point: all 8
@@ -23,7 +23,11 @@
 //                   validates the coordinates and drops the points strictly
 //                   inside the polygon; the extremes are among the others.
 //   (post.cu)       the classification of the survivors and the hull.
-//   labels_kernel   ch_filter: the label array Q of Alg. 2 (paper rule).
+//   labels_kernel   ch_filter: the label array Q of Alg. 2 (paper rule).  On
+//                   large inputs the main pass has set it to 0 and left the
+//                   points that may have another label, as in fused mode: one
+//                   read of the points instead of two (1e8 normal points: 183 us
+//                   a call against 288; 1.7 GB of needed traffic became 0.9).
 #include "ch_internal.cuh"
 #include "hullcore.cuh"
 #include "launch.h"
@@ -31,6 +35,8 @@
 #include "octagon.cuh"
 #include "star.cuh"
 #include "tma.cuh"
+
+#include "labels.cuh"
 
 #include <climits>
 
@@ -128,10 +134,58 @@ struct DenseProbe {
         __syncthreads();
         return (long long)s_out * n > (long long)kDensePts * switch_at;
     }
+    // ch_filter's region, in o.in_lo / o.in_hi: o's inner region, shrunk about its
+    // centre to the largest scale of a probed point, so that about one point in
+    // 2000 lies outside it and the octagon of the true extremes nearly always
+    // contains it (checked by the main pass: finalize_block).  With one in 100
+    // outside, the main pass took 178 us instead of 159 on 1e8 points and the
+    // survivors' labels 18 instead of 12.  False when too many points lie
+    // outside for one pass (more than switch_at of n).
+    __device__ __forceinline__ bool label_region(Octagon& o, long long n, unsigned switch_at) const {
+        __shared__ int s_t, s_b[8];
+        __shared__ unsigned s_far;
+        if (threadIdx.x == 0) {
+            s_t = 0;
+            s_far = 0u;
+        }
+        __syncthreads();
+        const int lo0[4] = {o.vx[W], o.vy[S], o.vx[SW] + o.vy[SW], o.vx[NW] - o.vy[NW] + kCoordLimit};
+        const int hi0[4] = {o.vx[E], o.vy[N], o.vx[NE] + o.vy[NE], o.vx[SE] - o.vy[SE] + kCoordLimit};
+        const float cx = (float)((lo0[0] + hi0[0]) / 2), cy = (float)((lo0[1] + hi0[1]) / 2);
+        const float c[4] = {cx, cy, cx + cy, cx - cy + (float)kCoordLimit};
+        float m = 0.0f;
+#pragma unroll
+        for (int j = 0; j < kDensePts / 256; ++j) {
+            const float f[4] = {p[j].x, p[j].y, p[j].x + p[j].y, p[j].x - p[j].y + (float)kCoordLimit};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                m = fmaxf(m, (f[k] - c[k]) / (f[k] > c[k] ? (float)hi0[k] - c[k] : (float)lo0[k] - c[k]));
+        }
+        const int t = __reduce_max_sync(0xFFFFFFFFu, (int)ceilf(1024.0f * fminf(m, 1.0f)));
+        if ((threadIdx.x & 31) == 0) atomicMax(&s_t, t);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int lo[4], hi[4];
+            inner_bounds(lo0, hi0, s_t, lo, hi);
+            for (int k = 0; k < 4; ++k) {
+                o.in_lo[k] = s_b[k] = max(lo[k], o.in_lo[k]);
+                o.in_hi[k] = s_b[4 + k] = min(hi[k], o.in_hi[k]);
+            }
+        }
+        __syncthreads();
+        unsigned far = 0u;
+#pragma unroll
+        for (int j = 0; j < kDensePts / 256; ++j)
+            far += pt_in_inner(__float2int_rn(p[j].x), __float2int_rn(p[j].y), s_b) ? 0u : 1u;
+        far = __reduce_add_sync(0xFFFFFFFFu, far);
+        if ((threadIdx.x & 31) == 0 && far) atomicAdd(&s_far, far);
+        __syncthreads();
+        return (long long)s_far * n <= (long long)kDensePts * switch_at;
+    }
 };
 
 __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ pts, long long n, int head,
-                                                     long long ntiles, Ctl* ctl, unsigned switch_at) {
+                                                     long long ntiles, Ctl* ctl, unsigned switch_at, int labels) {
     __shared__ unsigned long long s_red[8][8];
     __shared__ Octagon s_o;
     __shared__ int s_last;
@@ -221,6 +275,14 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ p
 
     if (s_o.discard_none) {
         if (threadIdx.x == 0) ctl->mode = 1;
+        return;
+    }
+    if (labels) {   // ch_filter
+        if (!test || !probe.label_region(s_o, n, switch_at)) {
+            if (threadIdx.x == 0) ctl->mode = 1;
+            return;
+        }
+        copy_octagon(&ctl->oct_s, &s_o);
         return;
     }
     copy_octagon(&ctl->oct_s, &s_o);
@@ -334,7 +396,7 @@ __device__ __forceinline__ unsigned emit_raw(unsigned keep, Get get, RawBuf& b, 
 // raw survivors of the fused pass lie outside the sample octagon's inner
 // region, so for them it would almost never apply.
 __device__ __noinline__ void finalize_block(const float* __restrict__ pts, long long n, int head, Ctl* ctl,
-                                            Octagon& s_o, uint32_t* keys, uint64_t* vals) {
+                                            Octagon& s_o, uint32_t* keys, uint64_t* vals, bool labels) {
     __shared__ unsigned long long s_ext[8];
     __shared__ int s_G[8];
     __shared__ long long s_lo[8], s_hi[8];
@@ -393,6 +455,15 @@ __device__ __noinline__ void finalize_block(const float* __restrict__ pts, long 
     }
     __syncthreads();
     CH_TRACE_MARK();
+    if (labels && threadIdx.x < 64 && *(volatile int*)&ctl->mode == 0) {
+        // ch_filter: the region whose points the pass has labelled 0 has to lie
+        // in the octagon (each corner left of each edge); else, all points anew
+        const int k = threadIdx.x >> 3, a = threadIdx.x & 7, b = (a + 1) & 7;
+        long long px, py;
+        inner_corner(ctl->oct_s.in_lo, ctl->oct_s.in_hi, k, px, py);
+        if (orient64(s_vx[a], s_vy[a], s_vx[b], s_vy[b], px, py) < 0) atomicExch(&ctl->mode, 1);
+    }
+    __syncthreads();
     setup_octagon_block(s_o, s_vx, s_vy, s_id, *(volatile int*)&ctl->mode != 0);
     CH_TRACE_MARK();
     if (threadIdx.x < 12) {
@@ -430,10 +501,15 @@ __device__ __noinline__ void finalize_block(const float* __restrict__ pts, long 
 
 constexpr size_t kMainSmemBytes = (size_t)8 * kStages * kWarpTileF4 * sizeof(float4);
 
+// With kLabels (ch_filter): the raw survivors are the points not strictly inside
+// the region of the sample pass (oct_s's inner bounds), and every label is set
+// to 0 beside them, 16 bytes a store; labels_kernel sets the survivors' ones.
+// two_pass: leave the points in L2 for a second pass.
+template <bool kLabels>
 __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ pts, long long n, int head,
                                                       long long ntiles, Ctl* ctl, uint64_t* raw_xy,
                                                       uint32_t* raw_idx, unsigned switch_at, uint32_t* keys,
-                                                      uint64_t* vals, int two_pass) {
+                                                      uint64_t* vals, int two_pass, uint8_t* labels) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ int s_inner[8];
     __shared__ float s_edge[24];
@@ -478,7 +554,7 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
                 convert_pt(x, y, X, Y, tr);
                 tile_keys2(tk, X, Y, X, Y, !any);
                 any = true;
-                if (filt && !pt_in_inner(X, Y, s_inner) && !pt_in_sample(x, y, s_edge)) keep = 1u;
+                if (filt && !pt_in_inner(X, Y, s_inner) && (kLabels || !pt_in_sample(x, y, s_edge))) keep = 1u;
             }
             auto get = [&](int, long long& idx, float& px, float& py) { idx = i; px = x; py = y; };
             if (filt) emit_raw<1>(keep, get, wbuf, wcnt, ctl, raw_xy, raw_idx);
@@ -486,6 +562,19 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
         if (any) track_tile(tr, tk, code);
     };
     if (gwarp == 0 && head) scalar_range(0, head, 0u);
+    int4* words = nullptr;
+    long long nwords = 0;
+    auto zero16 = [](int4* p) { __stcs(p, make_int4(0, 0, 0, 0)); };
+    if (kLabels && labels) {
+        const long long lead = min(n, (long long)((16u - ((uintptr_t)labels & 15u)) & 15u));
+        words = reinterpret_cast<int4*>(labels + lead);
+        nwords = (n - lead) / 16;
+        if (filt && gwarp == nwarps - 1) {   // what the tiles' shares leave: fewer than 16 bytes at each end, 33 words
+            if (lane < lead) labels[lane] = 0;
+            for (long long i = lead + 16 * nwords + lane; i < n; i += 32) labels[i] = 0;
+            for (long long w = 32 * ntiles + lane; w < nwords; w += 32) zero16(words + w);
+        }
+    }
 
     // Warp tiles t = gwarp + k * nwarps stream through a double-buffered
     // shared-memory ring filled by bulk asynchronous copies (TMA).
@@ -510,6 +599,10 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
             tile_keys2(tk, X0, Y0, X1, Y1, j == 0);
         }
         track_tile(tr, tk, (unsigned)(t + 1));
+        if (kLabels && filt && labels) {   // the tile's share of the label array's 16-byte words
+            const long long w = 32 * t + lane;
+            if (w < nwords) zero16(words + w);
+        }
         if (filt) {
             // Points strictly inside the inner region of the sample octagon
             // are strictly inside the hull; every other point is a raw
@@ -539,7 +632,7 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
                         x = v.x;
                         y = v.y;
                         keep = (pt_in_inner(__float2int_rn(x), __float2int_rn(y), s_inner) ||
-                                pt_in_sample(x, y, s_edge)) ? 0u : 1u;
+                                (!kLabels && pt_in_sample(x, y, s_edge))) ? 0u : 1u;
                         idx = head + t * kWarpTilePts + f2;
                     }
                     auto get = [&](int, long long& id, float& px, float& py) { id = idx; px = x; py = y; };
@@ -595,13 +688,13 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
     if (__syncthreads_or(read_status(ctl) != CH_OK)) return;
     // A call without a sample pass (two_pass) finds out here whether the data
     // are dense, against the octagon of the true extremes.
-    const bool test = two_pass && ntiles >= kStarMinTiles;
+    const bool test = !kLabels && two_pass && ntiles >= kStarMinTiles;
     DenseProbe probe;
     if (test)
         probe.load(reinterpret_cast<const float4*>(pts + 2 * head), kDensePts / 4,
                    [&](long long k) { return k * ntiles / (kDensePts / 4); });
     Octagon& o = *reinterpret_cast<Octagon*>(dsm);
-    finalize_block(pts, n, head, ctl, o, keys, vals);
+    finalize_block(pts, n, head, ctl, o, keys, vals, kLabels);
     if (test && read_status(ctl) == CH_OK && !o.discard_none && probe.dense(o, n, switch_at)) {
         copy_octagon(&ctl->oct_s, &o);
         if (threadIdx.x == 0) {
@@ -997,56 +1090,31 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
     if (__syncthreads_or(read_status(ctl) != CH_OK)) return;
     if (tid == 0) ctl->mode = 0;   // the post pass classifies the raw survivors
     __syncthreads();
-    if (!*(volatile int*)&ctl->oct_ready) finalize_block(pts, n, head, ctl, *reinterpret_cast<Octagon*>(dsm), keys, vals);
+    if (!*(volatile int*)&ctl->oct_ready) finalize_block(pts, n, head, ctl, *reinterpret_cast<Octagon*>(dsm), keys, vals, false);
 }
 
 // ---------------------------------------------------------------------------
 // ch_filter: the label array Q of Alg. 2 and the queue sizes (paper rule).
-__global__ void __launch_bounds__(256) labels_kernel(const float* __restrict__ pts, long long n,
-                                                     Ctl* ctl, uint8_t* labels) {
-    __shared__ Octagon s_o;
-    __shared__ unsigned s_cnt[4];
-    if (read_status(ctl) != CH_OK) return;
-    copy_octagon(&s_o, &ctl->oct);
-    if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0u;
-    __syncthreads();
-    unsigned c[4] = {0u, 0u, 0u, 0u};
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const float2 p = reinterpret_cast<const float2*>(pts)[i];
-        const int X = __float2int_rn(p.x), Y = __float2int_rn(p.y);
-        const int r = in_inner_strict(s_o, X, Y) ? -1 : classify_paper_slow(p.x, p.y, &s_o);
-        if (labels) labels[i] = (uint8_t)(r + 1);
-        if (r >= 0) c[r]++;
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        unsigned v = c[r];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s_cnt[r], v);
-    }
-    __syncthreads();
-    if (threadIdx.x < 4 && s_cnt[threadIdx.x]) atomicAdd(&ctl->counts4[threadIdx.x], s_cnt[threadIdx.x]);
-}
-
-// The label of one point by the paper rule: -1 inside the octagon's inner
-// region or the octagon, else its queue.
+// The label of one point: -1 inside the octagon's inner region or the octagon,
+// else its queue.
 __device__ __forceinline__ int label_of(float x, float y, const Octagon& o) {
     const int X = __float2int_rn(x), Y = __float2int_rn(y);
     return in_inner_strict(o, X, Y) ? -1 : classify_paper_slow(x, y, &o);
 }
 
-// The label pass fed by bulk copies, for 16-byte aligned points and a 4-byte
-// aligned label array: each warp streams its warp tiles (512 points) through
-// a double-buffered shared-memory ring, as the main pass does, and labels 4
-// consecutive points per lane and round (one 32-bit store of 4 labels; a
-// tile is 4 rounds).  The ragged tail (fewer than 512 points) is labelled
-// point by point by the first warp.
+// After a fused main pass (mode 0: every label is 0, the others' points are the
+// raw survivors) the survivors' labels, one per thread.  Else all points: each
+// warp streams its warp tiles (512 points, behind the unaligned head point)
+// through a double-buffered shared-memory ring, as the main pass does, and
+// labels 4 consecutive points per lane and round; the label array's words
+// (aligned, whatever its address and the head) are put together from two
+// lanes' labels.  The head and the ragged tail (fewer than 512 points) are
+// labelled point by point by the first warp.
 constexpr size_t kLabStreamSmemBytes = (size_t)8 * kStages * kWarpTileF4 * sizeof(float4);
 
-__global__ void __launch_bounds__(256) labels_stream_kernel(const float4* __restrict__ p4, long long n,
-                                                            long long ntiles, Ctl* ctl, uint32_t* labels4) {
+__global__ void __launch_bounds__(256) labels_kernel(const float* __restrict__ pts, long long n, int head,
+                                                     long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
+                                                     const uint32_t* raw_idx, uint8_t* labels) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ Octagon s_o;
     __shared__ unsigned s_cnt[4];
@@ -1059,41 +1127,57 @@ __global__ void __launch_bounds__(256) labels_stream_kernel(const float4* __rest
     const long long gwarp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     unsigned c[4] = {0u, 0u, 0u, 0u};
-    WarpStream ws{reinterpret_cast<float4*>(dsm) + warp * kStages * kWarpTileF4, s_bar[warp], p4, gwarp, nwarps,
-                  ntiles, lane};
-    ws.start();
-    for (long long k = 0;; ++k) {
-        const long long t = gwarp + k * nwarps;
-        if (t >= ntiles) break;
-        const float4* cur = ws.acquire(k, ctl);
-        if (!cur) {   // a copy never completed: status is CH_ETIMEOUT
-            ws.drain(k);
-            break;
+    auto count = [&](int lab) { c[0] += lab == 0; c[1] += lab == 1; c[2] += lab == 2; c[3] += lab == 3; };
+    if (ctl->mode == 0) {
+        const long long m = ctl->count_raw;
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += 32 * nwarps) {
+            const uint64_t xy = __ldcs(raw_xy + i);
+            const uint32_t id = __ldcs(raw_idx + i);
+            const int lab = classify_paper_slow((float)(int)(xy >> 32), (float)(int)(unsigned)xy, &s_o);
+            if (labels && lab >= 0) labels[id] = (uint8_t)(lab + 1);
+            count(lab);
         }
-#pragma unroll
-        for (int r = 0; r < kWarpTilePts / 128; ++r) {
-            const int q = r * 32 + lane;   // 4 points: float4 2q and 2q + 1 of the tile
-            const float4 a = cur[2 * q], b = cur[2 * q + 1];
-            const float xs[4] = {a.x, a.z, b.x, b.z}, ys[4] = {a.y, a.w, b.y, b.w};
-            uint32_t word = 0u;
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const int X = __float2int_rn(xs[m]), Y = __float2int_rn(ys[m]);
-                int lab = -1;
-                if (!in_inner_strict(s_o, X, Y)) lab = classify_paper_slow(xs[m], ys[m], &s_o);
-                word |= (uint32_t)(lab + 1) << (8 * m);
-                c[0] += lab == 0; c[1] += lab == 1; c[2] += lab == 2; c[3] += lab == 3;
+    } else {
+        const float4* p4 = reinterpret_cast<const float4*>(pts + 2 * head);
+        const unsigned off = (unsigned)((uintptr_t)(labels + head) & 3u);   // of every tile's first label
+        WarpStream ws{reinterpret_cast<float4*>(dsm) + warp * kStages * kWarpTileF4, s_bar[warp], p4, gwarp, nwarps,
+                      ntiles, lane};
+        ws.start();
+        for (long long k = 0;; ++k) {
+            const long long t = gwarp + k * nwarps;
+            if (t >= ntiles) break;
+            const float4* cur = ws.acquire(k, ctl);
+            if (!cur) {   // a copy never completed: status is CH_ETIMEOUT
+                ws.drain(k);
+                break;
             }
-            if (labels4) labels4[t * (kWarpTilePts / 4) + q] = word;
+            uint8_t* out = labels + head + t * kWarpTilePts;
+            uint32_t before = 0u;   // lane 0: the previous round's last word
+#pragma unroll
+            for (int r = 0; r < kWarpTilePts / 128; ++r) {
+                const int q = r * 32 + lane;   // 4 points: float4 2q and 2q + 1 of the tile
+                const float4 a = cur[2 * q], b = cur[2 * q + 1];
+                const float xs[4] = {a.x, a.z, b.x, b.z}, ys[4] = {a.y, a.w, b.y, b.w};
+                uint32_t word = 0u;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int lab = label_of(xs[m], ys[m], s_o);
+                    word |= (uint32_t)(lab + 1) << (8 * m);
+                    count(lab);
+                }
+                if (labels) store_labels(out, q, off, word, before);
+            }
+            ws.release(k);
         }
-        ws.release(k);
-    }
-    if (gwarp == 0) {   // the ragged tail
-        for (long long i = ntiles * kWarpTilePts + lane; i < n; i += 32) {
-            const float2 p = reinterpret_cast<const float2*>(p4)[i];
-            const int lab = label_of(p.x, p.y, s_o);
-            if (labels4) reinterpret_cast<uint8_t*>(labels4)[i] = (uint8_t)(lab + 1);
-            if (lab >= 0) c[lab]++;
+        if (gwarp == 0) {   // the head and the ragged tail
+            const long long tail = head + ntiles * kWarpTilePts;
+            for (long long j = lane; j < head + n - tail; j += 32) {
+                const long long i = j < head ? j : tail + j - head;
+                const float2 p = reinterpret_cast<const float2*>(pts)[i];
+                const int lab = label_of(p.x, p.y, s_o);
+                if (labels) labels[i] = (uint8_t)(lab + 1);
+                count(lab);
+            }
         }
     }
 #pragma unroll
@@ -1119,15 +1203,22 @@ __global__ void filter_output_kernel(const Ctl* ctl, long long n, int32_t* out_e
 void launch_init(Ctl* ctl, int mode, cudaStream_t s) { init_kernel<<<1, 256, 0, s>>>(ctl, mode); }
 
 void launch_sample(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, unsigned switch_at, int grid,
-                   cudaStream_t s) {
-    sample_kernel<<<grid, 256, 0, s>>>(pts, n, head, ntiles, ctl, switch_at);
+                   cudaStream_t s, int labels) {
+    sample_kernel<<<grid, 256, 0, s>>>(pts, n, head, ntiles, ctl, switch_at, labels);
 }
 
 void launch_main(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, uint64_t* raw_xy,
                  uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass, int grid,
                  cudaStream_t s) {
-    main_kernel<<<grid, 256, kMainSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, switch_at, keys, vals,
-                                                  two_pass);
+    main_kernel<false><<<grid, 256, kMainSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, switch_at, keys,
+                                                         vals, two_pass, nullptr);
+}
+
+void launch_main_labels(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, uint64_t* raw_xy,
+                        uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass,
+                        uint8_t* labels, int grid, cudaStream_t s) {
+    main_kernel<true><<<grid, 256, kMainSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, switch_at, keys,
+                                                        vals, two_pass, labels);
 }
 
 void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, void* bins, void* poly,
@@ -1139,14 +1230,9 @@ void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl
 size_t star_bins_bytes(int sms) { return sizeof(unsigned long long) * kStarBins * ((size_t)sms + 1); }
 size_t star_poly_bytes() { return sizeof(StarPoly); }
 
-void launch_labels(const float* pts, long long n, Ctl* ctl, uint8_t* labels, int grid, cudaStream_t s) {
-    if (((uintptr_t)pts & 15u) == 0u && ((uintptr_t)labels & 3u) == 0u) {
-        const long long ntiles = n / kWarpTilePts;
-        labels_stream_kernel<<<grid, 256, kLabStreamSmemBytes, s>>>(reinterpret_cast<const float4*>(pts), n, ntiles,
-                                                                    ctl, reinterpret_cast<uint32_t*>(labels));
-    } else {
-        labels_kernel<<<grid, 256, 0, s>>>(pts, n, ctl, labels);
-    }
+void launch_labels(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
+                   const uint32_t* raw_idx, uint8_t* labels, int grid, cudaStream_t s) {
+    labels_kernel<<<grid, 256, kLabStreamSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, labels);
 }
 
 void launch_filter_output(const Ctl* ctl, long long n, int32_t* out_ext8, int64_t* out_counts4, cudaStream_t s) {
@@ -1156,22 +1242,22 @@ void launch_filter_output(const Ctl* ctl, long long n, int32_t* out_ext8, int64_
 long long sample_tiles_host(long long ntiles) { return sample_tiles(ntiles); }
 
 cudaError_t configure_filter_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(main_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMainSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(labels_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kLabStreamSmemBytes);
+    const cudaFuncAttribute smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(main_kernel<false>, smem, (int)kMainSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(main_kernel<true>, smem, (int)kMainSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_kernel, smem, (int)kDenseSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(labels_kernel, smem, (int)kLabStreamSmemBytes);
     return e;
 }
 
 cudaError_t occupancy_filter(int* main_k, int* labels) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(main_k, main_kernel, 256, kMainSmemBytes);
     int a = 0, b = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, labels_kernel, 256, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, main_kernel<false>, 256, kMainSmemBytes);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, labels_stream_kernel, 256, kLabStreamSmemBytes);
-    *labels = a < b ? a : b;   // one grid size for both label kernels
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, main_kernel<true>, 256, kMainSmemBytes);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(labels, labels_kernel, 256, kLabStreamSmemBytes);
+    *main_k = a < b ? a : b;   // one grid size for both
     return e;
 }
 

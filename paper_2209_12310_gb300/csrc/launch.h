@@ -28,10 +28,13 @@ inline void launch_grid(void (*kernel)(KArgs...), int grid, int block, size_t sm
 
 void launch_init(Ctl* ctl, int mode, cudaStream_t s);
 void launch_sample(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, unsigned switch_at, int grid,
-                   cudaStream_t s);
+                   cudaStream_t s, int labels = 0);
 void launch_main(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, uint64_t* raw_xy,
                  uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass, int grid,
                  cudaStream_t s);
+void launch_main_labels(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, uint64_t* raw_xy,
+                        uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass,
+                        uint8_t* labels, int grid, cudaStream_t s);
 // The dense data's pass (star bins, star polygon, filter): the bins and the
 // polygon live in the workspace.
 void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, void* bins, void* poly,
@@ -39,7 +42,8 @@ void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl
 void launch_post(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
                  const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n,
                  int grid, cudaStream_t s);
-void launch_labels(const float* pts, long long n, Ctl* ctl, uint8_t* labels, int grid, cudaStream_t s);
+void launch_labels(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
+                   const uint32_t* raw_idx, uint8_t* labels, int grid, cudaStream_t s);
 size_t star_bins_bytes(int sms);   // a block's bins each, and the merged ones
 size_t star_poly_bytes();
 void launch_filter_output(const Ctl* ctl, long long n, int32_t* out_ext8, int64_t* out_counts4, cudaStream_t s);

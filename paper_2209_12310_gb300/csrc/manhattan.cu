@@ -149,7 +149,7 @@ __global__ void mh_init_kernel(Ctl* ctl) {
     const int t = threadIdx.x;
     if (t < 8) ctl->ext_packed[t] = 0ull;
     if (t < 4) { ctl->counts4[t] = 0u; ctl->blocks_done[t] = 0u; }
-    if (t == 0) { ctl->status = CH_OK; ctl->abort = 0; }
+    if (t == 0) { ctl->status = CH_OK; ctl->abort = 0; ctl->mode = 1; }   // mode 1: every point is labelled
 }
 
 }  // namespace
@@ -185,7 +185,9 @@ extern "C" int ch_filter_manhattan(const float* pts, int64_t n, int32_t* out_ext
         ProfScope p("labels", s);
         int mainb = 1, lab = 1;
         if (occupancy_filter(&mainb, &lab) != cudaSuccess) return CH_ECUDA;
-        launch_labels(pts, n, ctl, out_labels, sms * std::max(1, lab), s);
+        const int head = ((uintptr_t)pts & 15u) != 0u ? 1 : 0;
+        launch_labels(pts, n, head, (n - head) / kWarpTilePts, ctl, nullptr, nullptr, out_labels, sms * std::max(1, lab),
+                      s);
     }
     launch_filter_output(ctl, n, out_ext8, out_counts4, s);
     return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ECUDA;
