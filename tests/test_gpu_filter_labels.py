@@ -5,6 +5,7 @@ sends them back to a second read, and label arrays at every byte offset
 import numpy as np
 import pytest
 
+from oracle import filter16_ref as G
 from oracle import filter_ref as F
 from synth import workloads as W
 
@@ -70,3 +71,12 @@ def test_one_read_bad_coordinate(lib, bad):
 def test_label_offsets(lib, fn, n, shift, off):
     pts = W.make("ring" if n & 2 else "uniform", n, n)
     check((F.extremes(pts), F.labels(pts)), run(lib, fn, 8, pts, shift, off))
+
+
+@pytest.mark.parametrize("n", [1, 2, 511, 513, 1025, 70_001])
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("off", [0, 1, 2, 3])
+def test_label_offsets16(lib, n, shift, off):
+    pts = W.make("ring" if n & 2 else "uniform", n, n)
+    pts[n // 2:] = pts[:n - n // 2]      # ties: the lowest index wins, the head point among them
+    check((G.extremes16(pts), G.labels16(pts)), run(lib, "ch_filter16", 16, pts, shift, off))
