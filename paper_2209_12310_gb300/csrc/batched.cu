@@ -337,6 +337,86 @@ __global__ void __launch_bounds__(T) bt_extremes(BArgs a) {
     if (ts >= 0) bt_flush_track(tr, a.ctl + ts);
 }
 
+// All points of a set without a star slot, by the block that made its octagon o
+// (bt_octagon: a dense set, or a very small one; bt_filter passes over it).  A
+// warp of bt_filter took about 5 us per tile of such a set, whose points are
+// nearly all records, and one that met a run of them last ended long after the
+// others (filter and octagon of 768 mixed sets: 251 us before, 188 now; of 4096:
+// 737 and 657).  A kernel of its own with 1024 threads a set was no faster.
+__device__ __noinline__ void bt_classify_set(const BArgs& a, int i, const Octagon& o, long long base, int ni,
+                                             long long rb) {
+    __shared__ OctEdges s_e;
+    __shared__ unsigned s_cnt, s_q[4];
+    static_assert(kBStarMinPts / kBOctThreads < 255, "the tally's fields");
+    constexpr int kU = 4;   // points per thread in flight
+    Ctl* c = a.ctl + i;
+    const int tid = threadIdx.x, lane = tid & 31;
+    s_e.set(o, tid);
+    __syncthreads();   // the octagon's own records are counted
+    if (tid == 0) s_cnt = __ldcg(&c->count);
+    if (tid < 4) s_q[tid] = 0u;
+    __syncthreads();
+    const float2* p2 = reinterpret_cast<const float2*>(a.pts) + base;
+    QueueTally tally;
+    for (int j0 = tid - lane; j0 < ni; j0 += kU * kBOctThreads) {
+        float2 p[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int j = j0 + u * kBOctThreads + lane;
+            p[u] = j < ni ? __ldg(p2 + j) : make_float2(0.0f, 0.0f);
+        }
+        // two points a lane at a time: their chains interleave
+#pragma unroll
+        for (int u = 0; u < kU; u += 2) {
+            int X[2], Y[2], r[2];
+            bool keep[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 v = p[u + h];
+                X[h] = __float2int_rn(v.x);
+                Y[h] = __float2int_rn(v.y);
+                r[h] = classify_edges(v.x, v.y, s_e);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int j = j0 + (u + h) * kBOctThreads + lane;
+                if (j < ni && r[h] == kUndecided) r[h] = classify_hull_slow(p[u + h].x, p[u + h].y, &o);
+                keep[h] = j < ni && r[h] >= 0;
+                if (reduce_on_line(o, keep[h], X[h], Y[h], (unsigned)j, c)) keep[h] = false;
+                tally.add(keep[h], r[h]);
+            }
+            const unsigned b0 = __ballot_sync(0xFFFFFFFFu, keep[0]), b1 = __ballot_sync(0xFFFFFFFFu, keep[1]);
+            if (!(b0 | b1)) continue;
+            unsigned pos = 0u;
+            if (lane == 0) pos = atomicAdd(&s_cnt, (unsigned)(__popc(b0) + __popc(b1)));
+            pos = __shfl_sync(0xFFFFFFFFu, pos, 0);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (keep[h]) {
+                    uint32_t qu, qv;
+                    queue_frame(r[h], X[h], Y[h], qu, qv);
+                    const unsigned at = pos + (h ? (unsigned)__popc(b0) : 0u) +
+                                        (unsigned)__popc((h ? b1 : b0) & lanemask_lt());
+                    a.keys[rb + at] = make_key(r[h], qu);
+                    a.vals[rb + at] = make_val(qv, (uint32_t)(j0 + (u + h) * kBOctThreads + lane));
+                }
+            }
+        }
+    }
+    tally.fold();   // at most kBStarMinPts / kBOctThreads = 64 points a lane
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const unsigned w = tally.warp_total(q);
+        if (lane == 0 && w) atomicAdd(&s_q[q], w);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        c->count = s_cnt;
+        c->skip = 1;
+    }
+    if (tid < 4) c->counts4[tid] = __ldcg(&c->counts4[tid]) + s_q[tid];
+}
+
 // One block per set: the lowest index of each extreme (warp d rescans the
 // winning tile of direction d within the set), the octagon of the extremes
 // (with the inner region, which settles most points of bt_filter), the chain
@@ -459,6 +539,15 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
             c->star_cy = (s_vy[S] + s_vy[N]) / 2;
             a.star_list[atomicAdd(&a.star_ctr[0], 1u)] = i;
         }
+    } else {
+        // The same test (a point per thread) for the others.
+        const bool tiny = ni <= kBOctThreads;
+        bool out = tiny;
+        if (!tiny) {
+            const float2 p = __ldg(reinterpret_cast<const float2*>(a.pts) + base + tid * (ni / kBOctThreads));
+            out = !in_inner(s_o, __float2int_rn(p.x), __float2int_rn(p.y));
+        }
+        if (__syncthreads_count(out) * 16 > kBOctThreads) bt_classify_set(a, i, s_o, base, (int)ni, rb);
     }
 }
 
@@ -488,7 +577,7 @@ struct BtWarpSmem {
     Ctl* c;                          // the warp's set: control block, record region,
     long long rb, base;              // first point,
     int set;                         // its number (-1: none),
-    int skip;                        // empty, failed, or bt_dense's: nothing to classify
+    int skip;                        // empty, failed, classified already, or bt_dense's: nothing to classify
     unsigned qn;                     // points queued,
     unsigned cnt;                    // records staged,
     unsigned nq[4];                  // records per queue
@@ -628,8 +717,8 @@ __device__ __noinline__ void bt_warp_set(const BArgs& a, int q, BtWarpSmem& m) {
     const int lane = threadIdx.x & 31;
     bt_warp_done(a, m);
     Ctl* c = a.ctl + q;
-    // empty and failed sets (bt_octagon's verdict), and the sets with a star
-    // polygon, which bt_dense filters
+    // empty, failed and small dense sets (bt_octagon's verdict), and the sets with
+    // a star polygon, which bt_dense filters
     const int skip = c->skip;
     if (lane == 0) {
         m.c = c;

@@ -144,7 +144,7 @@ struct Ctl {
     int samp_dense;                     // dense data (oct_s: an octagon of input points): the star pass bins points
     int oct_ready;                      // the octagon of the true extremes and the end-point records stand
     int star_ok;                        // batched: the set is listed for a star polygon
-    int skip;                           // batched: nothing for bt_filter (empty, failed, or bt_dense's)
+    int skip;                           // batched: nothing for bt_filter (empty, failed, classified, or bt_dense's)
     int star_k;                         // the polygon's vertices, the dropped ones included
     int star_edges;                     // dense_kernel: the polygon's vertices in use (0: none)
     int star_final;                     // a polygon was built and accepted
