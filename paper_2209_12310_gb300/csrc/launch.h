@@ -26,6 +26,26 @@ inline void launch_grid(void (*kernel)(KArgs...), int grid, int block, size_t sm
     cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Launch of a kernel that may start before the stream's last kernel ends: as soon
+// as every block of that one has executed griddepcontrol.launch_dependents (or
+// ended).  The kernel itself ends with griddepcontrol.wait, so that what follows
+// it in the stream follows both.
+template <typename... KArgs, typename... Args>
+inline void launch_beside(void (*kernel)(KArgs...), int grid, int threads, size_t smem, cudaStream_t s,
+                          const Args&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 void launch_init(Ctl* ctl, int mode, cudaStream_t s);
 void launch_sample(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, unsigned switch_at, int grid,
                    cudaStream_t s, int labels = 0);

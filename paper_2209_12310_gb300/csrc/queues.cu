@@ -324,33 +324,7 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
     if (path == kPathQueues) {
         QcQueue& q = *reinterpret_cast<QcQueue*>(s_dyn);
         const unsigned m = ctl->count;
-        constexpr int kU = 4;   // records per thread in flight
-        for (unsigned j0 = 0; j0 < m; j0 += T * kU) {
-            uint32_t k[kU];
-            uint64_t w[kU];
-            bool own[kU];
-#pragma unroll
-            for (int e = 0; e < kU; ++e) {
-                const unsigned j = j0 + e * T + tid;
-                k[e] = j < m ? __ldcg(keys + j) : 0u;
-                own[e] = j < m && (int)(k[e] >> kKeyBits) == qq;
-            }
-#pragma unroll
-            for (int e = 0; e < kU; ++e) w[e] = own[e] ? __ldcg(vals + j0 + e * T + tid) : 0ull;
-#pragma unroll
-            for (int e = 0; e < kU; ++e) {
-                const unsigned bal = __ballot_sync(0xFFFFFFFFu, own[e]);
-                if (!bal) continue;
-                int pos = 0;
-                if (lane == 0) pos = atomicAdd(&s_n, __popc(bal));
-                pos = __shfl_sync(0xFFFFFFFFu, pos, 0) + __popc(bal & lanemask_lt());
-                if (own[e] && pos < QcQueue::kCap) {
-                    q.a[pos] = qc_pack(k[e] & kKeyMask, (unsigned)(w[e] >> 31), (unsigned)pos);
-                    q.si[pos] = (int)(w[e] & 0x7FFFFFFFull);
-                }
-            }
-        }
-        __syncthreads();
+        qc_gather<T, 4>(keys, vals, m, qq, q, &s_n);
         CH_TL(ctl, 19, 1);
         const int cnt = min(s_n, QcQueue::kCap);   // rec_q[qq], the two end points among them
         qc_sort<T>(q, cnt, s_m.lo[qq], s_m.hi[qq]);
