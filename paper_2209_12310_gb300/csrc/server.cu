@@ -5,8 +5,9 @@
 // admission queue (O(1), never touches the GPU, never copies: the caller's
 // buffer is read when the request is admitted into a batch and must stay
 // valid until ch_poll answers for it).  The engine thread repeatedly
-//   1. retires finished batches (result counts first, then the index lists,
-//      both copied back asynchronously and observed through CUDA events),
+//   1. retires finished batches (result counts and index lists, observed through
+//      CUDA events; a kernel packs the lists into the slot's pinned buffer when
+//      they fit, else they are copied one by one once the counts are known),
 //   2. forms a new batch from the queue head while a free stream slot exists
 //      and the arena has a contiguous block for the batch (admission by
 //      memory: a request waits until memory frees up),
@@ -91,6 +92,9 @@ class Arena {
     size_t size_ = 0;
 };
 
+constexpr int kMaxBatch = 4096;
+constexpr size_t kIdxCap = 1u << 19;   // indices of a slot's pinned buffer at first
+
 struct Slot {
     bool busy = false;
     int phase = 0;   // 1: waiting for counts, 2: waiting for indices
@@ -108,15 +112,66 @@ struct Slot {
     bool redone = false;
     int32_t* h_idx = nullptr;       // pinned result indices
     size_t h_idx_cap = 0;
+    size_t packed_cap = 0;          // of h_idx when the batch's pack kernel was launched
     size_t cap_k = 0;
     size_t arena_off = 0, arena_bytes = 0;
 };
 
 constexpr size_t kMaxQueue = 1u << 17;
+constexpr double kSpinSeconds = 2e-3;
 constexpr int kBatchTrace = 8;
 constexpr size_t kMaxTrace = 1u << 20;   // batches traced at most
-constexpr int kMaxBatch = 4096;
 constexpr int kSlots = 3;
+
+// The k sets' hulls, set i's n[i] indices at idx + off[i], one after the other
+// into out (pinned host memory) when they are at most cap in all; the host, which
+// has the counts at the same event, reads them from there.  Writes over the host
+// link from one kernel: a copy per set behind the counts' event cost a burst of
+// 32 requests about 100 us, and another round of waiting.
+constexpr int kPackThreads = 512;
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(const int32_t* __restrict__ idx,
+                                                            const int64_t* __restrict__ off,
+                                                            const int64_t* __restrict__ n, int k, int32_t* out,
+                                                            long long cap) {
+    __shared__ long long s_pos[kMaxBatch + 1];   // where each set's list starts
+    __shared__ long long s_sum[kPackThreads];
+    constexpr int kPer = kMaxBatch / kPackThreads;
+    const int t = threadIdx.x;
+    long long c[kPer], sum = 0;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        const int i = t * kPer + e;
+        // a set left to the single-hull path has no count yet
+        c[e] = i < k ? min(max(0ll, (long long)n[i]), (long long)(off[i + 1] - off[i])) : 0ll;
+        sum += c[e];
+    }
+    s_sum[t] = sum;
+    __syncthreads();
+    for (int o = 1; o < kPackThreads; o <<= 1) {
+        const long long v = t >= o ? s_sum[t - o] : 0ll;
+        __syncthreads();
+        s_sum[t] += v;
+        __syncthreads();
+    }
+    long long run = s_sum[t] - sum;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        s_pos[t * kPer + e] = run;
+        run += c[e];
+    }
+    __syncthreads();
+    const long long total = s_sum[kPackThreads - 1];
+    if (total > cap) return;
+    for (long long j = (long long)blockIdx.x * kPackThreads + t; j < total; j += (long long)gridDim.x * kPackThreads) {
+        int lo = 0, hi = k;   // s_pos[lo] <= j < s_pos[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) / 2;
+            if (s_pos[mid] <= j) lo = mid;
+            else hi = mid;
+        }
+        out[j] = idx[off[lo] + (j - s_pos[lo])];
+    }
+}
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 size_t batch_bytes(int64_t points, size_t k) {
@@ -178,10 +233,16 @@ bool Server::retire(Slot& sl) {
                 cudaMemsetAsync(d_n, 0xFF, 8 * k, sl.s);
             cudaMemcpyAsync(sl.h_n, d_n, 8 * k, cudaMemcpyDeviceToHost, sl.s);
             cudaEventRecord(sl.ev, sl.s);
+            sl.packed_cap = 0;   // the packed lists are from before
             sl.redo_sets = 0;
             for (size_t i = 0; i < k; ++i) sl.redo_sets += sl.h_redo[i] != 0;
             return true;
         }
+    }
+    if (sl.phase == 1) {
+        size_t hsum = 0;
+        for (size_t i = 0; i < k; ++i) hsum += sl.h_n[i] > 0 ? (size_t)sl.h_n[i] : 0;
+        if (hsum <= sl.packed_cap) sl.phase = 2;   // the lists came with the counts
     }
     if (sl.phase == 1) {
         size_t hsum = 0;
@@ -290,6 +351,14 @@ bool Server::launch(Slot& sl) {
         cudaMallocHost((void**)&sl.h_n, 8 * sl.cap_k);
         cudaMallocHost((void**)&sl.h_redo, sl.cap_k);
     }
+    if (!sl.h_idx) {
+        sl.h_idx_cap = kIdxCap;
+        if (cudaMallocHost((void**)&sl.h_idx, sl.h_idx_cap * sizeof(int32_t)) != cudaSuccess) {
+            cudaGetLastError();
+            sl.h_idx = nullptr;
+            sl.h_idx_cap = 0;
+        }
+    }
     sl.off.assign(k + 1, 0);
     for (size_t i = 0; i < k; ++i) sl.off[i + 1] = sl.off[i] + batch[i]->n;
     std::memcpy(sl.h_off, sl.off.data(), 8 * (k + 1));
@@ -314,6 +383,12 @@ bool Server::launch(Slot& sl) {
     if (st != CH_OK) cudaMemsetAsync(d_n, 0xFF, 8 * k, sl.s);   // -1 = CH_EINVAL per set
     cudaMemcpyAsync(sl.h_n, d_n, 8 * k, cudaMemcpyDeviceToHost, sl.s);
     cudaEventRecord(sl.te[2], sl.s);
+    sl.packed_cap = sl.h_idx ? sl.h_idx_cap : 0;
+    if (sl.packed_cap > 0) {
+        const int blocks = (int)std::min<size_t>(32, 1 + k / 4);
+        pack_kernel<<<blocks, kPackThreads, 0, sl.s>>>(d_idx, d_off, d_n, (int)k, sl.h_idx, (long long)sl.packed_cap);
+    }
+    cudaEventRecord(sl.te[3], sl.s);
     cudaEventRecord(sl.ev, sl.s);
     sl.reqs = std::move(batch);
     sl.arena_off = off;
@@ -325,11 +400,20 @@ bool Server::launch(Slot& sl) {
 
 void Server::run() {
     cudaSetDevice(device);
+    // While a batch is in flight, and for at most kSpinSeconds since anything
+    // happened, the thread looks again at once: a timed wait of 50 us lasts
+    // about twice that with the kernel's timer slack, a tenth of a small burst.
+    double last = 0;
     while (!stop.load()) {
-        bool progress = false;
+        bool progress = false, busy = false;
         for (auto& sl : slots) progress |= retire(sl);
         for (auto& sl : slots) progress |= launch(sl);
-        if (!progress) {
+        for (auto& sl : slots) busy |= sl.busy;
+        if (progress) last = now_s();
+        if (progress) continue;
+        if (busy && now_s() - last < kSpinSeconds) {
+            std::this_thread::yield();
+        } else {
             std::unique_lock<std::mutex> lk(mu);
             cv.wait_for(lk, std::chrono::microseconds(50));
         }
