@@ -255,11 +255,15 @@ static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, 
     // Raw survivors live in the B buffers until the post pass has turned them
     // into sort records in the A buffers.
     const unsigned switch_at = (unsigned)std::max<long long>(1 << 16, n >> 5);
-    const bool dense = ntiles >= kStarMinTiles;   // large enough for a star polygon
+    const bool dense = ntiles >= kStarMinTiles && n > kSmallMax;   // large enough for a star polygon
     // Inputs that stay in L2 take two passes: the extremes, then the filter
     // against their octagon.  Larger ones take one, with a sample's octagon.
     const bool two_pass = n <= kTwoPassMax;
-    if (two_pass) {
+    const bool one_block = n <= kSmallMax;   // one block does it all up to the large-survivor paths
+    if (one_block) {
+        ProfScope p("small", s);
+        launch_small(pts, n, ctl, kA, vA, out_idx, out_n, s);
+    } else if (two_pass) {
         { ProfScope p("init", s); launch_init(ctl, 1, s); }
         ProfScope p("main_filter", s);
         launch_main(pts, n, head, ntiles, ctl, nullptr, nullptr, switch_at, kA, vA, 1, di.sms * di.occ_main, s);
@@ -276,7 +280,7 @@ static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, 
         ProfScope p("main_filter", s);
         launch_main(pts, n, head, ntiles, ctl, vB, kB, switch_at, kA, vA, 0, di.sms * di.occ_main, s);
     }
-    {
+    if (!one_block) {
         ProfScope p("post", s);
         launch_post(pts, n, head, ntiles, ctl, vB, kB, kA, vA, out_idx, out_n, di.sms * di.occ_post, s);
     }

@@ -75,6 +75,7 @@ constexpr long long kStarMinTiles = 128;      // inputs below this many warp til
 // extremes come first and no sample is needed (the fused pass saves reads of
 // HBM at the price of one more kernel in the chain).
 constexpr long long kTwoPassMax = 1 << 22;
+constexpr long long kSmallMax = 8192;   // one block finds the records of so few points (small_kernel)
 // ch_filter's: its second read also stays in L2 up to 64 MB of points.
 constexpr long long kFilterTwoPassMax = 1 << 23;
 constexpr int kMaxLevels = 32;

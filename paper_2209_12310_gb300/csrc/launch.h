@@ -59,6 +59,8 @@ void launch_main_labels(const float* pts, long long n, int head, long long ntile
 // polygon live in the workspace.
 void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, void* bins, void* poly,
                   uint64_t* raw_xy, uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int sms, cudaStream_t s);
+void launch_small(const float* pts, long long n, Ctl* ctl, uint32_t* keys, uint64_t* vals, int32_t* out_idx,
+                  int64_t* out_n, cudaStream_t s);
 void launch_post(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
                  const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n,
                  int grid, cudaStream_t s);

@@ -8,10 +8,12 @@
 // computes the hull itself (quickhull rounds over the queues), so the
 // large-survivor path that follows finds ctl->done set and exits at once.
 #include "ch_internal.cuh"
+#include "extremes.cuh"
 #include "hullcore.cuh"
 #include "launch.h"
 #include "octagon.cuh"
 #include "records.cuh"
+#include "setup.cuh"
 
 #include <climits>
 
@@ -323,6 +325,89 @@ __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __re
 }
 
 // ---------------------------------------------------------------------------
+// Inputs of at most kSmallMax points: one block does the work of the init, main
+// and post kernels (their launches and the two grids' last blocks are most of
+// such a call: 39 us of device time for 1000 uniform points, 21 in one block;
+// 3000: 39 and 25; 8000: 41 and 38; past that the grid is the faster).
+__global__ void __launch_bounds__(kPostThreads, 1) small_kernel(const float* __restrict__ pts, int n, Ctl* ctl,
+                                                                uint32_t* keys, uint64_t* vals, int32_t* out_idx,
+                                                                int64_t* out_n) {
+    extern __shared__ __align__(16) char dyn[];
+    __shared__ Octagon s_o;
+    __shared__ unsigned long long s_best[8];
+    __shared__ int s_vx[8], s_vy[8], s_id[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float2* p2 = reinterpret_cast<const float2*>(pts);
+    reset_ctl(ctl, 1);
+    if (tid < 8) s_best[tid] = 0ull;
+    __syncthreads();
+    // extremes with the lowest index on ties; validity of every coordinate
+    unsigned long long best[8];
+#pragma unroll
+    for (int d = 0; d < 8; ++d) best[d] = 0ull;
+    bool bad = false;
+    for (int i = tid; i < n; i += kPostThreads) {
+        const float2 p = __ldg(p2 + i);
+        const int X = __float2int_rn(p.x), Y = __float2int_rn(p.y);
+        bad |= (__int2float_rn(X) != p.x) | (__int2float_rn(Y) != p.y) |
+               ((((unsigned)X | (unsigned)Y) >> kCoordBits) != 0u);
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            const unsigned k = (unsigned)dir_key(d, X, Y);
+            const unsigned long long w =
+                ((unsigned long long)(dir_is_max(d) ? k : 0xFFFFFFFFu - k) << 32) | (0xFFFFFFFFu - (unsigned)i);
+            best[d] = w > best[d] ? w : best[d];
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {
+        unsigned long long w = best[d];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xFFFFFFFFu, w, o);
+            w = v > w ? v : w;
+        }
+        if (lane == 0) atomicMax(&s_best[d], w);
+    }
+    if (__syncthreads_or(bad)) {
+        if (tid == 0) {
+            set_status(ctl, CH_ERANGE);
+            *out_n = CH_ERANGE;
+            ctl->done = 1;
+        }
+        return;
+    }
+    if (tid < 8) {
+        const int i = (int)(0xFFFFFFFFu - (unsigned)s_best[tid]);
+        s_id[tid] = i;
+        s_vx[tid] = __float2int_rn(p2[i].x);
+        s_vy[tid] = __float2int_rn(p2[i].y);
+    }
+    __syncthreads();
+    setup_octagon_block(s_o, s_vx, s_vy, s_id, false);   // a point per thread and step: no inner region needed
+    end_records(s_vx, s_vy, s_id, ctl, keys, vals);
+    copy_octagon(&ctl->oct, &s_o);
+    RecBuf& rb = reinterpret_cast<RecBuf*>(dyn)[warp];
+    unsigned rc = 0u;
+    QueueTally tally;
+    for (int i = tid; i - lane < n; i += kPostThreads) {
+        const bool valid = i < n;
+        const float2 p = valid ? __ldg(p2 + i) : make_float2(0.0f, 0.0f);
+        post_point(valid, p.x, p.y, (unsigned)i, s_o, rb, rc, ctl, keys, vals, tally);
+    }
+    __syncthreads();   // the end records are counted
+    rec_flush_block(rb, rc, ctl, keys, vals);
+    flush_queue_counts(tally, ctl);
+    __syncthreads();
+    post_last_block(pts, n, ctl, s_o, keys, vals, out_idx, out_n, dyn, false);
+}
+
+// ---------------------------------------------------------------------------
+void launch_small(const float* pts, long long n, Ctl* ctl, uint32_t* keys, uint64_t* vals, int32_t* out_idx,
+                  int64_t* out_n, cudaStream_t s) {
+    small_kernel<<<1, kPostThreads, kPostSmemBytes, s>>>(pts, (int)n, ctl, keys, vals, out_idx, out_n);
+}
+
 void launch_post(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
                  const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n,
                  int grid, cudaStream_t s) {
@@ -331,6 +416,9 @@ void launch_post(const float* pts, long long n, int head, long long ntiles, Ctl*
 }
 
 cudaError_t configure_post_kernel() {
+    const cudaError_t e =
+        cudaFuncSetAttribute(small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPostSmemBytes);
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(post_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPostSmemBytes);
 }
 
