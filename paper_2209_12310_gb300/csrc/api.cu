@@ -73,7 +73,6 @@ Layout make_layout(long long n) {
     // blocks of it run)
     const bool star = n / kWarpTilePts >= kStarMinTiles;
     L.off_star_poly = take(star ? star_poly_bytes() : 0);
-    L.off_star_bins = take(star ? star_bins_bytes(kStarBlocks) : 0);
     L.off_kA = take(4 * (size_t)L.cap);
     L.off_kB = take(4 * (size_t)L.cap);
     L.off_vA = take(8 * (size_t)L.cap);
@@ -81,6 +80,9 @@ Layout make_layout(long long n) {
     L.off_cu = take(4 * (size_t)L.ctcap * kChainTile);
     L.off_cv = take(4 * (size_t)L.ctcap * kChainTile);
     L.off_ci = take(4 * (size_t)L.ctcap * kChainTile);
+    // dense_kernel's bins, done with before the first chain is stored
+    L.off_star_bins = L.off_cu;
+    if (star) o = std::max(o, align_up(L.off_cu + star_bins_bytes(kStarBlocks)));
     L.off_clen = take(4 * (size_t)L.ctcap);
     L.total = o;
     return L;
