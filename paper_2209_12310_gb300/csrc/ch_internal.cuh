@@ -70,12 +70,15 @@ constexpr int kSampleTiles = 1024;            // warp tiles read by the sample p
 // Star polygon of dense data (star.cuh): angular bins around a centre.
 constexpr int kStarBins = 8192;
 constexpr int kStarBlocks = 160;              // blocks of dense_kernel at most
-constexpr long long kStarMinTiles = 128;      // inputs below this many warp tiles skip the star pass
+constexpr long long kStarMinTiles = 128;      // inputs below this many warp tiles get no star polygon
 // Inputs of at most this many points stay in L2 between two passes, so the
 // extremes come first and no sample is needed (the fused pass saves reads of
 // HBM at the price of one more kernel in the chain).
 constexpr long long kTwoPassMax = 1 << 22;
 constexpr long long kSmallMax = 8192;   // one block finds the records of so few points (small_kernel)
+// The label passes take a point per thread up to here, above warp tiles of 512
+// points (which leave most of the chip idle on small inputs).
+constexpr long long kPointsMax = 1 << 21;
 // ch_filter's: its second read also stays in L2 up to 64 MB of points.
 constexpr long long kFilterTwoPassMax = 1 << 23;
 constexpr int kMaxLevels = 32;
@@ -133,16 +136,16 @@ struct Ctl {
     int records_ready;                  // sort records complete before the re-classify stage
     unsigned int blocks_done[4];        // last-arriver counters (sample, main, stage C, roots)
     unsigned int barrier[3];            // grid barriers (dense_kernel, large_kernel, sort_kernel)
-    unsigned int tile_ctr[4];           // onesweep tile claim counters (0 .. 2), tile_chain_kernel's (3)
-    unsigned int digit_hist[kSortPasses][kDigits];   // sort fallback only (sort_hist_kernel)
+    unsigned int tile_ctr[4];           // onesweep tile claim counters (0 .. 2), the sorted tiles' (3)
+    unsigned int digit_hist[kSortPasses][kDigits];   // sort path only (sort_kernel)
     unsigned int rec_q[4];              // records per queue
-    unsigned int reg_end[4];            // chain length of queue r (queue_kernel, bt_queue_chain)
+    unsigned int reg_end[4];            // chain length of queue r (large_kernel, bt_queue_chain)
     unsigned int counts4[4];            // survivors per queue (ch_filter)
     unsigned long long line_ep[8];      // end points of survivors on the 4 axis support lines
     int bk_state;                       // large-survivor path: 0 unused, 1 queues / tiles / buckets, 2 full sort
     int path;                           // the single hull's large-survivor path (Path)
     unsigned int q_tile[5];             // path tiles: tiles of queue r are [q_tile[r], q_tile[r + 1])
-    int samp_dense;                     // dense data (oct_s: an octagon of input points): the star pass bins points
+    int samp_dense;                     // dense data (oct_s: an octagon of input points): dense_kernel's
     int oct_ready;                      // the octagon of the true extremes and the end-point records stand
     int star_ok;                        // batched: the set is listed for a star polygon
     int skip;                           // batched: nothing for bt_filter (empty, failed, classified, or bt_dense's)

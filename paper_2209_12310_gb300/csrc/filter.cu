@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ p
         return;
     }
     copy_octagon(&ctl->oct_s, &s_o);
-    // Dense data (points near a circle) goes to the star pass and dense_kernel
+    // Dense data (points near a circle) goes to dense_kernel
     // from the start; the main pass would find out by writing switch_at raw
     // survivors, and all points would be read again.
     const bool dense = test && !s_o.discard_none && probe.dense(s_o, n, switch_at);
@@ -1036,8 +1036,8 @@ __device__ __forceinline__ int label_of(float x, float y, const Octagon& o) {
 }
 
 // After a fused main pass (mode 0: every label is 0, the others' points are the
-// raw survivors) the survivors' labels, one per thread.  Else all points: each
-// warp streams its warp tiles (512 points, behind the unaligned head point)
+// raw survivors) the survivors' labels, one per thread.  Else all points: up to
+// kPointsMax one per thread, above each warp streams its warp tiles (512 points, behind the unaligned head point)
 // through a double-buffered shared-memory ring, as the main pass does, and
 // labels 4 consecutive points per lane and round; the label array's words
 // (aligned, whatever its address and the head) are put together from two
@@ -1068,6 +1068,13 @@ __global__ void __launch_bounds__(256) labels_kernel(const float* __restrict__ p
             const uint32_t id = __ldcs(raw_idx + i);
             const int lab = classify_paper_slow((float)(int)(xy >> 32), (float)(int)(unsigned)xy, &s_o);
             if (labels && lab >= 0) labels[id] = (uint8_t)(lab + 1);
+            count(lab);
+        }
+    } else if (n <= kPointsMax) {
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 32 * nwarps) {
+            const float2 p = reinterpret_cast<const float2*>(pts)[i];
+            const int lab = label_of(p.x, p.y, s_o);
+            if (labels) labels[i] = (uint8_t)(lab + 1);
             count(lab);
         }
     } else {

@@ -418,6 +418,119 @@ __global__ void __launch_bounds__(kF16Threads) f16_labels(const float* __restric
     if (t < 4 && s_cnt[t]) atomicAdd(&c->counts[t], s_cnt[t]);
 }
 
+// Inputs of at most kPointsMax points: a point per thread, per-point maxima and
+// exact labels.  Warp tiles of 512 points leave most of the chip idle there (a
+// call on 9000 ring points: 60 us by tiles, 29 by points, the host's part
+// included; 2 M uniform points 46 and 43, 4 M 52 and 70).
+__global__ void __launch_bounds__(kF16Threads) f16_extremes_points(const float2* __restrict__ pts, long long n,
+                                                            F16Ctl* c) {
+    __shared__ unsigned long long s_m[kF16Threads / 32][16];
+    int best[16];
+    unsigned arg[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        best[k] = INT_MIN;
+        arg[k] = 0u;
+    }
+    bool bad = false;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    // indices rise within a thread, so a strict improvement keeps the lowest
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const float2 p = __ldcs(pts + i);
+        const bool ok = p.x >= 0.0f && p.x < 16777216.0f && p.x == rintf(p.x) && p.y >= 0.0f && p.y < 16777216.0f &&
+                        p.y == rintf(p.y);
+        bad |= !ok;
+        const int X = ok ? __float2int_rz(p.x) : 0, Y = ok ? __float2int_rz(p.y) : 0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int v = key16(k, X, Y);
+            if (v > best[k]) {
+                best[k] = v;
+                arg[k] = (unsigned)i;
+            }
+        }
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        // keys exceed -2^26, so INT_MIN marks a thread without points
+        unsigned long long m = best[k] == INT_MIN
+                                   ? 0ull
+                                   : ((unsigned long long)(unsigned)(best[k] + kF16Bias) << 32) | (0xFFFFFFFFu - arg[k]);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) m = max_u64(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+        if (lane == 0) s_m[warp][k] = m;
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicCAS(&c->status, CH_OK, CH_ERANGE);
+    if (threadIdx.x < 16) {
+        unsigned long long m = 0ull;
+        for (int w = 0; w < kF16Threads / 32; ++w) m = max_u64(m, s_m[w][threadIdx.x]);
+        if (m) atomicMax(&c->packed[threadIdx.x], m);
+    }
+}
+
+__global__ void __launch_bounds__(kF16Threads) f16_labels_points(const float2* __restrict__ pts, long long n, F16Ctl* c,
+                                                          uint8_t* labels) {
+    __shared__ int s_vx[16], s_vy[16], s_live[16];
+    __shared__ int s_none;
+    __shared__ unsigned s_cnt[4];
+    if (*(volatile int*)&c->status != CH_OK) return;   // set before this launch: the same for every block
+    const int t = threadIdx.x;
+    if (t < 16) {
+        const unsigned idx = 0xFFFFFFFFu - (unsigned)(c->packed[t] & 0xFFFFFFFFull);
+        const float2 v = (long long)idx < n ? pts[idx] : make_float2(0.0f, 0.0f);
+        s_vx[t] = __float2int_rz(v.x);
+        s_vy[t] = __float2int_rz(v.y);
+    }
+    if (t < 4) s_cnt[t] = 0u;
+    __syncthreads();
+    if (t < 16) {
+        const int j = (t + 1) & 15;
+        s_live[t] = (s_vx[t] != s_vx[j] || s_vy[t] != s_vy[j]) ? 1 : 0;
+    }
+    if (t == 0) {
+        long long a2 = 0;
+        for (int k = 0; k < 16; ++k) {
+            const int j = (k + 1) & 15;
+            a2 += (long long)s_vx[k] * s_vy[j] - (long long)s_vx[j] * s_vy[k];
+        }
+        s_none = a2 == 0 ? 1 : 0;
+    }
+    __syncthreads();
+    const bool none = s_none != 0;
+    unsigned cnt[4] = {0u, 0u, 0u, 0u};
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i = (long long)blockIdx.x * blockDim.x + t; i < n; i += stride) {
+        const float2 p = __ldcs(pts + i);
+        const int X = __float2int_rz(p.x), Y = __float2int_rz(p.y);
+        bool inside = !none;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int j = (k + 1) & 15;
+            if (s_live[k] && orient64(s_vx[k], s_vy[k], s_vx[j], s_vy[j], X, Y) <= 0) inside = false;
+        }
+        int r = -1;
+        if (!inside) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {   // W->S, S->E, E->N, N->W
+                const int a = 4 * q, b = (4 * q + 4) & 15;
+                if (r < 0 && orient64(s_vx[a], s_vy[a], s_vx[b], s_vy[b], X, Y) < 0) r = q;
+            }
+        }
+        if (labels) labels[i] = (uint8_t)(r + 1);
+        if (r >= 0) cnt[r]++;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        unsigned v = cnt[q];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+        if ((t & 31) == 0 && v) atomicAdd(&s_cnt[q], v);
+    }
+    __syncthreads();
+    if (t < 4 && s_cnt[t]) atomicAdd(&c->counts[t], s_cnt[t]);
+}
+
 __global__ void f16_output(const F16Ctl* c, const Ctl* ctl, int32_t* out_ext16, int64_t* out_counts4) {
     const int t = threadIdx.x;
     const int st = c->status != CH_OK ? c->status : ctl->status;
@@ -442,17 +555,9 @@ extern "C" int ch_filter16(const float* pts, int64_t n, int32_t* out_ext16, uint
             return CH_ECUDA;
         return CH_OK;
     }
-    int dev = 0, sms = 0, occ_e = 0, occ_l = 0;
+    int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return CH_ECUDA;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return CH_ECUDA;
-    const cudaFuncAttribute smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if (cudaFuncSetAttribute(f16_extremes, smem, (int)kF16StreamSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(f16_labels, smem, (int)kF16StreamSmemBytes) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_e, f16_extremes, kF16Threads, kF16StreamSmemBytes) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_l, f16_labels, kF16Threads, kF16StreamSmemBytes) !=
-            cudaSuccess)
-        return CH_ECUDA;
     char* base = nullptr;
     Layout L;
     if ((st = get_workspace(dev, s, n, &base, &L)) != CH_OK) return st;
@@ -463,6 +568,29 @@ extern "C" int ch_filter16(const float* pts, int64_t n, int32_t* out_ext16, uint
     const long long want = std::max(1ll, (ntiles + kF16Threads / 32 - 1) / (kF16Threads / 32));
     const bool lab = out_labels || out_counts4;
     f16_init<<<1, 32, 0, s>>>(c, ctl);
+    if (n <= kPointsMax) {
+        const float2* p2 = reinterpret_cast<const float2*>(pts);
+        const int grid = (int)std::min<long long>((n + kF16Threads - 1) / kF16Threads, 4ll * sms);
+        {
+            ProfScope p("filter16_extremes", s);
+            f16_extremes_points<<<grid, kF16Threads, 0, s>>>(p2, n, c);
+        }
+        if (lab) {
+            ProfScope p("filter16_labels", s);
+            f16_labels_points<<<grid, kF16Threads, 0, s>>>(p2, n, c, out_labels);
+        }
+        f16_output<<<1, 32, 0, s>>>(c, ctl, out_ext16, out_counts4);
+        return cudaGetLastError() == cudaSuccess ? CH_OK : CH_ECUDA;
+    }
+    int occ_e = 0, occ_l = 0;
+    const cudaFuncAttribute smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (cudaFuncSetAttribute(f16_extremes, smem, (int)kF16StreamSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(f16_labels, smem, (int)kF16StreamSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_e, f16_extremes, kF16Threads, kF16StreamSmemBytes) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_l, f16_labels, kF16Threads, kF16StreamSmemBytes) !=
+            cudaSuccess)
+        return CH_ECUDA;
     {
         ProfScope p("filter16_extremes", s);
         const int grid = (int)std::min<long long>(want, (long long)sms * std::max(1, occ_e));

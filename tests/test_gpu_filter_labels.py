@@ -65,7 +65,7 @@ def test_one_read_bad_coordinate(lib, bad):
 
 
 @pytest.mark.parametrize("fn", ["ch_filter", "ch_filter_manhattan"])
-@pytest.mark.parametrize("n", [1, 511, 513, 1025, 70_001])
+@pytest.mark.parametrize("n", [1, 511, 513, 70_001, (1 << 21) + 1, (1 << 21) + 515])
 @pytest.mark.parametrize("shift", [0, 1])
 @pytest.mark.parametrize("off", [0, 1, 2, 3])
 def test_label_offsets(lib, fn, n, shift, off):
@@ -73,7 +73,7 @@ def test_label_offsets(lib, fn, n, shift, off):
     check((F.extremes(pts), F.labels(pts)), run(lib, fn, 8, pts, shift, off))
 
 
-@pytest.mark.parametrize("n", [1, 2, 511, 513, 1025, 70_001])
+@pytest.mark.parametrize("n", [1, 2, 511, 513, 70_001, (1 << 21) + 1, (1 << 21) + 515])
 @pytest.mark.parametrize("shift", [0, 1])
 @pytest.mark.parametrize("off", [0, 1, 2, 3])
 def test_label_offsets16(lib, n, shift, off):
