@@ -27,12 +27,6 @@ import time
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# Kernels per replayed hull: the filter part (init, sample, main, post) always;
-# the large-survivor part (8 bucket kernels, the sort's histogram and 3 passes,
-# which return at once on the bucketed path, and the chain merge) only when the
-# post pass raised its graph condition.
-FILTER_LAUNCHES = 4   # init, sample, main, post (the star pass adds one on large inputs)
-LARGE_LAUNCHES = 13   # bk_prep, bk_hist, bk_bsum, bk_bstart, bk_items, bk_part1, bk_part2, bk_hull, sort_hist, 3 sort passes, chain
 L2_BYTES = 129 * 1024 * 1024
 HBM_NOMINAL_GBS = 7900.0   # GB300 HBM3e, nominal (context beside the measured copy bandwidth)
 # One metric name for both arms (GPU library and the oracle's reference arm),
@@ -136,7 +130,10 @@ def algorithmic_bytes(n, counters):
     raw, m, two_pass = counters["raw"], counters["records"], counters["two_pass"]
     out = {"main_filter": 8.0 * n + 12.0 * raw,
            "post": (8.0 * n if two_pass else 12.0 * raw) + 12.0 * m}
+    if counters.get("star_vertices"):   # dense data: the dense pass reads the points, the main pass nothing
+        out = {"dense_filter": 8.0 * n + 12.0 * raw, "post": 12.0 * raw + 12.0 * m}
     if counters["stage"] >= 1:
+        out["large"] = 12.0 * m
         out.update({"bk_hist": 4.0 * m, "bk_part1": 24.0 * m, "bk_part2": 24.0 * m, "bk_hull": 12.0 * m})
     return out
 
@@ -386,12 +383,9 @@ def run_ours(args):
     kernels["_region"] = f"{prof_steps} profiled steps after the timed region"
     for k, v in per_kernel.items():
         kernels[k].update({kk: v[kk] for kk in ("algorithmic_bytes", "achieved_gbs", "frac_of_measured_hbm")})
-    # Kernels of a replayed step: the filter part, the star pass on its side
-    # branch when the input has enough tiles for it, and the large-survivor
-    # part when the call's counters say it ran (its graph node is skipped
-    # otherwise).
-    large = counters.get("stage", 0) >= 1
-    launches_per_step = FILTER_LAUNCHES + (1 if "star" in prof else 0) + (LARGE_LAUNCHES if large else 0)
+    # Kernels of a replayed step: one per profiled scope and step (those that the
+    # call's data do not need return at once, and are launches all the same).
+    launches_per_step = sum(v[0] for v in prof.values()) // max(prof_steps, 1)
 
     step_bytes = sum(v["algorithmic_bytes"] for v in per_kernel.values())
     step_roof = {"algorithmic_bytes": step_bytes, "achieved_gbs": step_bytes / (ms / args.steps / 1e3) / 1e9,
@@ -544,12 +538,13 @@ def run_filters(ch, torch, args, pts, n, sp, peak):
     """The filter on its own (labels and queue sizes) with the octagon
     (ch_filter) and with the 16-direction polygon (ch_filter16), on the
     resident input: device time per call, points kept, and the HBM fraction
-    of each pass (8 bytes a point read; the label pass also writes 1)."""
+    of each pass (8 bytes a point read; the pass that labels also writes 1:
+    ch_filter's only pass over a large input, the others' second)."""
     labels = torch.empty(max(n, 1), dtype=torch.uint8, device="cuda")
     counts = torch.empty(4, dtype=torch.int64, device="cuda")
     ext = torch.empty(16, dtype=torch.int32, device="cuda")
     out = {}
-    for name, fn, passes in (("octagon", ch.ch_filter, {"main_filter": 8.0, "labels": 9.0}),
+    for name, fn, passes in (("octagon", ch.ch_filter, {"main_filter": 9.0}),
                              ("octagon, two-kernel Manhattan extremes", ch.ch_filter_manhattan,
                               {"manhattan_axis": 8.0, "manhattan_corner": 8.0, "labels": 9.0}),
                              ("16-gon", ch.ch_filter16, {"filter16_extremes": 8.0, "filter16_labels": 9.0})):

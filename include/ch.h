@@ -252,10 +252,11 @@ int ch_reserve(int64_t n, int32_t k, void* stream);
  *   out[1]  sort records handed to the hull stage (the chain end points
  *           included): the survivors of the filter,
  *   out[2]  0 when the fused streaming pass did the extremes and the octagon
- *           filter; 1 when a second pass did the filter (small inputs, and
- *           dense data without a star polygon) or a star polygon did (out[5]),
- *   out[3]  hull stage: 0 finished by one block (few records), 1 bucketed
- *           chains, 2 the radix-sort fallback,
+ *           filter; 1 when a second pass did the filter (inputs of at most
+ *           2^22 points, and dense data without a star polygon) or a star
+ *           polygon did (out[5]),
+ *   out[3]  hull stage: 0 finished by one block (few records), 1 chains queue
+ *           by queue or by tiles of a queue, 2 the radix sort,
  *   out[4]  the call's status (CH_OK or the negative code it reported),
  *   out[5]  vertices of the star polygon that filtered dense data, those in
  *           its reflex dents (dropped before use) included (0 when the call

@@ -10,7 +10,8 @@
 //                set (Alg. 2, findExtremes) as packed (key, ~tile) maxima;
 //   bt_octagon   one block per set: the lowest index of each extreme (a
 //                rescan of its tile), octagon, inner region, chain end-point
-//                records; the density test that lists a set for a polygon;
+//                records; the density test that lists a set for a polygon
+//                (a small dense set's points are classified at once);
 //   bt_star_bin, bt_star_build  the listed sets' angular bins and star
 //                polygons (star.cuh; points near a circle, Table V);
 //   bt_dense     the filter of the sets with a polygon: runs of their points

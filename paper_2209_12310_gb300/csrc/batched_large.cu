@@ -1,6 +1,6 @@
 // batched_large.cu -- the sets of a batch whose survivors exceed one block,
-// all at once (the bucketed large-survivor path of bucket.cu and hull.cu,
-// segmented by set).  A segment is one (set, queue) pair.
+// all at once: buckets of equal width in u, a warp's chain per bucket and a
+// merge tree, segmented by set.  A segment is one (set, queue) pair.
 //   btl_prep     per segment: bucket count from its record count, bucket and
 //                chain-tile offsets (prefix over all segments), the bucket
 //                map (u range, scale); record tiles per set;

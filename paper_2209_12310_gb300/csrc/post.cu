@@ -128,7 +128,7 @@ __device__ __forceinline__ void flush_queue_counts(QueueTally& tally, Ctl* ctl) 
 // verdict, or more than a quarter of the points kept) the records are near the hull, mostly
 // vertices, and past kNearHullRec of them they would outgrow
 // the quickhull rounds' vertex capacity: the queues then, a block each (one
-// million points of a ring: 27,265 records, 13,024 vertices: queue_kernel takes
+// million points of a ring: 27,265 records, 13,024 vertices: large_kernel takes
 // the place of a partition into buckets, a warp's quickhull per bucket and a
 // radix sort when their chains overflow).  The sort takes what neither a
 // block nor the tiles are for: a queue too large for a block among few
