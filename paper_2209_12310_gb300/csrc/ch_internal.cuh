@@ -134,12 +134,15 @@ struct Ctl {
     int mode;                           // 0: fused single pass, 1: two streaming passes
     int done;                           // the hull has been written by a small-path block
     int records_ready;                  // sort records complete before the re-classify stage
-    unsigned int blocks_done[4];        // last-arriver counters (sample, main, stage C, roots)
+    unsigned int blocks_done[4];        // last-arriver counters (sample, main, post, a batched set's queues)
     unsigned int barrier[3];            // grid barriers (dense_kernel, large_kernel, sort_kernel)
     unsigned int tile_ctr[4];           // onesweep tile claim counters (0 .. 2), the sorted tiles' (3)
     unsigned int digit_hist[kSortPasses][kDigits];   // sort path only (sort_kernel)
     unsigned int rec_q[4];              // records per queue
     unsigned int reg_end[4];            // chain length of queue r (large_kernel, bt_queue_chain)
+    unsigned int joins_done;            // large_kernel: queues whose chain stands (or did not fit)
+    int join_over;                      // large_kernel: a queue's tile chains outgrew its block
+    unsigned int roots_done;            // sort_kernel: queue roots of the merge tree
     unsigned int counts4[4];            // survivors per queue (ch_filter)
     unsigned long long line_ep[8];      // end points of survivors on the 4 axis support lines
     int bk_state;                       // large-survivor path: 0 unused, 1 queues / tiles / buckets, 2 full sort

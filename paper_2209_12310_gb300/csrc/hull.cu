@@ -161,11 +161,10 @@ __global__ void __launch_bounds__(kChainThreads) sort_kernel(Ctl* ctl, uint32_t*
         // 5) the block completing the fourth queue root joins the chains.
         __threadfence();
         __syncthreads();
-        if (tid == 0) s_old = (int)atomicAdd(&ctl->blocks_done[3], 1u);
+        if (tid == 0) s_old = (int)atomicAdd(&ctl->roots_done, 1u);
         __syncthreads();
         if (s_old != 3) continue;
         __threadfence();
-        if (tid == 0) ctl->blocks_done[3] = 0u;
         int off[5];
         off[0] = 0;
         for (int q = 0; q < 4; ++q) off[q + 1] = off[q] + __ldcg(hb.clen + s_tb[q]) - 1;

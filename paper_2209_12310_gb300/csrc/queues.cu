@@ -273,7 +273,7 @@ static_assert(kLargeSmem <= 226 * 1024 && QcJoin::kCap < (1 << kQcPosBits), "one
 __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ QMap s_m;
-    __shared__ int s_path, s_n, s_last;
+    __shared__ int s_path, s_go, s_n, s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, qq = blockIdx.x;
     constexpr int T = kLargeThreads;
     Ctl* ctl = a.ctl;
@@ -302,7 +302,13 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
         CH_TL(ctl, 18, 1);
         go = go && grid_barrier(&ctl->barrier[1], 4u, ctl);
         if (!go && tid == 0) *a.out_n = CH_ETIMEOUT;
-        if (!go || qq >= 4 || *(volatile int*)&ctl->bk_state != 1) return;
+        if (!go || qq >= 4) return;
+        // A tile's chain that outgrew its block has set bk_state before the barrier;
+        // after it the word stays as it is until all four blocks have arrived
+        // below, so they agree on it (one read per block: its warps too).
+        if (tid == 0) s_go = *(volatile int*)&ctl->bk_state == 1;
+        __syncthreads();
+        if (!s_go) return;
     }
     const uint32_t* keys = a.keys;
     const uint64_t* vals = a.vals;
@@ -378,15 +384,17 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
     CH_TL(ctl, 21, 1);
     if (tid == 0) {
         ctl->reg_end[qq] = ok ? (unsigned)len : 0u;
-        if (!ok) ctl->bk_state = 2;   // the sort takes over (its input is untouched)
+        if (!ok) atomicExch(&ctl->join_over, 1);
     }
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-        s_last = atomicAdd(&ctl->blocks_done[3], 1u) == 3u;
-        if (s_last) ctl->blocks_done[3] = 0u;
+        s_last = atomicAdd(&ctl->joins_done, 1u) == 3u;
         __threadfence();
-        if (*(volatile int*)&ctl->bk_state != 1) s_last = 0;
+        if (s_last && *(volatile int*)&ctl->join_over) {
+            ctl->bk_state = 2;   // the sort takes over (its input is untouched)
+            s_last = 0;
+        }
     }
     __syncthreads();
     if (!s_last) return;

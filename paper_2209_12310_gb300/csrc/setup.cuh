@@ -35,6 +35,9 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
         ctl->records_ready = 0;
         ctl->bk_state = 0;
         ctl->path = kPathNone;
+        ctl->joins_done = 0u;
+        ctl->join_over = 0;
+        ctl->roots_done = 0u;
         ctl->samp_dense = 0;
         ctl->oct_ready = 0;
         ctl->star_ok = 0;

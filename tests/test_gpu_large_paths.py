@@ -1,0 +1,91 @@
+"""The single hull's ways through many survivors (queues.cu, hull.cu), each by
+the counters that name it and bit-exact with the oracle: circles without a
+width, whose queues' tile chains fit one block or hand over to the sort, and a
+tile whose own chain does."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+QUEUES_OR_TILES, SORT = 1, 2   # ch_hull_counters' stage
+
+
+def _circle(n, seed):
+    """n points of a circle, rounded: a queue's chain has about 10,400
+    vertices at 1e6 points, 13,700 at 4e6 (the oracle's)."""
+    a = np.random.default_rng(seed).uniform(0.0, 2.0 * math.pi, n)
+    r = float(1 << 23)
+    pts = np.stack([np.cos(a), np.sin(a)], 1) * r + r
+    return np.clip(np.rint(pts), 0, (1 << 24) - 1).astype(np.float32)
+
+
+def _calls(lib, pts, calls):
+    """Results and counters of calls on the same buffers (launched, captured,
+    replayed); out_idx is cleared in between."""
+    d = torch.from_numpy(pts).cuda()
+    out_idx = torch.empty(pts.shape[0], dtype=torch.int32, device="cuda")
+    out_n = torch.empty(1, dtype=torch.int64, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    for _ in range(calls):
+        out_idx.fill_(-7)
+        got = lib.hull(d, out_idx=out_idx, out_n=out_n)
+        yield got.cpu().numpy(), lib.ch_hull_counters(stream)
+
+
+@pytest.mark.parametrize("n,stage", [(1_000_000, QUEUES_OR_TILES), (4_000_003, SORT), (6_000_001, SORT)])
+def test_circle(lib, n, stage):
+    pts = _circle(n, n)
+    want = oracle.hull(pts)
+    # past 13,000 tile-chain points in a queue (a block's capacity) the sort takes over
+    assert (want.size > 4 * 13_000) == (stage == SORT)
+    for got, c in _calls(lib, pts, 100):
+        np.testing.assert_array_equal(got, want)
+        assert c["stage"] == stage, c
+
+
+def _steps(most_u, most_v, ok):
+    """Steps (du, dv) between points in the queue frame, one per slope, by slope."""
+    low = -most_v if most_v <= most_u else 0
+    got = [(du, dv) for du in range(1, most_u + 1) for dv in range(low, most_v + 1)
+           if (du + dv) % 2 == 0 and ok(du, dv) and math.gcd((dv + du) // 2, (dv - du) // 2) == 1]
+    return np.array(sorted(got, key=lambda s: s[1] / s[0]))
+
+
+def _long_tile(n):
+    """About n points beyond the upper right side of a triangle (its box's centre
+    is outside the hull: no star polygon).  In their queue's frame: a convex curve
+    of 9834 points, the 5229 falling ones once, the 4605 others, which lie
+    in one of the queue's 1024 equal u ranges, many times each."""
+    top = (1 << 24) - 1
+    fall = _steps(250, 250, lambda u, v: -0.55 * u < v < 0)
+    rise = _steps(20, 1600, lambda u, v: v > 0 and u / 19 + v / 1600 <= 1)
+    low = int(top * (math.sqrt(2.0) - 1.0))
+    start = np.array([int(math.ceil(-top + 512 * (2 * top + 1) / 1024)) + 600, low + 3000])
+    start[1] += (start[0] + start[1]) & 1
+    up = start + np.concatenate([[[0, 0]], np.cumsum(rise, axis=0)])
+    down = start - np.cumsum(fall[::-1], axis=0)
+
+    def xy(p):
+        return np.stack([(p[:, 1] + p[:, 0]) // 2, (p[:, 1] - p[:, 0]) // 2], 1)
+
+    corners = [np.array([[0, top], [top, 0], [low - 1000, 1000]])] * 2000
+    pts = np.concatenate(corners + [xy(down)] + [xy(up)] * ((n - 12_000) // len(up)))
+    pts = (top - pts)[np.random.default_rng(n).permutation(pts.shape[0])]
+    assert len(down) < 5900 and len(down) + len(up) > 9800 and pts.min() >= 0
+    return pts.astype(np.float32)
+
+
+@pytest.mark.parametrize("n", [905_000, 4_520_000])   # the extremes first, a sample first
+def test_tile_chain_over_its_block(lib, n):
+    """A tile of u ranges whose chain so far leaves its block no room for the
+    rest of its records; dense data without a star polygon."""
+    pts = _long_tile(n)
+    want = oracle.hull(pts)
+    for got, c in _calls(lib, pts, 10):
+        np.testing.assert_array_equal(got, want)
+        assert c["stage"] == SORT and c["star_vertices"] == 0 and c["two_pass"] == 1, c
