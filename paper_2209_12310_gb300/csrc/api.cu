@@ -62,13 +62,13 @@ Layout make_layout(long long n) {
         return r;
     };
     // zeroed at allocation: the control block, the sort's look-back status
-    // words, the merge tree's arrival counters and the tile
-    // counters (each kernel leaves them in that state for the next call)
+    // words and the merge tree's arrival counters (each kernel leaves them in that
+    // state for the next call)
     L.off_ctl = take(sizeof(Ctl));
     L.off_status = take(8 * (size_t)kDigits * L.sort_tiles);
     L.off_counters = take(4 * (size_t)kMaxLevels * L.ctcap);
-    L.off_tiles = take(tiles_bytes());           // large_kernel leaves its counters at zero
     L.zero_bytes = o;
+    L.off_tiles = take(tiles_bytes());
     // inputs that dense_kernel can take (device-independent: at most kStarBlocks
     // blocks of it run)
     const bool star = n / kWarpTilePts >= kStarMinTiles;
@@ -239,7 +239,7 @@ static void prof_drain() {
 // of kernels, each of which returns at once when the call does not need it (the
 // dense part on sparse data, the main pass on dense data, the large-survivor
 // paths not taken).  What a call may need beyond the sparse path is packed in
-// three cooperative kernels with grid barriers inside: an empty launch costs
+// three kernels whose blocks wait for one another inside: an empty launch costs
 // about 2 us, and a conditional graph node about 7 (measured on 65,537 points:
 // 50 us a call with one such node, 57 with two).
 static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, int64_t* out_n, cudaStream_t s,
@@ -250,6 +250,7 @@ static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, 
     Ctl* ctl = (Ctl*)(base + L.off_ctl);
     uint32_t *kA = (uint32_t*)(base + L.off_kA), *kB = (uint32_t*)(base + L.off_kB);
     uint64_t *vA = (uint64_t*)(base + L.off_vA), *vB = (uint64_t*)(base + L.off_vB);
+    unsigned* tiles = (unsigned*)(base + L.off_tiles);
     const int head = ((uintptr_t)pts & 15u) != 0u ? 1 : 0;
     const long long ntiles = (n - head) / kWarpTilePts;
     const long long samples = sample_tiles_host(ntiles);
@@ -284,9 +285,8 @@ static int enqueue_hull_direct(const float* pts, long long n, int32_t* out_idx, 
     }
     if (!one_block) {
         ProfScope p("post", s);
-        launch_post(pts, n, head, ntiles, ctl, vB, kB, kA, vA, out_idx, out_n, di.sms * di.occ_post, s);
+        launch_post(pts, n, head, ntiles, ctl, vB, kB, kA, vA, tiles, out_idx, out_n, di.sms * di.occ_post, s);
     }
-    unsigned* tiles = (unsigned*)(base + L.off_tiles);
     int *cu = (int*)(base + L.off_cu), *cv = (int*)(base + L.off_cv), *ci = (int*)(base + L.off_ci);
     const bool large = n + 16 > kQueueCap;   // else every queue fits a block
     {

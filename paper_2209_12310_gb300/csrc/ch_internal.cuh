@@ -96,7 +96,15 @@ __host__ __device__ __forceinline__ long long sample_tiles(long long ntiles) {
 constexpr float kEdgeTol = 268435456.0f;      // 2^28
 constexpr float kHugePositive = 1.0e30f;      // "always inside" coefficient of a skipped edge
 
-constexpr unsigned kSpinLimit = 1u << 20;     // bounded waits (onesweep look-back)
+constexpr unsigned kSpinLimit = 1u << 20;     // polls of a bounded wait (of a phase: without progress)
+
+// Phases of dense_kernel, large_kernel and sort_kernel whose end their blocks
+// wait for (claim_item, wait_phase).
+enum Phase {
+    kDenseBins = 0, kDenseMerge, kDensePoly, kDenseRadius,
+    kLargeHist, kLargeCut, kLargePart, kLargeChains,
+    kSortHist, kSortPass, kPhases = kSortPass + kSortPasses
+};
 
 // Directions of the 8 extremes in counter-clockwise octagon order.
 enum Dir { W = 0, SW, S, SE, E, NE, N, NW };
@@ -135,8 +143,9 @@ struct Ctl {
     int done;                           // the hull has been written by a small-path block
     int records_ready;                  // sort records complete before the re-classify stage
     unsigned int blocks_done[4];        // last-arriver counters (sample, main, post, a batched set's queues)
-    unsigned int barrier[3];            // grid barriers (dense_kernel, large_kernel, sort_kernel)
-    unsigned int tile_ctr[4];           // onesweep tile claim counters (0 .. 2), the sorted tiles' (3)
+    unsigned int claimed[kPhases];      // items of a phase that blocks have taken,
+    unsigned int finished[kPhases];     // and finished
+    unsigned int beat;                  // progress within long items
     unsigned int digit_hist[kSortPasses][kDigits];   // sort path only (sort_kernel)
     unsigned int rec_q[4];              // records per queue
     unsigned int reg_end[4];            // chain length of queue r (large_kernel, bt_queue_chain)
@@ -256,24 +265,56 @@ __device__ __forceinline__ bool spin_give_up(unsigned& spins, Ctl* ctl) {
     return false;
 }
 
-// Grid-wide barrier of a cooperative launch (all its blocks are resident): the
-// k-th (k = 1, 2, ...) use of the counter, which starts at zero.  Every wait is
-// bounded: false when it gave up (status CH_ETIMEOUT), and the kernel returns.
-// Whole block.
-__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned k, Ctl* ctl) {
-    __shared__ int s_ok;
+// Work of a phase that the whole grid shares.  Running blocks claim its items
+// one at a time until none is left and then wait for the phase's end, so a wait
+// is only ever for items that running blocks hold: it ends whatever share of the
+// grid is resident.  (Cooperative launches with grid barriers instead started
+// only once every SM was free, so that one block of another stream's kernel
+// held up the whole call, and a kernel that waited for the call's result never
+// saw it.)  All three: whole block.
+__device__ __forceinline__ unsigned claim_item(Ctl* ctl, int phase) {
+    __shared__ unsigned s_item;
+    __syncthreads();
+    if (threadIdx.x == 0) s_item = atomicAdd(&ctl->claimed[phase], 1u);
+    __syncthreads();
+    return s_item;
+}
+
+// The block's writes for n items stand; true in the one block that finishes the
+// phase's last (it sees the writes of all).
+__device__ __forceinline__ bool finish_items(Ctl* ctl, int phase, unsigned n, unsigned items) {
+    __shared__ int s_end;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned target = k * gridDim.x;
-        unsigned spins = 0u;
+        s_end = atomicAdd(&ctl->finished[phase], n) + n == items;
+        __threadfence();
+    }
+    __syncthreads();
+    return s_end != 0;
+}
+
+// Bounded: false when the wait gave up (status CH_ETIMEOUT), after kSpinLimit
+// polls in which no item of the phase was taken or finished and no block
+// reported progress within one (ctl->beat).
+__device__ __forceinline__ bool wait_phase(Ctl* ctl, int phase, unsigned items) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        volatile unsigned *claimed = &ctl->claimed[phase], *finished = &ctl->finished[phase], *beat = &ctl->beat;
+        unsigned spins = 0u, seen = 0u;
         s_ok = 1;
-        atomicAdd(counter, 1u);
-        while (*(volatile unsigned*)counter < target)
+        while (*finished < items) {
             if (spin_give_up(spins, ctl)) {
                 s_ok = 0;
                 break;
             }
+            if ((spins & 1023u) == 0u) {
+                const unsigned now = *claimed + *finished + *beat;
+                if (now != seen) spins = 0u;
+                seen = now;
+            }
+        }
         __threadfence();
     }
     __syncthreads();

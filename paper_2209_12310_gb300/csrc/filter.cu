@@ -640,8 +640,8 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// The main pass on dense data (points near a circle, Table V), one cooperative
-// launch of one block per SM:
+// The main pass on dense data (points near a circle, Table V), one launch of one
+// block per SM with waits between its phases (claim_item, wait_phase):
 //   1. the angular bins of the star polygon (star.cuh), per block in shared
 //      memory: a warp tile per warp, spread over the input.  Every point
 //      outside oct_s goes to its angular bin around that octagon's centre c,
@@ -830,44 +830,22 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
             s_edge[3 * tid + 1] = os.oct[tid].B;
             s_edge[3 * tid + 2] = os.oct[tid].C;
         }
-        __syncthreads();
         unsigned long long* mine = reinterpret_cast<unsigned long long*>(dsm);
-        for (int b = tid; b < kStarBins; b += kDenseThreads) mine[b] = 0ull;
-        __syncthreads();
-        const long long nt = min(ntiles, (long long)gridDim.x * kWarps), k = blockIdx.x + (long long)gridDim.x * warp;
-        if (k < nt)
-            star_tile_pass(p4, ((2 * k + 1) * ntiles) / (2 * nt), head, s_in, s_edge, cx, cy, mine, l2_evict_first());
-        __syncthreads();
-        for (int b = tid; b < kStarBins; b += kDenseThreads) bins[(size_t)blockIdx.x * kStarBins + b] = mine[b];
-        CH_TL(ctl, 7, 1);
-        if (!grid_barrier(&ctl->barrier[0], 1u, ctl)) return;
-    }
-    // 2. polygon: every block merges some bins and re-reads their points, one block makes the polygon of them, every block finds
-    // some bins' radius bounds
-    {
-        // 64 consecutive bins at a time, 16 threads each over the blocks' bins
-        constexpr int kSlots = 64, kGroups = kDenseThreads / kSlots;
-        unsigned long long* part = reinterpret_cast<unsigned long long*>(dsm);
-        const int slot = tid % kSlots, grp = tid / kSlots;
-        for (int b0 = (int)blockIdx.x * kSlots; b0 < kStarBins; b0 += (int)gridDim.x * kSlots) {
-            unsigned long long key = 0ull;
-            for (int g = grp; g < (int)gridDim.x; g += kGroups) {
-                const unsigned long long x = __ldcg(bins + (size_t)g * kStarBins + b0 + slot);
-                key = x > key ? x : key;
-            }
-            part[tid] = key;
+        const long long nt = min(ntiles, (long long)gridDim.x * kWarps);
+        for (unsigned g; (g = claim_item(ctl, kDenseBins)) < gridDim.x;) {   // gridDim.x shares
+            for (int b = tid; b < kStarBins; b += kDenseThreads) mine[b] = 0ull;
             __syncthreads();
-            if (tid < kSlots) {
-#pragma unroll
-                for (int g = 1; g < kGroups; ++g) key = part[g * kSlots + tid] > key ? part[g * kSlots + tid] : key;
-                merged[b0 + tid] = star_vertex(key, star_point(key, pts, n), b0 + tid, cx, cy);
-            }
+            const long long k = g + (long long)gridDim.x * warp;
+            if (k < nt)
+                star_tile_pass(p4, ((2 * k + 1) * ntiles) / (2 * nt), head, s_in, s_edge, cx, cy, mine, l2_evict_first());
             __syncthreads();
+            for (int b = tid; b < kStarBins; b += kDenseThreads) bins[(size_t)g * kStarBins + b] = mine[b];
+            finish_items(ctl, kDenseBins, 1u, gridDim.x);
         }
+        CH_TL(ctl, 7, 1);
+        if (!wait_phase(ctl, kDenseBins, gridDim.x)) return;
     }
-    CH_TL(ctl, 14, 1);
-    if (!grid_barrier(&ctl->barrier[0], 2u, ctl)) return;
-    if (blockIdx.x == 0) {
+    auto make_polygon = [&]() {
         StarPoly& M = *reinterpret_cast<StarPoly*>(dsm);
         unsigned long long* work = reinterpret_cast<unsigned long long*>(dsm + kDenseWorkOff);
         constexpr int kPer = kStarBins / kDenseThreads;
@@ -897,18 +875,46 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
             ctl->star_final = K ? 1 : 0;
         }
         CH_TL(ctl, 8, 1);
+    };
+    // 2. polygon: the blocks merge the bins and re-read their points, the one that
+    // finishes last makes the polygon of them, the blocks find the bins' radius bounds
+    {
+        // 64 consecutive bins at a time, 16 threads each over the blocks' bins
+        constexpr int kSlots = 64, kGroups = kDenseThreads / kSlots;
+        constexpr unsigned kItems = kStarBins / kSlots;
+        unsigned long long* part = reinterpret_cast<unsigned long long*>(dsm);
+        const int slot = tid % kSlots, grp = tid / kSlots;
+        for (unsigned it; (it = claim_item(ctl, kDenseMerge)) < kItems;) {
+            const int b0 = (int)it * kSlots;
+            unsigned long long key = 0ull;
+            for (int g = grp; g < (int)gridDim.x; g += kGroups) {
+                const unsigned long long x = __ldcg(bins + (size_t)g * kStarBins + b0 + slot);
+                key = x > key ? x : key;
+            }
+            part[tid] = key;
+            __syncthreads();
+            if (tid < kSlots) {
+#pragma unroll
+                for (int g = 1; g < kGroups; ++g) key = part[g * kSlots + tid] > key ? part[g * kSlots + tid] : key;
+                merged[b0 + tid] = star_vertex(key, star_point(key, pts, n), b0 + tid, cx, cy);
+            }
+            if (!finish_items(ctl, kDenseMerge, 1u, kItems)) continue;
+            CH_TL(ctl, 14, 1);
+            make_polygon();
+            finish_items(ctl, kDensePoly, 1u, 1u);
+        }
     }
-    if (!grid_barrier(&ctl->barrier[0], 3u, ctl)) return;
-    const int K = *(volatile int*)&ctl->star_edges;
+    if (!wait_phase(ctl, kDensePoly, 1u)) return;
+    const int K = *(volatile int*)&ctl->star_edges;   // the same for all from here on
     if (!K) return;
     {   // kStarWindow threads per bin, an edge of its window each
         constexpr int kSlots = kDenseThreads / kStarWindow;
+        constexpr unsigned kItems = kStarBins / kSlots;
         const int k = tid % kStarWindow;
-        for (int b0 = (int)blockIdx.x; b0 < kStarBins; b0 += (int)gridDim.x * kSlots) {
-            const int b = b0 + tid / kStarWindow * (int)gridDim.x;
-            const bool some = b < kStarBins;
+        for (unsigned it; (it = claim_item(ctl, kDenseRadius)) < kItems;) {
+            const int b = (int)it * kSlots + tid / kStarWindow;
             int first, count;
-            star_window(poly->tbl, K, some ? b : 0, first, count);
+            star_window(poly->tbl, K, b, first, count);
             unsigned r = 0xFFFFFFFFu;
             if (k < count && count <= kStarWindow) {
                 const int e = first + k < K ? first + k : first + k - K;
@@ -916,10 +922,11 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
             }
 #pragma unroll
             for (int d = kStarWindow / 2; d; d >>= 1) r = min(r, __shfl_xor_sync(0xFFFFFFFFu, r, d));
-            if (some && k == 0) poly->thr[b] = star_threshold(count <= kStarWindow ? r : 0u);
+            if (k == 0) poly->thr[b] = star_threshold(count <= kStarWindow ? r : 0u);
+            finish_items(ctl, kDenseRadius, 1u, kItems);
         }
+        if (!wait_phase(ctl, kDenseRadius, kItems)) return;
     }
-    if (!grid_barrier(&ctl->barrier[0], 4u, ctl)) return;
     CH_TL(ctl, 12, 1);
     // 3. the filter
     float* thr = reinterpret_cast<float*>(dsm);
@@ -1163,8 +1170,8 @@ void launch_main_labels(const float* pts, long long n, int head, long long ntile
 
 void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, void* bins, void* poly,
                   uint64_t* raw_xy, uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int sms, cudaStream_t s) {
-    launch_grid(dense_kernel, sms, kDenseThreads, kDenseSmemBytes, s, pts, n, head, ntiles, ctl,
-                (unsigned long long*)bins, (StarPoly*)poly, raw_xy, raw_idx, keys, vals);
+    dense_kernel<<<sms, kDenseThreads, kDenseSmemBytes, s>>>(pts, n, head, ntiles, ctl, (unsigned long long*)bins,
+                                                             (StarPoly*)poly, raw_xy, raw_idx, keys, vals);
 }
 
 size_t star_bins_bytes(int sms) { return sizeof(unsigned long long) * kStarBins * ((size_t)sms + 1); }

@@ -1,5 +1,5 @@
 // hull.cu -- the large-survivor path by sort: the radix sort (sort.cuh) and the
-// hull of the sorted survivors, in one cooperative launch.
+// hull of the sorted survivors, in one launch.
 //
 // The paper ends with "for i = 1..4: CH <- CH U hull(Q_i, n_i)" (Alg. 1): one
 // hull per queue, joined.  Here every queue r is a chain from quad vertex r
@@ -73,14 +73,10 @@ __global__ void __launch_bounds__(kChainThreads) sort_kernel(Ctl* ctl, uint32_t*
     if (go) {
         if (*(volatile int*)&ctl->bk_state != 2) return;
         SortSmem& sm = *reinterpret_cast<SortSmem*>(smem);
-        sort_hist(reinterpret_cast<unsigned(*)[kDigits]>(smem), kA, ctl);
-        go = grid_barrier(&ctl->barrier[2], 1u, ctl);
-        if (go) onesweep(sm, kA, vA, kB, vB, ctl, status, 0);
-        go = go && grid_barrier(&ctl->barrier[2], 2u, ctl);
-        if (go) onesweep(sm, kB, vB, kA, vA, ctl, status, 1);
-        go = go && grid_barrier(&ctl->barrier[2], 3u, ctl);
-        if (go) onesweep(sm, kA, vA, kB, vB, ctl, status, 2);
-        go = go && grid_barrier(&ctl->barrier[2], 4u, ctl);
+        go = wait_phase(ctl, kSortHist, sort_hist(reinterpret_cast<unsigned(*)[kDigits]>(smem), kA, ctl));
+        if (go) go = wait_phase(ctl, kSortPass, onesweep(sm, kA, vA, kB, vB, ctl, status, 0));
+        if (go) go = wait_phase(ctl, kSortPass + 1, onesweep(sm, kB, vB, kA, vA, ctl, status, 1));
+        if (go) go = wait_phase(ctl, kSortPass + 2, onesweep(sm, kA, vA, kB, vB, ctl, status, 2));
     }
     if (__syncthreads_or(!go || read_status(ctl) != CH_OK)) {   // a wait gave up: report it
         if (threadIdx.x == 0) *hb.out_n = read_status(ctl);
@@ -219,7 +215,7 @@ void launch_sort(Ctl* ctl, uint32_t* kA, uint64_t* vA, uint32_t* kB, uint64_t* v
     // its chains are built: the stitch's scratch
     const HullBufs hb{kB, vB, cu, cv, ci, clen, counters, ctcap, (int*)vA, (int*)kA, (int*)kB, (int*)vB, pts, n, out_idx,
                       out_n};
-    launch_grid(sort_kernel, grid, kChainThreads, chain_smem_bytes(), s, ctl, kA, vA, kB, vB, status, hb);
+    sort_kernel<<<grid, kChainThreads, chain_smem_bytes(), s>>>(ctl, kA, vA, kB, vB, status, hb);
 }
 
 cudaError_t configure_hull_kernels() {

@@ -9,23 +9,6 @@ namespace ch {
 
 struct Ctl;
 
-// Cooperative launch: every block is resident, so the blocks may meet at grid
-// barriers.  Errors are left for cudaGetLastError.
-template <typename... KArgs, typename... Args>
-inline void launch_grid(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeCooperative;
-    attr.val.cooperative = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
 // Launch of a kernel that may start before the stream's last kernel ends: as soon
 // as every block of that one has executed griddepcontrol.launch_dependents (or
 // ended).  The kernel itself ends with griddepcontrol.wait, so that what follows
@@ -62,8 +45,8 @@ void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl
 void launch_small(const float* pts, long long n, Ctl* ctl, uint32_t* keys, uint64_t* vals, int32_t* out_idx,
                   int64_t* out_n, cudaStream_t s);
 void launch_post(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
-                 const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n,
-                 int grid, cudaStream_t s);
+                 const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, unsigned* tiles, int32_t* out_idx,
+                 int64_t* out_n, int grid, cudaStream_t s);
 void launch_labels(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
                    const uint32_t* raw_idx, uint8_t* labels, int grid, cudaStream_t s);
 size_t star_bins_bytes(int sms);   // a block's bins each, and the merged ones
@@ -71,7 +54,8 @@ size_t star_poly_bytes();
 void launch_filter_output(const Ctl* ctl, long long n, int32_t* out_ext8, int64_t* out_counts4, cudaStream_t s);
 
 // The large-survivor path without a sort (queues.cu); tiles: tiles_bytes() of
-// the workspace, its first kPtGroups words zero at rest.
+// the workspace, its first kPtGroups words the records per group, which the post
+// pass clears when it picks the tiles.
 void launch_large(Ctl* ctl, const uint32_t* kA, const uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned* tiles, int* cu,
                   int* cv, int* ci, long long n, int32_t* out_idx, int64_t* out_n, int grid, cudaStream_t s);
 size_t tiles_bytes();

@@ -12,6 +12,7 @@
 #include "hullcore.cuh"
 #include "launch.h"
 #include "octagon.cuh"
+#include "partition.cuh"
 #include "records.cuh"
 #include "setup.cuh"
 
@@ -21,6 +22,7 @@ namespace ch {
 
 constexpr int kPostThreads = 512;
 static_assert(kPostThreads % 128 == 0, "mid_hull splits the block in four");
+static_assert(kSmallMax + 16 <= kQueueCap, "small_kernel's queues fit a block");
 
 // Records are staged per warp in shared memory; a full buffer goes out with
 // one atomic on the record counter, and at the end the block's remainders go
@@ -137,14 +139,14 @@ __device__ __forceinline__ void flush_queue_counts(QueueTally& tally, Ctl* ctl) 
 constexpr unsigned kNearHullRec = 512;
 
 __device__ void post_last_block(const float* __restrict__ pts, long long n, Ctl* ctl, const Octagon& o,
-                                uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n, char* dyn,
-                                bool dense) {
+                                uint32_t* keys, uint64_t* vals, unsigned* tiles, int32_t* out_idx, int64_t* out_n,
+                                char* dyn, bool dense) {
     __shared__ unsigned long long s_lep[8];
     __shared__ uint64_t s_lval[8];
     __shared__ unsigned s_lkey[8];
     __shared__ int s_lpos[8];
     __shared__ unsigned s_m, s_total;
-    __shared__ int s_mv;
+    __shared__ int s_mv, s_path;
     const int tid = threadIdx.x;
     CH_TRACE_DECL
     CH_TRACE_MARK();
@@ -177,9 +179,12 @@ __device__ void post_last_block(const float* __restrict__ pts, long long n, Ctl*
             for (int r = 0; r < 4; ++r) most = max(most, *(volatile unsigned*)&ctl->rec_q[r]);
             const int path = most <= (unsigned)kQueueCap ? kPathQueues
                              : *(volatile int*)&ctl->star_final || total > 4u * (unsigned)kQueueCap ? kPathTiles : kPathSort;
-            ctl->path = path;
+            ctl->path = s_path = path;
             ctl->bk_state = path == kPathSort ? 2 : 1;
         }
+        __syncthreads();
+        if (s_path == kPathTiles)   // large_kernel counts the records of each group of u there
+            for (int g = tid; g < kPtGroups; g += blockDim.x) tiles[g] = 0u;
         return;
     }
     __syncthreads();      // also makes this block's line records visible to it
@@ -220,7 +225,8 @@ constexpr size_t kPostSmemBytes =
 __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __restrict__ pts, long long n, int head,
                                                                long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
                                                                const uint32_t* raw_idx, uint32_t* keys,
-                                                               uint64_t* vals, int32_t* out_idx, int64_t* out_n) {
+                                                               uint64_t* vals, unsigned* tiles, int32_t* out_idx,
+                                                               int64_t* out_n) {
     extern __shared__ __align__(16) char dyn[];
     __shared__ Octagon s_o;
     __shared__ int s_flag, s_mode, s_dense;
@@ -320,7 +326,7 @@ __global__ void __launch_bounds__(kPostThreads, 1) post_kernel(const float* __re
     CH_TL(ctl, 5, 1);
     if (!last_block(&ctl->blocks_done[2], &s_flag)) return;
     CH_TL(ctl, 6, 0);
-    post_last_block(pts, n, ctl, s_o, keys, vals, out_idx, out_n, dyn, s_dense != 0);
+    post_last_block(pts, n, ctl, s_o, keys, vals, tiles, out_idx, out_n, dyn, s_dense != 0);
     CH_TL(ctl, 6, 1);
 }
 
@@ -399,7 +405,8 @@ __global__ void __launch_bounds__(kPostThreads, 1) small_kernel(const float* __r
     rec_flush_block(rb, rc, ctl, keys, vals);
     flush_queue_counts(tally, ctl);
     __syncthreads();
-    post_last_block(pts, n, ctl, s_o, keys, vals, out_idx, out_n, dyn, false);
+    // (at most kSmallMax + 16 records: every queue fits a block, so no tiles)
+    post_last_block(pts, n, ctl, s_o, keys, vals, nullptr, out_idx, out_n, dyn, false);
 }
 
 // ---------------------------------------------------------------------------
@@ -409,10 +416,10 @@ void launch_small(const float* pts, long long n, Ctl* ctl, uint32_t* keys, uint6
 }
 
 void launch_post(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, const uint64_t* raw_xy,
-                 const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, int32_t* out_idx, int64_t* out_n,
-                 int grid, cudaStream_t s) {
-    post_kernel<<<grid, kPostThreads, kPostSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, keys, vals, out_idx,
-                                                          out_n);
+                 const uint32_t* raw_idx, uint32_t* keys, uint64_t* vals, unsigned* tiles, int32_t* out_idx,
+                 int64_t* out_n, int grid, cudaStream_t s) {
+    post_kernel<<<grid, kPostThreads, kPostSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, keys, vals, tiles,
+                                                          out_idx, out_n);
 }
 
 cudaError_t configure_post_kernel() {

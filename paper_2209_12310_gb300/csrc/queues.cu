@@ -12,9 +12,10 @@
 // The lower chain of a set of points equals the lower chain of the chains of
 // any partition of it into u ranges, joined in u order.
 //
-// large_kernel is one cooperative launch for the first two ways: the phases of
-// the tiles (count, cut, move, reduce) meet at grid barriers.  As one kernel it
-// costs a call that needs none of it one empty launch.
+// large_kernel is one launch for the first two ways: its blocks share the phases
+// of the tiles (count, cut, move, reduce) by claimed items and wait for their
+// ends (claim_item, wait_phase).  As one kernel it costs a call that needs none of
+// it one empty launch.
 #include "ch_internal.cuh"
 #include "host.h"
 #include "hullcore.cuh"
@@ -73,7 +74,8 @@ struct LargeArgs {
 };
 
 // Records per group (shared-memory counts, then one atomic per group that
-// occurs).
+// occurs), by chunks of the records, as many as blocks unless those grow long.
+// Returns whether this block finished the last chunk.
 struct TileHistSmem {
     unsigned h[kPtGroups];     // records per group; in the cut, per tile
     unsigned beg[kPtGroups];
@@ -81,25 +83,30 @@ struct TileHistSmem {
     int tmp[33];
 };
 
-__device__ void tile_hist(const LargeArgs& a, TileHistSmem& sm, const QMap& m) {
+__device__ bool tile_hist(const LargeArgs& a, TileHistSmem& sm, const QMap& m) {
     const int tid = threadIdx.x;
     for (int g = tid; g < kPtGroups; g += kLargeThreads) sm.h[g] = 0u;
-    __syncthreads();
     const unsigned n = a.ctl->count;
-    const unsigned stride = gridDim.x * kLargeThreads;
+    const unsigned chunk = min(64u, (n - 1u) / (gridDim.x * kLargeThreads) + 1u) * kLargeThreads;
+    const unsigned chunks = (n - 1u) / chunk + 1u;
     constexpr int kU = 4;
-    for (unsigned i0 = blockIdx.x * kLargeThreads + tid; i0 < n; i0 += stride * kU) {
-        uint32_t k[kU];
+    unsigned taken = 0u;
+    for (unsigned c; (c = claim_item(a.ctl, kLargeHist)) < chunks; ++taken) {
+        const unsigned end = min(n, (c + 1u) * chunk);
+        for (unsigned i0 = c * chunk + tid; i0 < end; i0 += kLargeThreads * kU) {
+            uint32_t k[kU];
 #pragma unroll
-        for (int j = 0; j < kU; ++j)
-            if (i0 + j * stride < n) k[j] = __ldcg(a.keys + i0 + j * stride);
+            for (int j = 0; j < kU; ++j)
+                if (i0 + j * kLargeThreads < end) k[j] = __ldcg(a.keys + i0 + j * kLargeThreads);
 #pragma unroll
-        for (int j = 0; j < kU; ++j)
-            if (i0 + j * stride < n) atomicAdd(&sm.h[q_group(m, k[j])], 1u);
+            for (int j = 0; j < kU; ++j)
+                if (i0 + j * kLargeThreads < end) atomicAdd(&sm.h[q_group(m, k[j])], 1u);
+        }
     }
-    __syncthreads();
-    for (int g = tid; g < kPtGroups; g += kLargeThreads)
+    if (!taken) return false;
+    for (int g = tid; g < kPtGroups; g += kLargeThreads)   // behind the last claim's barriers
         if (sm.h[g]) atomicAdd(&a.ghist[g], sm.h[g]);
+    return finish_items(a.ctl, kLargeHist, taken, chunks);
 }
 
 // One block cuts the tiles: gtile maps a group to its tile, tile t's records go
@@ -112,7 +119,6 @@ __device__ void tile_cut(const LargeArgs& a, TileHistSmem& sm) {
 #pragma unroll
     for (int e = 0; e < kE; ++e) {
         c[e] = __ldcg(a.ghist + tid * kE + e);
-        a.ghist[tid * kE + e] = 0u;   // at rest again
         sum += c[e];
     }
     int tot;
@@ -163,17 +169,22 @@ struct TilePartSmem {
     unsigned short gtile[kPtGroups];
 };
 
-__device__ void tile_part(const LargeArgs& a, TilePartSmem& sm, const QMap& m) {
+// Returns the number of the phase's items.
+__device__ unsigned tile_part(const LargeArgs& a, TilePartSmem& sm, const QMap& m) {
     static_assert(kLargeThreads == kPtThreads, "partition block");
     const int tid = threadIdx.x;
     for (int g = tid; g < kPtGroups; g += kPtThreads) sm.gtile[g] = (unsigned short)__ldcg(a.gtile + g);
-    __syncthreads();
     const unsigned n = a.ctl->count, nt = *(volatile unsigned*)&a.ctl->q_tile[4];
-    for (unsigned i0 = blockIdx.x * kPtTile; i0 < n; i0 += gridDim.x * kPtTile)
+    const unsigned parts = (n - 1u) / kPtTile + 1u;
+    for (unsigned p; (p = claim_item(a.ctl, kLargePart)) < parts;) {
+        const unsigned i0 = p * kPtTile;
         partition_tile(
             sm.p, a.keys, a.vals, i0, min((unsigned)kPtTile, n - i0), nt,
             [&](uint32_t key) { return (unsigned)sm.gtile[q_group(m, key)]; },
             [&](unsigned g, unsigned cnt) { return atomicAdd(&a.tcur[g], cnt); }, a.kB, a.vB);
+        finish_items(a.ctl, kLargePart, 1u, parts);
+    }
+    return parts;
 }
 
 // The tiles' lower chains, to [tbeg[t], tbeg[t] + tlen[t]) of cu / cv / ci
@@ -181,17 +192,11 @@ __device__ void tile_part(const LargeArgs& a, TilePartSmem& sm, const QMap& m) {
 // pieces, the chain so far taken along with each; when that chain fills the
 // block, the call goes to the sort.
 __device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
-    __shared__ unsigned s_tile;
     const int tid = threadIdx.x;
     constexpr int T = kLargeThreads, kCap = QcQueue::kCap, kCarry = kCap * 3 / 4, kPer = kCap / T;
     static_assert(kCap % T == 0, "carried points per thread");
     const unsigned nt = *(volatile unsigned*)&a.ctl->q_tile[4];
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_tile = atomicAdd(&a.ctl->tile_ctr[3], 1u);
-        __syncthreads();
-        const unsigned t = s_tile;
-        if (t >= nt) return;
+    for (unsigned t; (t = claim_item(a.ctl, kLargeChains)) < nt;) {
         const unsigned beg = __ldcg(a.tbeg + t), cnt = __ldcg(a.tcur + t) - beg;
         unsigned long long *src = q.a, *dst = q.b;
         int len = 0;
@@ -237,6 +242,7 @@ __device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
             dst = q.b;
             len = qc_eliminate<T>(src, dst, len + take, q.tmp);
             c0 += (unsigned)take;
+            if (tid == 0) atomicAdd(&a.ctl->beat, 1u);   // a tile can hold any share of the records
             if (len > kCarry && c0 < cnt) {   // no room for the rest
                 if (tid == 0) a.ctl->bk_state = 2;
                 len = 0;
@@ -250,6 +256,7 @@ __device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
             a.ci[beg + j] = q.si[qc_pos(w)];
         }
         if (tid == 0) a.tlen[t] = len;
+        finish_items(a.ctl, kLargeChains, 1u, nt);
     }
 }
 
@@ -289,22 +296,25 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
     q_map(ctl->oct, s_m);
     __syncthreads();
     if (path == kPathTiles) {
-        tile_hist(a, *reinterpret_cast<TileHistSmem*>(s_dyn), s_m);
-        CH_TL(ctl, 15, 1);
-        bool go = grid_barrier(&ctl->barrier[1], 1u, ctl);
-        if (go && qq == 0) tile_cut(a, *reinterpret_cast<TileHistSmem*>(s_dyn));
-        go = go && grid_barrier(&ctl->barrier[1], 2u, ctl);
+        TileHistSmem& h = *reinterpret_cast<TileHistSmem*>(s_dyn);
+        if (tile_hist(a, h, s_m)) {
+            tile_cut(a, h);
+            finish_items(ctl, kLargeCut, 1u, 1u);
+        }
+        bool go = wait_phase(ctl, kLargeCut, 1u);
         CH_TL(ctl, 16, 1);
-        if (go) tile_part(a, *reinterpret_cast<TilePartSmem*>(s_dyn), s_m);
+        if (go) go = wait_phase(ctl, kLargePart, tile_part(a, *reinterpret_cast<TilePartSmem*>(s_dyn), s_m));
         CH_TL(ctl, 17, 1);
-        go = go && grid_barrier(&ctl->barrier[1], 3u, ctl);
-        if (go) tile_chains(a, *reinterpret_cast<QcQueue*>(s_dyn));
-        CH_TL(ctl, 18, 1);
-        go = go && grid_barrier(&ctl->barrier[1], 4u, ctl);
+        if (go) {
+            tile_chains(a, *reinterpret_cast<QcQueue*>(s_dyn));
+            CH_TL(ctl, 18, 1);
+            if (qq >= 4) return;
+            go = wait_phase(ctl, kLargeChains, *(volatile unsigned*)&ctl->q_tile[4]);
+        }
         if (!go && tid == 0) *a.out_n = CH_ETIMEOUT;
-        if (!go || qq >= 4) return;
-        // A tile's chain that outgrew its block has set bk_state before the barrier;
-        // after it the word stays as it is until all four blocks have arrived
+        if (!go) return;
+        // A tile's chain that outgrew its block has set bk_state before that phase's
+        // end; after it the word stays as it is until all four blocks have arrived
         // below, so they agree on it (one read per block: its warps too).
         if (tid == 0) s_go = *(volatile int*)&ctl->bk_state == 1;
         __syncthreads();
@@ -431,7 +441,7 @@ void launch_large(Ctl* ctl, const uint32_t* kA, const uint64_t* vA, uint32_t* kB
                   int* cv, int* ci, long long n, int32_t* out_idx, int64_t* out_n, int grid, cudaStream_t s) {
     const LargeArgs a{ctl, kA, vA, kB, vB, tiles, tiles + kPtGroups, tiles + 2 * kPtGroups, tiles + 3 * kPtGroups,
                       (int*)(tiles + 4 * kPtGroups), cu, cv, ci, n, out_idx, out_n};
-    launch_grid(large_kernel, grid, kLargeThreads, kLargeSmem, s, a);
+    large_kernel<<<grid, kLargeThreads, kLargeSmem, s>>>(a);
 }
 
 size_t tiles_bytes() { return sizeof(unsigned) * 5 * (size_t)kPtGroups; }

@@ -18,11 +18,13 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
         ctl->line_ep[t] = (t & 1) ? 0ull : ~0ull;   // even: minimum slot, odd: maximum slot
     }
     if (t < 4) {
-        ctl->tile_ctr[t] = 0u;
         ctl->counts4[t] = 0u;
         ctl->rec_q[t] = 0u;
         if (t) ctl->blocks_done[t] = 0u;
-        if (t < 3) ctl->barrier[t] = 0u;
+    }
+    if (t < kPhases) {
+        ctl->claimed[t] = 0u;
+        ctl->finished[t] = 0u;
     }
     if (t == 0) {
         ctl->status = CH_OK;
@@ -35,6 +37,7 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
         ctl->records_ready = 0;
         ctl->bk_state = 0;
         ctl->path = kPathNone;
+        ctl->beat = 0u;
         ctl->joins_done = 0u;
         ctl->join_over = 0;
         ctl->roots_done = 0u;

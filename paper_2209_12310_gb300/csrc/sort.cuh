@@ -10,7 +10,7 @@
 // preceding tiles, and scatters.  The digit histograms of all three passes
 // come from one counting pass over the records (sort_hist) before the first
 // scatter; the post pass keeps only per-queue counts.  These are phases of
-// sort_kernel (hull.cu), with grid barriers between them.
+// sort_kernel (hull.cu), whose blocks wait for each phase's end (wait_phase).
 //
 // Look-back waits are bounded (kSpinLimit polls with back-off); a wait that
 // gives up raises CH_ETIMEOUT and the abort flag, after which every other
@@ -61,7 +61,8 @@ struct SortSmem {
     unsigned tile;
 };
 
-__device__ void onesweep(SortSmem& sm, const uint32_t* kin, const uint64_t* vin, uint32_t* kout, uint64_t* vout, Ctl* ctl,
+// Returns the number of the pass's tiles.
+__device__ unsigned onesweep(SortSmem& sm, const uint32_t* kin, const uint64_t* vin, uint32_t* kout, uint64_t* vout, Ctl* ctl,
                          unsigned long long* status, int pass) {
     unsigned(&s_base)[kDigits] = sm.base;
     unsigned(&s_excl)[kDigits] = sm.excl;
@@ -75,8 +76,9 @@ __device__ void onesweep(SortSmem& sm, const uint32_t* kin, const uint64_t* vin,
     const int shift = pass * kDigitBits;
 
     bool have_base = false;
-    for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->tile_ctr[pass], 1u);
+    unsigned taken = 0u;
+    for (;; ++taken) {
+        if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->claimed[kSortPass + pass], 1u);
         for (int i = threadIdx.x; i < (kSortThreads / 32) * kDigits; i += kSortThreads)
             (&s_wcnt[0][0])[i] = 0;
         __syncthreads();
@@ -176,23 +178,33 @@ __device__ void onesweep(SortSmem& sm, const uint32_t* kin, const uint64_t* vin,
         }
         __syncthreads();
     }
+    if (taken) finish_items(ctl, kSortPass + pass, taken, ntiles);
+    return ntiles;
 }
 
-// Digit histograms of the records for the three passes.
-__device__ void sort_hist(unsigned (*s_h)[kDigits], const uint32_t* keys, Ctl* ctl) {
+// Digit histograms of the records for the three passes, by chunks of the
+// records, as many as blocks unless those grow long.  Returns their number.
+__device__ unsigned sort_hist(unsigned (*s_h)[kDigits], const uint32_t* keys, Ctl* ctl) {
     for (int i = threadIdx.x; i < kSortPasses * kDigits; i += blockDim.x) (&s_h[0][0])[i] = 0u;
-    __syncthreads();
     const unsigned count = ctl->count;
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-        const uint32_t k = keys[i];
+    const unsigned chunk = min(256u, (count - 1u) / (gridDim.x * blockDim.x) + 1u) * blockDim.x;
+    const unsigned chunks = (count - 1u) / chunk + 1u;
+    unsigned taken = 0u;
+    for (unsigned c; (c = claim_item(ctl, kSortHist)) < chunks; ++taken) {
+        const unsigned end = min(count, (c + 1u) * chunk);
+        for (unsigned i = c * chunk + threadIdx.x; i < end; i += blockDim.x) {
+            const uint32_t k = keys[i];
 #pragma unroll
-        for (int p = 0; p < kSortPasses; ++p) atomicAdd(&s_h[p][(k >> (p * kDigitBits)) & (kDigits - 1)], 1u);
+            for (int p = 0; p < kSortPasses; ++p) atomicAdd(&s_h[p][(k >> (p * kDigitBits)) & (kDigits - 1)], 1u);
+        }
     }
-    __syncthreads();
+    if (!taken) return chunks;
     for (int i = threadIdx.x; i < kSortPasses * kDigits; i += blockDim.x) {
         const unsigned c = (&s_h[0][0])[i];
         if (c) atomicAdd(&(&ctl->digit_hist[0][0])[i], c);
     }
+    finish_items(ctl, kSortHist, taken, chunks);
+    return chunks;
 }
 
 }  // namespace ch
