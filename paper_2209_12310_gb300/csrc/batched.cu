@@ -1679,11 +1679,11 @@ __global__ void __launch_bounds__(T) bt_queue_chain(BArgs a) {
             continue;
         }
         qc_gather<T, kBQGather>(a.keys + rb, a.vals + rb, m, qq, q, &s_n);
-        const int n = min(s_n, Q::kCap);   // counts4[qq], the chain's two end points among them
+        int n = min(s_n, Q::kCap);   // counts4[qq], the chain's two end points among them
         uint32_t ulo, uhi, v;
         queue_frame(qq, c->oct.vx[2 * qq], c->oct.vy[2 * qq], ulo, v);
         queue_frame(qq, c->oct.vx[(2 * qq + 2) & 7], c->oct.vy[(2 * qq + 2) & 7], uhi, v);
-        qc_sort<T>(q, n, (int)ulo, (int)uhi);
+        n = qc_sort<T>(q, n, (int)ulo, (int)uhi);
         unsigned long long *src = q.a, *dst = q.b;
         const int len = qc_eliminate<T>(src, dst, n, q.tmp);
         for (int j = tid; j < len; j += T) {

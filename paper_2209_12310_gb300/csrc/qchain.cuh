@@ -102,87 +102,49 @@ __device__ __forceinline__ void qc_gather(const uint32_t* keys, const uint64_t* 
     __syncthreads();
 }
 
-// The n points of q.a (u in [lo, hi]) in order, in place.  Whole block of T
-// threads.  Buckets of equal width in u hold about two points each; every point
-// counts the points of its bucket before it (independent loads, where an
-// insertion sort per bucket is a chain of them: records that a polygon leaves
-// can crowd a few buckets by the hundred; by words, the indices compared only
-// among equal points: with qc_less throughout this loop was 23,000 of the sort's
-// 32,000 cycles for 8000 points).  When some bucket holds more than
-// kQcBucket, the whole array goes through a bitonic sort instead.
-constexpr unsigned kQcBucket = 512;
-
-template <int T, class Q>
-__device__ void qc_sort(Q& q, int n, int lo, int hi) {
-    const int tid = threadIdx.x;
-    const int nb = min(Q::kBuckets, n / 2 + 1);
-    const float scale = (float)nb / (float)(hi - lo + 1);
-    auto bucket = [&](unsigned long long w) { return max(0, min(nb - 1, (int)((float)(qc_u(w) - lo) * scale))); };
-    for (int b = tid; b < nb; b += T) q.cnt[b] = 0u;
-    if (tid == 0) q.big = 0;
-    __syncthreads();
-    for (int j = tid; j < n; j += T) atomicAdd(&q.cnt[bucket(q.a[j])], 1u);
-    __syncthreads();
-    const int per = (nb + T - 1) / T, b0 = min(nb, tid * per), b1 = min(nb, b0 + per);
-    unsigned sum = 0u, most = 0u;
-    for (int b = b0; b < b1; ++b) {
-        sum += q.cnt[b];
-        most = max(most, q.cnt[b]);
+// Whether point w can still be a strict vertex beside the lower chain of some of
+// its queue's points: not when it lies on or above an edge, or above a vertex.  A
+// copy of a vertex goes too, its index kept at the vertex if it is lower.
+__device__ __forceinline__ bool qc_beside(unsigned long long w, int id, const unsigned long long* chain, int len, int* si) {
+    const int u = qc_u(w), v = qc_v(w);
+    int lo = 0, hi = len;   // the first vertex with no smaller u
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (qc_u(chain[mid]) < u) lo = mid + 1;
+        else hi = mid;
     }
-    if (most > kQcBucket) q.big = 1;
-    int tot;
-    unsigned run = (unsigned)block_excl_scan((int)sum, q.tmp, &tot);
-    if (q.big) {   // block-uniform: set before the scan's barriers
-        int P = 1;
-        while (P < n) P <<= 1;   // n <= CAP < 2^14 <= 2 CAP words in a and b
-        unsigned long long* s = q.a;
-        for (int j = n + tid; j < P; j += T) s[j] = kQcPad;
-        __syncthreads();
-        for (int k = 2; k <= P; k <<= 1)
-            for (int d = k >> 1; d > 0; d >>= 1) {
-                for (int i = tid; i < P; i += T) {
-                    const int l = i ^ d;
-                    if (l > i) {
-                        const unsigned long long x = s[i], y = s[l];
-                        const bool up = (i & k) == 0;
-                        if (up ? qc_less(y, x, q.si) : qc_less(x, y, q.si)) {
-                            s[i] = y;
-                            s[l] = x;
-                        }
+    if (lo == len) return true;
+    const unsigned long long c = chain[lo];
+    const int cu = qc_u(c), cv = qc_v(c);
+    if (cu == u) {
+        if (v != cv) return v < cv;
+        if (qc_pos(c) == qc_pos(w)) return true;   // the vertex itself
+        if (id < si[qc_pos(c)]) atomicMin(&si[qc_pos(c)], id);
+        return false;
+    }
+    if (lo == 0) return true;
+    const unsigned long long p = chain[lo - 1];
+    return (long long)(cu - qc_u(p)) * (v - qc_v(p)) < (long long)(cv - qc_v(p)) * (u - qc_u(p));
+}
+
+// The P words of s in order, P a power of two (a bitonic network).  Whole block.
+template <int T>
+__device__ __forceinline__ void qc_bitonic(unsigned long long* s, int P, const int* si) {
+    for (int k = 2; k <= P; k <<= 1)
+        for (int d = k >> 1; d > 0; d >>= 1) {
+            for (int i = threadIdx.x; i < P; i += T) {
+                const int l = i ^ d;
+                if (l > i) {
+                    const unsigned long long x = s[i], y = s[l];
+                    const bool up = (i & k) == 0;
+                    if (up ? qc_less(y, x, si) : qc_less(x, y, si)) {
+                        s[i] = y;
+                        s[l] = x;
                     }
                 }
-                __syncthreads();
             }
-        return;
-    }
-    for (int b = b0; b < b1; ++b) {
-        const unsigned c = q.cnt[b];
-        q.cnt[b] = run;
-        run += c;
-    }
-    __syncthreads();
-    for (int j = tid; j < n; j += T) {
-        const unsigned long long w = q.a[j];
-        q.b[atomicAdd(&q.cnt[bucket(w)], 1u)] = w;
-    }
-    __syncthreads();
-    for (int j = tid; j < n; j += T) {
-        const unsigned long long w = q.b[j];
-        const int b = bucket(w);   // cnt[b] is now the end of bucket b
-        const int s = b ? (int)q.cnt[b - 1] : 0, e = (int)q.cnt[b];
-        int r = s, same = 0;   // same: points of equal (u, v), this one among them
-        for (int i = s; i < e; ++i) {
-            const unsigned long long x = q.b[i];
-            r += x < w ? 1 : 0;
-            same += ((x ^ w) >> kQcPosBits) == 0ull ? 1 : 0;
+            __syncthreads();
         }
-        if (same > 1) {   // by index
-            r = s;
-            for (int i = s; i < e; ++i) r += qc_less(q.b[i], w, q.si) ? 1 : 0;
-        }
-        q.a[r] = w;
-    }
-    __syncthreads();
 }
 
 // The lower chain of the n >= 1 points in src, ordered by (u, v, index):
@@ -248,6 +210,128 @@ __device__ int qc_eliminate(unsigned long long*& src, unsigned long long*& dst, 
         dst = t;
         n = tot;
     }
+}
+
+// Drops, of the n > kQcSample points of q.a, those that the lower chain of
+// kQcSample of them rules out; returns how many are left.  Whole block.
+constexpr int kQcSample = 512;
+
+template <int T, class Q>
+__device__ __noinline__ int qc_thin(Q& q, int n) {
+    static_assert(Q::kCap % T == 0 && Q::kCap >= 2 * kQcSample, "points per thread; the sample and its chain in b");
+    constexpr int kPer = Q::kCap / T;
+    const int tid = threadIdx.x;
+    for (int j = tid; j < kQcSample; j += T) q.b[j] = q.a[(int)((long long)j * n / kQcSample)];
+    __syncthreads();
+    qc_bitonic<T>(q.b, kQcSample, q.si);
+    unsigned long long *src = q.b, *dst = q.b + kQcSample;
+    const int len = qc_eliminate<T>(src, dst, kQcSample, q.tmp);
+    unsigned long long w[kPer];
+    unsigned kept = 0u;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+        const int j = e * T + tid;
+        w[e] = j < n ? q.a[j] : 0ull;
+        if (j < n && qc_beside(w[e], q.si[qc_pos(w[e])], src, len, q.si)) kept |= 1u << e;
+    }
+    int tot;
+    int at = block_excl_scan(__popc(kept), q.tmp, &tot);   // its barriers: every word is read
+#pragma unroll
+    for (int e = 0; e < kPer; ++e)
+        if ((kept >> e) & 1u) q.a[at++] = w[e];
+    __syncthreads();
+    return tot;
+}
+
+// The n points of q.a (u in [lo, hi]) in order, in place, less some that are no
+// vertices; returns how many are left.  Whole block of T threads.  Buckets of
+// equal width in u hold about two points each; every point
+// counts the points of its bucket before it (independent loads, where an
+// insertion sort per bucket is a chain of them: records that a polygon leaves
+// can crowd a few buckets by the hundred; by words, the indices compared only
+// among equal points: with qc_less throughout this loop was 23,000 of the sort's
+// 32,000 cycles for 8000 points).  When some bucket holds more than kQcBucket,
+// the points are thinned first (copies of one vertex all share a bucket) and the
+// buckets span what is left; still crowded, the whole array goes through a
+// bitonic sort.
+constexpr unsigned kQcBucket = 512;
+static_assert(kQcBucket >= kQcSample, "crowded: more points than the sample");
+
+template <int T, class Q>
+__device__ int qc_sort(Q& q, int n, int lo, int hi) {
+    const int tid = threadIdx.x;
+    int nb;
+    float scale;
+    auto bucket = [&](unsigned long long w) { return max(0, min(nb - 1, (int)((float)(qc_u(w) - lo) * scale))); };
+    for (int turn = 0;; ++turn) {
+        nb = min(Q::kBuckets, n / 2 + 1);
+        scale = (float)nb / (float)(hi - lo + 1);
+        for (int b = tid; b < nb; b += T) q.cnt[b] = 0u;
+        if (tid == 0) q.big = 0;
+        __syncthreads();
+        for (int j = tid; j < n; j += T) atomicAdd(&q.cnt[bucket(q.a[j])], 1u);
+        __syncthreads();
+        const int per = (nb + T - 1) / T, b0 = min(nb, tid * per), b1 = min(nb, b0 + per);
+        unsigned sum = 0u, most = 0u;
+        for (int b = b0; b < b1; ++b) {
+            sum += q.cnt[b];
+            most = max(most, q.cnt[b]);
+        }
+        if (most > kQcBucket) q.big = 1;
+        int tot;
+        unsigned run = (unsigned)block_excl_scan((int)sum, q.tmp, &tot);
+        if (!q.big) {   // block-uniform: set before the scan's barriers
+            for (int b = b0; b < b1; ++b) {
+                const unsigned c = q.cnt[b];
+                q.cnt[b] = run;
+                run += c;
+            }
+            __syncthreads();
+            break;
+        }
+        __syncthreads();   // read by all before the next turn writes it
+        if (turn == 0) {
+            n = qc_thin<T>(q, n);
+            lo = INT_MAX;
+            hi = INT_MIN;
+            for (int j = tid; j < n; j += T) {
+                lo = min(lo, qc_u(q.a[j]));
+                hi = max(hi, qc_u(q.a[j]));
+            }
+            lo = block_reduce<int>(lo, [](int x, int y) { return min(x, y); }, q.tmp);
+            hi = block_reduce<int>(hi, [](int x, int y) { return max(x, y); }, q.tmp);
+            continue;
+        }
+        int P = 1;
+        while (P < n) P <<= 1;   // n <= CAP < 2^14 <= 2 CAP words in a and b
+        for (int j = n + tid; j < P; j += T) q.a[j] = kQcPad;
+        __syncthreads();
+        qc_bitonic<T>(q.a, P, q.si);
+        return n;
+    }
+    for (int j = tid; j < n; j += T) {
+        const unsigned long long w = q.a[j];
+        q.b[atomicAdd(&q.cnt[bucket(w)], 1u)] = w;
+    }
+    __syncthreads();
+    for (int j = tid; j < n; j += T) {
+        const unsigned long long w = q.b[j];
+        const int b = bucket(w);   // cnt[b] is now the end of bucket b
+        const int s = b ? (int)q.cnt[b - 1] : 0, e = (int)q.cnt[b];
+        int r = s, same = 0;   // same: points of equal (u, v), this one among them
+        for (int i = s; i < e; ++i) {
+            const unsigned long long x = q.b[i];
+            r += x < w ? 1 : 0;
+            same += ((x ^ w) >> kQcPosBits) == 0ull ? 1 : 0;
+        }
+        if (same > 1) {   // by index
+            r = s;
+            for (int i = s; i < e; ++i) r += qc_less(q.b[i], w, q.si) ? 1 : 0;
+        }
+        q.a[r] = w;
+    }
+    __syncthreads();
+    return n;
 }
 
 // ---------------------------------------------------------------------------

@@ -189,11 +189,79 @@ __device__ unsigned tile_part(const LargeArgs& a, TilePartSmem& sm, const QMap& 
 
 // The tiles' lower chains, to [tbeg[t], tbeg[t] + tlen[t]) of cu / cv / ci
 // (u, v, index).  A tile with more records than the block holds goes in
-// pieces, the chain so far taken along with each; when that chain fills the
-// block, the call goes to the sort.
+// pieces: the records after the first piece are tested against the chain so far
+// as they are read, and only those that it leaves (few, unless the records are
+// mostly vertices; none of a vertex's copies) are sorted with it.  (Every piece
+// sorted whole, a million points with 600,000 copies of one hull vertex took
+// 23 ms; see tile_read.)  When the chain fills the block, the call goes to the
+// sort.
+constexpr int kReadU = 2;                                         // records per thread and step
+constexpr int kCarry = QcQueue::kCap - kReadU * kLargeThreads;    // vertices carried at most
+
+// Reads the tile's records from c0 on (at beg + c0, cnt in all), while a step's
+// fit the block; q.a and q.si [0, len) hold the chain so far, what it leaves goes
+// behind.  Returns the number of points in q.a, *next the first record not read.
+__device__ int tile_read(const LargeArgs& a, QcQueue& q, unsigned beg, unsigned cnt, unsigned c0, int len, unsigned* next) {
+    __shared__ int s_fill;
+    constexpr int T = kLargeThreads, U = kReadU;
+    const int tid = threadIdx.x, lane = tid & 31;
+    uint32_t k[U];
+    uint64_t w[U];
+    auto load = [&]() {
+#pragma unroll
+        for (int e = 0; e < U; ++e) {
+            const unsigned j = c0 + e * T + tid;
+            k[e] = j < cnt ? __ldcg(a.kB + beg + j) & kKeyMask : 0u;
+            w[e] = j < cnt ? __ldcg(a.vB + beg + j) : 0ull;
+        }
+    };
+    if (tid == 0) s_fill = len;
+    load();
+    int fill = len;
+    for (unsigned step = 0u; c0 < cnt && fill <= QcQueue::kCap - U * T; ++step) {
+        unsigned long long x[U];
+        int id[U];
+        bool keep[U];
+#pragma unroll
+        for (int e = 0; e < U; ++e) {
+            x[e] = qc_pack(k[e], (unsigned)(w[e] >> 31), (1u << kQcPosBits) - 1u);   // no slot of a vertex
+            id[e] = (int)(w[e] & 0x7FFFFFFFull);
+            keep[e] = c0 + e * T + tid < cnt;
+        }
+        c0 += U * T;
+        load();   // the next step's, while this one's are tested
+        __syncthreads();   // s_fill and q.a [0, len) stand
+#pragma unroll
+        for (int e = 0; e < U; ++e) {
+            keep[e] = keep[e] && qc_beside(x[e], id[e], q.a, len, q.si);
+            // of a warp's copies of one point, the lowest index
+            unsigned bal = __ballot_sync(0xFFFFFFFFu, keep[e]);
+            if (bal == 0u) continue;
+            if (keep[e]) {
+                const unsigned same = __match_any_sync(bal, x[e]);
+                keep[e] = (unsigned)id[e] == __reduce_min_sync(same, (unsigned)id[e]);
+            }
+            bal = __ballot_sync(0xFFFFFFFFu, keep[e]);
+            int pos = 0;
+            if (lane == 0) pos = atomicAdd(&s_fill, __popc(bal));
+            pos = __shfl_sync(0xFFFFFFFFu, pos, 0) + __popc(bal & lanemask_lt());
+            if (keep[e]) {
+                q.a[pos] = (x[e] & ~((1ull << kQcPosBits) - 1ull)) | (unsigned)pos;
+                q.si[pos] = id[e];
+            }
+        }
+        __syncthreads();
+        fill = s_fill;
+        if (tid == 0 && (step & 63u) == 63u) atomicAdd(&a.ctl->beat, 1u);
+    }
+    __syncthreads();
+    *next = min(c0, cnt);
+    return fill;
+}
+
 __device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
     const int tid = threadIdx.x;
-    constexpr int T = kLargeThreads, kCap = QcQueue::kCap, kCarry = kCap * 3 / 4, kPer = kCap / T;
+    constexpr int T = kLargeThreads, kCap = QcQueue::kCap, kPer = kCap / T;
     static_assert(kCap % T == 0, "carried points per thread");
     const unsigned nt = *(volatile unsigned*)&a.ctl->q_tile[4];
     for (unsigned t; (t = claim_item(a.ctl, kLargeChains)) < nt;) {
@@ -201,8 +269,18 @@ __device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
         unsigned long long *src = q.a, *dst = q.b;
         int len = 0;
         for (unsigned c0 = 0; c0 < cnt;) {
-            const int take = (int)min(cnt - c0, (unsigned)(kCap - len));
-            if (len) {   // the carried chain first, in slots 0 .. len - 1
+            int n;
+            if (len == 0) {
+                n = (int)min(cnt, (unsigned)kCap);
+#pragma unroll 5
+                for (int j = tid; j < n; j += T) {
+                    const uint32_t k = __ldcg(a.kB + beg + j);
+                    const uint64_t w = __ldcg(a.vB + beg + j);
+                    q.a[j] = qc_pack(k & kKeyMask, (unsigned)(w >> 31), (unsigned)j);
+                    q.si[j] = (int)(w & 0x7FFFFFFFull);
+                }
+                c0 = (unsigned)n;
+            } else {   // the chain so far in slots 0 .. len - 1
                 unsigned long long w[kPer];
                 int id[kPer];
 #pragma unroll
@@ -220,28 +298,25 @@ __device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
                         q.si[j] = id[e];
                     }
                 }
-            }
-#pragma unroll 5
-            for (int j = tid; j < take; j += T) {
-                const uint32_t k = __ldcg(a.kB + beg + c0 + j);
-                const uint64_t w = __ldcg(a.vB + beg + c0 + j);
-                q.a[len + j] = qc_pack(k & kKeyMask, (unsigned)(w >> 31), (unsigned)(len + j));
-                q.si[len + j] = (int)(w & 0x7FFFFFFFull);
+                src = q.a;
+                dst = q.b;
+                n = tile_read(a, q, beg, cnt, c0, len, &c0);
             }
             __syncthreads();
-            // the buckets span the points' own range, which is the tile's
-            int lo = INT_MAX, hi = INT_MIN;
-            for (int j = tid; j < len + take; j += T) {
-                lo = min(lo, qc_u(q.a[j]));
-                hi = max(hi, qc_u(q.a[j]));
+            if (n > len) {
+                // the buckets span the points' own range, which is the tile's
+                int lo = INT_MAX, hi = INT_MIN;
+                for (int j = tid; j < n; j += T) {
+                    lo = min(lo, qc_u(q.a[j]));
+                    hi = max(hi, qc_u(q.a[j]));
+                }
+                lo = block_reduce<int>(lo, [](int x, int y) { return min(x, y); }, q.tmp);
+                hi = block_reduce<int>(hi, [](int x, int y) { return max(x, y); }, q.tmp);
+                n = qc_sort<T>(q, n, lo, hi);
+                src = q.a;
+                dst = q.b;
+                len = qc_eliminate<T>(src, dst, n, q.tmp);
             }
-            lo = block_reduce<int>(lo, [](int x, int y) { return min(x, y); }, q.tmp);
-            hi = block_reduce<int>(hi, [](int x, int y) { return max(x, y); }, q.tmp);
-            qc_sort<T>(q, len + take, lo, hi);
-            src = q.a;
-            dst = q.b;
-            len = qc_eliminate<T>(src, dst, len + take, q.tmp);
-            c0 += (unsigned)take;
             if (tid == 0) atomicAdd(&a.ctl->beat, 1u);   // a tile can hold any share of the records
             if (len > kCarry && c0 < cnt) {   // no room for the rest
                 if (tid == 0) a.ctl->bk_state = 2;
@@ -343,11 +418,11 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
         qc_gather<T, 4>(keys, vals, m, qq, q, &s_n);
         CH_TL(ctl, 19, 1);
         const int cnt = min(s_n, QcQueue::kCap);   // rec_q[qq], the two end points among them
-        qc_sort<T>(q, cnt, s_m.lo[qq], s_m.hi[qq]);
+        const int left = qc_sort<T>(q, cnt, s_m.lo[qq], s_m.hi[qq]);
         CH_TL(ctl, 20, 1);
         src = q.a;
         dst = q.b;
-        len = qc_eliminate<T>(src, dst, cnt, q.tmp);
+        len = qc_eliminate<T>(src, dst, left, q.tmp);
         for (int j = tid; j < len; j += T) {
             vout[pre[qq] + j] = src[j] >> kQcPosBits;
             iout[pre[qq] + j] = q.si[qc_pos(src[j])];

@@ -89,3 +89,65 @@ def test_tile_chain_over_its_block(lib, n):
     for got, c in _calls(lib, pts, 10):
         np.testing.assert_array_equal(got, want)
         assert c["stage"] == SORT and c["star_vertices"] == 0 and c["two_pass"] == 1, c
+
+
+def _far_copies(n, order, cluster=0.0):
+    """n points on the GPU: a normal cloud inside eight extremes, and 60 % copies
+    of one more hull vertex (or, with cluster > 0, points this far from it), which
+    the octagon of the extremes does not hold; the hull's indices with it."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    c, rho, m = float(1 << 23), 6.0e6, int(0.6 * n)
+    pts = torch.randn((n, 2), generator=g, device="cuda").mul_(6.0e5).add_(c)
+    far = torch.tensor([c + rho * math.cos(math.pi / 8), c + rho * math.sin(math.pi / 8)], device="cuda")
+    pts[:m] = far
+    if cluster:
+        pts[:m] += torch.randn((m, 2), generator=g, device="cuda").mul_(cluster)
+    for k in range(8):
+        pts[m + k] = torch.tensor([c + rho * math.cos(k * math.pi / 4), c + rho * math.sin(k * math.pi / 4)])
+    pts.round_()
+    if order == "shuffled":
+        pts = pts[torch.randperm(n, generator=g, device="cuda")]
+    return pts.contiguous()
+
+
+@pytest.mark.parametrize("n,order", [(3000, "shuffled"), (15_000, "shuffled"), (20_000, "sorted"), (60_000, "shuffled"),
+                                     (1_000_000, "shuffled"), (1_000_003, "sorted"), (50_000_000, "shuffled")])
+def test_copies_of_a_vertex(lib, n, order):
+    """Every copy lies in one range of u: in a queue's block, in the sort (a run of
+    equal keys over several of its tiles), and in one tile of u ranges."""
+    pts = _far_copies(n, order)
+    few = torch.unique(pts, dim=0)   # the hull's coordinates, then their lowest indices
+    want = few[torch.from_numpy(oracle.hull(few.cpu().numpy())).cuda().long()]
+    assert want.shape[0] == 9
+    first = [int((pts == v).all(1).nonzero()[0]) for v in want]
+    got = lib.hull(pts)
+    assert got.tolist() == first
+
+
+@pytest.mark.parametrize("n", [30_000, 3_000_000])
+def test_cluster_beyond_the_octagon(lib, n):
+    pts = _far_copies(n, "shuffled", 3.0e4)
+    np.testing.assert_array_equal(lib.hull(pts).cpu().numpy(), oracle.hull(pts.cpu().numpy()))
+
+
+def _stairs(m, copies, seed):
+    """A convex curve of m points in the range of few others' u, each copied;
+    the copies of one point follow each other."""
+    i = np.arange(m, dtype=np.int64)
+    arc = np.stack([i * 1500, np.concatenate([[0], np.cumsum(i[:-1] - m // 2)])], 1)
+    arc[:, 1] += 5 - arc[:, 1].min()
+    return np.repeat(arc[np.random.default_rng(seed).permutation(m)], copies, axis=0).astype(np.float32)
+
+
+@pytest.mark.parametrize("m,copies", [(300, 60), (5000, 4), (300, 3000)])
+def test_copies_of_every_vertex(lib, m, copies):
+    pts = _stairs(m, copies, m)
+    want = oracle.hull(pts)
+    assert want.size == m
+    d = torch.from_numpy(pts).cuda()
+    np.testing.assert_array_equal(lib.hull(d).cpu().numpy(), want)
+    off = np.array([0, pts.shape[0], 2 * pts.shape[0], 2 * pts.shape[0] + 1000])
+    sets = lib.hull_batched(torch.cat([d, d.flip(0), d[:1000]]), off)
+    np.testing.assert_array_equal(sets[0].cpu().numpy(), want)
+    np.testing.assert_array_equal(sets[1].cpu().numpy(), oracle.hull(np.ascontiguousarray(pts[::-1])))
