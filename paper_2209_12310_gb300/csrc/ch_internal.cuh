@@ -98,12 +98,14 @@ constexpr float kHugePositive = 1.0e30f;      // "always inside" coefficient of 
 
 constexpr unsigned kSpinLimit = 1u << 20;     // polls of a bounded wait (of a phase: without progress)
 
+constexpr int kJoinRounds = 8;                // rounds that join a queue's tile chains, at most
+
 // Phases of dense_kernel, large_kernel and sort_kernel whose end their blocks
 // wait for (claim_item, wait_phase).
 enum Phase {
     kDenseBins = 0, kDenseMerge, kDensePoly, kDenseRadius,
-    kLargeHist, kLargeCut, kLargePart, kLargeChains,
-    kSortHist, kSortPass, kPhases = kSortPass + kSortPasses
+    kLargeHist, kLargeCut, kLargePart, kLargeChains, kLargeJoin,
+    kSortHist = kLargeJoin + kJoinRounds, kSortPass, kPhases = kSortPass + kSortPasses
 };
 
 // Directions of the 8 extremes in counter-clockwise octagon order.
@@ -149,8 +151,9 @@ struct Ctl {
     unsigned int digit_hist[kSortPasses][kDigits];   // sort path only (sort_kernel)
     unsigned int rec_q[4];              // records per queue
     unsigned int reg_end[4];            // chain length of queue r (large_kernel, bt_queue_chain)
-    unsigned int joins_done;            // large_kernel: queues whose chain stands (or did not fit)
-    int join_over;                      // large_kernel: a queue's tile chains outgrew its block
+    unsigned int joins_done;            // large_kernel: queues whose chain stands
+    unsigned int join_n[kJoinRounds + 1][4];   // large_kernel: points of each queue's tile chains,
+                                        // and after each round that joins them
     unsigned int roots_done;            // sort_kernel: queue roots of the merge tree
     unsigned int counts4[4];            // survivors per queue (ch_filter)
     unsigned long long line_ep[8];      // end points of survivors on the 4 axis support lines

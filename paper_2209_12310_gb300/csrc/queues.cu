@@ -6,9 +6,10 @@
 //           and reduces it to its lower chain in shared memory (qchain.cuh);
 //   tiles   the u range of each queue is cut into tiles of some thousand
 //           records, which a block each reduces the same way, and a block per
-//           queue reduces its tiles' chains, joined in u order, to its chain;
-//   sort    the radix sort and the merge tree (sort.cuh, hull.cu), also when
-//           a tile's or a queue's chain outgrows shared memory.
+//           queue reduces its tiles' chains, joined in u order, to its chain
+//           (all blocks in rounds, when those outgrow shared memory);
+//   sort    the radix sort and the merge tree (sort.cuh, hull.cu), also when a
+//           tile's chain outgrows shared memory.
 // The lower chain of a set of points equals the lower chain of the chains of
 // any partition of it into u ranges, joined in u order.
 //
@@ -66,6 +67,7 @@ struct LargeArgs {
     uint32_t* kB;            // the records by tile; then scratch and
     uint64_t* vB;            // the queues' chains (u, v)
     unsigned *ghist, *gtile, *tbeg, *tcur;   // kPtGroups each
+    unsigned* seg[2];        // as many: ghist and gtile again, once the tiles stand
     int* tlen;
     int *cu, *cv, *ci;       // the tiles' chains; then (cu) the queues' chains (index)
     long long n;
@@ -330,7 +332,12 @@ __device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
             a.cv[beg + j] = qc_v(w);
             a.ci[beg + j] = q.si[qc_pos(w)];
         }
-        if (tid == 0) a.tlen[t] = len;
+        if (tid == 0) {
+            a.tlen[t] = len;
+            int r = 0;
+            while (r < 3 && t >= *(volatile unsigned*)&a.ctl->q_tile[r + 1]) ++r;
+            atomicAdd(&a.ctl->join_n[0][r], (unsigned)len);
+        }
         finish_items(a.ctl, kLargeChains, 1u, nt);
     }
 }
@@ -343,19 +350,171 @@ struct QcJoin {
     unsigned off[kPtGroups];   // tile chains' places in the queue
     int tmp[33];
 };
+// Tile chains of a queue that are too long for one block, joined by all blocks in
+// rounds.  The queues' points, in u order, are cut into segments; a block
+// reduces a segment, with the point before and the point after it as fixed ends,
+// to its lower chain (what that drops lies on or above a segment between two
+// input points), and the next round cuts at other places.  A round that drops
+// nothing has found every three neighbours turning strictly left: the chains
+// stand.  (Of a circle's points a few at the tiles' ends go in the first round.
+// 4e6 points 1.15 ms a call with the radix sort and the merge tree as the way out,
+// 0.45 now; 2e7 3.4 and 1.26.)
+// Round j reads the tiles' chains (j = 0), else what round j - 1 left, a segment's
+// points at its place (cu / cv / ci after odd rounds, vB / kB after even ones), its
+// count in seg[(j - 1) & 1].
+struct JoinPlan {
+    unsigned n[4], first[5];   // points and first segment of each queue
+    unsigned shift;            // the first segment is shorter by this much
+    __device__ __forceinline__ void set(const Ctl* ctl, int j, unsigned size) {
+        shift = (j & 1) ? size / 2u : 0u;
+        first[0] = 0u;
+        for (int r = 0; r < 4; ++r) {
+            n[r] = __ldcg(&ctl->join_n[j][r]);
+            first[r + 1] = first[r] + (n[r] + shift + size - 1u) / size;
+        }
+    }
+    __device__ __forceinline__ unsigned low(unsigned k, unsigned size) const { return k ? k * size - shift : 0u; }
+};
+constexpr unsigned kJoinLeast = 2048, kJoinMost = 8192;   // points of a segment
+static_assert(kJoinMost + 2 <= QcQueue::kCap && QcQueue::kBuckets >= kPtGroups, "a segment's points, the pieces' places");
+
+// Segment k of queue r in round j.
+__device__ void join_segment(const LargeArgs& a, QcQueue& q, const JoinPlan& p, const JoinPlan& was, int j, int r,
+                             unsigned k, unsigned size, unsigned pre) {
+    constexpr int T = kLargeThreads, kE = kPtGroups / T;
+    const int tid = threadIdx.x;
+    Ctl* ctl = a.ctl;
+    // the places of the pieces that round j - 1 left of the queue
+    const unsigned t0 = j ? was.first[r] : __ldcg(&ctl->q_tile[r]);
+    const unsigned np = (j ? was.first[r + 1] : __ldcg(&ctl->q_tile[r + 1])) - t0;
+    const unsigned* lens = j ? a.seg[(j - 1) & 1] : reinterpret_cast<const unsigned*>(a.tlen);
+    unsigned c[kE], sum = 0u;
+#pragma unroll
+    for (int e = 0; e < kE; ++e) {
+        const unsigned t = tid * kE + e;
+        c[e] = t < np ? __ldcg(lens + t0 + t) : 0u;
+        sum += c[e];
+    }
+    int tot;
+    unsigned run = (unsigned)block_excl_scan((int)sum, q.tmp, &tot);
+#pragma unroll
+    for (int e = 0; e < kE; ++e) {
+        q.cnt[tid * kE + e] = run;
+        run += c[e];
+    }
+    __syncthreads();
+    const unsigned lo = p.low(k, size), hi = min(p.n[r], (k + 1u) * size - p.shift);
+    const unsigned left = lo ? 1u : 0u, right = hi < p.n[r] ? 1u : 0u;
+    const int m = (int)(hi - lo + left + right);
+    for (int x = tid; x < m; x += T) {
+        const unsigned i = lo - left + x;
+        unsigned b = 0u, e = np;   // the last piece that begins at or before i (empty ones begin where the next does)
+        while (e - b > 1u) {
+            const unsigned mid = (b + e) >> 1;
+            if (q.cnt[mid] <= i) b = mid;
+            else e = mid;
+        }
+        unsigned u, v;
+        int id;
+        if (j & 1) {
+            const size_t at = (size_t)pre + was.low(b, size) + (i - q.cnt[b]);
+            const uint64_t w = __ldcg(a.vB + at);
+            u = (unsigned)(w >> kKeyBits);
+            v = (unsigned)(w & kKeyMask);
+            id = (int)__ldcg(a.kB + at);
+        } else {
+            const size_t at = (j ? (size_t)pre + was.low(b, size) : (size_t)__ldcg(a.tbeg + t0 + b)) + (i - q.cnt[b]);
+            u = (unsigned)__ldcg(a.cu + at);
+            v = (unsigned)__ldcg(a.cv + at);
+            id = __ldcg(a.ci + at);
+        }
+        q.a[x] = qc_pack(u, v, (unsigned)x);
+        q.si[x] = id;
+    }
+    __syncthreads();
+    unsigned long long *src = q.a, *dst = q.b;
+    const int len = qc_eliminate<T>(src, dst, m, q.tmp) - (int)(left + right);   // the ends stay
+    for (int x = tid; x < len; x += T) {
+        const unsigned long long w = src[x + left];
+        const size_t at = (size_t)pre + lo + x;
+        if (j & 1) {
+            a.cu[at] = qc_u(w);
+            a.cv[at] = qc_v(w);
+            a.ci[at] = q.si[qc_pos(w)];
+        } else {
+            a.vB[at] = w >> kQcPosBits;
+            a.kB[at] = (uint32_t)q.si[qc_pos(w)];
+        }
+    }
+    if (tid == 0) {
+        a.seg[j & 1][p.first[r] + k] = (unsigned)len;
+        atomicAdd(&ctl->join_n[j + 1][r], (unsigned)len);
+    }
+}
+
+// All blocks.  Returns the last round in the one block that finished it (the
+// queues' chains are at their places, without gaps), else -1; *go is false when a
+// wait gave up.
+__device__ int join_rounds(const LargeArgs& a, QcQueue& q, const unsigned (&pre)[5], bool* go) {
+    __shared__ JoinPlan s_p[2];
+    __shared__ unsigned s_size;
+    const int tid = threadIdx.x;
+    Ctl* ctl = a.ctl;
+    if (tid == 0) {
+        unsigned n = 0u;
+        for (int r = 0; r < 4; ++r) n += __ldcg(&ctl->join_n[0][r]);
+        s_size = max(kJoinLeast, min(kJoinMost, (n / gridDim.x + 2u) & ~1u));
+    }
+    __syncthreads();
+    const unsigned size = s_size;
+    for (int j = 0; j < kJoinRounds; ++j) {
+        JoinPlan &p = s_p[j & 1], &was = s_p[(j & 1) ^ 1];
+        if (tid == 0) p.set(ctl, j, size);
+        __syncthreads();
+        const unsigned items = p.first[4];
+        bool last = false;
+        if (items <= (unsigned)kPtGroups) {
+            for (unsigned it; (it = claim_item(ctl, kLargeJoin + j)) < items;) {
+                const int r = it >= p.first[2] ? (it >= p.first[3] ? 3 : 2) : (it >= p.first[1] ? 1 : 0);
+                join_segment(a, q, p, was, j, r, it - p.first[r], size, pre[r]);
+                last = finish_items(ctl, kLargeJoin + j, 1u, items);
+            }
+            if (!wait_phase(ctl, kLargeJoin + j, items)) {
+                *go = false;
+                return -1;
+            }
+        } else {   // too many points: the sort
+            last = blockIdx.x == 0;
+        }
+        unsigned before = 0u, after = 0u;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            before += p.n[r];
+            after += __ldcg(&ctl->join_n[j + 1][r]);
+        }
+        if (items <= (unsigned)kPtGroups && before == after) return last ? j : -1;
+        if (items > (unsigned)kPtGroups || j + 1 == kJoinRounds) {
+            if (last && tid == 0) ctl->bk_state = 2;   // the sort takes over (its input is untouched)
+            return -1;
+        }
+    }
+    return -1;
+}
+
 constexpr size_t large_max(size_t x, size_t y) { return x > y ? x : y; }
 constexpr size_t kLargeSmem = large_max(large_max(sizeof(QcJoin), sizeof(QcQueue)),
                                         large_max(sizeof(TileHistSmem), sizeof(TilePartSmem)));
 static_assert(kLargeSmem <= 226 * 1024 && QcJoin::kCap < (1 << kQcPosBits), "one block's shared memory");
 
 // Blocks 0 .. 3 end with a queue each: its chain from its records (path queues)
-// or from its tiles' chains (path tiles), left at the queue's records' place in
-// vB (u, v) and cu (index; each queue's own tiles' chains lie there, consumed by
-// then); the block that finishes last joins the four.
+// or from its tiles' chains (path tiles, while they fit), left at the queue's
+// records' place in vB (u, v) and cu (index; each queue's own tiles' chains lie
+// there, consumed by then); the block that finishes last joins the four.  Longer
+// tile chains are all blocks' work (join_rounds).
 __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ QMap s_m;
-    __shared__ int s_path, s_go, s_n, s_last;
+    __shared__ int s_path, s_way, s_n, s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, qq = blockIdx.x;
     constexpr int T = kLargeThreads;
     Ctl* ctl = a.ctl;
@@ -383,17 +542,22 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
         if (go) {
             tile_chains(a, *reinterpret_cast<QcQueue*>(s_dyn));
             CH_TL(ctl, 18, 1);
-            if (qq >= 4) return;
             go = wait_phase(ctl, kLargeChains, *(volatile unsigned*)&ctl->q_tile[4]);
         }
-        if (!go && tid == 0) *a.out_n = CH_ETIMEOUT;
-        if (!go) return;
-        // A tile's chain that outgrew its block has set bk_state before that phase's
-        // end; after it the word stays as it is until all four blocks have arrived
-        // below, so they agree on it (one read per block: its warps too).
-        if (tid == 0) s_go = *(volatile int*)&ctl->bk_state == 1;
+        if (!go) {
+            if (tid == 0) *a.out_n = CH_ETIMEOUT;
+            return;
+        }
+        // What follows is the same for every block: the totals stand, and a tile's
+        // chain that outgrew its block has set bk_state before the phase's end (one
+        // read per block: its warps too).
+        if (tid == 0) {
+            bool fit = true;
+            for (int r = 0; r < 4; ++r) fit = fit && __ldcg(&ctl->join_n[0][r]) <= (unsigned)QcJoin::kCap;
+            s_way = *(volatile int*)&ctl->bk_state != 1 ? kPathSort : fit ? kPathQueues : kPathTiles;
+        }
         __syncthreads();
-        if (!s_go) return;
+        if (s_way == kPathSort || (s_way == kPathQueues && qq >= 4)) return;
     }
     const uint32_t* keys = a.keys;
     const uint64_t* vals = a.vals;
@@ -410,9 +574,13 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) pre[r + 1] = pre[r] + ctl->rec_q[r];
     unsigned long long *src, *dst;
-    int len = 0;
-    bool ok = true;
-    if (path == kPathQueues) {
+    int len = 0, round = -1;
+    if (path == kPathTiles && s_way == kPathTiles) {   // too long for a block each
+        bool go = true;
+        round = join_rounds(a, *reinterpret_cast<QcQueue*>(s_dyn), pre, &go);
+        if (!go && tid == 0) *out_n = CH_ETIMEOUT;
+        if (round < 0) return;
+    } else if (path == kPathQueues) {
         QcQueue& q = *reinterpret_cast<QcQueue*>(s_dyn);
         const unsigned m = ctl->count;
         qc_gather<T, 4>(keys, vals, m, qq, q, &s_n);
@@ -446,52 +614,52 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
             run += c[e];
         }
         __syncthreads();
-        ok = tot <= QcJoin::kCap;
-        if (ok) {
-            for (unsigned t = warp; t < nt; t += T / 32) {
-                const unsigned o = q.off[t], l = (unsigned)__ldcg(tlen + t0 + t), b = __ldcg(tbeg + t0 + t);
-                for (unsigned j = lane; j < l; j += 32) {
-                    q.a[o + j] = qc_pack((unsigned)__ldcg(cu + b + j), (unsigned)__ldcg(cv + b + j), o + j);
-                    scratch[pre[qq] + o + j] = (unsigned)__ldcg(ci + b + j);
-                }
+        for (unsigned t = warp; t < nt; t += T / 32) {
+            const unsigned o = q.off[t], l = (unsigned)__ldcg(tlen + t0 + t), b = __ldcg(tbeg + t0 + t);
+            for (unsigned j = lane; j < l; j += 32) {
+                q.a[o + j] = qc_pack((unsigned)__ldcg(cu + b + j), (unsigned)__ldcg(cv + b + j), o + j);
+                scratch[pre[qq] + o + j] = (unsigned)__ldcg(ci + b + j);
             }
-            __syncthreads();
-            CH_TL(ctl, 19, 1);
-            src = q.a;
-            dst = q.b;
-            len = qc_eliminate<T>(src, dst, tot, q.tmp);
-            for (int j = tid; j < len; j += T) {
-                vout[pre[qq] + j] = src[j] >> kQcPosBits;
-                iout[pre[qq] + j] = (int)scratch[pre[qq] + qc_pos(src[j])];
-            }
+        }
+        __syncthreads();
+        CH_TL(ctl, 19, 1);
+        src = q.a;
+        dst = q.b;
+        len = qc_eliminate<T>(src, dst, tot, q.tmp);
+        for (int j = tid; j < len; j += T) {
+            vout[pre[qq] + j] = src[j] >> kQcPosBits;
+            iout[pre[qq] + j] = (int)scratch[pre[qq] + qc_pos(src[j])];
         }
     }
     CH_TL(ctl, 21, 1);
-    if (tid == 0) {
-        ctl->reg_end[qq] = ok ? (unsigned)len : 0u;
-        if (!ok) atomicExch(&ctl->join_over, 1);
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        s_last = atomicAdd(&ctl->joins_done, 1u) == 3u;
+    if (round < 0) {
+        if (tid == 0) ctl->reg_end[qq] = (unsigned)len;
         __threadfence();
-        if (s_last && *(volatile int*)&ctl->join_over) {
-            ctl->bk_state = 2;   // the sort takes over (its input is untouched)
-            s_last = 0;
+        __syncthreads();
+        if (tid == 0) {
+            s_last = atomicAdd(&ctl->joins_done, 1u) == 3u;
+            __threadfence();
         }
+        __syncthreads();
+        if (!s_last) return;
     }
-    __syncthreads();
-    if (!s_last) return;
     CH_TL(ctl, 22, 1);
+    const unsigned* lens = round < 0 ? ctl->reg_end : ctl->join_n[round + 1];
+    const bool spread = round >= 0 && (round & 1);   // in cu, cv, ci
+    const int* idx = round < 0 ? iout : spread ? ci : (const int*)a.kB;
     int off[5];
     off[0] = 0;
-    for (int r = 0; r < 4; ++r) off[r + 1] = off[r] + max((int)__ldcg(&ctl->reg_end[r]) - 1, 0);
+    for (int r = 0; r < 4; ++r) off[r + 1] = off[r] + max((int)__ldcg(lens + r) - 1, 0);
     auto get = [&](int r, int j, int& pu, int& pv, int& pi) {
-        const uint64_t x = __ldcg(vout + pre[r] + j);
-        pu = (int)(x >> kKeyBits);
-        pv = (int)(x & kKeyMask);
-        pi = __ldcg(iout + pre[r] + j);
+        if (spread) {
+            pu = __ldcg(cu + pre[r] + j);
+            pv = __ldcg(cv + pre[r] + j);
+        } else {
+            const uint64_t x = __ldcg(vout + pre[r] + j);
+            pu = (int)(x >> kKeyBits);
+            pv = (int)(x & kKeyMask);
+        }
+        pi = __ldcg(idx + pre[r] + j);
     };
     if (off[4] > kStitchLong) {
         stitch_long(off, get, n, ctl, out_idx, out_n);
@@ -515,7 +683,7 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
 void launch_large(Ctl* ctl, const uint32_t* kA, const uint64_t* vA, uint32_t* kB, uint64_t* vB, unsigned* tiles, int* cu,
                   int* cv, int* ci, long long n, int32_t* out_idx, int64_t* out_n, int grid, cudaStream_t s) {
     const LargeArgs a{ctl, kA, vA, kB, vB, tiles, tiles + kPtGroups, tiles + 2 * kPtGroups, tiles + 3 * kPtGroups,
-                      (int*)(tiles + 4 * kPtGroups), cu, cv, ci, n, out_idx, out_n};
+                      {tiles, tiles + kPtGroups}, (int*)(tiles + 4 * kPtGroups), cu, cv, ci, n, out_idx, out_n};
     large_kernel<<<grid, kLargeThreads, kLargeSmem, s>>>(a);
 }
 

@@ -22,6 +22,7 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
         ctl->rec_q[t] = 0u;
         if (t) ctl->blocks_done[t] = 0u;
     }
+    if (t < 4 * (kJoinRounds + 1)) (&ctl->join_n[0][0])[t] = 0u;
     if (t < kPhases) {
         ctl->claimed[t] = 0u;
         ctl->finished[t] = 0u;
@@ -39,7 +40,6 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
         ctl->path = kPathNone;
         ctl->beat = 0u;
         ctl->joins_done = 0u;
-        ctl->join_over = 0;
         ctl->roots_done = 0u;
         ctl->samp_dense = 0;
         ctl->oct_ready = 0;

@@ -1,7 +1,7 @@
 """The single hull's ways through many survivors (queues.cu, hull.cu), each by
 the counters that name it and bit-exact with the oracle: circles without a
-width, whose queues' tile chains fit one block or hand over to the sort, and a
-tile whose own chain does."""
+width, whose queues' tile chains fit one block or are joined in rounds, a tile
+whose own chain goes to the sort, and records crowded in one range of u."""
 import math
 
 import numpy as np
@@ -37,15 +37,15 @@ def _calls(lib, pts, calls):
         yield got.cpu().numpy(), lib.ch_hull_counters(stream)
 
 
-@pytest.mark.parametrize("n,stage", [(1_000_000, QUEUES_OR_TILES), (4_000_003, SORT), (6_000_001, SORT)])
-def test_circle(lib, n, stage):
+@pytest.mark.parametrize("n", [1_000_000, 4_000_003, 6_000_001, 20_000_003])
+def test_circle(lib, n):
     pts = _circle(n, n)
     want = oracle.hull(pts)
-    # past 13,000 tile-chain points in a queue (a block's capacity) the sort takes over
-    assert (want.size > 4 * 13_000) == (stage == SORT)
+    # past 13,000 tile-chain points in a queue (a block's capacity) all blocks join them in rounds
+    assert (want.size > 4 * 13_000) == (n > 1_000_000)
     for got, c in _calls(lib, pts, 100):
         np.testing.assert_array_equal(got, want)
-        assert c["stage"] == stage, c
+        assert c["stage"] == QUEUES_OR_TILES, c
 
 
 def _steps(most_u, most_v, ok):
