@@ -468,8 +468,8 @@ int ch_filter(const float* pts, int64_t n, int32_t* out_ext8, uint8_t* out_label
     uint32_t* kB = (uint32_t*)(base + L.off_kB);
     uint64_t* vB = (uint64_t*)(base + L.off_vB);
     const bool lab = out_labels || out_counts4;
-    // One read of the points that labels those of a region inside a sample's
-    // octagon at once and leaves the others for labels_kernel; inputs that stay
+    // One read of the points, which finds those of a region inside a sample's
+    // octagon (label 0) and leaves the others for labels_kernel; inputs that stay
     // in L2, or want no labels: the extremes first.
     const bool fused = lab && n > kFilterTwoPassMax;
     const unsigned switch_at = fused ? (unsigned)(n >> 5) : 0xFFFFFFFFu;
@@ -483,8 +483,8 @@ int ch_filter(const float* pts, int64_t n, int32_t* out_ext8, uint8_t* out_label
     }
     {
         ProfScope p("main_filter", s);
-        launch_main_labels(pts, n, head, ntiles, ctl, vB, kB, switch_at, kA, vA, lab && !fused, out_labels,
-                           di.sms * di.occ_main, s);
+        launch_main_labels(pts, n, head, ntiles, ctl, vB, kB, switch_at, kA, vA, lab && !fused, di.sms * di.occ_main,
+                           s);
     }
     if (lab) {
         ProfScope p("labels", s);

@@ -100,12 +100,12 @@ constexpr unsigned kSpinLimit = 1u << 20;     // polls of a bounded wait (of a p
 
 constexpr int kJoinRounds = 8;                // rounds that join a queue's tile chains, at most
 
-// Phases of dense_kernel, large_kernel and sort_kernel whose end their blocks
+// Phases of dense_kernel, large_kernel, sort_kernel and labels_kernel whose end their blocks
 // wait for (claim_item, wait_phase).
 enum Phase {
     kDenseBins = 0, kDenseMerge, kDensePoly, kDenseRadius,
     kLargeHist, kLargeCut, kLargePart, kLargeChains, kLargeJoin,
-    kSortHist = kLargeJoin + kJoinRounds, kSortPass, kPhases = kSortPass + kSortPasses
+    kSortHist = kLargeJoin + kJoinRounds, kSortPass, kLabelZero = kSortPass + kSortPasses, kPhases
 };
 
 // Directions of the 8 extremes in counter-clockwise octagon order.

@@ -24,10 +24,10 @@
 //                   inside the polygon; the extremes are among the others.
 //   (post.cu)       the classification of the survivors and the hull.
 //   labels_kernel   ch_filter: the label array Q of Alg. 2 (paper rule).  On
-//                   large inputs the main pass has set it to 0 and left the
-//                   points that may have another label, as in fused mode: one
-//                   read of the points instead of two (1e8 normal points: 183 us
-//                   a call against 288; 1.7 GB of needed traffic became 0.9).
+//                   large inputs the main pass has left the points that may have
+//                   a label other than 0, as in fused mode: one read of the
+//                   points instead of two (1e8 normal points: 183 us a call
+//                   against 288; 1.7 GB of needed traffic became 0.9).
 #include "ch_internal.cuh"
 #include "hullcore.cuh"
 #include "launch.h"
@@ -435,14 +435,13 @@ __device__ __noinline__ void finalize_block(const float* __restrict__ pts, long 
 constexpr size_t kMainSmemBytes = (size_t)8 * kStages * kWarpTileF4 * sizeof(float4);
 
 // With kLabels (ch_filter): the raw survivors are the points not strictly inside
-// the region of the sample pass (oct_s's inner bounds), and every label is set
-// to 0 beside them, 16 bytes a store; labels_kernel sets the survivors' ones.
-// two_pass: leave the points in L2 for a second pass.
+// the region of the sample pass (oct_s's inner bounds).  two_pass: leave the
+// points in L2 for a second pass.
 template <bool kLabels>
 __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ pts, long long n, int head,
                                                       long long ntiles, Ctl* ctl, uint64_t* raw_xy,
                                                       uint32_t* raw_idx, unsigned switch_at, uint32_t* keys,
-                                                      uint64_t* vals, int two_pass, uint8_t* labels) {
+                                                      uint64_t* vals, int two_pass) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ int s_inner[8];
     __shared__ float s_edge[24];
@@ -495,20 +494,6 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
         if (any) track_tile(tr, tk, code);
     };
     if (gwarp == 0 && head) scalar_range(0, head, 0u);
-    int4* words = nullptr;
-    long long nwords = 0;
-    auto zero16 = [](int4* p) { __stcs(p, make_int4(0, 0, 0, 0)); };
-    if (kLabels && labels) {
-        const long long lead = min(n, (long long)((16u - ((uintptr_t)labels & 15u)) & 15u));
-        words = reinterpret_cast<int4*>(labels + lead);
-        nwords = (n - lead) / 16;
-        if (filt && gwarp == nwarps - 1) {   // what the tiles' shares leave: fewer than 16 bytes at each end, 33 words
-            if (lane < lead) labels[lane] = 0;
-            for (long long i = lead + 16 * nwords + lane; i < n; i += 32) labels[i] = 0;
-            for (long long w = 32 * ntiles + lane; w < nwords; w += 32) zero16(words + w);
-        }
-    }
-
     // Warp tiles t = gwarp + k * nwarps stream through a double-buffered
     // shared-memory ring filled by bulk asynchronous copies (TMA).
     WarpStream ws{reinterpret_cast<float4*>(dsm) + warp * kStages * kWarpTileF4, s_bar[warp],
@@ -532,10 +517,6 @@ __global__ void __launch_bounds__(256, 2) main_kernel(const float* __restrict__ 
             tile_keys2(tk, X0, Y0, X1, Y1, j == 0);
         }
         track_tile(tr, tk, (unsigned)(t + 1));
-        if (kLabels && filt && labels) {   // the tile's share of the label array's 16-byte words
-            const long long w = 32 * t + lane;
-            if (w < nwords) zero16(words + w);
-        }
         if (filt) {
             // Points strictly inside the inner region of the sample octagon
             // are strictly inside the hull; every other point is a raw
@@ -1042,8 +1023,26 @@ __device__ __forceinline__ int label_of(float x, float y, const Octagon& o) {
     return in_inner_strict(o, X, Y) ? -1 : classify_paper_slow(x, y, &o);
 }
 
-// After a fused main pass (mode 0: every label is 0, the others' points are the
-// raw survivors) the survivors' labels, one per thread.  Else all points: up to
+// After a fused main pass (mode 0): every label 0, 16 bytes a store, a share of
+// the words per item.  Not beside the main pass's reads (181 us a call on 1e8
+// points, 183 here, 191 by a kernel of its own): the caller's labels stay as they
+// are when that pass meets a bad coordinate.  Whole block.
+__device__ __forceinline__ void zero_labels(uint8_t* labels, long long n, Ctl* ctl) {
+    const long long lead = min(n, (long long)((16u - ((uintptr_t)labels & 15u)) & 15u)), words = (n - lead) / 16;
+    int4* w = reinterpret_cast<int4*>(labels + lead);
+    for (unsigned it; (it = claim_item(ctl, kLabelZero)) < gridDim.x;) {
+        const long long end = words * (it + 1) / gridDim.x;
+        for (long long j = words * it / gridDim.x + threadIdx.x; j < end; j += blockDim.x) __stcs(w + j, make_int4(0, 0, 0, 0));
+        if (it == 0u && threadIdx.x < 16) {   // what the words leave at each end
+            if (threadIdx.x < lead) labels[threadIdx.x] = 0;
+            if (threadIdx.x < n - lead - 16 * words) labels[lead + 16 * words + threadIdx.x] = 0;
+        }
+        finish_items(ctl, kLabelZero, 1u, gridDim.x);
+    }
+}
+
+// After a fused main pass (mode 0) every label is set to 0, then the raw
+// survivors' labels, one per thread.  Else all points: up to
 // kPointsMax one per thread, above each warp streams its warp tiles (512 points, behind the unaligned head point)
 // through a double-buffered shared-memory ring, as the main pass does, and
 // labels 4 consecutive points per lane and round; the label array's words
@@ -1069,14 +1068,24 @@ __global__ void __launch_bounds__(256) labels_kernel(const float* __restrict__ p
     unsigned c[4] = {0u, 0u, 0u, 0u};
     auto count = [&](int lab) { c[0] += lab == 0; c[1] += lab == 1; c[2] += lab == 2; c[3] += lab == 3; };
     if (ctl->mode == 0) {
+        // the first survivor's loads are in flight while the zeros go out
         const long long m = ctl->count_raw;
-        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += 32 * nwarps) {
-            const uint64_t xy = __ldcs(raw_xy + i);
-            const uint32_t id = __ldcs(raw_idx + i);
-            const int lab = classify_paper_slow((float)(int)(xy >> 32), (float)(int)(unsigned)xy, &s_o);
+        long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        uint64_t xy = i < m ? __ldcs(raw_xy + i) : 0ull;
+        uint32_t id = i < m ? __ldcs(raw_idx + i) : 0u;
+        if (labels) zero_labels(labels, n, ctl);
+        bool zeroed = !labels;
+        do {
+            int lab = -1;
+            if (i < m) lab = classify_paper_slow((float)(int)(xy >> 32), (float)(int)(unsigned)xy, &s_o);
+            if (!zeroed && !wait_phase(ctl, kLabelZero, gridDim.x)) return;
+            zeroed = true;
             if (labels && lab >= 0) labels[id] = (uint8_t)(lab + 1);
             count(lab);
-        }
+            i += 32 * nwarps;
+            xy = i < m ? __ldcs(raw_xy + i) : 0ull;
+            id = i < m ? __ldcs(raw_idx + i) : 0u;
+        } while (i < m);
     } else if (n <= kPointsMax) {
         for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 32 * nwarps) {
             const float2 p = reinterpret_cast<const float2*>(pts)[i];
@@ -1158,14 +1167,14 @@ void launch_main(const float* pts, long long n, int head, long long ntiles, Ctl*
                  uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass, int grid,
                  cudaStream_t s) {
     main_kernel<false><<<grid, 256, kMainSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, switch_at, keys,
-                                                         vals, two_pass, nullptr);
+                                                         vals, two_pass);
 }
 
 void launch_main_labels(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, uint64_t* raw_xy,
-                        uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass,
-                        uint8_t* labels, int grid, cudaStream_t s) {
+                        uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass, int grid,
+                        cudaStream_t s) {
     main_kernel<true><<<grid, 256, kMainSmemBytes, s>>>(pts, n, head, ntiles, ctl, raw_xy, raw_idx, switch_at, keys,
-                                                        vals, two_pass, labels);
+                                                        vals, two_pass);
 }
 
 void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, void* bins, void* poly,

@@ -36,8 +36,8 @@ void launch_main(const float* pts, long long n, int head, long long ntiles, Ctl*
                  uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass, int grid,
                  cudaStream_t s);
 void launch_main_labels(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, uint64_t* raw_xy,
-                        uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass,
-                        uint8_t* labels, int grid, cudaStream_t s);
+                        uint32_t* raw_idx, unsigned switch_at, uint32_t* keys, uint64_t* vals, int two_pass, int grid,
+                        cudaStream_t s);
 // The dense data's pass (star bins, star polygon, filter): the bins and the
 // polygon live in the workspace.
 void launch_dense(const float* pts, long long n, int head, long long ntiles, Ctl* ctl, void* bins, void* poly,
