@@ -71,10 +71,11 @@ constexpr int kSampleTiles = 1024;            // warp tiles read by the sample p
 constexpr int kStarBins = 8192;
 constexpr int kStarBlocks = 160;              // blocks of dense_kernel at most
 constexpr long long kStarMinTiles = 128;      // inputs below this many warp tiles get no star polygon
-// Inputs of at most this many points stay in L2 between two passes, so the
-// extremes come first and no sample is needed (the fused pass saves reads of
-// HBM at the price of one more kernel in the chain).
-constexpr long long kTwoPassMax = 1 << 22;
+// Inputs of at most this many points take two passes: the extremes first, without
+// a sample, and the second read from L2.  Past it a sample and one pass are the
+// faster (uniform points: 68 us by two passes and 71 by one at 2.0 M, 75 and 66 at
+// 2.5 M, 86 and 72 at 4.2 M).
+constexpr long long kTwoPassMax = 1 << 21;
 constexpr long long kSmallMax = 8192;   // one block finds the records of so few points (small_kernel)
 // The label passes take a point per thread up to here, above warp tiles of 512
 // points (which leave most of the chip idle on small inputs).
