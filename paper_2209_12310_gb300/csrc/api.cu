@@ -483,8 +483,8 @@ int ch_filter(const float* pts, int64_t n, int32_t* out_ext8, uint8_t* out_label
     }
     {
         ProfScope p("main_filter", s);
-        launch_main_labels(pts, n, head, ntiles, ctl, vB, kB, switch_at, kA, vA, lab && !fused, di.sms * di.occ_main,
-                           s);
+        launch_main_labels(pts, n, head, ntiles, ctl, vB, kB, switch_at, kA, vA, lab && n <= kFilterKeepMax,
+                           di.sms * di.occ_main, s);
     }
     if (lab) {
         ProfScope p("labels", s);

@@ -80,8 +80,13 @@ constexpr long long kSmallMax = 8192;   // one block finds the records of so few
 // The label passes take a point per thread up to here, above warp tiles of 512
 // points (which leave most of the chip idle on small inputs).
 constexpr long long kPointsMax = 1 << 21;
-// ch_filter's: its second read also stays in L2 up to 64 MB of points.
-constexpr long long kFilterTwoPassMax = 1 << 23;
+// ch_filter: up to kFilterTwoPassMax points two reads (the second from L2 while the
+// points are 64 MB at most), above one and a sample before it, which only pays when
+// nearly all points lie inside the sample's region (8.5 M uniform points 62 us by
+// two reads and 67 by one, 16.7 M 84 and 80, 1e8 288 and 183; of a triangle, which
+// is read twice all the same, 79 and 88, 124 and 134).
+constexpr long long kFilterKeepMax = 1 << 23;
+constexpr long long kFilterTwoPassMax = 1 << 24;
 constexpr int kMaxLevels = 32;
 
 // Warp tiles read by the sample pass: about 1/32 of the input, at most
