@@ -147,7 +147,8 @@ __device__ __forceinline__ void qc_bitonic(unsigned long long* s, int P, const i
         }
 }
 
-// The lower chain of the n >= 1 points in src, ordered by (u, v, index):
+// The lower chain of the n >= 1 points in src, ordered by (u, v), the first of
+// equal points with their lowest index:
 // returns its length; src points at it (the two buffers change roles).  Of
 // points of equal u only the first can be a vertex: the others are skipped
 // where they follow it.  Whole block of T threads.  Runs have an odd length,
@@ -248,9 +249,8 @@ __device__ __noinline__ int qc_thin(Q& q, int n) {
 // equal width in u hold about two points each; every point
 // counts the points of its bucket before it (independent loads, where an
 // insertion sort per bucket is a chain of them: records that a polygon leaves
-// can crowd a few buckets by the hundred; by words, the indices compared only
-// among equal points: with qc_less throughout this loop was 23,000 of the sort's
-// 32,000 cycles for 8000 points).  When some bucket holds more than kQcBucket,
+// can crowd a few buckets by the hundred; by words, not indices: with qc_less this
+// loop was 23,000 of the sort's 32,000 cycles for 8000 points).  When some bucket holds more than kQcBucket,
 // the points are thinned first (copies of one vertex all share a bucket) and the
 // buckets span what is left; still crowded, the whole array goes through a
 // bitonic sort.
@@ -318,16 +318,14 @@ __device__ int qc_sort(Q& q, int n, int lo, int hi) {
         const unsigned long long w = q.b[j];
         const int b = bucket(w);   // cnt[b] is now the end of bucket b
         const int s = b ? (int)q.cnt[b - 1] : 0, e = (int)q.cnt[b];
-        int r = s, same = 0;   // same: points of equal (u, v), this one among them
+        int r = s;
+        unsigned long long first = w;   // of the points of equal (u, v): the one that can be a vertex
         for (int i = s; i < e; ++i) {
             const unsigned long long x = q.b[i];
             r += x < w ? 1 : 0;
-            same += ((x ^ w) >> kQcPosBits) == 0ull ? 1 : 0;
+            if (((x ^ w) >> kQcPosBits) == 0ull) first = x < first ? x : first;
         }
-        if (same > 1) {   // by index
-            r = s;
-            for (int i = s; i < e; ++i) r += qc_less(q.b[i], w, q.si) ? 1 : 0;
-        }
+        if (first != w) atomicMin(&q.si[qc_pos(first)], q.si[qc_pos(w)]);   // it takes the lowest index
         q.a[r] = w;
     }
     __syncthreads();
