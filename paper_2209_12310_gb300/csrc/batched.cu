@@ -585,23 +585,27 @@ struct BtWarpSmem {
 };
 
 // The inner region of an octagon as four scaled keys: a point is inside when
-// |key * scale + offset| <= 1 for x, y, x + y and x - y.  The region is taken 8
-// units smaller on each side (16 for x + y) than the octagon's: the three
-// roundings of a scaled key are below 2^-23 (|key| + |centre|), 4 units (8 and
-// 2 for the sum), so a point that passes is inside.
+// |key * scale + offset| <= 1 for x, y, x + y and x - y.  Keys are integers, so the
+// bounds lie half a unit outside lo and hi; the roundings (of the bounds' sum, the
+// scale, the offset and the key x + y) move them by less than 7 parts in 2^24 of
+// the larger of |lo| and |hi|, so they are taken 8 parts further in: a point that
+// passes is inside.  (A fixed margin of 8 units lost most of the region of a set
+// with small coordinates: 256 sets of 200,000 points in [0, 50)^2 took 667 us, 267
+// with integer keys, 250 now.)
 struct BtInner {
     float sx, ox, sy, oy, ss, os, sd, od;
-    __device__ __forceinline__ void axis(int lo, int hi, float margin, float& s, float& o) const {
-        const float h = 0.5f * (float)(hi - lo) - margin;
+    __device__ __forceinline__ void axis(int lo, int hi, float& s, float& o) const {
+        const float margin = (float)max(abs(lo), abs(hi)) * (1.0f / 2097152.0f);
+        const float h = 0.5f * (float)(hi - lo) + (0.5f - margin);
         const bool some = lo <= hi && h > 0.0f;
         s = some ? 1.0f / h : 0.0f;
         o = some ? -0.5f * ((float)lo + (float)hi) * s : 2.0f;
     }
     __device__ __forceinline__ void set(const Octagon& o) {
-        axis(o.in_lo[0], o.in_hi[0], 8.0f, sx, ox);
-        axis(o.in_lo[1], o.in_hi[1], 8.0f, sy, oy);
-        axis(o.in_lo[2], o.in_hi[2], 16.0f, ss, os);
-        axis(o.in_lo[3] - kCoordLimit, o.in_hi[3] - kCoordLimit, 8.0f, sd, od);
+        axis(o.in_lo[0], o.in_hi[0], sx, ox);
+        axis(o.in_lo[1], o.in_hi[1], sy, oy);
+        axis(o.in_lo[2], o.in_hi[2], ss, os);
+        axis(o.in_lo[3] - kCoordLimit, o.in_hi[3] - kCoordLimit, sd, od);
     }
     __device__ __forceinline__ bool outside(float x, float y) const {
         float m;
