@@ -429,17 +429,19 @@ __device__ __forceinline__ long long qh_depth(const Q& q, int a, int b, int u, i
 // The four chains; on success the joined cycle (every chain without its end
 // vertex, which starts the next chain) is in q.ru / q.rv / q.ri as x, y,
 // index, and its length in *mv.  False when a limit is exceeded (the caller
-// falls back to the sort-based path).  Whole block; m records in q.
-template <class Q>
+// falls back to the sort-based path; with kEarly also after three rounds, when
+// more than half the records are still outside the chains and would, as vertices,
+// exceed the capacity).  Whole block; m records in q.
+template <bool kEarly = false, class Q>
 static __device__ bool qh_chains(Q& q, int m, int* mv) {
     constexpr int kQhCap = Q::kVertices;
     __shared__ unsigned long long s_s[4], s_e[4];
-    __shared__ int s_si[4], s_ei[4], s_len[4], s_nvert, s_changed, s_fail;
+    __shared__ int s_si[4], s_ei[4], s_len[4], s_nvert, s_changed, s_fail, s_live;
     const int tid = threadIdx.x, T = blockDim.x;
     constexpr int kVBits = kKeyBits;   // v < 2^25 in every frame
     constexpr unsigned long long kVMask = (1ull << kVBits) - 1ull;
     if (tid < 4) { s_s[tid] = ~0ull; s_e[tid] = 0ull; s_si[tid] = INT_MAX; s_ei[tid] = INT_MAX; }
-    if (tid == 0) { s_nvert = 8; s_fail = 0; s_changed = 0; }
+    if (tid == 0) { s_nvert = 8; s_fail = 0; s_changed = 0; s_live = 0; }
     for (int a = tid; a < kQhCap; a += T) { q.segmax[a] = 0ull; q.segarg[a] = ~0ull; q.splitu[a] = -1; }
     __syncthreads();
     // S = minimum (u, v); E = maximum u, then minimum v; then lowest indices
@@ -481,6 +483,7 @@ static __device__ bool qh_chains(Q& q, int m, int* mv) {
     for (int round = 0;; ++round) {
         const int nv = s_nvert;
         // depths; each segment's maximum
+        int live = 0;
         for (int i = tid; i < m; i += T) {
             int a = q.rs[i];
             if (a < 0) continue;
@@ -500,8 +503,11 @@ static __device__ bool qh_chains(Q& q, int m, int* mv) {
                     atomicMax(&q.segmax[a], (unsigned long long)d);
             }
             q.rs[i] = a;
+            live += a >= 0;
         }
+        if (kEarly && round == 3 && live) atomicAdd(&s_live, live);
         __syncthreads();
+        if (kEarly && round == 3 && 2 * s_live > m && s_live + nv > kQhCap) return false;
         CH_TRACE_MARK();
         if (tid == 0) s_changed = 0;
         // the deepest record per segment: smallest u, then index
