@@ -44,6 +44,7 @@ constexpr size_t kF16StreamSmemBytes = (size_t)(kF16Threads / 32) * kStages * kW
 // Up to here the extremes pass leaves the points in L2 for the label pass (96 MB;
 // 20 M points took 98 us a call evicted first, the two reads from HBM).
 constexpr long long kF16Keep = 12ll << 20;
+constexpr long long kF16PointsMax = 3ll << 20;   // a point per thread up to here (f16_extremes_points)
 constexpr int kF16Bias = 1 << 26;   // makes every key positive below 2^27
 
 struct F16Ctl {
@@ -54,8 +55,7 @@ struct F16Ctl {
     unsigned long long tile_packed[16];
     unsigned done;                  // last-arriver counter
     int ready;                      // the last block filled the fields below
-    int vx[16], vy[16], live[16];   // the 16-gon's vertices, edges of non-zero length
-    int none;                       // zero area: nothing is inside
+    int vx[16], vy[16];             // the 16-gon's vertices
     Octagon oct;                    // octagon of the even directions, with its inner region
 };
 static_assert(kF16Threads == 256, "eight warps find the 16 directions' points");
@@ -293,26 +293,14 @@ __global__ void __launch_bounds__(kF16Threads, 2) f16_extremes(const float* __re
         c->vy[k] = __float2int_rn(p.y);
     }
     __syncthreads();
-    // what the label pass needs: live edges, zero area, and the octagon of the
-    // even directions with its inner region (inside the 16-gon)
+    // what the label pass needs beside the vertices: the octagon of the even
+    // directions with its inner region (inside the 16-gon)
     __shared__ int s_vx[8], s_vy[8], s_id[8];
     __shared__ Octagon s_o;
-    if (threadIdx.x < 16) {
-        const int k = threadIdx.x, j = (k + 1) & 15;
-        c->live[k] = (c->vx[k] != c->vx[j] || c->vy[k] != c->vy[j]) ? 1 : 0;
-    }
     if (threadIdx.x < 8) {
         s_vx[threadIdx.x] = c->vx[2 * threadIdx.x];
         s_vy[threadIdx.x] = c->vy[2 * threadIdx.x];
         s_id[threadIdx.x] = (int)(0xFFFFFFFFu - (unsigned)(c->packed[2 * threadIdx.x] & 0xFFFFFFFFull));
-    }
-    if (threadIdx.x == 0) {
-        long long a2 = 0;
-        for (int k = 0; k < 16; ++k) {
-            const int j = (k + 1) & 15;
-            a2 += (long long)c->vx[k] * c->vy[j] - (long long)c->vx[j] * c->vy[k];
-        }
-        c->none = a2 == 0 ? 1 : 0;
     }
     __syncthreads();
     setup_octagon_block(s_o, s_vx, s_vy, s_id, true);
@@ -330,68 +318,126 @@ __global__ void __launch_bounds__(kF16Threads, 2) f16_extremes(const float* __re
 // are settled inline (that octagon lies inside the 16-gon), the others by the
 // exact 16-edge test; the head and the ragged tail are labelled point by point
 // by the first warp.
-// Out of line: the inner-region test settles most points, and the streaming
-// loop stays small.
-static __device__ __noinline__ int f16_label_exact(int X, int Y, const int* vx, const int* vy, const int* live,
-                                                   bool none) {
-    bool inside = !none;
+// Edge a -> b as a float function e(p) = A x + B y + C, positive left of the edge,
+// its coefficients divided by the length |dx| + |dy|.  The factor 1 / length is off
+// by 2 parts in 2^24, A and B (|A| + |B| = 1) by 3 and C (below 2^24) by 4, so by
+// less than 3 and 4 in e; the two multiply-adds stay below 2^25 and round by 2 at
+// most: e is off by less than kF16Tol, whatever the edge's length.  (With the
+// octagon's one bound for all lengths a short edge left every point undecided: 20 M
+// points of a triangle took 220 us, 157 now.)  A zero-length edge is a huge constant.
+constexpr float kF16Tol = 16.0f;
+__device__ __forceinline__ float4 f16_edge(int ax, int ay, int bx, int by) {
+    const long long dx = bx - ax, dy = by - ay;
+    const long long len = (dx < 0 ? -dx : dx) + (dy < 0 ? -dy : dy);
+    if (len == 0) return make_float4(0.0f, 0.0f, kHugePositive, 0.0f);
+    const float inv = 1.0f / __ll2float_rn(len);
+    return make_float4((float)-dy * inv, (float)dx * inv, __ll2float_rn(dy * ax - dx * ay) * inv, 0.0f);
+}
+__device__ __forceinline__ float f16_value(const float4& e, float x, float y) { return fmaf(e.x, x, fmaf(e.y, y, e.z)); }
+
+// The label from the edge functions in float: inside when surely left of every
+// edge, else, when surely right of one (or the polygon has no area), the first
+// quadrilateral edge it is surely right of while surely left of those before;
+// kF16Undecided where the error bound leaves that open.  The exact test of 16
+// int64 orientations decided every point outside the inner region before: 90 us a
+// call on 2.2 M ring points, 52 now.
+__device__ __forceinline__ int f16_label_float(float x, float y, const float4* e, bool none) {
+    float m = kHugePositive;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const int j = (k + 1) & 15;
-        if (live[k] && orient64(vx[k], vy[k], vx[j], vy[j], X, Y) <= 0) inside = false;
-    }
-    int r = -1;
-    if (!inside) {
+    for (int k = 0; k < 16; ++k) m = fminf(m, f16_value(e[k], x, y));
+    if (!none && m > kF16Tol) return -1;
+    if (!none && m >= -kF16Tol) return kF16Undecided;
+    int r = kF16Undecided;   // right of no edge: near
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {   // W->S, S->E, E->N, N->W
-            const int a = 4 * q, b = (4 * q + 4) & 15;
-            if (r < 0 && orient64(vx[a], vy[a], vx[b], vy[b], X, Y) < 0) r = q;
-        }
+    for (int k = 3; k >= 0; --k) {
+        const float v = f16_value(e[16 + k], x, y);
+        r = v < -kF16Tol ? k : v <= kF16Tol ? (int)kF16Undecided : r;
     }
     return r;
 }
 
-// The label from the edge functions in float (error below kEdgeTol, octagon.cuh):
-// inside when surely left of every edge, else, when surely right of one (or the
-// polygon has no area), the first quadrilateral edge it is surely right of while
-// surely left of those before; kF16Undecided where the error bound leaves that
-// open.  The exact test of 16 int64 orientations decided every point outside
-// the inner region before: 90 us a call on 2.2 M ring points, 52 now.
-__device__ __forceinline__ int f16_label_float(float x, float y, const float4* e, bool none) {
-    float m = kHugePositive;
+// The polygon's and the quadrilateral's edges, for a block.
+struct F16Poly {
+    float4 e[20];            // the 16 edges' functions, then the quadrilateral's
+    float2 v[16];            // the vertices,
+    int vx[16], vy[16];
+    int lab[16];             // and their labels: on the polygon, so outside
+    int none;                // zero area: nothing is inside
+    // The rest from vx and vy, by the first warp; a barrier before and after.
+    __device__ __forceinline__ void set(int t) {
+        if (t < 20) {
+            const int a = t < 16 ? t : 4 * (t - 16), b = (t < 16 ? t + 1 : a + 4) & 15;
+            e[t] = f16_edge(vx[a], vy[a], vx[b], vy[b]);
+        }
+        if (t < 16) {
+            v[t] = make_float2((float)vx[t], (float)vy[t]);
+            int r = -1;
+            for (int q = 3; q >= 0; --q) {   // W->S, S->E, E->N, N->W
+                const int a = 4 * q, b = (4 * q + 4) & 15;
+                if (orient64(vx[a], vy[a], vx[b], vy[b], vx[t], vy[t]) < 0) r = q;
+            }
+            lab[t] = r;
+        }
+        if (t < 32) {
+            const int k = t & 15, j = (k + 1) & 15;
+            long long a2 = (long long)vx[k] * vy[j] - (long long)vx[j] * vy[k];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) m = fminf(m, fmaf(e[k].x, x, fmaf(e[k].y, y, e[k].z)));
-    if (!none && m > kEdgeTol) return -1;
-    if (!none && m >= -kEdgeTol) return kF16Undecided;
-    int r = kF16Undecided;   // right of no edge: the exact test
-#pragma unroll
-    for (int k = 3; k >= 0; --k) {
-        const float v = fmaf(e[16 + k].x, x, fmaf(e[16 + k].y, y, e[16 + k].z));
-        r = v < -kEdgeTol ? k : v <= kEdgeTol ? (int)kF16Undecided : r;
+            for (int o = 8; o; o >>= 1) a2 += __shfl_xor_sync(0xFFFFFFFFu, a2, o);
+            if (t == 0) none = a2 == 0 ? 1 : 0;
+        }
     }
-    return r;
+};
+
+// The same where the bound leaves edges open: copies of a vertex have its label,
+// the others take int64 orientations of those edges.  Out of line: most points are
+// settled before, and the streaming loop stays small.  With all orientations exact,
+// 5 M points with 60 % copies of a vertex took 140 us, 92 now.
+static __device__ __noinline__ int f16_label_near(float x, float y, const F16Poly& p) {
+    int at = -1;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) at = x == p.v[k].x && y == p.v[k].y ? k : at;
+    if (at >= 0) return p.lab[at];
+    const int X = __float2int_rn(x), Y = __float2int_rn(y);
+    unsigned open = 0u;   // not surely left of the edge
+    bool inside = !p.none;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const float v = f16_value(p.e[k], x, y);
+        open |= v <= kF16Tol ? 1u << k : 0u;
+        inside = inside && v >= -kF16Tol;
+    }
+    for (; inside && open; open &= open - 1u) {
+        const int a = __ffs((int)open) - 1, b = (a + 1) & 15;
+        inside = orient64(p.vx[a], p.vy[a], p.vx[b], p.vy[b], X, Y) > 0;
+    }
+    if (inside) return -1;
+    for (int q = 0; q < 4; ++q) {   // W->S, S->E, E->N, N->W
+        const float v = f16_value(p.e[16 + q], x, y);
+        const int a = 4 * q, b = (4 * q + 4) & 15;
+        if (v < -kF16Tol || (v <= kF16Tol && orient64(p.vx[a], p.vy[a], p.vx[b], p.vy[b], X, Y) < 0)) return q;
+    }
+    return -1;
 }
 
 __global__ void __launch_bounds__(kF16Threads) f16_labels(const float* __restrict__ pts, long long n, int head,
                                                           long long ntiles, F16Ctl* c, Ctl* ctl, uint8_t* labels) {
     extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ int s_vx[16], s_vy[16], s_live[16];
-    __shared__ float4 s_edge[20];   // the 16 edges' functions, then the quadrilateral's
+    __shared__ F16Poly s_p;
     __shared__ Octagon s_o;
     __shared__ unsigned s_cnt[4];
     __shared__ unsigned long long s_bar[kF16Threads / 32][kStages];
     if (*(volatile int*)&c->status != CH_OK || !c->ready) return;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    if (t < 16) { s_vx[t] = c->vx[t]; s_vy[t] = c->vy[t]; s_live[t] = c->live[t]; }
-    if (t < 4) s_cnt[t] = 0u;
-    if (t < 20) {
-        const int a = t < 16 ? t : 4 * (t - 16), b = (t < 16 ? t + 1 : a + 4) & 15;
-        const Edge e = make_edge(c->vx[a], c->vy[a], c->vx[b], c->vy[b]);
-        s_edge[t] = make_float4(e.A, e.B, e.C, 0.0f);
+    if (t < 16) {
+        s_p.vx[t] = c->vx[t];
+        s_p.vy[t] = c->vy[t];
     }
+    if (t < 4) s_cnt[t] = 0u;
     copy_octagon(&s_o, &c->oct);
     __syncthreads();
-    const bool none = c->none != 0;
+    s_p.set(t);
+    __syncthreads();
+    const bool none = s_p.none != 0;
     const long long gwarp = ((long long)blockIdx.x * blockDim.x + t) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     unsigned cnt[4] = {0u, 0u, 0u, 0u};
@@ -399,8 +445,8 @@ __global__ void __launch_bounds__(kF16Threads) f16_labels(const float* __restric
         const int X = __float2int_rn(x), Y = __float2int_rn(y);
         int lab = -1;
         if (!in_inner_strict(s_o, X, Y)) {
-            lab = f16_label_float(x, y, s_edge, none);
-            if (lab == kF16Undecided) lab = f16_label_exact(X, Y, s_vx, s_vy, s_live, none);
+            lab = f16_label_float(x, y, s_p.e, none);
+            if (lab == kF16Undecided) lab = f16_label_near(x, y, s_p);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) cnt[q] += lab == q;
@@ -450,10 +496,10 @@ __global__ void __launch_bounds__(kF16Threads) f16_labels(const float* __restric
     if (t < 4 && s_cnt[t]) atomicAdd(&c->counts[t], s_cnt[t]);
 }
 
-// Inputs of at most kPointsMax points: a point per thread, per-point maxima and
-// exact labels.  Warp tiles of 512 points leave most of the chip idle there (a
-// call on 9000 ring points: 60 us by tiles, 29 by points, the host's part
-// included; 2 M uniform points 46 and 43, 4 M 52 and 70).
+// Inputs of at most kF16PointsMax points: a point per thread, per-point maxima and
+// labels.  Warp tiles of 512 points leave most of the chip idle there (uniform
+// points: 37 us a call by points at 1 M, 45 and 50 by tiles at 2 M, 55 and 55 at
+// 3 M, 72 and 63 at 5 M; of a ring 48 and 58, 58 and 69, 78 and 83).
 __global__ void __launch_bounds__(kF16Threads) f16_extremes_points(const float2* __restrict__ pts, long long n,
                                                             F16Ctl* c) {
     __shared__ unsigned long long s_m[kF16Threads / 32][16];
@@ -503,52 +549,27 @@ __global__ void __launch_bounds__(kF16Threads) f16_extremes_points(const float2*
 
 __global__ void __launch_bounds__(kF16Threads) f16_labels_points(const float2* __restrict__ pts, long long n, F16Ctl* c,
                                                           uint8_t* labels) {
-    __shared__ int s_vx[16], s_vy[16], s_live[16];
-    __shared__ int s_none;
+    __shared__ F16Poly s_p;
     __shared__ unsigned s_cnt[4];
     if (*(volatile int*)&c->status != CH_OK) return;   // set before this launch: the same for every block
     const int t = threadIdx.x;
     if (t < 16) {
         const unsigned idx = 0xFFFFFFFFu - (unsigned)(c->packed[t] & 0xFFFFFFFFull);
         const float2 v = (long long)idx < n ? pts[idx] : make_float2(0.0f, 0.0f);
-        s_vx[t] = __float2int_rz(v.x);
-        s_vy[t] = __float2int_rz(v.y);
+        s_p.vx[t] = __float2int_rz(v.x);
+        s_p.vy[t] = __float2int_rz(v.y);
     }
     if (t < 4) s_cnt[t] = 0u;
     __syncthreads();
-    if (t < 16) {
-        const int j = (t + 1) & 15;
-        s_live[t] = (s_vx[t] != s_vx[j] || s_vy[t] != s_vy[j]) ? 1 : 0;
-    }
-    if (t == 0) {
-        long long a2 = 0;
-        for (int k = 0; k < 16; ++k) {
-            const int j = (k + 1) & 15;
-            a2 += (long long)s_vx[k] * s_vy[j] - (long long)s_vx[j] * s_vy[k];
-        }
-        s_none = a2 == 0 ? 1 : 0;
-    }
+    s_p.set(t);
     __syncthreads();
-    const bool none = s_none != 0;
+    const bool none = s_p.none != 0;
     unsigned cnt[4] = {0u, 0u, 0u, 0u};
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + t; i < n; i += stride) {
         const float2 p = __ldcs(pts + i);
-        const int X = __float2int_rz(p.x), Y = __float2int_rz(p.y);
-        bool inside = !none;
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const int j = (k + 1) & 15;
-            if (s_live[k] && orient64(s_vx[k], s_vy[k], s_vx[j], s_vy[j], X, Y) <= 0) inside = false;
-        }
-        int r = -1;
-        if (!inside) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {   // W->S, S->E, E->N, N->W
-                const int a = 4 * q, b = (4 * q + 4) & 15;
-                if (r < 0 && orient64(s_vx[a], s_vy[a], s_vx[b], s_vy[b], X, Y) < 0) r = q;
-            }
-        }
+        int r = f16_label_float(p.x, p.y, s_p.e, none);
+        if (r == kF16Undecided) r = f16_label_near(p.x, p.y, s_p);
         if (labels) labels[i] = (uint8_t)(r + 1);
         if (r >= 0) cnt[r]++;
     }
@@ -600,7 +621,7 @@ extern "C" int ch_filter16(const float* pts, int64_t n, int32_t* out_ext16, uint
     const long long want = std::max(1ll, (ntiles + kF16Threads / 32 - 1) / (kF16Threads / 32));
     const bool lab = out_labels || out_counts4;
     f16_init<<<1, 32, 0, s>>>(c, ctl);
-    if (n <= kPointsMax) {
+    if (n <= kF16PointsMax) {
         const float2* p2 = reinterpret_cast<const float2*>(pts);
         const int grid = (int)std::min<long long>((n + kF16Threads - 1) / kF16Threads, 4ll * sms);
         {
