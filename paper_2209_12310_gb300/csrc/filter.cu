@@ -1058,7 +1058,7 @@ __global__ void __launch_bounds__(256) labels_kernel(const float* __restrict__ p
     __shared__ Octagon s_o;
     __shared__ unsigned s_cnt[4];
     __shared__ unsigned long long s_bar[8][kStages];
-    if (read_status(ctl) != CH_OK) return;
+    if (__syncthreads_or(read_status(ctl) != CH_OK)) return;   // (a wait below may set it meanwhile)
     copy_octagon(&s_o, &ctl->oct);
     if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0u;
     __syncthreads();

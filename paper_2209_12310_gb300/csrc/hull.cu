@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kChainThreads) sort_kernel(Ctl* ctl, uint32_t*
     __shared__ int s_mv[kChainThreads / 2][3];   // per pair: destination, source, count
 
     if (*(volatile int*)&ctl->done) return;
-    bool go = read_status(ctl) == CH_OK;
+    bool go = !__syncthreads_or(read_status(ctl) != CH_OK);   // (a wait below may set it meanwhile)
     if (go) {
         if (*(volatile int*)&ctl->bk_state != 2) return;
         SortSmem& sm = *reinterpret_cast<SortSmem*>(smem);
