@@ -191,6 +191,7 @@ struct Server {
     std::mutex mu;
     std::condition_variable cv;
     std::deque<Req*> queue;
+    std::atomic<size_t> waiting{0};   // queue.size(), for the engine thread to look at without the lock
     std::unordered_map<uint64_t, Req*> reqs;
     uint64_t next_ticket = 1;
     std::atomic<bool> stop{false};
@@ -308,7 +309,7 @@ bool Server::retire(Slot& sl) {
 }
 
 bool Server::launch(Slot& sl) {
-    if (sl.busy) return false;
+    if (sl.busy || waiting.load() == 0) return false;
     std::vector<Req*> batch;
     int64_t points = 0;
     size_t off = 0, bytes = 0;
@@ -338,6 +339,7 @@ bool Server::launch(Slot& sl) {
             points -= r->n;
             queue.push_front(r);
         }
+        waiting.store(queue.size());
         if (batch.empty()) return false;
         for (Req* r : batch) r->state = 1;
     }
@@ -400,9 +402,11 @@ bool Server::launch(Slot& sl) {
 
 void Server::run() {
     cudaSetDevice(device);
-    // While a batch is in flight, and for at most kSpinSeconds since anything
-    // happened, the thread looks again at once: a timed wait of 50 us lasts
-    // about twice that with the kernel's timer slack, a tenth of a small burst.
+    // While a batch is in flight and something happened in the last kSpinSeconds
+    // (2 ms: a small burst's batches), the thread looks again at once, which keeps
+    // a core busy; longer batches and an idle server are looked at by timed waits,
+    // of 50 us and the kernel's timer slack (about as much again, a tenth of a
+    // small burst).
     double last = 0;
     while (!stop.load()) {
         bool progress = false, busy = false;
@@ -493,6 +497,7 @@ int ch_submit(void* srv, const float* pts_host, int64_t n, uint64_t* ticket) {
     if (S->t_first == 0) S->t_first = r->t_submit;
     S->reqs[r->ticket] = r;
     S->queue.push_back(r);
+    S->waiting.store(S->queue.size());
     *ticket = r->ticket;
     S->cv.notify_one();
     return CH_OK;
