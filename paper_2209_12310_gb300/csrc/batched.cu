@@ -134,7 +134,6 @@ __global__ void __launch_bounds__(256) bt_init(BArgs a) {
         c->count = 8u;
         c->done = 0;
         c->bk_state = 0;
-        c->star_ok = 0;
         c->skip = 0;
         c->star_k = 0;
         c->star_cx = 0;
@@ -544,7 +543,6 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
         if (lane == 0 && out) atomicAdd(&s_out, out);
         __syncthreads();
         if (tid == 0 && s_out * (sure ? 16u : 4u) > (unsigned)kBDenseSample) {
-            c->star_ok = 1;
             c->star_cx = (s_vx[W] + s_vx[E]) / 2;   // the centre of the extremes' box
             c->star_cy = (s_vy[S] + s_vy[N]) / 2;
             a.star_list[atomicAdd(&a.star_ctr[0], 1u)] = i;
@@ -1007,7 +1005,7 @@ __global__ void __launch_bounds__(kBStarBinThreads) bt_star_bin(BArgs a) {
 // Star polygons of the dense sets (bt_octagon's list), one block per set,
 // persistent over the list: the polygon of the set's bins (star_finish,
 // star.cuh: vertices re-read from the input by index, checked exactly) is
-// built in shared memory and copied to the set's slot, for bt_filter.  A
+// built in shared memory and copied to the set's slot, for bt_dense.  A
 // set without one keeps star_k = 0 and is filtered by its octagon alone.
 constexpr int kBStarThreads = 512;
 constexpr size_t kBStarAOff = (sizeof(StarPoly) + 15) / 16 * 16;
@@ -1657,7 +1655,7 @@ __global__ void __launch_bounds__(T) bt_queue_chain(BArgs a) {
     extern __shared__ __align__(16) char dyn[];
     Q& q = *reinterpret_cast<Q*>(dyn);
     __shared__ int s_item, s_n, s_last;
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x;
     // the small shape's blocks start beside the large one's and read nothing of theirs
     if (kLarge) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned items = 4u * a.star_ctr[kLarge ? 10 : 9];

@@ -149,7 +149,6 @@ struct Ctl {
     unsigned int epoch;                 // onesweep status epoch (incremented per call)
     int mode;                           // 0: fused single pass, 1: two streaming passes
     int done;                           // the hull has been written by a small-path block
-    int records_ready;                  // sort records complete before the re-classify stage
     unsigned int blocks_done[4];        // last-arriver counters (sample, main, post, a batched set's queues)
     unsigned int claimed[kPhases];      // items of a phase that blocks have taken,
     unsigned int finished[kPhases];     // and finished
@@ -168,7 +167,6 @@ struct Ctl {
     unsigned int q_tile[5];             // path tiles: tiles of queue r are [q_tile[r], q_tile[r + 1])
     int samp_dense;                     // dense data (oct_s: an octagon of input points): dense_kernel's
     int oct_ready;                      // the octagon of the true extremes and the end-point records stand
-    int star_ok;                        // batched: the set is listed for a star polygon
     int skip;                           // batched: nothing for bt_filter (empty, failed, classified, or bt_dense's)
     int star_k;                         // the polygon's vertices, the dropped ones included
     int star_edges;                     // dense_kernel: the polygon's vertices in use (0: none)

@@ -123,19 +123,6 @@ static __device__ __noinline__ int classify_paper_slow(float x, float y, const O
     return -1;
 }
 
-// Strictly outside the closed octagon (the survivor test against a sample
-// octagon; no queue needed).  Degenerate octagons keep everything.
-static __device__ __noinline__ bool outside_closed_slow(float x, float y, const Octagon* op) {
-    const Octagon& o = *op;
-    if (o.discard_none) return true;
-    float m = kHugePositive;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) m = fminf(m, edge_float(o.oct[k], x, y));
-    if (m > kEdgeTol) return false;
-    if (m < -kEdgeTol) return true;
-    return !in_closed_octagon_exact(o, (long long)x, (long long)y);
-}
-
 // Inner region I(t): the 8-direction bounds of the octagon's own vertices,
 // shrunk about their centre by t/1024.  Its candidate vertices (the
 // intersections of consecutive bounding lines, integer points) span a polygon

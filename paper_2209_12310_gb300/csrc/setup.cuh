@@ -35,7 +35,6 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
         ctl->epoch += 1u;
         ctl->mode = mode;
         ctl->done = 0;
-        ctl->records_ready = 0;
         ctl->bk_state = 0;
         ctl->path = kPathNone;
         ctl->beat = 0u;
@@ -43,7 +42,6 @@ __device__ __forceinline__ void reset_ctl(Ctl* ctl, int mode) {
         ctl->roots_done = 0u;
         ctl->samp_dense = 0;
         ctl->oct_ready = 0;
-        ctl->star_ok = 0;
         ctl->star_k = 0;
         ctl->star_final = 0;
     }
