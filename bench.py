@@ -29,6 +29,7 @@ sys.path.insert(0, ROOT)
 
 L2_BYTES = 129 * 1024 * 1024
 HBM_NOMINAL_GBS = 7900.0   # GB300 HBM3e, nominal (context beside the measured copy bandwidth)
+TWO_PASS_MAX = 1 << 21     # points up to which the main pass comes first (kTwoPassMax, ch_internal.cuh)
 # One metric name for both arms (GPU library and the oracle's reference arm),
 # so that their lines can be divided.
 METRIC = "points/s (filter+hull, device-timed)"
@@ -130,8 +131,10 @@ def algorithmic_bytes(n, counters):
     raw, m, two_pass = counters["raw"], counters["records"], counters["two_pass"]
     out = {"main_filter": 8.0 * n + 12.0 * raw,
            "post": (8.0 * n if two_pass else 12.0 * raw) + 12.0 * m}
-    if counters.get("star_vertices"):   # dense data: the dense pass reads the points, the main pass nothing
+    if counters.get("star_vertices"):   # dense data: the dense pass reads the points and leaves the survivors
         out = {"dense_filter": 8.0 * n + 12.0 * raw, "post": 12.0 * raw + 12.0 * m}
+        if n <= TWO_PASS_MAX:           # its verdict is the main pass's, which has read them for the extremes
+            out["main_filter"] = 8.0 * n
     if counters["stage"] >= 1:
         out["large"] = 12.0 * m
         out.update({"bk_hist": 4.0 * m, "bk_part1": 24.0 * m, "bk_part2": 24.0 * m, "bk_hull": 12.0 * m})
