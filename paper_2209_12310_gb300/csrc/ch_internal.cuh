@@ -150,16 +150,9 @@ struct Ctl {
     int mode;                           // 0: fused single pass, 1: two streaming passes
     int done;                           // the hull has been written by a small-path block
     unsigned int blocks_done[4];        // last-arriver counters (sample, main, post, a batched set's queues)
-    unsigned int claimed[kPhases];      // items of a phase that blocks have taken,
-    unsigned int finished[kPhases];     // and finished
-    unsigned int beat;                  // progress within long items
     unsigned int digit_hist[kSortPasses][kDigits];   // sort path only (sort_kernel)
     unsigned int rec_q[4];              // records per queue
     unsigned int reg_end[4];            // chain length of queue r (large_kernel, bt_queue_chain)
-    unsigned int joins_done;            // large_kernel: queues whose chain stands
-    unsigned int join_n[kJoinRounds + 1][4];   // large_kernel: points of each queue's tile chains,
-                                        // and after each round that joins them
-    unsigned int roots_done;            // sort_kernel: queue roots of the merge tree
     unsigned int counts4[4];            // survivors per queue (ch_filter)
     unsigned long long line_ep[8];      // end points of survivors on the 4 axis support lines
     int bk_state;                       // large-survivor path: 0 unused, 1 queues / tiles / buckets, 2 full sort
@@ -174,6 +167,13 @@ struct Ctl {
     int star_cx, star_cy;               // its centre (vertices are stored relative to it)
     Octagon oct;                        // octagon of the true extremes
     Octagon oct_s;                      // octagon of a sample's extremes
+    unsigned int claimed[kPhases];      // items of a phase that blocks have taken,
+    unsigned int finished[kPhases];     // and finished
+    unsigned int beat;                  // progress within long items
+    unsigned int joins_done;            // large_kernel: queues whose chain stands
+    unsigned int join_n[kJoinRounds + 1][4];   // large_kernel: points of each queue's tile chains,
+                                        // and after each round that joins them
+    unsigned int roots_done;            // sort_kernel: queue roots of the merge tree
 #if defined(CH_TRACE) || defined(CH_TIMELINE)
     unsigned long long tl[24][2];       // debug builds: first start / last end per phase (%globaltimer)
 #endif
@@ -278,7 +278,7 @@ __device__ __forceinline__ bool spin_give_up(unsigned& spins, Ctl* ctl) {
 // grid is resident.  (Cooperative launches with grid barriers instead started
 // only once every SM was free, so that one block of another stream's kernel
 // held up the whole call, and a kernel that waited for the call's result never
-// saw it.)  All three: whole block.
+// saw it.)  All four: whole block.
 __device__ __forceinline__ unsigned claim_item(Ctl* ctl, int phase) {
     __shared__ unsigned s_item;
     __syncthreads();
@@ -301,13 +301,34 @@ __device__ __forceinline__ bool finish_items(Ctl* ctl, int phase, unsigned n, un
     return s_end != 0;
 }
 
-// Bounded: false when the wait gave up (status CH_ETIMEOUT), after kSpinLimit
-// polls in which no item of the phase was taken or finished and no block
-// reported progress within one (ctl->beat).
-__device__ __forceinline__ bool wait_phase(Ctl* ctl, int phase, unsigned items) {
-    __shared__ int s_ok;
+// The same for one item, and the claim of the phase's next one, whose latency is
+// the same (one after the other on both sides of every phase: 4 us more on a dense
+// hull's three phases).  *last: as finish_items returns.
+__device__ __forceinline__ unsigned finish_and_claim(Ctl* ctl, int phase, unsigned items, bool* last = nullptr) {
+    __shared__ unsigned s_next, s_end;
+    __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
+        const unsigned before = atomicAdd(&ctl->finished[phase], 1u);
+        s_next = atomicAdd(&ctl->claimed[phase], 1u);
+        s_end = before + 1u == items;
+        if (last && s_end) __threadfence();
+    }
+    __syncthreads();
+    if (last) *last = s_end != 0u;
+    return s_next;
+}
+
+// Bounded: false when the wait gave up (status CH_ETIMEOUT), after kSpinLimit
+// polls in which no item of the phase was taken or finished and no block
+// reported progress within one (ctl->beat).  Meanwhile claims an item of phase
+// next, to be worked on after the wait.
+__device__ __forceinline__ bool wait_phase(Ctl* ctl, int phase, unsigned items, int next = -1, unsigned* item = nullptr) {
+    __shared__ int s_ok;
+    __shared__ unsigned s_claim;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (item) s_claim = atomicAdd(&ctl->claimed[next], 1u);
         volatile unsigned *claimed = &ctl->claimed[phase], *finished = &ctl->finished[phase], *beat = &ctl->beat;
         unsigned spins = 0u, seen = 0u;
         s_ok = 1;
@@ -325,6 +346,7 @@ __device__ __forceinline__ bool wait_phase(Ctl* ctl, int phase, unsigned items) 
         __threadfence();
     }
     __syncthreads();
+    if (item) *item = s_claim;
     return s_ok != 0;
 }
 

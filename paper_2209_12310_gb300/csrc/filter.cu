@@ -801,6 +801,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
     const int cx = (os.vx[W] + os.vx[E]) / 2, cy = (os.vy[S] + os.vy[N]) / 2;
     const float4* p4 = reinterpret_cast<const float4*>(pts + 2 * head);
     unsigned long long* merged = bins + (size_t)gridDim.x * kStarBins;
+    unsigned item;   // of the phase at hand
     {   // 1. bins
         if (tid < 4) {
             s_in[tid] = os.in_lo[tid];
@@ -813,7 +814,9 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
         }
         unsigned long long* mine = reinterpret_cast<unsigned long long*>(dsm);
         const long long nt = min(ntiles, (long long)gridDim.x * kWarps);
-        for (unsigned g; (g = claim_item(ctl, kDenseBins)) < gridDim.x;) {   // gridDim.x shares
+        item = claim_item(ctl, kDenseBins);
+        while (item < gridDim.x) {   // gridDim.x shares
+            const unsigned g = item;
             for (int b = tid; b < kStarBins; b += kDenseThreads) mine[b] = 0ull;
             __syncthreads();
             const long long k = g + (long long)gridDim.x * warp;
@@ -821,10 +824,10 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
                 star_tile_pass(p4, ((2 * k + 1) * ntiles) / (2 * nt), head, s_in, s_edge, cx, cy, mine, l2_evict_first());
             __syncthreads();
             for (int b = tid; b < kStarBins; b += kDenseThreads) bins[(size_t)g * kStarBins + b] = mine[b];
-            finish_items(ctl, kDenseBins, 1u, gridDim.x);
+            item = finish_and_claim(ctl, kDenseBins, gridDim.x);
         }
         CH_TL(ctl, 7, 1);
-        if (!wait_phase(ctl, kDenseBins, gridDim.x)) return;
+        if (!wait_phase(ctl, kDenseBins, gridDim.x, kDenseMerge, &item)) return;
     }
     auto make_polygon = [&]() {
         StarPoly& M = *reinterpret_cast<StarPoly*>(dsm);
@@ -865,8 +868,8 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
         constexpr unsigned kItems = kStarBins / kSlots;
         unsigned long long* part = reinterpret_cast<unsigned long long*>(dsm);
         const int slot = tid % kSlots, grp = tid / kSlots;
-        for (unsigned it; (it = claim_item(ctl, kDenseMerge)) < kItems;) {
-            const int b0 = (int)it * kSlots;
+        while (item < kItems) {
+            const int b0 = (int)item * kSlots;
             unsigned long long key = 0ull;
             for (int g = grp; g < (int)gridDim.x; g += kGroups) {
                 const unsigned long long x = __ldcg(bins + (size_t)g * kStarBins + b0 + slot);
@@ -879,21 +882,23 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
                 for (int g = 1; g < kGroups; ++g) key = part[g * kSlots + tid] > key ? part[g * kSlots + tid] : key;
                 merged[b0 + tid] = star_vertex(key, star_point(key, pts, n), b0 + tid, cx, cy);
             }
-            if (!finish_items(ctl, kDenseMerge, 1u, kItems)) continue;
+            bool last;
+            item = finish_and_claim(ctl, kDenseMerge, kItems, &last);
+            if (!last) continue;
             CH_TL(ctl, 14, 1);
             make_polygon();
             finish_items(ctl, kDensePoly, 1u, 1u);
         }
     }
-    if (!wait_phase(ctl, kDensePoly, 1u)) return;
+    if (!wait_phase(ctl, kDensePoly, 1u, kDenseRadius, &item)) return;
     const int K = *(volatile int*)&ctl->star_edges;   // the same for all from here on
     if (!K) return;
     {   // kStarWindow threads per bin, an edge of its window each
         constexpr int kSlots = kDenseThreads / kStarWindow;
         constexpr unsigned kItems = kStarBins / kSlots;
         const int k = tid % kStarWindow;
-        for (unsigned it; (it = claim_item(ctl, kDenseRadius)) < kItems;) {
-            const int b = (int)it * kSlots + tid / kStarWindow;
+        while (item < kItems) {
+            const int b = (int)item * kSlots + tid / kStarWindow;
             int first, count;
             star_window(poly->tbl, K, b, first, count);
             unsigned r = 0xFFFFFFFFu;
@@ -904,7 +909,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) dense_kernel(const float* __
 #pragma unroll
             for (int d = kStarWindow / 2; d; d >>= 1) r = min(r, __shfl_xor_sync(0xFFFFFFFFu, r, d));
             if (k == 0) poly->thr[b] = star_threshold(count <= kStarWindow ? r : 0u);
-            finish_items(ctl, kDenseRadius, 1u, kItems);
+            item = finish_and_claim(ctl, kDenseRadius, kItems);
         }
         if (!wait_phase(ctl, kDenseRadius, kItems)) return;
     }

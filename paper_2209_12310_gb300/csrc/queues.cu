@@ -87,13 +87,14 @@ struct TileHistSmem {
 
 __device__ bool tile_hist(const LargeArgs& a, TileHistSmem& sm, const QMap& m) {
     const int tid = threadIdx.x;
-    for (int g = tid; g < kPtGroups; g += kLargeThreads) sm.h[g] = 0u;
     const unsigned n = a.ctl->count;
     const unsigned chunk = min(64u, (n - 1u) / (gridDim.x * kLargeThreads) + 1u) * kLargeThreads;
     const unsigned chunks = (n - 1u) / chunk + 1u;
     constexpr int kU = 4;
-    unsigned taken = 0u;
-    for (unsigned c; (c = claim_item(a.ctl, kLargeHist)) < chunks; ++taken) {
+    bool last = false;
+    for (unsigned c = claim_item(a.ctl, kLargeHist); c < chunks; c = finish_and_claim(a.ctl, kLargeHist, chunks, &last)) {
+        for (int g = tid; g < kPtGroups; g += kLargeThreads) sm.h[g] = 0u;
+        __syncthreads();
         const unsigned end = min(n, (c + 1u) * chunk);
         for (unsigned i0 = c * chunk + tid; i0 < end; i0 += kLargeThreads * kU) {
             uint32_t k[kU];
@@ -104,11 +105,11 @@ __device__ bool tile_hist(const LargeArgs& a, TileHistSmem& sm, const QMap& m) {
             for (int j = 0; j < kU; ++j)
                 if (i0 + j * kLargeThreads < end) atomicAdd(&sm.h[q_group(m, k[j])], 1u);
         }
+        __syncthreads();
+        for (int g = tid; g < kPtGroups; g += kLargeThreads)
+            if (sm.h[g]) atomicAdd(&a.ghist[g], sm.h[g]);
     }
-    if (!taken) return false;
-    for (int g = tid; g < kPtGroups; g += kLargeThreads)   // behind the last claim's barriers
-        if (sm.h[g]) atomicAdd(&a.ghist[g], sm.h[g]);
-    return finish_items(a.ctl, kLargeHist, taken, chunks);
+    return last;
 }
 
 // One block cuts the tiles: gtile maps a group to its tile, tile t's records go
@@ -171,20 +172,20 @@ struct TilePartSmem {
     unsigned short gtile[kPtGroups];
 };
 
-// Returns the number of the phase's items.
-__device__ unsigned tile_part(const LargeArgs& a, TilePartSmem& sm, const QMap& m) {
+// item: claimed already.  Returns the number of the phase's items.
+__device__ unsigned tile_part(const LargeArgs& a, TilePartSmem& sm, const QMap& m, unsigned item) {
     static_assert(kLargeThreads == kPtThreads, "partition block");
     const int tid = threadIdx.x;
     for (int g = tid; g < kPtGroups; g += kPtThreads) sm.gtile[g] = (unsigned short)__ldcg(a.gtile + g);
     const unsigned n = a.ctl->count, nt = *(volatile unsigned*)&a.ctl->q_tile[4];
     const unsigned parts = (n - 1u) / kPtTile + 1u;
-    for (unsigned p; (p = claim_item(a.ctl, kLargePart)) < parts;) {
+    __syncthreads();
+    for (unsigned p = item; p < parts; p = finish_and_claim(a.ctl, kLargePart, parts)) {
         const unsigned i0 = p * kPtTile;
         partition_tile(
             sm.p, a.keys, a.vals, i0, min((unsigned)kPtTile, n - i0), nt,
             [&](uint32_t key) { return (unsigned)sm.gtile[q_group(m, key)]; },
             [&](unsigned g, unsigned cnt) { return atomicAdd(&a.tcur[g], cnt); }, a.kB, a.vB);
-        finish_items(a.ctl, kLargePart, 1u, parts);
     }
     return parts;
 }
@@ -261,12 +262,12 @@ __device__ int tile_read(const LargeArgs& a, QcQueue& q, unsigned beg, unsigned 
     return fill;
 }
 
-__device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
+__device__ void tile_chains(const LargeArgs& a, QcQueue& q, unsigned item) {
     const int tid = threadIdx.x;
     constexpr int T = kLargeThreads, kCap = QcQueue::kCap, kPer = kCap / T;
     static_assert(kCap % T == 0, "carried points per thread");
     const unsigned nt = *(volatile unsigned*)&a.ctl->q_tile[4];
-    for (unsigned t; (t = claim_item(a.ctl, kLargeChains)) < nt;) {
+    for (unsigned t = item; t < nt; t = finish_and_claim(a.ctl, kLargeChains, nt)) {
         const unsigned beg = __ldcg(a.tbeg + t), cnt = __ldcg(a.tcur + t) - beg;
         unsigned long long *src = q.a, *dst = q.b;
         int len = 0;
@@ -338,7 +339,6 @@ __device__ void tile_chains(const LargeArgs& a, QcQueue& q) {
             while (r < 3 && t >= *(volatile unsigned*)&a.ctl->q_tile[r + 1]) ++r;
             atomicAdd(&a.ctl->join_n[0][r], (unsigned)len);
         }
-        finish_items(a.ctl, kLargeChains, 1u, nt);
     }
 }
 
@@ -535,12 +535,15 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_kernel(LargeArgs a) {
             tile_cut(a, h);
             finish_items(ctl, kLargeCut, 1u, 1u);
         }
-        bool go = wait_phase(ctl, kLargeCut, 1u);
+        unsigned item;
+        bool go = wait_phase(ctl, kLargeCut, 1u, kLargePart, &item);
         CH_TL(ctl, 16, 1);
-        if (go) go = wait_phase(ctl, kLargePart, tile_part(a, *reinterpret_cast<TilePartSmem*>(s_dyn), s_m));
+        if (go)
+            go = wait_phase(ctl, kLargePart, tile_part(a, *reinterpret_cast<TilePartSmem*>(s_dyn), s_m, item), kLargeChains,
+                            &item);
         CH_TL(ctl, 17, 1);
         if (go) {
-            tile_chains(a, *reinterpret_cast<QcQueue*>(s_dyn));
+            tile_chains(a, *reinterpret_cast<QcQueue*>(s_dyn), item);
             CH_TL(ctl, 18, 1);
             go = wait_phase(ctl, kLargeChains, *(volatile unsigned*)&ctl->q_tile[4]);
         }
