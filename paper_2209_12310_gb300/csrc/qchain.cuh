@@ -318,14 +318,20 @@ __device__ int qc_sort(Q& q, int n, int lo, int hi) {
         const unsigned long long w = q.b[j];
         const int b = bucket(w);   // cnt[b] is now the end of bucket b
         const int s = b ? (int)q.cnt[b - 1] : 0, e = (int)q.cnt[b];
-        int r = s;
-        unsigned long long first = w;   // of the points of equal (u, v): the one that can be a vertex
+        int r = s, same = 0;   // same: points of equal (u, v), this one among them
         for (int i = s; i < e; ++i) {
             const unsigned long long x = q.b[i];
             r += x < w ? 1 : 0;
-            if (((x ^ w) >> kQcPosBits) == 0ull) first = x < first ? x : first;
+            same += ((x ^ w) >> kQcPosBits) == 0ull ? 1 : 0;
         }
-        if (first != w) atomicMin(&q.si[qc_pos(first)], q.si[qc_pos(w)]);   // it takes the lowest index
+        if (same > 1) {   // the first of them, which can be a vertex, takes the lowest index
+            unsigned long long first = w;
+            for (int i = s; i < e; ++i) {
+                const unsigned long long x = q.b[i];
+                if (((x ^ w) >> kQcPosBits) == 0ull && x < first) first = x;
+            }
+            if (first != w) atomicMin(&q.si[qc_pos(first)], q.si[qc_pos(w)]);
+        }
         q.a[r] = w;
     }
     __syncthreads();
