@@ -70,6 +70,7 @@ constexpr int kBOctThreads = 256;      // threads of bt_octagon: a warp per dire
 // around the centre of the box of the set's extremes, over a sample of
 // kBStarParts evenly spread runs of the set (up to kBStarRun points each).
 constexpr long long kBStarMinPts = 16384;
+constexpr long long kBFewPts = 2048;         // smaller sets are classified where their octagon is made (bt_octagon)
 constexpr long long kBStarSurePts = 32768;   // smaller ones only when much denser (bt_octagon)
 constexpr int kBStarParts = 16;
 constexpr int kBStarRun = 16384;
@@ -549,16 +550,17 @@ __global__ void __launch_bounds__(kBOctThreads) bt_octagon(BArgs a) {
         }
     } else {
         // For the others: more than half outside the inner region (a point per
-        // thread), or a very small set: this block classifies them all.  (At
-        // 1 / 16, 256 sets of 9000 uniform points took 155 us, 136 now; of points in
-        // [0, 50)^2 199 and 124; rings are the same.)
+        // thread; 1 / 16 in a small set), or a very small set: this block classifies
+        // them all.  (At 1 / 16 for all, 256 sets of 9000 uniform points took 155 us,
+        // 135 now; of points in [0, 50)^2 199 and 124; rings are the same.  At 1 / 2
+        // for all, 20 sets of up to 1355 points took 122 us, 114 now.)
         const bool tiny = ni <= kBOctThreads;
         bool out = tiny;
         if (!tiny) {
             const float2 p = __ldg(reinterpret_cast<const float2*>(a.pts) + base + tid * (ni / kBOctThreads));
             out = !in_inner(s_o, __float2int_rn(p.x), __float2int_rn(p.y));
         }
-        if (__syncthreads_count(out) * 2 > kBOctThreads) bt_classify_set(a, i, s_o, base, (int)ni, rb);
+        if (__syncthreads_count(out) * (ni <= kBFewPts ? 16 : 2) > kBOctThreads) bt_classify_set(a, i, s_o, base, (int)ni, rb);
     }
 }
 
@@ -1491,6 +1493,8 @@ __global__ void __launch_bounds__(kBStarThreads, 1) bt_star_refine(BArgs a) {
 constexpr int kBSmallRec = 2048;        // records of a small set
 constexpr int kBSmallVert = 256;        // quickhull vertices of a small set
 constexpr int kBSmallThreads = 256;
+constexpr int kBDenseRec = 256;         // records of a dense set that try the quickhull rounds, in a batch of
+constexpr int kBFewSets = 608;          // at most this many sets (four blocks per SM)
 using QhSmall = QhSmemT<kBSmallRec, kBSmallVert>;
 
 // bt_queue_chain's two shapes: a queue of at most kBQSmall records by 256
@@ -1559,10 +1563,22 @@ __global__ void __launch_bounds__(kBSmallThreads) bt_hull_small(BArgs a) {
         a.vals[rb + s_lpos[tid]] = s_lval[tid];
         atomicAdd(&c->counts4[s_lkey[tid] >> kKeyBits], 1u);
     }
-    if (total > (unsigned)kBSmallRec) {
-        // Records near the hull (a star polygon left them, or more than a quarter
-        // of the points survived the octagon) are mostly vertices: queue by queue.
-        const bool dense = c->star_k > 0 || 4ll * total > ni;
+    // Records near the hull (a star polygon left them, or more than a quarter
+    // of the points survived the octagon) are mostly vertices: queue by queue.
+    // Many sets try the rounds first, which leave early on vertices; while every
+    // set has a block of its own at once, that would only delay the queues' kernel
+    // (39 sets of up to 594,402 points with 2 % distortion: 251 us, 288 with), but
+    // for copies of a few points, which end the rounds (256 sets of 1000 points, 60 %
+    // copies: 156 us queue by queue, 112).
+    const bool dense = c->star_k > 0 || 4ll * total > ni;
+    bool rounds = total <= (unsigned)kBSmallRec;
+    if (rounds && dense && total > (unsigned)kBDenseRec && a.k <= kBFewSets) {
+        int same = 0;
+        if (tid < 32)
+            same = __popc(__match_any_sync(0xFFFFFFFFu, __ldcg(a.keys + rb + (size_t)tid * total / 32)));
+        rounds = __syncthreads_or(same >= 8);
+    }
+    if (!rounds) {
         __syncthreads();   // the queue counts are complete
         if (tid == 0) {
             if (!dense && total <= (unsigned)kMidCap) a.hull_list[atomicAdd(&a.star_ctr[5], 1u)] = i;
