@@ -541,13 +541,14 @@ def run_filters(ch, torch, args, pts, n, sp, peak):
     """The filter on its own (labels and queue sizes) with the octagon
     (ch_filter) and with the 16-direction polygon (ch_filter16), on the
     resident input: device time per call, points kept, and the HBM fraction
-    of each pass (8 bytes a point read; the pass that labels also writes 1:
-    ch_filter's only pass over a large input, the others' second)."""
+    of each pass (8 bytes a point read; a pass that labels also writes 1:
+    the others' second; ch_filter reads a large input once and its second
+    kernel only writes)."""
     labels = torch.empty(max(n, 1), dtype=torch.uint8, device="cuda")
     counts = torch.empty(4, dtype=torch.int64, device="cuda")
     ext = torch.empty(16, dtype=torch.int32, device="cuda")
     out = {}
-    for name, fn, passes in (("octagon", ch.ch_filter, {"main_filter": 9.0}),
+    for name, fn, passes in (("octagon", ch.ch_filter, {"main_filter": 8.0, "labels": 1.0}),
                              ("octagon, two-kernel Manhattan extremes", ch.ch_filter_manhattan,
                               {"manhattan_axis": 8.0, "manhattan_corner": 8.0, "labels": 9.0}),
                              ("16-gon", ch.ch_filter16, {"filter16_extremes": 8.0, "filter16_labels": 9.0})):
