@@ -73,9 +73,10 @@ typedef enum {
  *            device wait timed out (CH_ETIMEOUT).
  * Returns CH_OK on enqueue.  On sparse data (few points outside the octagon)
  * the points are streamed once (8 bytes per point): the extremes and the
- * filter share one pass.  When most points survive that pass's filter (points
- * near a circle, Table V) a second streaming pass classifies every point.  The
- * hull stage touches only the survivors.
+ * filter share one pass (inputs of at most 2^21 points: two, the second from
+ * L2).  Dense data (points near a circle, Table V, where most points survive the
+ * octagon) are streamed once through a star polygon of thousands of their own
+ * points instead.  The hull stage touches only the survivors.
  */
 int ch_hull(const float* pts, int64_t n, int32_t* out_idx, int64_t* out_n, void* stream);
 
@@ -151,6 +152,7 @@ int ch_batched_config(int64_t total_points, int32_t k, int32_t* threads, int32_t
  *                point is strictly inside the octagon W..NW (or in no queue),
  *                else its queue 1..4: 1 = strictly right of W->S, 2 = right of
  *                S->E, 3 = right of E->N, 4 = right of N->W (first match).
+ *                Not written on a data error.
  *   out_counts4  device int64[4] or NULL: number of points in each queue, or
  *                all four set to a negative ch_status on a data error.
  */
@@ -253,7 +255,7 @@ int ch_reserve(int64_t n, int32_t k, void* stream);
  *           included): the survivors of the filter,
  *   out[2]  0 when the fused streaming pass did the extremes and the octagon
  *           filter; 1 when a second pass did the filter (inputs of at most
- *           2^22 points, and dense data without a star polygon) or a star
+ *           2^21 points, and dense data without a star polygon) or a star
  *           polygon did (out[5]),
  *   out[3]  hull stage: 0 finished by one block (few records), 1 chains queue
  *           by queue or by tiles of a queue, 2 the radix sort,

@@ -126,16 +126,14 @@ __device__ __forceinline__ void flush_queue_counts(QueueTally& tally, Ctl* ctl) 
 
 // The block that finished last: support-line records, then the hull of few
 // records (at most kMidCap: quickhull rounds, else the sort-based mid_hull), or
-// the path of the large-survivor part.  On dense data (an earlier pass's
-// verdict, or more than a quarter of the points kept) the records are near the hull, mostly
-// vertices, and past kNearHullRec of them they would outgrow
-// the quickhull rounds' vertex capacity: the queues then, a block each (one
-// million points of a ring: 27,265 records, 13,024 vertices: large_kernel takes
-// the place of a partition into buckets, a warp's quickhull per bucket and a
-// radix sort when their chains overflow).  The sort takes what neither a
-// block nor the tiles are for: a queue too large for a block among few
-// records in all.  Every other record is already in keys/vals and in the
-// per-queue counts.
+// the path of the large-survivor part.  On dense data (an earlier pass's verdict,
+// or more than a quarter of the points kept) the records are near the hull, mostly
+// vertices, and past kNearHullRec of them the rounds take longer than the queues,
+// a block each: calls on 300 and 700 points of a ring 51 and 78 us by the rounds,
+// 35 and 36 by the queues (with 60 % copies of a vertex 26 and 27, 26 and 49; the
+// line lies between).  The sort takes what neither a block nor the tiles are for: a
+// queue too large for a block among few records in all.  Every other record is
+// already in keys/vals and in the per-queue counts.
 constexpr unsigned kNearHullRec = 512;
 
 __device__ void post_last_block(const float* __restrict__ pts, long long n, Ctl* ctl, const Octagon& o,

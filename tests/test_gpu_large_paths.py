@@ -3,6 +3,7 @@ the counters that name it and bit-exact with the oracle: circles without a
 width, whose queues' tile chains fit one block or are joined in rounds, a tile
 whose own chain goes to the sort, and records crowded in one range of u."""
 import math
+import time
 
 import numpy as np
 import pytest
@@ -151,3 +152,39 @@ def test_copies_of_every_vertex(lib, m, copies):
     sets = lib.hull_batched(torch.cat([d, d.flip(0), d[:1000]]), off)
     np.testing.assert_array_equal(sets[0].cpu().numpy(), want)
     np.testing.assert_array_equal(sets[1].cpu().numpy(), oracle.hull(np.ascontiguousarray(pts[::-1])))
+
+
+LEFT_TO_THE_SINGLE_HULL = 2   # ch_batched_counters' stage
+
+
+def test_batched_sets_left_to_the_single_hull(lib):
+    """Circles of more than 10,240 records a queue, whose bucket chains overflow,
+    beside sets that the batch finishes itself."""
+    sets = [_circle(n, n) for n in (120_000, 3000, 250_000, 60_000)]
+    off = np.zeros(len(sets) + 1, np.int64)
+    off[1:] = np.cumsum([s.shape[0] for s in sets])
+    got = lib.hull_batched(torch.from_numpy(np.concatenate(sets)).cuda(), off)
+    stages = [c["stage"] for c in lib.ch_batched_counters(len(sets), torch.cuda.current_stream().cuda_stream)]
+    assert stages[0] == stages[2] == LEFT_TO_THE_SINGLE_HULL and stages[1] != LEFT_TO_THE_SINGLE_HULL
+    for i, s in enumerate(sets):
+        np.testing.assert_array_equal(got[i].cpu().numpy(), oracle.hull(s), err_msg=str(i))
+
+
+def test_served_request_left_to_the_single_hull(lib):
+    reqs = [_circle(120_000, 1), _circle(5000, 2), _circle(200_000, 3)]
+    srv = lib.ch_server_create(2 << 30, 0)
+    try:
+        tickets = [lib.ch_submit(srv, p.ctypes.data, p.shape[0])[1] for p in reqs]
+        left, end = set(range(len(reqs))), time.time() + 60.0
+        while left and time.time() < end:
+            for i in list(left):
+                buf = np.empty(reqs[i].shape[0], np.int32)
+                status, h = lib.ch_poll(srv, tickets[i], buf.ctypes.data, buf.size)
+                if status != lib.CH_PENDING:
+                    assert status == lib.CH_OK, lib.ch_strerror(status)
+                    np.testing.assert_array_equal(buf[:h], oracle.hull(reqs[i]), err_msg=str(i))
+                    left.discard(i)
+        assert not left
+        assert sum(batch[7] for batch in lib.ch_server_trace(srv)) == 2   # sets redone
+    finally:
+        lib.ch_server_destroy(srv)
